@@ -324,12 +324,29 @@ static int qkv_project(const a3_handle* h, int layer, const bf16* a, const int32
   return A3_OK;
 }
 
+// C += A B^T, then (next_gain given) a_out = RMSNorm(C) * next_gain.  Few rows: the GEMM's k-slices are added by the
+// norm's kernel; otherwise the GEMM updates C itself and the norm follows.
+static int residual_then_norm(const a3_handle* h, const GemmArgs& g, const LayerWs& w, const bf16* next_gain, cudaStream_t st) {
+  const a3_model_desc& m = h->m;
+  const int slices = residual_slices(h, g.M, g.seg[0].n, g.K, w.attn_part_bytes);
+  if (slices > 1) {  // the attention's partial results were consumed before the projection that follows it: their room is free
+    A3_TRY(gemm_residual_split(h, g, slices, (float*)w.attn_part, st));
+    return add_slices_rmsnorm(h, g.C, (const float*)w.attn_part, slices, next_gain, m.rms_eps, g.M, m.d_model, w.a, st);
+  }
+  A3_TRY(gemm_bf16(h, EPI_RESIDUAL, g, st));
+  if (!next_gain) return A3_OK;
+  return rmsnorm_rows(h, g.C, next_gain, m.rms_eps, g.M, m.d_model, w.a, st);
+}
+
+// One decoder layer.  normed: w.a already holds the attention norm of x (the previous layer's last step left it there);
+// next_gain: leave RMSNorm(x) * next_gain of the result in w.a for the layer that follows on the same rows.
 static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const int32_t* pos, int M, bf16* kc, bf16* vc,
-                                int kv_len, float* lse_out, const LayerWs& w, cudaStream_t st) {
+                                int kv_len, float* lse_out, const LayerWs& w, cudaStream_t st, bool normed = false,
+                                const bf16* next_gain = nullptr) {
   const a3_model_desc& m = h->m;
   const a3_layer_weights& lw = h->layers[layer];
   const int qd = m.n_q_heads * m.head_dim;
-  A3_TRY(rmsnorm_rows(h, x, (const bf16*)lw.attn_norm, m.rms_eps, M, m.d_model, w.a, st));
+  if (!normed) A3_TRY(rmsnorm_rows(h, x, (const bf16*)lw.attn_norm, m.rms_eps, M, m.d_model, w.a, st));
   A3_TRY(qkv_project(h, layer, w.a, pos, M, 0, w.q, kc, vc, kv_len, st));
   A3_TRY(attention_rows(h, w.q, pos, M, kc, vc, kv_len, w.o, lse_out, w.attn_part, w.attn_part_bytes, st));
   GemmArgs g{};
@@ -340,8 +357,7 @@ static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const in
   g.seg[0] = {(const bf16*)lw.wo, nullptr, m.d_model, 0};
   g.C = x;
   g.ldc = m.d_model;
-  A3_TRY(gemm_bf16(h, EPI_RESIDUAL, g, st));
-  A3_TRY(rmsnorm_rows(h, x, (const bf16*)lw.mlp_norm, m.rms_eps, M, m.d_model, w.a, st));
+  A3_TRY(residual_then_norm(h, g, w, (const bf16*)lw.mlp_norm, st));
   GemmArgs u{};
   u.A = w.a;
   u.M = M;
@@ -360,8 +376,7 @@ static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const in
   d.seg[0] = {(const bf16*)lw.w_down, nullptr, m.d_model, 0};
   d.C = x;
   d.ldc = m.d_model;
-  A3_TRY(gemm_bf16(h, EPI_RESIDUAL, d, st));
-  return A3_OK;
+  return residual_then_norm(h, d, w, next_gain, st);
 }
 }  // namespace a3
 
@@ -552,8 +567,9 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     if (((uintptr_t)r->k_evicted | (uintptr_t)r->v_evicted) & 15) return A3_EINVAL;
   }
   // one layer for rows whose last nq entries are the question rows, then (optionally) its eviction
-  auto layer_step = [&](int l, bf16* x, const int32_t* pos, int rows) -> int {
-    A3_TRY(recompute_layer_impl(h, l, x, pos, rows, kl(l), vl(l), n, evict ? lw.lse : nullptr, lw, st));
+  auto layer_step = [&](int l, bf16* x, const int32_t* pos, int rows, bool normed, bool norm_next) -> int {
+    const bf16* next_gain = norm_next && l + 1 < m.n_layers ? (const bf16*)h->layers[l + 1].attn_norm : nullptr;
+    A3_TRY(recompute_layer_impl(h, l, x, pos, rows, kl(l), vl(l), n, evict ? lw.lse : nullptr, lw, st, normed, next_gain));
     if (!evict) return A3_OK;
     const size_t first_q = (size_t)(rows - nq);
     return a3_evict_layer(h, lw.q + first_q * m.n_q_heads * m.head_dim, pos + first_q, nq, lw.lse + first_q * m.n_q_heads, kl(l), vl(l), n,
@@ -572,8 +588,9 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     if (nq > 0) {
       bf16* xq = w.x_all;  // [nq][d] scratch for the question rows
       A3_CUDA(cudaMemcpyAsync(xq, (const bf16*)r->x0 + (size_t)r->n_ctx * m.d_model, (size_t)nq * m.d_model * 2, cudaMemcpyDeviceToDevice, st));
-      for (int l = 0; l < ls; ++l) A3_TRY(recompute_layer_impl(h, l, xq, q_pos, nq, kl(l), vl(l), n, nullptr, lw, st));
-      A3_TRY(rmsnorm_rows(h, xq, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, nq, m.d_model, lw.a, st));
+      for (int l = 0; l < ls; ++l)
+        A3_TRY(recompute_layer_impl(h, l, xq, q_pos, nq, kl(l), vl(l), n, nullptr, lw, st, l > 0, (const bf16*)h->layers[l + 1].attn_norm));
+      if (ls == 0) A3_TRY(rmsnorm_rows(h, xq, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, nq, m.d_model, lw.a, st));
       A3_TRY(qkv_project(h, ls, lw.a, q_pos, nq, 0, lw.q, kl(ls), vl(ls), n, st));
       A3_TRY(scores_with_stats(h, lw.q, q_pos, nq, kl(ls), n, r->n_system, r->n_ctx, w.lse_q, lw.attn_part, lw.attn_part_bytes,
                                r->scores_out, st));
@@ -586,7 +603,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     if (M == 0) return A3_OK;
     A3_TRY(check_rows(h, r->rows_out, M, n, st));
     A3_TRY(a3_gather_rows(h, r->x0, n, r->rows_out, M, m.d_model, r->x_out, stream));
-    for (int l = 0; l < m.n_layers; ++l) A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M));
+    for (int l = 0; l < m.n_layers; ++l) A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, l > 0, true));
     return A3_OK;
   }
 
@@ -608,16 +625,17 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
       // block 0 on this panel of rows: they attend to the rows before them, whose K/V the earlier panels have written
       if (i == 0) A3_TRY(feed_to(ls + 1 + FEED_AHEAD));  // a full block is long: several layers' copies fit under it
       if (i + 1 < panels) A3_TRY(recompute_layer_impl(h, 0, w.x_all + (size_t)r0 * m.d_model, w.all_pos + r0, r1 - r0, kl(0), vl(0), n, nullptr, lw, st));
-      else A3_TRY(layer_step(0, w.x_all + (size_t)r0 * m.d_model, w.all_pos + r0, r1 - r0));
+      else A3_TRY(layer_step(0, w.x_all + (size_t)r0 * m.d_model, w.all_pos + r0, r1 - r0, false, panels == 1));
     }
   }
   for (int l = 1; l < ls; ++l) {
     A3_TRY(feed_to(ls + 1 + FEED_AHEAD * (l + 1)));
-    A3_TRY(layer_step(l, w.x_all, w.all_pos, n));
+    A3_TRY(layer_step(l, w.x_all, w.all_pos, n, l > 1 || panels == 1, true));
   }
   A3_TRY(feed_to(ls + 1 + FEED_AHEAD));
   // selection layer: true K, V for all rows, queries of the question rows, scores, Re (Eq. 3)
-  A3_TRY(rmsnorm_rows(h, w.x_all, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, n, m.d_model, lw.a, st));
+  if (ls == 0 || (ls == 1 && panels > 1))  // otherwise the last full block left the norm of all rows
+    A3_TRY(rmsnorm_rows(h, w.x_all, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, n, m.d_model, lw.a, st));
   A3_TRY(qkv_project(h, ls, lw.a, w.all_pos, n, r->n_ctx, lw.q, kl(ls), vl(ls), n, st));
   A3_CUDA(cudaMemsetAsync(r->scores_out, 0, (size_t)n * 4, st));
   if (r->selector == A3_SELECT_VALUE_DEVIATION) {
@@ -649,7 +667,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
       A3_CUDA(cudaStreamWaitEvent(st, layer_ready[l], 0));
       A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, l, l + 1, stream));
     }
-    A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M));
+    A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, l > ls, true));
   }
   return A3_OK;
 }
@@ -670,7 +688,8 @@ extern "C" int a3_precompute_chunk(const a3_handle* h, void* x_chunk, int T, voi
   A3_TRY(iota_rows(h, w.all_pos, 0, T, st));
   for (int l = 0; l < m.n_layers; ++l)
     A3_TRY(recompute_layer_impl(h, l, (bf16*)x_chunk, w.all_pos, T, (bf16*)((char*)k_chunk + (size_t)l * layer_stride),
-                                (bf16*)((char*)v_chunk + (size_t)l * layer_stride), T, nullptr, lw, st));
+                                (bf16*)((char*)v_chunk + (size_t)l * layer_stride), T, nullptr, lw, st, l > 0,
+                                l + 1 < m.n_layers ? (const bf16*)h->layers[l + 1].attn_norm : nullptr));
   return A3_OK;
 }
 

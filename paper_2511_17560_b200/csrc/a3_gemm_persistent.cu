@@ -42,6 +42,8 @@ struct SpParams {
   int tok_tiles, tok_n;  // token tiles and tokens per tile (multiple of 16, at most 256)
   int n_fblocks;         // feature blocks (one per CTA pair and unit): units = n_fblocks x tok_tiles
   int group;             // feature blocks per group of the unit order (1: feature blocks outermost)
+  int k_slices;          // SPLIT: slices of the k-loop per (feature block, token tile); 1 otherwise
+  float* part;           // SPLIT: fp32 partial sums [k_slices][M][F]
   int n_units, n_pairs;
   int stages, stage_bytes, sub_bytes;  // ring depth; bytes per stage = SP_SUB x sub_bytes (A + this CTA's half of the token tile for one k-block, 1024-byte multiple)
   bf16* C;
@@ -98,6 +100,12 @@ __device__ __forceinline__ void sp_unit(int u, int n_fblocks, int tok_tiles, int
   fb = g * group + (r - tt * gsz);
 }
 
+// SPLIT: ring stages [first, first + count) of slice ks of a k-loop of `steps` stages
+__device__ __forceinline__ void sp_slice(int ks, int k_slices, int steps, int& first, int& count) {
+  first = (int)((long long)steps * ks / k_slices);
+  count = (int)((long long)steps * (ks + 1) / k_slices) - first;
+}
+
 // D += A B over the CTA pair (accumulating form: no predicate to set up)
 __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
   asm volatile(
@@ -114,7 +122,10 @@ __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc
 // heads of the concatenated list, one per CTA of the pair, times one token tile; the epilogue adds the bias, rotates
 // q and k at the tokens' positions (the two halves of a rotation pair sit 64 lanes apart and meet through shared
 // memory, like gate and up) and writes q to its buffer and k, v into the cache rows pos[token] (the scatter of Eq. 5).
-template <int EPI>
+// SPLIT: a launch with fewer units than CTA pairs cuts the k-loop of every unit into k_slices and the epilogue writes
+// the slice's fp32 sums to `part` instead; the kernel that follows (RMSNorm, which reads these rows anyway) adds the
+// slices in order.  See residual_slices below for when and why.
+template <int EPI, bool SPLIT = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
               const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmW, const SpParams p) {
@@ -123,7 +134,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // same offset in both CTAs of the pair
   unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const int S = p.stages;
-  const int xch_off = S * p.stage_bytes, bar_off = xch_off + (EPI == EPI_SWIGLU ? SP_XCH_BYTES : (EPI == EPI_QKV ? SP_QKV_EXTRA : 0));
+  const int xch_off = S * p.stage_bytes, bar_off = xch_off + (SPLIT ? 0 : EPI == EPI_SWIGLU ? SP_XCH_BYTES : (EPI == EPI_QKV ? SP_QKV_EXTRA : 0));
   // barriers (8 bytes each): full[8] (used in the leader), empty[8], tmem_full[2], tmem_empty[2] (used in the leader)
   const uint32_t bars = base + bar_off;
   auto full_bar = [&](int s) { return bars + 8u * s; };
@@ -151,7 +162,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     for (int b = 0; b < 2; ++b) {
       mbar_init(tmem_full(b), 1);
       // SwiGLU: the gate warps and the up warps of both warp sets of each CTA; residual and QKV: every epilogue warp
-      mbar_init(tmem_empty(b), EPI == EPI_SWIGLU ? 8 : 16);
+      mbar_init(tmem_empty(b), EPI == EPI_SWIGLU && !SPLIT ? 8 : 16);
     }
     abort_flag[0] = 0;
     abort_flag[1] = 0;
@@ -182,8 +193,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       bool ok = true;
       if (EPI == EPI_QKV) tmap_prefetch(&tmW);
       for (int u = pair; u < p.n_units && ok; u += p.n_pairs) {
-        int fb, tt;
-        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        int fb, tt, kb0 = 0, kb1 = KT;
+        sp_unit(SPLIT ? u / p.k_slices : u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        if (SPLIT) {
+          sp_slice(u % p.k_slices, p.k_slices, KT / SP_SUB, kb0, kb1);
+          kb0 *= SP_SUB;
+          kb1 = kb0 + kb1 * SP_SUB;
+        }
         int f0 = fb * (2 * ROWS) + (int)rank * ROWS;
         const CUtensorMap* mapA = &tmG;
         if (EPI == EPI_QKV) {
@@ -196,7 +212,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           mapA = sg == 0 ? &tmG : (sg == 1 ? &tmU : &tmW);
         }
         const int t0 = tt * p.tok_n + (int)rank * half_n;
-        for (int kb = 0; kb < KT; kb += SP_SUB, ++kbg) {
+        for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
           if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
             ok = false;
             break;
@@ -205,7 +221,6 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           // the leader announces the bytes of both CTAs; a copy of the peer that completes earlier cannot end the
           // phase, because the leader's own arrival is still pending until its expect_tx
           if (leader) mbar_expect_tx(full_bar(s), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
-#pragma unroll
 #pragma unroll
           for (int j = 0; j < SP_SUB; ++j) {
             const uint32_t sa = base + s * p.stage_bytes + j * p.sub_bytes, sb = sa + SP_A_BYTES;
@@ -242,9 +257,16 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       const uint64_t da0 = smem_desc_sw128(base), db0 = smem_desc_sw128(base + SP_A_BYTES);
       // descriptor address fields count 16-byte units: stage and k-step offsets are added to the first stage's
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, sub16 = (uint32_t)p.sub_bytes >> 4;
-      const int per_unit = KT / SP_SUB;
-      const int my_units = pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0;
-      const int total = my_units * per_unit;
+      int per_unit = KT / SP_SUB, total = 0;
+      if (SPLIT) {
+        for (int u = pair, first; u < p.n_units; u += p.n_pairs) {
+          int count;
+          sp_slice(u % p.k_slices, p.k_slices, KT / SP_SUB, first, count);
+          total += count;
+        }
+      } else {
+        total = (pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0) * per_unit;
+      }
       int s = 0, it = 0, in_unit = 0;
       uint32_t ph = 0, stage_off = 0, d = tmem_base;
       bool ok = total > 0, ready = false;
@@ -255,6 +277,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           ok = mbar_wait(tmem_empty(b), ((it >> 1) & 1) ^ 1, abort_flag, p.status);
           if (!ok) break;
           d = tmem_base + (uint32_t)b * 256u;
+          if (SPLIT) {
+            int first;
+            sp_slice((pair + it * p.n_pairs) % p.k_slices, p.k_slices, KT / SP_SUB, first, per_unit);
+          }
         }
         if (!ready) ok = mbar_wait(full_bar(s), ph, abort_flag, p.status);
         if (!ok) break;
@@ -290,6 +316,43 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         ph = phn;
         stage_off = offn;
       }
+    }
+  } else if (SPLIT) {
+    // ---------------- epilogue of a k-slice: warps 2..9 of both CTAs, lane = feature (of the one matrix or of this CTA's
+    // head), warp set 0 the first half of the token columns, set 1 the second; a warp writes 32 consecutive fp32 sums of
+    // one token (128 bytes) per instruction.
+    const int quarter = warp & 3;
+    const int set = (warp - 2) >> 2;
+    const int ep_tid = (warp - 2) * 32 + lane;
+    const int set_n = p.tok_n >> 1;
+    const int n_chunks = (set_n + 31) >> 5;
+    int it = 0;
+    for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
+      const int b = it & 1;
+      int fb, tt;
+      sp_unit(u / p.k_slices, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+      const int f = fb * (2 * ROWS) + (int)rank * ROWS + quarter * 32 + lane;
+      const int t0 = tt * p.tok_n + set * set_n;
+      float* prow = p.part + ((size_t)(u % p.k_slices) * p.M + t0) * p.F + f;
+      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+      named_bar_sync(1, 256);
+      if (!ep_ok[0]) break;  // uniform for the 256 threads
+      tc_fence_after();
+      const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+      for (int c = 0; c < n_chunks; ++c) {
+        const int w = min(32, set_n - c * 32);
+        float v[32];
+        __syncwarp();
+        sp_ld_chunk(trow + c * 32, w, v);
+        const int valid = f < p.F ? min(w, p.M - (t0 + c * 32)) : 0;
+#pragma unroll
+        for (int e = 0; e < 32; ++e)
+          if (e < valid) prow[(size_t)(c * 32 + e) * p.F] = v[e];
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
     }
   } else if (EPI == EPI_SWIGLU) {
     // ---------------- epilogue: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31.
@@ -595,6 +658,71 @@ static SpTiling choose_tiling(const a3_handle* h, int M, int n_fblocks, int pair
   return best;
 }
 
+// How many k-slices the residual GEMM of few rows is cut into (1: not at all).  With one unit per 256 features x 256
+// tokens, M <= 512 rows leave most of the 74 CTA pairs idle: a down projection of 75 rows x 3 584 features ran on 28 SMs
+// and streamed its 136 MB of weights at 1.4 TB/s.  Compared are, in clocks, the 256 x 256 tile kernel (a k-block costs its
+// 512 tensor clocks) and rounds of the split units (a k-block costs the larger of its tensor time and the arrival of its
+// operands, see choose_tiling) plus the fp32 partial sums, which are written and read once each through L2 (about 3 KB a
+// clock), at most `part_bytes` of them.  A slice is at least 1 024 deep: shorter ones are all pipeline fill.
+// Pinned kernel variants (a3_set_option) are compared bit for bit and therefore keep the undivided sums.
+constexpr int SP_SLICE_MIN_KB = 16;
+static bool split_allowed(const a3_handle* h) {
+  return h->opt[A3_OPT_RESIDUAL_T] == 1 && h->opt[A3_OPT_QKV_T] == 1 && h->opt[A3_OPT_SWIGLU_PAIR] == 1 &&
+         h->opt[A3_OPT_GEMM_TILING] == 0;
+}
+static int choose_slices(int M, int F, int K, int n_fblocks, int pairs, long long unsplit, size_t part_bytes) {
+  const int tiles = cdiv(M, 256), n = cdiv(cdiv(M, tiles), 16) * 16, kt = K / TC_BK;
+  const int per_kb = 2 * n > 256 + n ? 2 * n : 256 + n;
+  int best = 1;
+  for (int s = 2; s <= 16 && s * SP_SLICE_MIN_KB <= kt; ++s) {
+    if ((size_t)s * M * F * 4 > part_bytes) break;
+    const long long cost = (long long)cdiv((long long)n_fblocks * tiles * s, pairs) * ((long long)cdiv(kt / SP_SUB, s) * SP_SUB * per_kb + 2000) +
+                           (long long)s * M * F * 8 / 3000 + 2000;
+    if (cost < unsplit) {
+      unsplit = cost;
+      best = s;
+    }
+  }
+  return best;
+}
+int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) {
+  if (!split_allowed(h) || h->opt[A3_OPT_GEMM_BN_RESIDUAL] != 0 || M <= 0 || K % (SP_SUB * TC_BK) || N % 32) return 1;
+  const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2, blocks = cdiv(N, 4 * SP_FEAT);
+  if (blocks * cdiv(M, 256) > pairs / 2) return 1;  // the pairs are busy with whole units
+  return choose_slices(M, N, K, blocks, pairs, (long long)(K / TC_BK) * 512, part_bytes);
+}
+
+int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st) {
+  SpParams p{};
+  p.M = a.M;
+  p.K = a.K;
+  p.F = a.seg[0].n;
+  const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2;
+  p.n_fblocks = cdiv(p.F, 4 * SP_FEAT);
+  p.tok_tiles = cdiv(a.M, 256);
+  p.tok_n = cdiv(cdiv(a.M, p.tok_tiles), 16) * 16;
+  p.k_slices = slices;
+  p.part = part;
+  p.n_units = p.n_fblocks * p.tok_tiles * slices;
+  p.group = 1;
+  p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
+  p.status = h->dev_status;
+  p.sub_bytes = SP_A_BYTES + (int)align_up((size_t)(p.tok_n / 2) * TC_BK * 2, 1024);
+  p.stage_bytes = SP_SUB * p.sub_bytes;
+  p.stages = (SP_SMEM_LIMIT - 256 - 1024) / p.stage_bytes;
+  if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
+  const int smem_bytes = p.stages * p.stage_bytes + 256 + 1024;
+  CUtensorMap tX, tG;
+  A3_TRY(make_tmap(&tX, a.A, a.M, a.K, p.tok_n / 2));
+  A3_TRY(make_tmap(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT));
+  static SmemAttrOnce attr;
+  A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI_RESIDUAL, true>, SP_SMEM_LIMIT));
+  ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
+  A3_CUDA(launch_pdl(pair_t_kernel<EPI_RESIDUAL, true>, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tG, tG, p));
+  A3_LAUNCHED();
+  return A3_OK;
+}
+
 template <int EPI>
 static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   constexpr int ROWS = EPI == EPI_SWIGLU ? SP_FEAT : 2 * SP_FEAT;  // output features per CTA
@@ -610,6 +738,7 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   p.tok_n = til.n;
   p.n_units = p.n_fblocks * p.tok_tiles;
   p.group = unit_group(a.M, a.K);
+  p.k_slices = 1;
   p.n_pairs = p.n_units < sms / 2 ? p.n_units : sms / 2;
   p.C = a.C;
   p.ldc = a.ldc;
@@ -664,6 +793,7 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   p.tok_n = til.n;
   p.n_fblocks = head_pairs;
   p.group = unit_group(a.M, a.K);
+  p.k_slices = 1;
   p.n_units = head_pairs * p.tok_tiles;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;

@@ -128,6 +128,9 @@ inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 // out[m] = rmsnorm(x[m]) * gain, rows of width d.
 int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps, int M, int d, bf16* out, cudaStream_t st);
+// x[m] += part[0][m] + part[1][m] + ... (fp32 [slices][M][d], rounded once), then out[m] as above (gain null: no norm).
+int add_slices_rmsnorm(const a3_handle* h, bf16* x, const float* part, int slices, const bf16* gain, float eps, int M, int d, bf16* out,
+                       cudaStream_t st);
 
 enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_SWIGLU = 1, EPI_QKV = 2 };
 
@@ -160,6 +163,10 @@ int gemm_swiglu_pair(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
 // C += A B^T with the same kernel structure (weights on the M side, persistent CTA pairs).
 bool residual_t_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_residual_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
+// The same product of few rows, its k-loop cut into slices: fp32 partial sums [slices][M][N] for add_slices_rmsnorm.
+// residual_slices: how many slices suit the shape (1: use gemm_bf16), given room for part_bytes of partial sums.
+int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes);
+int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st);
 // QKV projection (bias, RoPE, scatter in the epilogue) with one head per CTA of a pair
 bool qkv_t_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
