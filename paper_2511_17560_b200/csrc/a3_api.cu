@@ -292,6 +292,7 @@ static int qkv_project(const a3_handle* h, int layer, const bf16* a, const int32
   const int qd = m.n_q_heads * m.head_dim, kvd = m.n_kv_heads * m.head_dim;
   GemmArgs g{};
   g.K = m.d_model;
+  g.early_weights = true;
   g.q_out = q_out;
   g.k_cache = kc;
   g.v_cache = vc;
@@ -353,6 +354,7 @@ static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const in
   g.A = w.o;
   g.M = M;
   g.K = qd;
+  g.early_weights = true;
   g.nseg = 1;
   g.seg[0] = {(const bf16*)lw.wo, nullptr, m.d_model, 0};
   g.C = x;
@@ -362,6 +364,7 @@ static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const in
   u.A = w.a;
   u.M = M;
   u.K = m.d_model;
+  u.early_weights = true;
   u.nseg = 1;
   u.seg[0] = {(const bf16*)lw.w_gate, nullptr, m.d_ff, 0};
   u.B2 = (const bf16*)lw.w_up;
@@ -372,6 +375,7 @@ static int recompute_layer_impl(const a3_handle* h, int layer, bf16* x, const in
   d.A = w.hmid;
   d.M = M;
   d.K = m.d_ff;
+  d.early_weights = true;
   d.nseg = 1;
   d.seg[0] = {(const bf16*)lw.w_down, nullptr, m.d_model, 0};
   d.C = x;

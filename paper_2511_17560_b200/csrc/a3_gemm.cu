@@ -455,8 +455,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();  // the peer's barriers exist before anything is signalled on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();
   pdl_launch_dependents();
+  // as in the persistent kernel: the weights may be read before the preceding kernel has finished (see GemmArgs)
+  if (warp >= 2 || !p.early) pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own rows of A, own half of B
@@ -472,19 +473,24 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       tmap_prefetch(&tmA);
       tmap_prefetch(mapB);
-      int issued = 0;
-      for (int kb = 0; kb < KT; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (kb / STAGES) & 1;
-        if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) break;
-        const uint32_t sa = base + s * L::STAGE_BYTES, sb = sa + L::A_BYTES;
-        const uint32_t full_leader = full_bar(s) & PAIR_LEADER_MASK;
+      auto load_weights = [&](int s, int kb) {
         // The leader announces the bytes of both CTAs.  A copy of the peer may complete before that: the phase
         // cannot end early, because the leader's own arrival is still pending until its expect_tx.
         if (leader) mbar_expect_tx(full_bar(s), 2 * L::STAGE_BYTES);
-        tma_load_2d_pair(sa, &tmA, kb * TC_BK, m0, full_leader);
-        tma_load_2d_pair(sb, mapB, kb * TC_BK, brow0, full_leader);
-        issued = kb + 1;
+        tma_load_2d_pair(base + s * L::STAGE_BYTES + L::A_BYTES, mapB, kb * TC_BK, brow0, full_bar(s) & PAIR_LEADER_MASK);
+      };
+      const int early = p.early ? min(STAGES, KT) : 0;
+      for (int kb = 0; kb < early; ++kb) load_weights(kb, kb);
+      if (p.early) pdl_wait();
+      int issued = early;
+      for (int kb = 0; kb < KT; ++kb) {
+        const int s = kb % STAGES;
+        if (kb >= early) {
+          if (!mbar_wait(empty_bar(s), ((kb / STAGES) & 1) ^ 1, abort_flag, p.status)) break;
+          load_weights(s, kb);
+        }
+        tma_load_2d_pair(base + s * L::STAGE_BYTES, &tmA, kb * TC_BK, m0, full_bar(s) & PAIR_LEADER_MASK);
+        issued = max(issued, kb + 1);
       }
       if (*abort_flag) {
         // let the copies already issued land before the CTA can exit (bounded)
@@ -737,6 +743,7 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
   p.max_pos = h->m.max_positions;
   p.tab = h->rope_tab;
   p.status = h->dev_status;
+  p.early = a.early_weights;
   if (pair) bn = 512;
   if (epi == EPI_RESIDUAL) return dispatch_tc<EPI_RESIDUAL>(h, a, p, tiles, bn, stages, st);
   if (epi == EPI_SWIGLU) return dispatch_tc<EPI_SWIGLU>(h, a, p, tiles, bn, stages, st);

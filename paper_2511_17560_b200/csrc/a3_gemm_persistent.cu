@@ -42,6 +42,7 @@ struct SpParams {
   int tok_tiles, tok_n;  // token tiles and tokens per tile (multiple of 16, at most 256)
   int n_fblocks;         // feature blocks (one per CTA pair and unit): units = n_fblocks x tok_tiles
   int group;             // feature blocks per group of the unit order (1: feature blocks outermost)
+  int early;             // the first ring stages' weights may be loaded before the preceding kernels are waited for
   int k_slices;          // SPLIT: slices of the k-loop per (feature block, token tile); 1 otherwise
   float* part;           // SPLIT: fp32 partial sums [k_slices][M][F]
   int n_units, n_pairs;
@@ -178,8 +179,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   cluster_sync_all();  // the peer's barriers exist before anything is signalled on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();
   pdl_launch_dependents();
+  // Only the threads that touch what earlier kernels wrote wait for them: the producer before the first token tile, the
+  // epilogue warps.  The weights are nobody's output, so the producer has already filled the ring's weight half by then
+  // (16 KiB x 2 per stage and CTA, most of what a launch of few rows spends its first microseconds on).
+  if (warp >= 2 || !p.early) pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own gate/up rows, own half of the token tile
@@ -192,6 +196,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       uint32_t ph = 0;  // k-block is a long dependent chain in a one-thread role
       bool ok = true;
       if (EPI == EPI_QKV) tmap_prefetch(&tmW);
+      int early = p.early ? S : 0;  // ring stages whose weights are requested ahead of pdl_wait (within the first unit)
       for (int u = pair; u < p.n_units && ok; u += p.n_pairs) {
         int fb, tt, kb0 = 0, kb1 = KT;
         sp_unit(SPLIT ? u / p.k_slices : u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
@@ -212,23 +217,37 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           mapA = sg == 0 ? &tmG : (sg == 1 ? &tmU : &tmW);
         }
         const int t0 = tt * p.tok_n + (int)rank * half_n;
-        for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
-          if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
-            ok = false;
-            break;
-          }
-          const uint32_t full_leader = full_bar(s) & PAIR_LEADER_MASK;
+        auto load_weights = [&](int stage, int kb) {
+          const uint32_t full_leader = full_bar(stage) & PAIR_LEADER_MASK;
           // the leader announces the bytes of both CTAs; a copy of the peer that completes earlier cannot end the
           // phase, because the leader's own arrival is still pending until its expect_tx
-          if (leader) mbar_expect_tx(full_bar(s), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
+          if (leader) mbar_expect_tx(full_bar(stage), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
 #pragma unroll
           for (int j = 0; j < SP_SUB; ++j) {
-            const uint32_t sa = base + s * p.stage_bytes + j * p.sub_bytes, sb = sa + SP_A_BYTES;
+            const uint32_t sa = base + stage * p.stage_bytes + j * p.sub_bytes;
             tma_load_2d_pair(sa, mapA, (kb + j) * TC_BK, f0, full_leader);
             if (EPI == EPI_SWIGLU) tma_load_2d_pair(sa + SP_A_BYTES / 2, &tmU, (kb + j) * TC_BK, f0, full_leader);
-            tma_load_2d_pair(sb, &tmX, (kb + j) * TC_BK, t0, full_leader);
           }
-          issued = kbg + 1;
+        };
+        if (early && kbg == 0) {
+          early = min(early, (kb1 - kb0) / SP_SUB);
+          for (int i = 0; i < early; ++i) load_weights(i, kb0 + i * SP_SUB);
+          issued = early;
+          pdl_wait();
+        }
+        for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
+          if (kbg >= early) {
+            if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
+              ok = false;
+              break;
+            }
+            load_weights(s, kb);
+          }
+          const uint32_t full_leader = full_bar(s) & PAIR_LEADER_MASK;
+#pragma unroll
+          for (int j = 0; j < SP_SUB; ++j)
+            tma_load_2d_pair(base + s * p.stage_bytes + j * p.sub_bytes + SP_A_BYTES, &tmX, (kb + j) * TC_BK, t0, full_leader);
+          issued = max(issued, kbg + 1);
           if (++s == S) {
             s = 0;
             ph ^= 1;
@@ -702,6 +721,7 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   p.tok_tiles = cdiv(a.M, 256);
   p.tok_n = cdiv(cdiv(a.M, p.tok_tiles), 16) * 16;
   p.k_slices = slices;
+  p.early = a.early_weights;
   p.part = part;
   p.n_units = p.n_fblocks * p.tok_tiles * slices;
   p.group = 1;
@@ -739,6 +759,7 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   p.n_units = p.n_fblocks * p.tok_tiles;
   p.group = unit_group(a.M, a.K);
   p.k_slices = 1;
+  p.early = a.early_weights;
   p.n_pairs = p.n_units < sms / 2 ? p.n_units : sms / 2;
   p.C = a.C;
   p.ldc = a.ldc;
@@ -794,6 +815,7 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   p.n_fblocks = head_pairs;
   p.group = unit_group(a.M, a.K);
   p.k_slices = 1;
+  p.early = a.early_weights;
   p.n_units = head_pairs * p.tok_tiles;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;

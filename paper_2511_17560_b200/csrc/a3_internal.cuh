@@ -147,6 +147,10 @@ struct GemmArgs {
   GemmSegment seg[3];
   int nseg;
   const bf16* B2;  // EPI_SWIGLU: the "up" matrix, same shape as seg[0].B (gate)
+  // The launch follows another kernel of this library in the same call: the weights, which the caller leaves alone while
+  // calls are queued, may be read before that kernel has finished (programmatic dependent launch).  Off for a GEMM that
+  // is the first launch of its call, whose predecessor is the caller's.
+  bool early_weights;
   bf16* C;         // EPI_RESIDUAL: [M][N] in/out (C += A B^T); EPI_SWIGLU: [M][N] out
   int ldc;
   // EPI_QKV

@@ -345,6 +345,12 @@ int check_rows(const a3_handle* h, const int32_t* pos, int M, int kv_len, cudaSt
 constexpr int RN_THREADS = 128, RN_VPT = 4;
 __global__ void __launch_bounds__(RN_THREADS)
 rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gain, float eps, int row_vecs, uint4* __restrict__ out) {
+  uint4 gv[RN_VPT];  // the gains, cold in every layer, are on their way before the preceding kernel has finished
+#pragma unroll
+  for (int i = 0; i < RN_VPT; ++i) {
+    const int idx = threadIdx.x + i * RN_THREADS;
+    gv[i] = idx < row_vecs ? __ldg(gain + idx) : make_uint4(0, 0, 0, 0);
+  }
   pdl_wait();
   pdl_launch_dependents();
   const uint4* xr = x + (size_t)blockIdx.x * row_vecs;
@@ -384,7 +390,7 @@ rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gain, floa
     if (idx < row_vecs) {
       float f[8], g[8], r[8];
       unpack8(v[i], f);
-      unpack8(__ldg(gain + idx), g);
+      unpack8(gv[i], g);
 #pragma unroll
       for (int e = 0; e < 8; ++e) r[e] = f[e] * inv * g[e];
       orow[idx] = pack8(r);
@@ -444,6 +450,12 @@ template <int SLICES>
 __global__ void __launch_bounds__(RS_THREADS)
 add_slices_rmsnorm_kernel(uint4* __restrict__ x, const float4* __restrict__ part, int slices, const uint4* __restrict__ gain, float eps,
                           int row_vecs, uint4* __restrict__ out) {
+  uint4 gv[RS_VPT];
+#pragma unroll
+  for (int i = 0; i < RS_VPT; ++i) {
+    const int idx = threadIdx.x + i * RS_THREADS;
+    gv[i] = gain && idx < row_vecs ? __ldg(gain + idx) : make_uint4(0, 0, 0, 0);
+  }
   pdl_wait();
   pdl_launch_dependents();
   uint4* xr = x + (size_t)blockIdx.x * row_vecs;
@@ -483,10 +495,10 @@ add_slices_rmsnorm_kernel(uint4* __restrict__ x, const float4* __restrict__ part
   for (int w = 0; w < RS_THREADS / 32; ++w) tot += sums[w];
   const float inv = rsqrtf(tot / (float)(row_vecs * 8) + eps);
   uint4* orow = out + (size_t)blockIdx.x * row_vecs;
-  auto scaled = [&](const uint4& xv, int idx) {
+  auto scaled = [&](const uint4& xv, const uint4& gain_v, int idx) {
     float f[8], g[8];
     unpack8(xv, f);
-    unpack8(__ldg(gain + idx), g);
+    unpack8(gain_v, g);
 #pragma unroll
     for (int e = 0; e < 8; ++e) f[e] = f[e] * inv * g[e];
     orow[idx] = pack8(f);
@@ -494,9 +506,9 @@ add_slices_rmsnorm_kernel(uint4* __restrict__ x, const float4* __restrict__ part
 #pragma unroll
   for (int i = 0; i < RS_VPT; ++i) {
     const int idx = threadIdx.x + i * RS_THREADS;
-    if (idx < row_vecs) scaled(v[i], idx);
+    if (idx < row_vecs) scaled(v[i], gv[i], idx);
   }
-  for (int idx = threadIdx.x + RS_VPT * RS_THREADS; idx < row_vecs; idx += RS_THREADS) scaled(xr[idx], idx);
+  for (int idx = threadIdx.x + RS_VPT * RS_THREADS; idx < row_vecs; idx += RS_THREADS) scaled(xr[idx], __ldg(gain + idx), idx);
 }
 
 int add_slices_rmsnorm(const a3_handle* h, bf16* x, const float* part, int slices, const bf16* gain, float eps, int M, int d, bf16* out,
