@@ -46,7 +46,7 @@ struct SpParams {
   int k_slices;          // SPLIT: slices of the k-loop per (feature block, token tile); 1 otherwise
   float* part;           // SPLIT: fp32 partial sums [k_slices][M][F]
   int n_units, n_pairs;
-  int stages, stage_bytes, sub_bytes;  // ring depth; bytes per stage = SP_SUB x sub_bytes (A + this CTA's half of the token tile for one k-block, 1024-byte multiple)
+  int stages, stage_bytes;  // ring depth; bytes per stage: SP_SUB k-blocks of weights, then SP_SUB of this CTA's half of the token tile
   bf16* C;
   int ldc;
   uint32_t* status;
@@ -147,7 +147,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   volatile int* ep_ok = abort_flag + 2;  // the epilogue's one waiter tells the other 127 threads how its wait ended
   float* xch = reinterpret_cast<float*>(base_ptr + xch_off);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int pair = blockIdx.x >> 1;
@@ -187,15 +187,18 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own gate/up rows, own half of the token tile
-    if (lane == 0) {
-      tmap_prefetch(&tmX);
-      tmap_prefetch(&tmG);
-      if (EPI == EPI_SWIGLU) tmap_prefetch(&tmU);
+    // as a whole warp, one elected lane issuing; a stage's k-blocks of an operand are one copy of a 3-D map ([k-block][row][64])
+    {
+      if (elect_one()) {
+        tmap_prefetch(&tmX);
+        tmap_prefetch(&tmG);
+        if (EPI != EPI_RESIDUAL) tmap_prefetch(&tmU);
+        if (EPI == EPI_QKV) tmap_prefetch(&tmW);
+      }
       int kbg = 0, issued = 0;
       int s = 0;        // ring position and phase, kept by counting: S is a run-time value and a division per
       uint32_t ph = 0;  // k-block is a long dependent chain in a one-thread role
       bool ok = true;
-      if (EPI == EPI_QKV) tmap_prefetch(&tmW);
       int early = p.early ? S : 0;  // ring stages whose weights are requested ahead of pdl_wait (within the first unit)
       for (int u = pair; u < p.n_units && ok; u += p.n_pairs) {
         int fb, tt, kb0 = 0, kb1 = KT;
@@ -218,16 +221,23 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         }
         const int t0 = tt * p.tok_n + (int)rank * half_n;
         auto load_weights = [&](int stage, int kb) {
-          const uint32_t full_leader = full_bar(stage) & PAIR_LEADER_MASK;
+          const uint32_t full_leader = full_bar(stage) & PAIR_LEADER_MASK, sa = base + stage * p.stage_bytes;
           // the leader announces the bytes of both CTAs; a copy of the peer that completes earlier cannot end the
           // phase, because the leader's own arrival is still pending until its expect_tx
-          if (leader) mbar_expect_tx(full_bar(stage), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
+          if (elect_one()) {
+            if (leader) mbar_expect_tx(full_bar(stage), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
+            if (EPI == EPI_SWIGLU) {
+              // a k-block's operand is gate rows, then up rows
 #pragma unroll
-          for (int j = 0; j < SP_SUB; ++j) {
-            const uint32_t sa = base + stage * p.stage_bytes + j * p.sub_bytes;
-            tma_load_2d_pair(sa, mapA, (kb + j) * TC_BK, f0, full_leader);
-            if (EPI == EPI_SWIGLU) tma_load_2d_pair(sa + SP_A_BYTES / 2, &tmU, (kb + j) * TC_BK, f0, full_leader);
+              for (int j = 0; j < SP_SUB; ++j) {
+                tma_load_3d_pair(sa + j * SP_A_BYTES, &tmG, f0, kb + j, full_leader);
+                tma_load_3d_pair(sa + j * SP_A_BYTES + SP_A_BYTES / 2, &tmU, f0, kb + j, full_leader);
+              }
+            } else {
+              tma_load_3d_pair(sa, mapA, f0, kb, full_leader);
+            }
           }
+          __syncwarp();
         };
         if (early && kbg == 0) {
           early = min(early, (kb1 - kb0) / SP_SUB);
@@ -237,16 +247,15 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         }
         for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
           if (kbg >= early) {
-            if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
+            if (!mbar_wait_warp(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
               ok = false;
               break;
             }
             load_weights(s, kb);
           }
-          const uint32_t full_leader = full_bar(s) & PAIR_LEADER_MASK;
-#pragma unroll
-          for (int j = 0; j < SP_SUB; ++j)
-            tma_load_2d_pair(base + s * p.stage_bytes + j * p.sub_bytes + SP_A_BYTES, &tmX, (kb + j) * TC_BK, t0, full_leader);
+          if (elect_one())
+            tma_load_3d_pair(base + s * p.stage_bytes + SP_SUB * SP_A_BYTES, &tmX, t0, kb, full_bar(s) & PAIR_LEADER_MASK);
+          __syncwarp();
           issued = max(issued, kbg + 1);
           if (++s == S) {
             s = 0;
@@ -254,7 +263,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           }
         }
       }
-      if (*abort_flag) {
+      if (lane == 0 && *abort_flag) {
         // let the copies already issued land before the CTA can exit (bounded)
         if (leader) {
           for (int k = max(0, issued - S); k < issued; ++k)
@@ -268,14 +277,14 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: the leader alone, for both CTAs.
-    // The tensor pipe queues only about two instructions, so everything this thread does between two of them has
-    // to fit into some 200 clocks or the pipe runs dry.  The look at the next stage's barrier therefore happens in
-    // the middle of a stage (after its first four instructions), the commit and the ring arithmetic at its end.
-    if (lane == 0 && leader) {
+    // The whole warp walks the loop, one elected lane issues (see uniform_warp in a3_tc.cuh).  Back to back at 804 rows x
+    // 28 672 columns 167 -> 156 us, at 133 rows 54.3 -> 51.1, a single unit alone (no contention) 19.7 -> 16.0.
+    if (leader) {
       const uint32_t idesc = idesc_bf16_pair(p.tok_n);
-      const uint64_t da0 = smem_desc_sw128(base), db0 = smem_desc_sw128(base + SP_A_BYTES);
+      const uint64_t da0 = smem_desc_sw128(base), db0 = smem_desc_sw128(base + SP_SUB * SP_A_BYTES);
       // descriptor address fields count 16-byte units: stage and k-step offsets are added to the first stage's
-      const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, sub16 = (uint32_t)p.sub_bytes >> 4;
+      const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, a_sub16 = SP_A_BYTES >> 4, b_sub16 = (uint32_t)half_n * (TC_BK * 2) >> 4;
+      const uint32_t tmem_acc = __shfl_sync(0xffffffffu, tmem_base, 0);
       int per_unit = KT / SP_SUB, total = 0;
       if (SPLIT) {
         for (int u = pair, first; u < p.n_units; u += p.n_pairs) {
@@ -287,53 +296,45 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         total = (pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0) * per_unit;
       }
       int s = 0, it = 0, in_unit = 0;
-      uint32_t ph = 0, stage_off = 0, d = tmem_base;
-      bool ok = total > 0, ready = false;
+      uint32_t ph = 0, stage_off = 0, d = tmem_acc;
+      bool ok = total > 0;
       for (int g = 0; g < total && ok; ++g) {
         if (in_unit == 0) {
           // the epilogues of both CTAs have drained this accumulator (first use: passes at once)
           const int b = it & 1;
-          ok = mbar_wait(tmem_empty(b), ((it >> 1) & 1) ^ 1, abort_flag, p.status);
+          ok = mbar_wait_warp(tmem_empty(b), ((it >> 1) & 1) ^ 1, abort_flag, p.status);
           if (!ok) break;
-          d = tmem_base + (uint32_t)b * 256u;
+          d = tmem_acc + (uint32_t)b * 256u;
           if (SPLIT) {
             int first;
             sp_slice((pair + it * p.n_pairs) % p.k_slices, p.k_slices, KT / SP_SUB, first, per_unit);
           }
         }
-        if (!ready) ok = mbar_wait(full_bar(s), ph, abort_flag, p.status);
+        ok = mbar_wait_warp(full_bar(s), ph, abort_flag, p.status);
         if (!ok) break;
         tc_fence_after();
         const uint64_t da_s = da0 + stage_off, db_s = db0 + stage_off;
-        tc_mma_pair_f16(d, da_s, db_s, idesc, in_unit != 0);
+        if (elect_one()) {
+          tc_mma_pair_f16(d, da_s, db_s, idesc, in_unit != 0);
 #pragma unroll
-        for (int k = 1; k < TC_BK / 16; ++k) tc_mma_pair_acc(d, da_s + (uint64_t)(2 * k), db_s + (uint64_t)(2 * k), idesc);
-        // next ring position, and one look at its barrier while the pipe works on the instructions above
-        int sn = s + 1;
-        uint32_t phn = ph, offn = stage_off + stage16;
-        if (sn == S) {
-          sn = 0;
-          phn ^= 1;
-          offn = 0;
-        }
-        ready = g + 1 < total && mbar_try_wait(full_bar(sn), phn);
-#pragma unroll
-        for (int j = 1; j < SP_SUB; ++j) {
-#pragma unroll
-          for (int k = 0; k < TC_BK / 16; ++k) {
-            const uint64_t koff = (uint64_t)(j * sub16 + 2 * k);
-            tc_mma_pair_acc(d, da_s + koff, db_s + koff, idesc);
+          for (int i = 1; i < SP_SUB * (TC_BK / 16); ++i) {
+            const int j = i / (TC_BK / 16), k = i % (TC_BK / 16);
+            tc_mma_pair_acc(d, da_s + (uint64_t)(j * a_sub16 + 2 * k), db_s + (uint64_t)(j * b_sub16 + 2 * k), idesc);
           }
+          tc_commit_pair(empty_bar(s), 3);  // frees this stage in both CTAs once the instructions above have read it
+          if (in_unit + 1 == per_unit) tc_commit_pair(tmem_full(it & 1), 3);  // publishes the accumulator in both CTAs
         }
-        tc_commit_pair(empty_bar(s), 3);  // frees this stage in both CTAs once the instructions above have read it
+        __syncwarp();
         if (++in_unit == per_unit) {
-          tc_commit_pair(tmem_full(it & 1), 3);  // publishes the accumulator in both CTAs
           in_unit = 0;
           ++it;
         }
-        s = sn;
-        ph = phn;
-        stage_off = offn;
+        stage_off += stage16;
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+          stage_off = 0;
+        }
       }
     }
   } else if (SPLIT) {
@@ -727,14 +728,13 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   p.group = 1;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;
-  p.sub_bytes = SP_A_BYTES + (int)align_up((size_t)(p.tok_n / 2) * TC_BK * 2, 1024);
-  p.stage_bytes = SP_SUB * p.sub_bytes;
+  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
   p.stages = (SP_SMEM_LIMIT - 256 - 1024) / p.stage_bytes;
   if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
   const int smem_bytes = p.stages * p.stage_bytes + 256 + 1024;
   CUtensorMap tX, tG;
-  A3_TRY(make_tmap(&tX, a.A, a.M, a.K, p.tok_n / 2));
-  A3_TRY(make_tmap(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT));
+  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
+  A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB));
   static SmemAttrOnce attr;
   A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI_RESIDUAL, true>, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
@@ -765,15 +765,14 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   p.ldc = a.ldc;
   p.status = h->dev_status;
   // as many ring stages as fit beside the exchange buffers
-  p.sub_bytes = SP_A_BYTES + (int)align_up((size_t)(p.tok_n / 2) * TC_BK * 2, 1024);
-  p.stage_bytes = SP_SUB * p.sub_bytes;
+  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
   p.stages = (SP_SMEM_LIMIT - XCH - 256 - 1024) / p.stage_bytes;
   if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
   const int smem_bytes = p.stages * p.stage_bytes + XCH + 256 + 1024;
   CUtensorMap tX, tG, tU;
-  A3_TRY(make_tmap(&tX, a.A, a.M, a.K, p.tok_n / 2));
-  A3_TRY(make_tmap(&tG, a.seg[0].B, p.F, a.K, ROWS));
-  if (EPI == EPI_SWIGLU) A3_TRY(make_tmap(&tU, a.B2, p.F, a.K, ROWS));
+  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
+  A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, ROWS, EPI == EPI_SWIGLU ? 1 : SP_SUB));
+  if (EPI == EPI_SWIGLU) A3_TRY(make_tmap_kblocks(&tU, a.B2, p.F, a.K, ROWS, 1));
   else tU = tG;
   static SmemAttrOnce attr;
   A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI>, SP_SMEM_LIMIT));
@@ -829,15 +828,14 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   p.layout = h->m.rope_layout;
   p.max_pos = h->m.max_positions;
   p.tab = h->rope_tab;
-  p.sub_bytes = SP_A_BYTES + (int)align_up((size_t)(p.tok_n / 2) * TC_BK * 2, 1024);
-  p.stage_bytes = SP_SUB * p.sub_bytes;
+  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
   p.stages = (SP_SMEM_LIMIT - SP_QKV_EXTRA - 256 - 1024) / p.stage_bytes;
   if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
   const int smem_bytes = p.stages * p.stage_bytes + SP_QKV_EXTRA + 256 + 1024;
   CUtensorMap tX, tW[3];
-  A3_TRY(make_tmap(&tX, a.A, a.M, a.K, p.tok_n / 2));
+  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   for (int s = 0; s < 3; ++s) {
-    if (s < a.nseg) A3_TRY(make_tmap(&tW[s], a.seg[s].B, a.seg[s].n, a.K, 128));
+    if (s < a.nseg) A3_TRY(make_tmap_kblocks(&tW[s], a.seg[s].B, a.seg[s].n, a.K, 128, SP_SUB));
     else tW[s] = tW[0];
   }
   static SmemAttrOnce attr;

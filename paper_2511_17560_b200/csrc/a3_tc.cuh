@@ -71,6 +71,47 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
   }
 }
+// One look at a barrier that never suspends the caller (try_wait may).
+__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done;
+}
+// Roles of one thread run as whole warps: every lane walks the loop with the same values and elect_one() picks the one
+// that issues.  tcgen05 and TMA instructions take their operands from uniform registers; under `if (lane == 0)` nothing is
+// known to be uniform and every descriptor is moved over on its own, which made the issuing thread the limit of short
+// products (475 clocks per k-block of four instructions that the pipe runs in 192 at N = 16).
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(is));
+  return is != 0;
+}
+// mbar_wait for a whole warp: the same answer in every lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t* status,
+                                               unsigned long long limit_ns = TC_WAIT_NS) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 32; ++i)
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    if (__any_sync(0xffffffffu, global_ns() - t0 > limit_ns)) {
+      if ((threadIdx.x & 31) == 0) {
+        *abort_flag = 1;
+        atomicOr(status, A3_DEV_WAIT_EXHAUSTED);
+      }
+      return false;
+    }
+  }
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
@@ -169,6 +210,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
                ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
                : "memory");
 }
+// same, 3-D map of k-blocks (make_tmap_kblocks): rows from y of k-blocks from z
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+               ::"r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(cta_mask) : "memory");
 }
@@ -220,5 +267,23 @@ static inline int make_tmap(CUtensorMap* map, const void* ptr, long long rows, l
   return A3_OK;
 }
 
+// The same matrix as [cols / 64][rows][64]: one copy brings `kblocks` consecutive 64-column blocks of box_rows rows, block
+// after block, each laid out as make_tmap's box (cols a multiple of 64)
+static inline int make_tmap_kblocks(CUtensorMap* map, const void* ptr, long long rows, long long cols, int box_rows, int kblocks) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return A3_ECUDA;
+  cuuint64_t dims[3] = {(cuuint64_t)TC_BK, (cuuint64_t)rows, (cuuint64_t)(cols / TC_BK)};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)TC_BK * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows, (cuuint32_t)kblocks};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    g_last_cuda_error = (int)r;
+    return A3_ECUDA;
+  }
+  return A3_OK;
+}
 
 }  // namespace a3
