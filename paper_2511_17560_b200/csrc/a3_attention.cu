@@ -116,7 +116,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::BAR_OFF + 8 * 27 + 8);
   float2* xch = reinterpret_cast<float2*>(base_ptr + L::XCH_OFF);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int G = Hq / Hkv;
   const int rows_total = M * G;
   const int row_tiles = (rows_total + ATC_BM - 1) / ATC_BM;
@@ -163,94 +163,125 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const uint32_t tmem_s0 = tmem_base, tmem_o = tmem_base + 256;
 
   if (warp == 0) {
-    // ---------------- TMA producer
-    if (lane == 0) {
+    // ---------------- TMA producer (the whole warp walks, one elected lane issues)
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmK) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmV) : "memory");
-      uint32_t it = 0;
-      bool ok = true;
-      for (int r = 0; r < rounds && ok; ++r) {
-        const int i = item_index(r);
-        if (i < 0) continue;
-        const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
-        if (!w.valid) continue;
-        for (int kt = 0; kt < w.nkt; ++kt, ++it) {
-          const int s = it % L::KV_STAGES;
-          const uint32_t ph = (it / L::KV_STAGES) & 1;
-          const uint32_t sk = base + L::KV_OFF + s * L::KV_STAGE, sv = sk + (D / 64) * L::SUB;
-          ok = mbar_wait(k_empty(s), ph ^ 1, abort_flag, status);
-          if (!ok) break;
+    }
+    uint32_t s = 0, ph = 0;  // ring stage and phase, kept by counting
+    bool ok = true;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int i = item_index(r);
+      if (i < 0) continue;
+      const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
+      const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0), row0 = __shfl_sync(0xffffffffu, w.kt0 * ATC_BN, 0);
+      for (int kt = 0; kt < nkt; ++kt) {
+        const uint32_t sk = base + L::KV_OFF + s * L::KV_STAGE, sv = sk + (D / 64) * L::SUB;
+        ok = mbar_wait_warp(k_empty(s), ph ^ 1, abort_flag, status);
+        if (!ok) break;
+        if (elect_one()) {
           mbar_expect_tx(k_full(s), L::KV_STAGE / 2);
 #pragma unroll
-          for (int j = 0; j < D / 64; ++j) tma_load_2d(sk + j * L::SUB, &tmK, w.g * D + 64 * j, (w.kt0 + kt) * ATC_BN, k_full(s));
-          if (want_o) {  // the statistics-only pass never reads V
-            ok = mbar_wait(v_empty(s), ph ^ 1, abort_flag, status);
-            if (!ok) break;
+          for (int j = 0; j < D / 64; ++j) tma_load_2d(sk + j * L::SUB, &tmK, w.g * D + 64 * j, row0 + kt * ATC_BN, k_full(s));
+        }
+        __syncwarp();
+        if (want_o) {  // the statistics-only pass never reads V
+          ok = mbar_wait_warp(v_empty(s), ph ^ 1, abort_flag, status);
+          if (!ok) break;
+          if (elect_one()) {
             mbar_expect_tx(v_full(s), L::KV_STAGE / 2);
 #pragma unroll
-            for (int j = 0; j < D / 64; ++j) tma_load_2d(sv + j * L::SUB, &tmV, w.g * D + 64 * j, (w.kt0 + kt) * ATC_BN, v_full(s));
+            for (int j = 0; j < D / 64; ++j) tma_load_2d(sv + j * L::SUB, &tmV, w.g * D + 64 * j, row0 + kt * ATC_BN, v_full(s));
           }
+          __syncwarp();
+        }
+        if (++s == L::KV_STAGES) {
+          s = 0;
+          ph ^= 1;
         }
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc(ATC_BN, 0);
-      constexpr uint32_t idesc_o = idesc(D, 1);
-      const uint32_t sq = base + L::Q_OFF;
-      auto issue_s = [&](uint32_t t) {  // S of running key tile t into S buffer t & 1, from K stage t mod 3
-        const uint32_t sk = base + L::KV_OFF + (t % L::KV_STAGES) * L::KV_STAGE;
+    // ---------------- MMA issuer (the whole warp walks, one elected lane issues)
+    constexpr uint32_t idesc_s = idesc(ATC_BN, 0);
+    constexpr uint32_t idesc_o = idesc(D, 1);
+    const uint64_t dq = desc_k_sw128(base + L::Q_OFF), dk0 = desc_k_sw128(base + L::KV_OFF);
+    const uint64_t dv0 = desc_mn_sw128(base + L::KV_OFF + (D / 64) * L::SUB, L::SUB);
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+    auto issue_s = [&](uint32_t b, uint32_t stage) {  // S of a key tile into S buffer b, from K stage `stage`
+      const uint64_t dk = dk0 + stage * (L::KV_STAGE >> 4);
+      if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
-          const uint32_t sub = (k / 4) * L::SUB + (k % 4) * 32;
-          mma_f16(tmem_s0 + (t & 1) * 128, desc_k_sw128(sq + sub), desc_k_sw128(sk + sub), idesc_s, k != 0);
+          const uint32_t sub = ((k / 4) * L::SUB + (k % 4) * 32) >> 4;
+          mma_f16(tmem_u + b * 128, dq + sub, dk + sub, idesc_s, k != 0);
         }
-        commit(s_full(t & 1));
-        commit(k_empty(t % L::KV_STAGES));  // the K stage is free once these MMAs have read it
-      };
-      uint32_t it = 0, qn = 0;
-      bool ok = true;
-      for (int r = 0; r < rounds && ok; ++r) {
-        const int i = item_index(r);
-        if (i < 0) continue;
-        const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
-        if (!w.valid || w.nkt == 0) continue;
-        ok = mbar_wait(q_ready, qn & 1, abort_flag, status);
-        ++qn;
-        ok = ok && mbar_wait(k_full(it % L::KV_STAGES), (it / L::KV_STAGES) & 1, abort_flag, status);
-        if (!ok) break;
-        fence_after();
-        issue_s(it);
-        for (int kt = 0; kt < w.nkt; ++kt, ++it) {
-          if (kt + 1 < w.nkt) {
-            ok = mbar_wait(k_full((it + 1) % L::KV_STAGES), ((it + 1) / L::KV_STAGES) & 1, abort_flag, status);
-            if (!ok) break;
-            fence_after();
-            issue_s(it + 1);
-          }
-          ok = mbar_wait(p_ready(it & 1), (it >> 1) & 1, abort_flag, status);
+        commit(s_full(b));
+        commit(k_empty(stage));  // the K stage is free once these MMAs have read it
+      }
+      __syncwarp();
+    };
+    uint32_t it = 0, qn = 0;
+    uint32_t ks = 0, kph = 0, vs = 0, vph = 0;  // ring positions of the next K and V tile
+    auto k_next = [&]() {  // waits for the next K tile and returns its stage; L::KV_STAGES on failure
+      if (!mbar_wait_warp(k_full(ks), kph, abort_flag, status)) return (uint32_t)L::KV_STAGES;
+      const uint32_t at = ks;
+      if (++ks == L::KV_STAGES) {
+        ks = 0;
+        kph ^= 1;
+      }
+      return at;
+    };
+    bool ok = true;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int i = item_index(r);
+      if (i < 0) continue;
+      const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
+      const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0);
+      if (nkt == 0) continue;
+      ok = mbar_wait_warp(q_ready, qn & 1, abort_flag, status);
+      ++qn;
+      if (!ok) break;
+      uint32_t stage = k_next();
+      ok = stage < L::KV_STAGES;
+      if (!ok) break;
+      fence_after();
+      issue_s(it & 1, stage);
+      for (int kt = 0; kt < nkt; ++kt, ++it) {
+        if (kt + 1 < nkt) {
+          stage = k_next();
+          ok = stage < L::KV_STAGES;
           if (!ok) break;
-          if (want_o) {
-            ok = mbar_wait(v_full(it % L::KV_STAGES), (it / L::KV_STAGES) & 1, abort_flag, status);
-            if (!ok) break;
-          }
           fence_after();
-          if (want_o) {
-            const uint32_t sv = base + L::KV_OFF + (it % L::KV_STAGES) * L::KV_STAGE + (D / 64) * L::SUB;
-            // P of this tile lies over the first half of each thread's S columns (see the softmax warps): keys
-            // 64 h + 16 kk .. + 15 in the eight 32-bit columns at 64 h + 8 kk of S buffer it & 1.  The next S into
-            // that buffer is issued after these MMAs and the tensor pipe runs in order.
-            const uint32_t tp = tmem_s0 + (it & 1) * 128;
+          issue_s((it + 1) & 1, stage);
+        }
+        ok = mbar_wait_warp(p_ready(it & 1), (it >> 1) & 1, abort_flag, status);
+        if (!ok) break;
+        if (want_o) {
+          ok = mbar_wait_warp(v_full(vs), vph, abort_flag, status);
+          if (!ok) break;
+          fence_after();
+          const uint64_t dv = dv0 + vs * (L::KV_STAGE >> 4);
+          // P of this tile lies over the first half of each thread's S columns (see the softmax warps): keys
+          // 64 h + 16 kk .. + 15 in the eight 32-bit columns at 64 h + 8 kk of S buffer it & 1.  The next S into
+          // that buffer is issued after these MMAs and the tensor pipe runs in order.
+          const uint32_t tp = tmem_u + (it & 1) * 128;
+          if (elect_one()) {
 #pragma unroll
             for (int k = 0; k < ATC_BN / 16; ++k) {
-              const uint64_t db = desc_mn_sw128(sv + k * 16 * 128, L::SUB);
               // each half of the tile's keys accumulates into an output of its own (see the softmax warps)
-              mma_f16_ts(tmem_o + (k / 4) * D, tp + (k / 4) * 64 + (k % 4) * 8, db, idesc_o, (kt | (k % 4)) != 0);
+              mma_f16_ts(tmem_u + 256 + (k / 4) * D, tp + (k / 4) * 64 + (k % 4) * 8, dv + ((k * 16 * 128) >> 4), idesc_o, (kt | (k % 4)) != 0);
             }
             commit(p_free(it & 1));  // P V of this tile is complete: the outputs hold tiles 0..kt
-            commit(v_empty(it % L::KV_STAGES));
+            commit(v_empty(vs));
           }
+          __syncwarp();
+          if (++vs == L::KV_STAGES) {
+            vs = 0;
+            vph ^= 1;
+          }
+        } else {
+          fence_after();
         }
       }
     }

@@ -98,7 +98,7 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::BAR_OFF + 8 * 21);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::BAR_OFF + 8 * 21 + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int G = Hq / Hkv;
   const int rows_total = M * G;
   const int row_tiles = (rows_total + ATC_BM - 1) / ATC_BM;
@@ -141,124 +141,137 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   pdl_launch_dependents();
 
   if (warp == 0) {
-    // ---------------- TMA producer: K(t) then V(t) of every key tile the item walks
-    if (lane == 0) {
+    // ---------------- TMA producer: K(t) then V(t) of every key tile the item walks (whole warp, one elected lane issues)
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmK) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmV) : "memory");
-      uint32_t it = 0;
-      bool ok = true;
-      for (int r = 0; r < rounds && ok; ++r) {
-        const int i = item_index(r);
-        if (i < 0) continue;
-        const At2Item w = at2_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_pairs);
-        for (int t = 0; t < w.T; ++t, ++it) {
-          const int s = it & 1;
-          const uint32_t ph = (it >> 1) & 1;
-          ok = mbar_wait(k_empty(s), ph ^ 1, abort_flag, status);
-          if (!ok) break;
+    }
+    uint32_t it = 0;
+    bool ok = true;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int i = item_index(r);
+      if (i < 0) continue;
+      const At2Item w = at2_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_pairs);
+      const int T = __shfl_sync(0xffffffffu, w.T, 0);
+      for (int t = 0; t < T; ++t, ++it) {
+        const uint32_t s = it & 1, ph = (it >> 1) & 1;
+        ok = mbar_wait_warp(k_empty(s), ph ^ 1, abort_flag, status);
+        if (!ok) break;
+        if (elect_one()) {
           mbar_expect_tx(k_full(s), L::TILE);
           tma_load_2d(base + L::K_OFF + s * L::TILE, &tmK, w.g * D, t * ATC_BN, k_full(s));
           tma_load_2d(base + L::K_OFF + s * L::TILE + L::SUB, &tmK, w.g * D + 64, t * ATC_BN, k_full(s));
-          ok = mbar_wait(v_empty(s), ph ^ 1, abort_flag, status);
-          if (!ok) break;
+        }
+        __syncwarp();
+        ok = mbar_wait_warp(v_empty(s), ph ^ 1, abort_flag, status);
+        if (!ok) break;
+        if (elect_one()) {
           mbar_expect_tx(v_full(s), L::TILE);
           tma_load_2d(base + L::V_OFF + s * L::TILE, &tmV, w.g * D, t * ATC_BN, v_full(s));
           tma_load_2d(base + L::V_OFF + s * L::TILE + L::SUB, &tmV, w.g * D + 64, t * ATC_BN, v_full(s));
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1 || warp == 10) {
-    // ---------------- MMA issuers: this thread owns row tile x; K and V stages are released by both threads
-    if (lane == 0) {
-      const int x = warp == 1 ? 0 : 1;
-      constexpr uint32_t idesc_s = idesc(ATC_BN / 2, 0);
-      constexpr uint32_t idesc_o = idesc(D, 1);
-      uint32_t it = 0, qn = 0, cx = 0;  // running key tile; items; tiles this row tile has done (barrier phases)
-      // logits of 64 keys (half hh of the key tile in K stage `kstage`)
-      auto issue_s = [&](int hh, uint32_t kstage) {
-        const uint32_t sq = base + L::Q_OFF + x * L::TILE, sk = base + L::K_OFF + kstage * L::TILE + hh * (64 * 128);
+    // ---------------- MMA issuers: this warp owns row tile x (it walks whole, one elected lane issues); K and V stages are
+    // released by both
+    const int x = warp == 1 ? 0 : 1;
+    constexpr uint32_t idesc_s = idesc(ATC_BN / 2, 0);
+    constexpr uint32_t idesc_o = idesc(D, 1);
+    const uint64_t dq = desc_k_sw128(base + L::Q_OFF) + x * (L::TILE >> 4), dk0 = desc_k_sw128(base + L::K_OFF);
+    const uint64_t dv0 = desc_mn_sw128(base + L::V_OFF, L::SUB);
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint32_t ts_x = tmem_u + x * 128, to_x = tmem_u + 256 + x * 128;
+    uint32_t it = 0, qn = 0, cx = 0;  // running key tile; items; tiles this row tile has done (barrier phases)
+    // logits of 64 keys (half hh of the key tile in K stage `kstage`); release: the stage has been read for the last time
+    auto issue_s = [&](int hh, uint32_t kstage, bool release) {
+      const uint64_t dk = dk0 + kstage * (L::TILE >> 4) + hh * (64 * 128 >> 4);
+      if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
-          const uint32_t sub = (k / 4) * L::SUB + (k % 4) * 32;
-          mma_f16(tmem_base + x * 128 + hh * 64, desc_k_sw128(sq + sub), desc_k_sw128(sk + sub), idesc_s, k != 0);
+          const uint32_t sub = ((k / 4) * L::SUB + (k % 4) * 32) >> 4;
+          mma_f16(ts_x + hh * 64, dq + sub, dk + sub, idesc_s, k != 0);
         }
         commit(s_full(x, hh));
-      };
-      // P V of 64 keys: P of half hh lies over the first 32 columns of that half of S_X
-      auto issue_pv_half = [&](int hh, uint32_t vstage, bool first) {
-        const uint32_t sv = base + L::V_OFF + vstage * L::TILE;
+        if (release) commit(k_empty(kstage));
+      }
+      __syncwarp();
+    };
+    // P V of 64 keys: P of half hh lies over the first 32 columns of that half of S_X
+    auto issue_pv_half = [&](int hh, uint32_t vstage, bool first) {
+      const uint64_t dv = dv0 + vstage * (L::TILE >> 4);
+      if (elect_one()) {
 #pragma unroll
-        for (int k = 4 * hh; k < 4 * hh + 4; ++k) {
-          const uint64_t db = desc_mn_sw128(sv + k * 16 * 128, L::SUB);
-          mma_f16_ts(tmem_base + 256 + x * 128, tmem_base + x * 128 + hh * 64 + (k - 4 * hh) * 8, db, idesc_o, !(first && k == 0));
-        }
+        for (int kk = 0; kk < 4; ++kk)
+          mma_f16_ts(to_x, ts_x + hh * 64 + kk * 8, dv + (((4 * hh + kk) * 16 * 128) >> 4), idesc_o, !(first && hh == 0 && kk == 0));
         commit(hh == 0 ? pv0_done(x) : pv_done(x));
-      };
-      bool ok = true;
-      for (int r = 0; r < rounds && ok; ++r) {
-        const int i = item_index(r);
-        if (i < 0) continue;
-        const At2Item w = at2_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_pairs);
-        const int nkt = w.nkt[x];
-        ok = mbar_wait(q_ready, qn & 1, abort_flag, status);
-        ++qn;
-        if (!ok) break;
-        if (w.T == 0) continue;
-        ok = mbar_wait(k_full(it & 1), (it >> 1) & 1, abort_flag, status);
-        if (!ok) break;
-        fence_after();
-        if (nkt > 0) {
-          issue_s(0, it & 1);
-          issue_s(1, it & 1);
-          commit(k_empty(it & 1));
+        if (hh == 1) commit(v_empty(vstage));
+      }
+      __syncwarp();
+    };
+    auto release = [&](uint32_t bar) {
+      if (elect_one()) mbar_arrive(bar);
+      __syncwarp();
+    };
+    bool ok = true;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int i = item_index(r);
+      if (i < 0) continue;
+      const At2Item w = at2_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_pairs);
+      const int nkt = __shfl_sync(0xffffffffu, w.nkt[x], 0), T = __shfl_sync(0xffffffffu, w.T, 0);
+      ok = mbar_wait_warp(q_ready, qn & 1, abort_flag, status);
+      ++qn;
+      if (!ok) break;
+      if (T == 0) continue;
+      ok = mbar_wait_warp(k_full(it & 1), (it >> 1) & 1, abort_flag, status);
+      if (!ok) break;
+      fence_after();
+      if (nkt > 0) {
+        issue_s(0, it & 1, false);
+        issue_s(1, it & 1, true);
+      } else {
+        release(k_empty(it & 1));
+      }
+      for (int t = 0; t < T && ok; ++t, ++it) {
+        const bool more = t + 1 < T;
+        const uint32_t vs = it & 1, vph = (it >> 1) & 1, kn = (it + 1) & 1, kph = ((it + 1) >> 1) & 1;
+        if (t < nkt) {
+          const bool next = t + 1 < nkt;
+          // halves in key order.  Each P V is followed by the same half of the next key tile's logits: P V has read
+          // the columns they go to, and the pipe runs this warp's instructions in order.
+          ok = mbar_wait_warp(p0_ready(x), cx & 1, abort_flag, status) && mbar_wait_warp(v_full(vs), vph, abort_flag, status);
+          if (!ok) break;
+          fence_after();
+          issue_pv_half(0, vs, t == 0);
+          if (next) {
+            ok = mbar_wait_warp(k_full(kn), kph, abort_flag, status);
+            if (!ok) break;
+            fence_after();
+            issue_s(0, kn, false);
+          }
+          ok = mbar_wait_warp(p_ready(x), cx & 1, abort_flag, status);
+          if (!ok) break;
+          fence_after();
+          issue_pv_half(1, vs, t == 0);
+          if (next) issue_s(1, kn, true);
+          ++cx;
+          if (more && !next) {
+            // this row tile is done, the other walks on: its stages still need this warp's arrival, and an
+            // arrival must not run ahead of the stage's use (it would be counted in the wrong phase): wait
+            // until the tile has landed
+            ok = mbar_wait_warp(k_full(kn), kph, abort_flag, status);
+            if (!ok) break;
+            release(k_empty(kn));
+          }
         } else {
-          mbar_arrive(k_empty(it & 1));
-        }
-        for (int t = 0; t < w.T && ok; ++t, ++it) {
-          const bool more = t + 1 < w.T;
-          const uint32_t vs = it & 1, vph = (it >> 1) & 1, kn = (it + 1) & 1, kph = ((it + 1) >> 1) & 1;
-          if (t < nkt) {
-            const bool next = t + 1 < nkt;
-            // halves in key order.  Each P V is followed by the same half of the next key tile's logits: P V has read
-            // the columns they go to, and the pipe runs this thread's instructions in order.
-            ok = mbar_wait(p0_ready(x), cx & 1, abort_flag, status) && mbar_wait(v_full(vs), vph, abort_flag, status);
+          ok = mbar_wait_warp(v_full(vs), vph, abort_flag, status);
+          if (!ok) break;
+          release(v_empty(vs));
+          if (more) {
+            ok = mbar_wait_warp(k_full(kn), kph, abort_flag, status);
             if (!ok) break;
-            fence_after();
-            issue_pv_half(0, vs, t == 0);
-            if (next) {
-              ok = mbar_wait(k_full(kn), kph, abort_flag, status);
-              if (!ok) break;
-              fence_after();
-              issue_s(0, kn);
-            }
-            ok = mbar_wait(p_ready(x), cx & 1, abort_flag, status);
-            if (!ok) break;
-            fence_after();
-            issue_pv_half(1, vs, t == 0);
-            if (next) issue_s(1, kn);
-            ++cx;
-            commit(v_empty(vs));
-            if (more) {
-              if (next) {
-                commit(k_empty(kn));
-              } else {
-                // this row tile is done, the other walks on: its stages still need this thread's arrival, and an
-                // arrival must not run ahead of the stage's use (it would be counted in the wrong phase): wait
-                // until the tile has landed
-                ok = mbar_wait(k_full(kn), kph, abort_flag, status);
-                if (!ok) break;
-                mbar_arrive(k_empty(kn));
-              }
-            }
-          } else {
-            ok = mbar_wait(v_full(vs), vph, abort_flag, status);
-            if (!ok) break;
-            mbar_arrive(v_empty(vs));
-            if (more) {
-              ok = mbar_wait(k_full(kn), kph, abort_flag, status);
-              if (!ok) break;
-              mbar_arrive(k_empty(kn));
-            }
+            release(k_empty(kn));
           }
         }
       }

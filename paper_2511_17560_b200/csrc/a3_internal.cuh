@@ -234,6 +234,16 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&t);
 }
 
+// Roles of one thread run as whole warps: every lane walks the loop with the same values and elect_one() picks the one
+// that issues.  tcgen05 and TMA instructions take their operands from uniform registers; under `if (lane == 0)` nothing is
+// known to be uniform and every descriptor is moved over on its own, which made the issuing thread the limit of short
+// products (475 clocks per k-block of four instructions that the pipe runs in 192 at N = 16).
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(is));
+  return is != 0;
+}
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool pred) {

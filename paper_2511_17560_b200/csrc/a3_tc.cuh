@@ -71,28 +71,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
   }
 }
-// One look at a barrier that never suspends the caller (try_wait may).
-__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done;
-}
-// Roles of one thread run as whole warps: every lane walks the loop with the same values and elect_one() picks the one
-// that issues.  tcgen05 and TMA instructions take their operands from uniform registers; under `if (lane == 0)` nothing is
-// known to be uniform and every descriptor is moved over on its own, which made the issuing thread the limit of short
-// products (475 clocks per k-block of four instructions that the pipe runs in 192 at N = 16).
-__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
-__device__ __forceinline__ bool elect_one() {
-  uint32_t is;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(is));
-  return is != 0;
-}
 // mbar_wait for a whole warp: the same answer in every lane.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t* status,
                                                unsigned long long limit_ns = TC_WAIT_NS) {
