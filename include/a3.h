@@ -156,7 +156,7 @@ typedef enum {
   A3_OPT_ATTN_MAX_CTAS,         /* cap on the persistent attention grid; 0 = one CTA per SM (default) */
   A3_OPT_SWIGLU_NARROW,         /* one-CTA gate/up GEMM: 0 uniform tiles, 1 narrower last wave (default), 16..120 forced width */
   A3_OPT_SWIGLU_PAIR,           /* persistent CTA-pair gate/up GEMM: 0 never, 1 whenever the shape allows (default) */
-  A3_OPT_RESIDUAL_T,            /* persistent CTA-pair C += A B^T: 0 never, 1 by shape (default), 2 whenever the shape allows */
+  A3_OPT_RESIDUAL_T,            /* persistent CTA-pair C += A B^T: 0 never, 1 whenever the shape allows, few rows in k-slices (default), 2 never in k-slices */
   A3_OPT_GEMM_BN_RESIDUAL,      /* tile width of the tile GEMMs per epilogue; 0 = choose; 512 = the 256 x 256 CTA-pair tile */
   A3_OPT_GEMM_BN_SWIGLU,
   A3_OPT_GEMM_BN_QKV,

@@ -21,6 +21,8 @@
 // abort flag and the device status bit, all roles leave their loops, tensor memory is released and the CTA returns.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "a3_internal.cuh"
 #include "a3_tc.cuh"
 
@@ -31,10 +33,15 @@ constexpr int SP_MAX_STAGES = 8;
 constexpr int SP_SUB = 2;  // k-blocks of 64 per ring stage: one barrier hand-shake and one commit per 8 MMAs
 constexpr int SP_FEAT = 64;                              // features per CTA (64 gate lanes + 64 up lanes)
 constexpr int SP_A_BYTES = 2 * SP_FEAT * TC_BK * 2;      // 16 KiB: gate rows, then up rows
-constexpr int SP_XCH_BYTES = 2 * 2 * 32 * SP_FEAT * 4;   // per warp set: two buffers of float [32 tokens][64 features]
-constexpr int SP_QKV_SET_FLOATS = 4 * (32 * 32 + 4);            // QKV: per warp set, four quarters of [32 tokens][32 features] fp32, 16 bytes apart in the banks
-constexpr int SP_QKV_XCH_BYTES = 2 * SP_QKV_SET_FLOATS * 4 + 128;  // + room to keep the next field 256-byte aligned
-constexpr int SP_QKV_EXTRA = SP_QKV_XCH_BYTES + 256;              // ... and the checked positions of a chunk's tokens per set
+// Exchange buffers of the epilogues, which take `chunk` tokens at a time (32 where that costs no ring stage, else 16 or 8: see
+// set_stages).  SwiGLU: per warp set two buffers of float [chunk][64 features]; QKV and residual: per warp set four
+// quarters of [chunk][32 features] fp32, 16 bytes apart in the banks.
+__host__ __device__ constexpr int sp_set_floats(int epi, int chunk) {
+  return epi == EPI_SWIGLU ? 2 * chunk * SP_FEAT : 4 * (chunk * 32 + 4);
+}
+// both sets, 256-byte aligned, and for QKV the checked positions of a chunk's tokens per set behind them
+__host__ __device__ constexpr int sp_xch_floats_bytes(int epi, int chunk) { return (2 * sp_set_floats(epi, chunk) * 4 + 255) & ~255; }
+__host__ __device__ constexpr int sp_xch_bytes(int epi, int chunk) { return sp_xch_floats_bytes(epi, chunk) + (epi == EPI_QKV ? 256 : 0); }
 constexpr int SP_SMEM_LIMIT = 227 * 1024;
 
 struct SpParams {
@@ -47,6 +54,7 @@ struct SpParams {
   float* part;           // SPLIT: fp32 partial sums [k_slices][M][F]
   int n_units, n_pairs;
   int stages, stage_bytes;  // ring depth; bytes per stage: SP_SUB k-blocks of weights, then SP_SUB of this CTA's half of the token tile
+  int chunk;             // tokens per exchange of the epilogue: 32, 16 or (not QKV) 8
   bf16* C;
   int ldc;
   uint32_t* status;
@@ -73,16 +81,24 @@ __device__ __forceinline__ void mbar_arrive_in_cta(uint32_t bar, uint32_t cta) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(cta));
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
 }
-// w (8, 16, 24 or 32; uniform for the warp) consecutive accumulator columns of this thread's lane
+// w (8 .. CH in steps of 8; uniform for the warp) consecutive accumulator columns of this thread's lane
+template <int CH>
 __device__ __forceinline__ void sp_ld_chunk(uint32_t taddr, int w, float* v) {
-  if (w == 32) {
+  if (CH == 32 && w == 32) {
     tc_ld32(taddr, v);
   } else {  // static register indices: the array must not go to local memory
-    if (w >= 8) tc_ld8(taddr, v);
-    if (w >= 16) tc_ld8(taddr + 8, v + 8);
-    if (w >= 24) tc_ld8(taddr + 16, v + 16);
+#pragma unroll
+    for (int i = 0; i < CH / 8; ++i)
+      if (w >= 8 * i + 8) tc_ld8(taddr + 8 * i, v + 8 * i);
   }
   tc_wait_ld();
+}
+// f(std::integral_constant<int, chunk>) for the chunk of this launch
+template <bool MAY_8, typename F>
+__device__ __forceinline__ bool sp_with_chunk(int chunk, F f) {
+  if (chunk == 32) return f(std::integral_constant<int, 32>());
+  if (!MAY_8 || chunk == 16) return f(std::integral_constant<int, 16>());
+  return f(std::integral_constant<int, 8>());
 }
 
 // Unit u -> (feature block, token tile).  Units are numbered in groups of `group` feature blocks, token tiles next,
@@ -135,7 +151,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // same offset in both CTAs of the pair
   unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const int S = p.stages;
-  const int xch_off = S * p.stage_bytes, bar_off = xch_off + (SPLIT ? 0 : EPI == EPI_SWIGLU ? SP_XCH_BYTES : (EPI == EPI_QKV ? SP_QKV_EXTRA : 0));
+  const int xch_off = S * p.stage_bytes, bar_off = xch_off + (SPLIT ? 0 : sp_xch_bytes(EPI, p.chunk));
   // barriers (8 bytes each): full[8] (used in the leader), empty[8], tmem_full[2], tmem_empty[2] (used in the leader)
   const uint32_t bars = base + bar_off;
   auto full_bar = [&](int s) { return bars + 8u * s; };
@@ -364,7 +380,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         const int w = min(32, set_n - c * 32);
         float v[32];
         __syncwarp();
-        sp_ld_chunk(trow + c * 32, w, v);
+        sp_ld_chunk<32>(trow + c * 32, w, v);
         const int valid = f < p.F ? min(w, p.M - (t0 + c * 32)) : 0;
 #pragma unroll
         for (int e = 0; e < 32; ++e)
@@ -389,64 +405,67 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int feat = (quarter & 1) * 32 + lane;  // feature within this CTA's 64
     const int ep_tid = (warp - 2) * 32 + lane;
     const int set_n = p.tok_n >> 1;              // token columns of a set (multiple of 8)
-    const int n_chunks = (set_n + 31) >> 5;
     const int my_units = pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0;
-    const int total_chunks = my_units * n_chunks;
     const int bar_written = 2 + set * 4, bar_read = 4 + set * 4, bar_group = 10 + set * 2 + (up_warp ? 0 : 1);
-    float* xset = xch + set * (2 * 32 * SP_FEAT);
-    int it = 0, cc = 0;
-    for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
-      const int b = it & 1;
-      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
-      named_bar_sync(1, 256);
-      if (!ep_ok[0]) break;  // uniform for the 256 threads
-      tc_fence_after();
-      const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
-      int fb, tt;
-      sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
-      const int f = fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + feat;
-      const int t0 = tt * p.tok_n + set * set_n;
-      bf16* out = p.C + f;
+    sp_with_chunk<true>(p.chunk, [&](auto chunk) {
+      constexpr int CH = decltype(chunk)::value;
+      const int n_chunks = (set_n + CH - 1) / CH, total_chunks = my_units * n_chunks;
+      float* xset = xch + set * sp_set_floats(EPI, CH);
+      int it = 0, cc = 0;
+      for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
+        const int b = it & 1;
+        if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+        named_bar_sync(1, 256);
+        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        tc_fence_after();
+        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+        int fb, tt;
+        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        const int f = fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + feat;
+        const int t0 = tt * p.tok_n + set * set_n;
+        bf16* out = p.C + f;
 #pragma unroll 1
-      for (int c = 0; c < n_chunks; ++c, ++cc) {
-        const int buf = cc & 1;
-        const int w = min(32, set_n - c * 32);
-        float* xb = xset + buf * (32 * SP_FEAT);
-        float v[32];
-        __syncwarp();
-        sp_ld_chunk(trow + c * 32, w, v);
-        const bool writer = up_warp == (buf == 0);
-        if (writer) {
-          if (cc >= 2) named_bar_sync(bar_read + buf, 128);  // the readers are done with what this buffer held
-          if (w == 32) {
+        for (int c = 0; c < n_chunks; ++c, ++cc) {
+          const int buf = cc & 1;
+          const int w = min(CH, set_n - c * CH);
+          float* xb = xset + buf * (CH * SP_FEAT);
+          float v[CH];
+          __syncwarp();
+          sp_ld_chunk<CH>(trow + c * CH, w, v);
+          const bool writer = up_warp == (buf == 0);
+          if (writer) {
+            if (cc >= 2) named_bar_sync(bar_read + buf, 128);  // the readers are done with what this buffer held
+            if (w == CH) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) xb[e * SP_FEAT + feat] = v[e];
+              for (int e = 0; e < CH; ++e) xb[e * SP_FEAT + feat] = v[e];
+            } else {
+#pragma unroll
+              for (int e = 0; e < CH; ++e)
+                if (e < w) xb[e * SP_FEAT + feat] = v[e];
+            }
+            named_bar_arrive(bar_written + buf, 128);
           } else {
+            named_bar_sync(bar_written + buf, 128);
+            bf16* orow = out + (size_t)(t0 + c * CH) * p.ldc;
+            const int valid = min(w, p.M - (t0 + c * CH));  // tokens of this chunk that exist
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (e < w) xb[e * SP_FEAT + feat] = v[e];
+            for (int e = 0; e < CH; ++e) {
+              const float o = xb[e * SP_FEAT + feat];
+              const float g = up_warp ? o : v[e], uv = up_warp ? v[e] : o;
+              const float r = silu_mul(g, uv);
+              if (e < valid) orow[(size_t)e * p.ldc] = __float2bfloat16_rn(r);
+            }
+            if (cc + 2 < total_chunks) named_bar_arrive(bar_read + buf, 128);  // nobody waits for the last two
           }
-          named_bar_arrive(bar_written + buf, 128);
-        } else {
-          named_bar_sync(bar_written + buf, 128);
-          bf16* orow = out + (size_t)(t0 + c * 32) * p.ldc;
-          const int valid = min(w, p.M - (t0 + c * 32));  // tokens of this chunk that exist
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float o = xb[e * SP_FEAT + feat];
-            const float g = up_warp ? o : v[e], uv = up_warp ? v[e] : o;
-            const float r = silu_mul(g, uv);
-            if (e < valid) orow[(size_t)e * p.ldc] = __float2bfloat16_rn(r);
-          }
-          if (cc + 2 < total_chunks) named_bar_arrive(bar_read + buf, 128);  // nobody waits for the last two
         }
+        // this half of the set has read its part of the accumulator (wait::ld in sp_ld_chunk): one arrival per half,
+        // set and CTA on the leader's barrier hands it back to the MMA issuer
+        tc_fence_before();
+        named_bar_sync(bar_group, 64);
+        if (lane == 0 && (quarter == 0 || quarter == 2)) mbar_arrive_in_cta(tmem_empty(b), 0);
       }
-      // this half of the set has read its part of the accumulator (wait::ld in sp_ld_chunk): one arrival per half,
-      // set and CTA on the leader's barrier hands it back to the MMA issuer
-      tc_fence_before();
-      named_bar_sync(bar_group, 64);
-      if (lane == 0 && (quarter == 0 || quarter == 2)) mbar_arrive_in_cta(tmem_empty(b), 0);
-    }
+      return true;
+    });
   } else if (EPI == EPI_QKV) {
     // ---------------- epilogue, q / k / v heads: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31,
     // lane = feature of this CTA's head; warp set 0 (warps 2..5) takes the first half of the token columns, set 1 the
@@ -462,161 +481,182 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int ep_tid = (warp - 2) * 32 + lane;
     const int st = quarter * 32 + lane;  // thread within the set
     const int set_n = p.tok_n >> 1;
-    const int n_chunks = (set_n + 31) >> 5;
-    float* xset = xch + set * SP_QKV_SET_FLOATS;
-    int* posbuf = reinterpret_cast<int*>(base_ptr + xch_off + SP_QKV_XCH_BYTES) + set * 32;
     const int bar_set = 2 + set;
-    // phase 2 assignment: token e2 (+16 in the second pass), features f0 .. f0 + 7 and 64 + f0 .. 64 + f0 + 7
-    const int e2 = st >> 3, f0 = (st & 7) * 8;
-    const float* xlo = xset + (f0 >> 5) * (32 * 32 + 4) + (f0 & 31);
-    const float* xhi = xset + (2 + (f0 >> 5)) * (32 * 32 + 4) + (f0 & 31);
-    float* xmine = xset + quarter * (32 * 32 + 4) + lane;
-    int it = 0;
-    for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
-      const int b = it & 1;
-      int fb, tt;
-      sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
-      const int hd = 2 * fb + (int)rank;
-      const bool live = hd < p.n_heads;
-      const int hde = live ? hd : 0;
-      const int sg = (hde >= p.seg_heads_end[0]) + (hde >= p.seg_heads_end[1]);
-      const int head_in_seg = hde - (sg == 0 ? 0 : p.seg_heads_end[sg - 1]);
-      const int kind = p.kind[sg];
-      const int t0 = tt * p.tok_n + set * set_n;
-      const float bias = p.bias[sg] ? __bfloat162float(p.bias[sg][head_in_seg * 128 + quarter * 32 + lane]) : 0.f;
-      const bool rotate = kind != 2;
-      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
-      named_bar_sync(1, 256);
-      if (!ep_ok[0]) break;  // uniform for the 256 threads
-      tc_fence_after();
-      const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+    sp_with_chunk<false>(p.chunk, [&](auto chunk) {
+      constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4;
+      const int n_chunks = (set_n + CH - 1) / CH;
+      float* xset = xch + set * sp_set_floats(EPI, CH);
+      int* posbuf = reinterpret_cast<int*>(base_ptr + xch_off + sp_xch_floats_bytes(EPI, CH)) + set * 32;
+      // phase 2 assignment: token e2 (+16 in the second pass), features f0 .. f0 + 7 and 64 + f0 .. 64 + f0 + 7
+      const int e2 = st >> 3, f0 = (st & 7) * 8;
+      const float* xlo = xset + (f0 >> 5) * QUARTER + (f0 & 31);
+      const float* xhi = xset + (2 + (f0 >> 5)) * QUARTER + (f0 & 31);
+      float* xmine = xset + quarter * QUARTER + lane;
+      int it = 0;
+      for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
+        const int b = it & 1;
+        int fb, tt;
+        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        const int hd = 2 * fb + (int)rank;
+        const bool live = hd < p.n_heads;
+        const int hde = live ? hd : 0;
+        const int sg = (hde >= p.seg_heads_end[0]) + (hde >= p.seg_heads_end[1]);
+        const int head_in_seg = hde - (sg == 0 ? 0 : p.seg_heads_end[sg - 1]);
+        const int kind = p.kind[sg];
+        const int t0 = tt * p.tok_n + set * set_n;
+        const float bias = p.bias[sg] ? __bfloat162float(p.bias[sg][head_in_seg * 128 + quarter * 32 + lane]) : 0.f;
+        const bool rotate = kind != 2;
+        if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+        named_bar_sync(1, 256);
+        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        tc_fence_after();
+        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-      for (int c = 0; c < n_chunks; ++c) {
-        const int w = min(32, set_n - c * 32);
-        const int valid = min(w, p.M - (t0 + c * 32));  // tokens of this chunk that exist (may be <= 0)
-        float v[32];
+        for (int c = 0; c < n_chunks; ++c) {
+          const int w = min(CH, set_n - c * CH);
+          const int valid = min(w, p.M - (t0 + c * CH));  // tokens of this chunk that exist (may be <= 0)
+          float v[CH];
+          __syncwarp();
+          sp_ld_chunk<CH>(trow + c * CH, w, v);
+          if (quarter == 0) {  // positions of the chunk's tokens, checked: -1 where nothing is to be written
+            int ps = -1;
+            if (lane < valid) {
+              ps = p.pos[t0 + c * CH + lane];
+              if (ps < 0 || ps >= p.kv_len || ps >= p.max_pos) {
+                if (live) atomicOr(p.status, A3_DEV_BAD_POSITION);
+                ps = -1;
+              }
+            }
+            posbuf[lane] = ps;
+          }
+#pragma unroll
+          for (int e = 0; e < CH; ++e) xmine[e * 32] = v[e] + bias;
+          named_bar_sync(bar_set, 128);
+#pragma unroll
+          for (int pass = 0; pass < CH / 16; ++pass) {
+            const int e = e2 + 16 * pass;
+            const int ps = posbuf[e];
+            if (ps < 0 || !live) continue;
+            float a[8], bq[8], ra[8], rb[8];
+            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(xlo + e * 32);
+            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(xlo + e * 32 + 4);
+            *reinterpret_cast<float4*>(bq) = *reinterpret_cast<const float4*>(xhi + e * 32);
+            *reinterpret_cast<float4*>(bq + 4) = *reinterpret_cast<const float4*>(xhi + e * 32 + 4);
+            if (!rotate) {
+#pragma unroll
+              for (int k = 0; k < 8; ++k) ra[k] = a[k], rb[k] = bq[k];
+            } else if (p.layout == 0) {
+              // pairs (i, i + 64): the thread's first 8 features rotate with the 8 that lie 64 further, frequencies f0 .. f0 + 7
+              const float4* tr = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + f0);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const float4 t = __ldg(tr + k);  // (cos, sin) of two frequencies
+                ra[2 * k] = a[2 * k] * t.x - bq[2 * k] * t.y;
+                rb[2 * k] = a[2 * k] * t.y + bq[2 * k] * t.x;
+                ra[2 * k + 1] = a[2 * k + 1] * t.z - bq[2 * k + 1] * t.w;
+                rb[2 * k + 1] = a[2 * k + 1] * t.w + bq[2 * k + 1] * t.z;
+              }
+            } else {
+              // pairs (2i, 2i + 1): both groups of 8 hold four pairs of their own, frequencies f0/2 .. and 32 + f0/2 ..
+              const float4* tl = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + (f0 >> 1));
+              const float4* th = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + 32 + (f0 >> 1));
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const float4 t = __ldg(tl + k), u4 = __ldg(th + k);
+                ra[4 * k] = a[4 * k] * t.x - a[4 * k + 1] * t.y;
+                ra[4 * k + 1] = a[4 * k] * t.y + a[4 * k + 1] * t.x;
+                ra[4 * k + 2] = a[4 * k + 2] * t.z - a[4 * k + 3] * t.w;
+                ra[4 * k + 3] = a[4 * k + 2] * t.w + a[4 * k + 3] * t.z;
+                rb[4 * k] = bq[4 * k] * u4.x - bq[4 * k + 1] * u4.y;
+                rb[4 * k + 1] = bq[4 * k] * u4.y + bq[4 * k + 1] * u4.x;
+                rb[4 * k + 2] = bq[4 * k + 2] * u4.z - bq[4 * k + 3] * u4.w;
+                rb[4 * k + 3] = bq[4 * k + 2] * u4.w + bq[4 * k + 3] * u4.z;
+              }
+            }
+            bf16* dst = kind == 0 ? p.q_out + (size_t)(t0 + c * CH + e) * (p.Hq * 128) + head_in_seg * 128
+                      : (kind == 1 ? p.k_cache : p.v_cache) + (size_t)ps * (p.Hkv * 128) + head_in_seg * 128;
+            *reinterpret_cast<uint4*>(dst + f0) = pack8(ra);
+            *reinterpret_cast<uint4*>(dst + 64 + f0) = pack8(rb);
+          }
+          named_bar_sync(bar_set, 128);  // everybody has read this chunk's values and positions
+        }
+        // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
+        tc_fence_before();
         __syncwarp();
-        sp_ld_chunk(trow + c * 32, w, v);
-        if (quarter == 0) {  // positions of the chunk's tokens, checked: -1 where nothing is to be written
-          int ps = -1;
-          if (lane < valid) {
-            ps = p.pos[t0 + c * 32 + lane];
-            if (ps < 0 || ps >= p.kv_len || ps >= p.max_pos) {
-              if (live) atomicOr(p.status, A3_DEV_BAD_POSITION);
-              ps = -1;
-            }
-          }
-          posbuf[lane] = ps;
-        }
-#pragma unroll
-        for (int e = 0; e < 32; ++e) xmine[e * 32] = v[e] + bias;
-        named_bar_sync(bar_set, 128);
-#pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          const int e = e2 + 16 * pass;
-          const int ps = posbuf[e];
-          if (ps < 0 || !live) continue;
-          float a[8], bq[8], ra[8], rb[8];
-          *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(xlo + e * 32);
-          *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(xlo + e * 32 + 4);
-          *reinterpret_cast<float4*>(bq) = *reinterpret_cast<const float4*>(xhi + e * 32);
-          *reinterpret_cast<float4*>(bq + 4) = *reinterpret_cast<const float4*>(xhi + e * 32 + 4);
-          if (!rotate) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) ra[k] = a[k], rb[k] = bq[k];
-          } else if (p.layout == 0) {
-            // pairs (i, i + 64): the thread's first 8 features rotate with the 8 that lie 64 further, frequencies f0 .. f0 + 7
-            const float4* tr = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + f0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float4 t = __ldg(tr + k);  // (cos, sin) of two frequencies
-              ra[2 * k] = a[2 * k] * t.x - bq[2 * k] * t.y;
-              rb[2 * k] = a[2 * k] * t.y + bq[2 * k] * t.x;
-              ra[2 * k + 1] = a[2 * k + 1] * t.z - bq[2 * k + 1] * t.w;
-              rb[2 * k + 1] = a[2 * k + 1] * t.w + bq[2 * k + 1] * t.z;
-            }
-          } else {
-            // pairs (2i, 2i + 1): both groups of 8 hold four pairs of their own, frequencies f0/2 .. and 32 + f0/2 ..
-            const float4* tl = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + (f0 >> 1));
-            const float4* th = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + 32 + (f0 >> 1));
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              const float4 t = __ldg(tl + k), u4 = __ldg(th + k);
-              ra[4 * k] = a[4 * k] * t.x - a[4 * k + 1] * t.y;
-              ra[4 * k + 1] = a[4 * k] * t.y + a[4 * k + 1] * t.x;
-              ra[4 * k + 2] = a[4 * k + 2] * t.z - a[4 * k + 3] * t.w;
-              ra[4 * k + 3] = a[4 * k + 2] * t.w + a[4 * k + 3] * t.z;
-              rb[4 * k] = bq[4 * k] * u4.x - bq[4 * k + 1] * u4.y;
-              rb[4 * k + 1] = bq[4 * k] * u4.y + bq[4 * k + 1] * u4.x;
-              rb[4 * k + 2] = bq[4 * k + 2] * u4.z - bq[4 * k + 3] * u4.w;
-              rb[4 * k + 3] = bq[4 * k + 2] * u4.w + bq[4 * k + 3] * u4.z;
-            }
-          }
-          bf16* dst = kind == 0 ? p.q_out + (size_t)(t0 + c * 32 + e) * (p.Hq * 128) + head_in_seg * 128
-                    : (kind == 1 ? p.k_cache : p.v_cache) + (size_t)ps * (p.Hkv * 128) + head_in_seg * 128;
-          *reinterpret_cast<uint4*>(dst + f0) = pack8(ra);
-          *reinterpret_cast<uint4*>(dst + 64 + f0) = pack8(rb);
-        }
-        named_bar_sync(bar_set, 128);  // everybody has read this chunk's values and positions
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
       }
-      // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
-    }
+      return true;
+    });
   } else if (EPI == EPI_RESIDUAL) {
     // ---------------- epilogue, C += A B^T: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31,
-    // lane = output feature; warp set 0 (warps 2..5) takes the first half of the token columns, set 1 the second.
-    // A warp reads and writes 32 consecutive features of one token (64 bytes) per instruction.
+    // lane = output feature; warp set 0 (warps 2..5) takes the first half of the token columns, set 1 the second.  A chunk of
+    // tokens at a time in the two phases of the QKV epilogue: feature-major out of tensor memory into shared memory, then
+    // token-major, a thread taking 8 consecutive features of a token (16 bytes of C, 256 contiguous bytes per token).
+    // All old values of a unit (at most 16 vectors per thread) are requested while its main loop still runs: a launch with
+    // one unit per pair has nothing else to hide them under.
     const int quarter = warp & 3;
     const int set = (warp - 2) >> 2;
     const int ep_tid = (warp - 2) * 32 + lane;
+    const int st = quarter * 32 + lane;  // thread within the set
     const int set_n = p.tok_n >> 1;
-    const int n_chunks = (set_n + 31) >> 5;
-    int it = 0;
-    for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
-      const int b = it & 1;
-      int fb, tt;
-      sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
-      const int f = fb * (2 * ROWS) + (int)rank * ROWS + quarter * 32 + lane;
-      const int t0 = tt * p.tok_n + set * set_n;
-      const bool f_ok = f < p.F;  // the last feature block may reach past the matrix (zero-filled loads)
-      bf16* crow = p.C + (size_t)t0 * p.ldc + (f_ok ? f : 0);
-      // the old values of the first chunk are on their way while the main loop still runs
-      bf16 old[32];
-      {
-        const int valid = f_ok ? min(min(32, set_n), p.M - t0) : 0;
+    const int bar_set = 2 + set;
+    // phase 2 assignment: tokens e2, e2 + 8, .. of a chunk, features 8 (st & 15) .. + 7
+    const int e2 = st >> 4, fg = st & 15;
+    sp_with_chunk<true>(p.chunk, [&](auto chunk) {
+      constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4;
+      const int n_chunks = (set_n + CH - 1) / CH;
+      float* xset = xch + set * sp_set_floats(EPI, CH);
+      float* xmine = xset + quarter * QUARTER + lane;
+      const float* xrow = xset + (fg >> 2) * QUARTER + (fg & 3) * 8;
+      int it = 0;
+      for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
+        const int b = it & 1;
+        int fb, tt;
+        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        const int f = fb * (2 * ROWS) + (int)rank * ROWS + fg * 8;
+        const int t0 = tt * p.tok_n + set * set_n;
+        // tokens of this set that exist; none where the last feature block reaches past the matrix (zero-filled loads)
+        const int valid = f < p.F ? min(set_n, p.M - t0) : 0;
+        bf16* crow = p.C + (size_t)(valid > 0 ? t0 : 0) * p.ldc + (valid > 0 ? f : 0);
+        uint4 old[16];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) old[e] = e < valid ? crow[(size_t)e * p.ldc] : __float2bfloat16_rn(0.f);
-      }
-      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
-      named_bar_sync(1, 256);
-      if (!ep_ok[0]) break;  // uniform for the 256 threads
-      tc_fence_after();
-      const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
-#pragma unroll 1
-      for (int c = 0; c < n_chunks; ++c) {
-        const int w = min(32, set_n - c * 32);
-        float v[32];
-        __syncwarp();
-        sp_ld_chunk(trow + c * 32, w, v);
-        bf16* orow = crow + (size_t)(c * 32) * p.ldc;
-        const int valid = f_ok ? min(w, p.M - (t0 + c * 32)) : 0;
+        for (int i = 0; i < 16; ++i)
+          old[i] = i * 8 + e2 < valid ? *reinterpret_cast<const uint4*>(crow + (size_t)(i * 8 + e2) * p.ldc) : make_uint4(0, 0, 0, 0);
+        if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+        named_bar_sync(1, 256);
+        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        tc_fence_after();
+        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (e < valid) orow[(size_t)e * p.ldc] = __float2bfloat16_rn(v[e] + __bfloat162float(old[e]));
-        if (c + 1 < n_chunks) {  // the next chunk's old values
-          const int nvalid = f_ok ? min(min(32, set_n - (c + 1) * 32), p.M - (t0 + (c + 1) * 32)) : 0;
-          const bf16* nrow = orow + (size_t)32 * p.ldc;
+        for (int c = 0; c < 128 / CH; ++c) {
+          if (c >= n_chunks) break;
+          float v[CH];
+          __syncwarp();
+          sp_ld_chunk<CH>(trow + c * CH, min(CH, set_n - c * CH), v);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) old[e] = e < nvalid ? nrow[(size_t)e * p.ldc] : __float2bfloat16_rn(0.f);
+          for (int e = 0; e < CH; ++e) xmine[e * 32] = v[e];
+          named_bar_sync(bar_set, 128);
+#pragma unroll
+          for (int i = 0; i < CH / 8; ++i) {
+            const int e = i * 8 + e2;
+            if (c * CH + e >= valid) continue;
+            float a[8], o[8];
+            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(xrow + e * 32);
+            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(xrow + e * 32 + 4);
+            unpack8(old[c * (CH / 8) + i], o);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a[k] += o[k];
+            *reinterpret_cast<uint4*>(crow + (size_t)(c * CH + e) * p.ldc) = pack8(a);
+          }
+          named_bar_sync(bar_set, 128);  // everybody has read this chunk's values
         }
+        // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
       }
-      // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
-    }
+      return true;
+    });
   }
   tc_fence_before();
   cluster_sync_all();  // neither CTA releases tensor or shared memory while the other may still use it
@@ -628,17 +668,12 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
 bool swiglu_pair_usable(const a3_handle* h, const GemmArgs& a) {
   return h->opt[A3_OPT_SWIGLU_PAIR] != 0 && a.M > 0 && a.K % (SP_SUB * TC_BK) == 0 && a.seg[0].n % (2 * SP_FEAT) == 0 && a.seg[0].bias == nullptr;
 }
-// Measured at Llama-8B width: with several units per CTA pair (5 152 rows: 336 units on 74 pairs) this kernel hides
-// every epilogue but the last and wins (output projection 139 vs 165 us, down projection 522 vs 533 us); with at most
-// one unit per pair (804 rows: 64 units) it has nothing to hide and the 256 x 256 CTA-pair kernel is as fast or faster
-// (26 vs 28 us, 85 vs 82 us).  A3_OPT_RESIDUAL_T: 0 never, 1 by that rule (default), 2 whenever the shape allows.
+// A3_OPT_RESIDUAL_T: 0 never, otherwise whenever the shape allows.  Against the 256 x 256 tile kernel, output + down projection
+// of a layer: 513 rows 110 -> 81 us, 804 rows 116 -> 105, 1 024 rows 118 -> 119 (Llama width); 550 rows 133 -> 94, 804 rows
+// 142 -> 110 (Qwen width).
 bool residual_t_usable(const a3_handle* h, const GemmArgs& a) {
-  const int g_residual_t = h->opt[A3_OPT_RESIDUAL_T];
-  if (g_residual_t == 0 || a.M <= 0 || a.K % (SP_SUB * TC_BK) != 0 || a.nseg != 1 || a.seg[0].n % 32 != 0 || a.seg[0].bias != nullptr)
-    return false;
-  if (g_residual_t == 2) return true;
-  const int sms = h->sm_count > 0 ? h->sm_count : 148;
-  return cdiv(a.seg[0].n, 4 * SP_FEAT) * cdiv(a.M, 256) > sms / 2;
+  return h->opt[A3_OPT_RESIDUAL_T] != 0 && a.M > 0 && a.K % (SP_SUB * TC_BK) == 0 && a.nseg == 1 && a.seg[0].n % 32 == 0 &&
+         a.seg[0].bias == nullptr;
 }
 
 // Token tiling of a launch: `tiles` tiles of `n` tokens (a multiple of 16, at most 256) that divide the row count
@@ -680,19 +715,20 @@ static SpTiling choose_tiling(const a3_handle* h, int M, int n_fblocks, int pair
 
 // How many k-slices the residual GEMM of few rows is cut into (1: not at all).  With one unit per 256 features x 256
 // tokens, M <= 512 rows leave most of the 74 CTA pairs idle: a down projection of 75 rows x 3 584 features ran on 28 SMs
-// and streamed its 136 MB of weights at 1.4 TB/s.  Compared are, in clocks, the 256 x 256 tile kernel (a k-block costs its
-// 512 tensor clocks) and rounds of the split units (a k-block costs the larger of its tensor time and the arrival of its
-// operands, see choose_tiling) plus the fp32 partial sums, which are written and read once each through L2 (about 3 KB a
-// clock), at most `part_bytes` of them.  A slice is at least 1 024 deep: shorter ones are all pipeline fill.
+// and streamed its 136 MB of weights at 1.4 TB/s.  Compared are, in clocks, one round of whole units and rounds of the
+// split ones (a k-block costs the larger of its tensor time and the arrival of its operands, see choose_tiling) plus the
+// fp32 partial sums, which are written and read once each through L2 (about 3 KB a clock), at most `part_bytes` of them.
+// A slice is at least 1 024 deep: shorter ones are all pipeline fill.
 // Pinned kernel variants (a3_set_option) are compared bit for bit and therefore keep the undivided sums.
 constexpr int SP_SLICE_MIN_KB = 16;
 static bool split_allowed(const a3_handle* h) {
   return h->opt[A3_OPT_RESIDUAL_T] == 1 && h->opt[A3_OPT_QKV_T] == 1 && h->opt[A3_OPT_SWIGLU_PAIR] == 1 &&
          h->opt[A3_OPT_GEMM_TILING] == 0;
 }
-static int choose_slices(int M, int F, int K, int n_fblocks, int pairs, long long unsplit, size_t part_bytes) {
+static int choose_slices(int M, int F, int K, int n_fblocks, int pairs, size_t part_bytes) {
   const int tiles = cdiv(M, 256), n = cdiv(cdiv(M, tiles), 16) * 16, kt = K / TC_BK;
   const int per_kb = 2 * n > 256 + n ? 2 * n : 256 + n;
+  long long unsplit = (long long)kt * per_kb;
   int best = 1;
   for (int s = 2; s <= 16 && s * SP_SLICE_MIN_KB <= kt; ++s) {
     if ((size_t)s * M * F * 4 > part_bytes) break;
@@ -709,7 +745,27 @@ int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) 
   if (!split_allowed(h) || h->opt[A3_OPT_GEMM_BN_RESIDUAL] != 0 || M <= 0 || K % (SP_SUB * TC_BK) || N % 32) return 1;
   const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2, blocks = cdiv(N, 4 * SP_FEAT);
   if (blocks * cdiv(M, 256) > pairs / 2) return 1;  // the pairs are busy with whole units
-  return choose_slices(M, N, K, blocks, pairs, (long long)(K / TC_BK) * 512, part_bytes);
+  return choose_slices(M, N, K, blocks, pairs, part_bytes);
+}
+
+// Ring depth and epilogue chunk of a launch: the widest chunk among those that leave the ring deepest (a stage more is 8 %
+// at 513 rows, where 32-token chunks leave three stages of 176 tokens and 8-token chunks four).  Returns the dynamic
+// shared memory.
+static int set_stages(SpParams& p, int epi, bool split) {
+  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
+  p.stages = 0;
+  int xch = 0;
+  for (int chunk = 32; chunk >= (epi == EPI_QKV ? 16 : 8); chunk /= 2) {
+    const int x = split ? 0 : sp_xch_bytes(epi, chunk);
+    int stages = (SP_SMEM_LIMIT - x - 256 - 1024) / p.stage_bytes;
+    if (stages > SP_MAX_STAGES) stages = SP_MAX_STAGES;
+    if (stages > p.stages) {
+      p.stages = stages;
+      p.chunk = chunk;
+      xch = x;
+    }
+  }
+  return p.stages * p.stage_bytes + xch + 256 + 1024;
 }
 
 int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st) {
@@ -728,10 +784,7 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   p.group = 1;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;
-  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
-  p.stages = (SP_SMEM_LIMIT - 256 - 1024) / p.stage_bytes;
-  if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
-  const int smem_bytes = p.stages * p.stage_bytes + 256 + 1024;
+  const int smem_bytes = set_stages(p, EPI_RESIDUAL, true);
   CUtensorMap tX, tG;
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB));
@@ -746,7 +799,6 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
 template <int EPI>
 static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   constexpr int ROWS = EPI == EPI_SWIGLU ? SP_FEAT : 2 * SP_FEAT;  // output features per CTA
-  constexpr int XCH = EPI == EPI_SWIGLU ? SP_XCH_BYTES : 0;
   SpParams p{};
   p.M = a.M;
   p.K = a.K;
@@ -764,11 +816,7 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   p.C = a.C;
   p.ldc = a.ldc;
   p.status = h->dev_status;
-  // as many ring stages as fit beside the exchange buffers
-  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
-  p.stages = (SP_SMEM_LIMIT - XCH - 256 - 1024) / p.stage_bytes;
-  if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
-  const int smem_bytes = p.stages * p.stage_bytes + XCH + 256 + 1024;
+  const int smem_bytes = set_stages(p, EPI, false);
   CUtensorMap tX, tG, tU;
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, ROWS, EPI == EPI_SWIGLU ? 1 : SP_SUB));
@@ -828,10 +876,7 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   p.layout = h->m.rope_layout;
   p.max_pos = h->m.max_positions;
   p.tab = h->rope_tab;
-  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
-  p.stages = (SP_SMEM_LIMIT - SP_QKV_EXTRA - 256 - 1024) / p.stage_bytes;
-  if (p.stages > SP_MAX_STAGES) p.stages = SP_MAX_STAGES;
-  const int smem_bytes = p.stages * p.stage_bytes + SP_QKV_EXTRA + 256 + 1024;
+  const int smem_bytes = set_stages(p, EPI_QKV, false);
   CUtensorMap tX, tW[3];
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   for (int s = 0; s < 3; ++s) {
