@@ -43,31 +43,46 @@ struct AtcLayout {
   static constexpr int SMEM_BYTES = XCH_OFF + 2048;      // the dynamic shared window must be 1024-byte aligned (checked)
 };
 
-// One unit of work: a 128-row tile of one KV head and one segment of its key tiles.
-struct AtcItem {
-  int g, r0, maxpos, minpos;
+// One unit of work: a 128-row tile of one KV head and one segment of its key tiles.  Where it lies follows from its number
+// alone; how many key tiles it has from the positions of its rows.
+struct AtcPlace {
+  int g, r0;
+  int z;  // segment index
+};
+struct AtcItem : AtcPlace {
+  int maxpos, minpos;
   int nkt_all;   // key tiles the row tile needs in total
   int kt0, nkt;  // this segment: first key tile and count
-  int z;         // segment index
   bool valid;    // the segment exists for this row tile
   bool partial;  // the row tile has several segments: leave unnormalised partial results for the combine kernel
 };
 
 // Items are numbered longest row tile first (rows are sorted by position, so the last tile sees the most keys),
 // then segment, then KV head.
-__device__ __forceinline__ AtcItem atc_item(int i, const int32_t* __restrict__ pos, int M, int G, int Hkv, int kv_len,
-                                            int row_tiles, int n_split, int tiles_per_split) {
-  AtcItem it;
+__device__ __forceinline__ AtcPlace atc_place(int i, int Hkv, int row_tiles, int n_split) {
+  AtcPlace pl;
   const int per_tile = n_split * Hkv;
   const int tile = row_tiles - 1 - i / per_tile;
   const int rem = i % per_tile;
-  it.z = rem / Hkv;
-  it.g = rem % Hkv;
-  it.r0 = tile * ATC_BM;
+  pl.z = rem / Hkv;
+  pl.g = rem % Hkv;
+  pl.r0 = tile * ATC_BM;
+  return pl;
+}
+// `unsplit`: every item has at least one key tile, also when no key is visible (invalid positions): all of it is masked, and
+// the output is zero.  Its K tile may then be requested before the positions are known.
+__device__ __forceinline__ AtcItem atc_item(const AtcPlace& pl, const int32_t* __restrict__ pos, int M, int G, int kv_len, int tiles_per_split,
+                                            bool unsplit) {
+  AtcItem it;
+  static_cast<AtcPlace&>(it) = pl;
   const int last_tok = min(M - 1, (it.r0 + ATC_BM - 1) / G);
   it.maxpos = min(pos[last_tok], kv_len - 1);
   it.minpos = pos[it.r0 / G];
   it.nkt_all = it.maxpos < 0 ? 0 : it.maxpos / ATC_BN + 1;
+  if (unsplit && it.nkt_all == 0) {
+    it.nkt_all = 1;
+    it.maxpos = it.minpos = -1;
+  }
   const int n_active = (it.nkt_all + tiles_per_split - 1) / tiles_per_split;
   it.valid = it.z < max(n_active, 1);
   it.kt0 = it.z * tiles_per_split;
@@ -130,6 +145,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     return i < n_items ? i : -1;
   };
   const int rounds = (n_items + C - 1) / C;
+  // The first item's place (a chain of divisions) is worked out before the preceding kernel has finished; then its Q rows
+  // and its first K tile are requested without waiting for the positions: of the 13 400 clocks that a launch with one key
+  // tile took from there, 5 600 went by before its first product (3 900 now).
+  const AtcPlace first = atc_place(item_index(0) < 0 ? 0 : item_index(0), Hkv, row_tiles, n_split);
+  const bool k_ahead = n_split == 1 && item_index(0) >= 0;  // an unsplit item starts at key tile 0
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < L::KV_STAGES; ++i) {
@@ -170,21 +190,28 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
     uint32_t s = 0, ph = 0;  // ring stage and phase, kept by counting
     bool ok = true;
+    auto load_k = [&](int g, int row) {
+      const uint32_t sk = base + L::KV_OFF + s * L::KV_STAGE;
+      if (elect_one()) {
+        mbar_expect_tx(k_full(s), L::KV_STAGE / 2);
+#pragma unroll
+        for (int j = 0; j < D / 64; ++j) tma_load_2d(sk + j * L::SUB, &tmK, g * D + 64 * j, row, k_full(s));
+      }
+      __syncwarp();
+    };
+    if (k_ahead) load_k(first.g, 0);
     for (int r = 0; r < rounds && ok; ++r) {
       const int i = item_index(r);
       if (i < 0) continue;
-      const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
+      const AtcItem w = atc_item(r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split), pos, M, G, kv_len, tiles_per_split, n_split == 1);
       const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0), row0 = __shfl_sync(0xffffffffu, w.kt0 * ATC_BN, 0);
       for (int kt = 0; kt < nkt; ++kt) {
-        const uint32_t sk = base + L::KV_OFF + s * L::KV_STAGE, sv = sk + (D / 64) * L::SUB;
-        ok = mbar_wait_warp(k_empty(s), ph ^ 1, abort_flag, status);
-        if (!ok) break;
-        if (elect_one()) {
-          mbar_expect_tx(k_full(s), L::KV_STAGE / 2);
-#pragma unroll
-          for (int j = 0; j < D / 64; ++j) tma_load_2d(sk + j * L::SUB, &tmK, w.g * D + 64 * j, row0 + kt * ATC_BN, k_full(s));
+        const uint32_t sv = base + L::KV_OFF + s * L::KV_STAGE + (D / 64) * L::SUB;
+        if (!(k_ahead && r == 0 && kt == 0)) {
+          ok = mbar_wait_warp(k_empty(s), ph ^ 1, abort_flag, status);
+          if (!ok) break;
+          load_k(w.g, row0 + kt * ATC_BN);
         }
-        __syncwarp();
         if (want_o) {  // the statistics-only pass never reads V
           ok = mbar_wait_warp(v_empty(s), ph ^ 1, abort_flag, status);
           if (!ok) break;
@@ -236,7 +263,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     for (int r = 0; r < rounds && ok; ++r) {
       const int i = item_index(r);
       if (i < 0) continue;
-      const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
+      const AtcItem w = atc_item(r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split), pos, M, G, kv_len, tiles_per_split, n_split == 1);
       const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0);
       if (nkt == 0) continue;
       ok = mbar_wait_warp(q_ready, qn & 1, abort_flag, status);
@@ -316,17 +343,22 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     for (int r = 0; r < rounds && ok; ++r) {
       const int i = item_index(r);
       if (i < 0) continue;
-      const AtcItem w = atc_item(i, pos, M, G, Hkv, kv_len, row_tiles, n_split, tiles_per_split);
-      if (!w.valid) continue;
-      const int fr = w.r0 + row;
+      const AtcPlace pl = r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split);
+      const int fr = pl.r0 + row;
       const bool row_ok = fr < rows_total;
       const int tok = row_ok ? fr / G : 0;
-      const int hq = w.g * G + (row_ok ? fr % G : 0);
+      const int hq = pl.g * G + (row_ok ? fr % G : 0);
+      uint4 qv[D / 16];  // this thread's half of the Q row, on its way while the positions are read
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c)
+        qv[c] = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + ((size_t)tok * Hq + hq) * D) + half * (D / 16) + c) : make_uint4(0, 0, 0, 0);
+      const AtcItem w = atc_item(pl, pos, M, G, kv_len, tiles_per_split, n_split == 1);
+      if (!w.valid) continue;
       const int lim = row_ok ? min(pos[tok], kv_len - 1) : -1;
       const size_t prow = ((size_t)w.z * Hkv + w.g) * (size_t)rows_pad + fr;  // partial-result row
 
       if (w.nkt == 0) {
-        // no visible key at all (only with invalid positions): defined output, no pipeline work
+        // no visible key in this segment (only with invalid positions): defined output, no pipeline work
         if (row_ok && want_o && !w.partial) {
           uint4* dst = reinterpret_cast<uint4*>(o + ((size_t)tok * Hq + hq) * D + half * (D / 2));
 #pragma unroll
@@ -340,12 +372,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       // Q row -> shared memory, swizzled K-major sub-tiles (each thread copies half of the row's 16-byte chunks).
       // The previous item's S MMAs have all completed (their last s_full was waited for), so the Q buffer is free.
       {
-        const uint4* src = reinterpret_cast<const uint4*>(q + ((size_t)tok * Hq + hq) * D);
 #pragma unroll
         for (int cc = 0; cc < D / 16; ++cc) {
           const int c = half * (D / 16) + cc;
-          uint4 v = row_ok ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
-          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (c / 8) * L::SUB + swz(row, c % 8)) = v;
+          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (c / 8) * L::SUB + swz(row, c % 8)) = qv[cc];
         }
         fence_async_smem();
         mbar_arrive(q_ready);
@@ -363,69 +393,59 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const uint32_t ts = tmem_s0 + (it & 1) * 128 + lane_addr + half * 64;
         const int key0 = (w.kt0 + kt) * ATC_BN + half * 64;  // first key of this thread's columns
         const bool need_mask = (w.kt0 + kt) * ATC_BN + ATC_BN - 1 > w.minpos;
-        // The row's 64 logits of this thread, raw, into registers
         float x[64];
-        ld32(ts, x);
-        ld32(ts + 32, x + 32);
-        wait_ld();
+        // The row's 64 logits of this thread into registers, those of keys the row does not see as -inf (which the scale, the
+        // maximum and ex2 carry through: one path for masked and whole tiles, since every instruction that a launch meets
+        // for the first time is fetched from far away)
+        auto load_logits = [&]() {
+          ld32(ts, x);
+          ld32(ts + 32, x + 32);
+          wait_ld();
+          if (need_mask) {
+            const int seen = lim - key0;  // columns 0 .. seen
+#pragma unroll
+            for (int e = 0; e < 64; ++e) x[e] = e <= seen ? x[e] : -INFINITY;
+          }
+        };
+        load_logits();
         if (want_o && it >= 2) {
           // keeps every phase of p_free[b] observed in order, so that the parity waits below cannot mistake an older
           // completion for the one they mean (P V of running tile it-2 finished long ago: this does not block)
           ok = __all_sync(0xffffffffu, mbar_wait(p_free(it & 1), ((it >> 1) & 1) ^ 1, abort_flag, status));
           if (!ok) break;
         }
-        // maximum of the scaled, masked logits (first tile and the rare re-reference only)
-        auto row_max = [&]() {
+        auto row_max = [&]() {  // maximum of the scaled logits (first tile and the rare re-reference only)
           float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int e = 0; e < 64; ++e) {
-            const float t = (need_mask && key0 + e > lim) ? -INFINITY : x[e] * scale_log2;
-            m4[e & 3] = fmaxf(m4[e & 3], t);
-          }
-          return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-        };
-        // x <- exp2(x * scale - m_ref) (one FMA and one ex2.approx per element; ex2 maps -inf to +0); returns the sum
-        auto to_probabilities = [&]() {
-          float ls[4] = {0.f, 0.f, 0.f, 0.f};
-          const float neg_ref = -m_ref;
-          if (need_mask) {
-#pragma unroll
-            for (int e = 0; e < 64; ++e) {
-              float t = fmaf(x[e], scale_log2, neg_ref);
-              if (key0 + e > lim) t = -INFINITY;
-              x[e] = ex2_approx(t);
-              ls[e & 3] += x[e];
-            }
-          } else {
-            // packed fp32 pairs (fma.rn.f32x2 / add.rn.f32x2): half the issue slots for the FMA and the sum
-            const float2 sc2 = make_float2(scale_log2, scale_log2), nr2 = make_float2(neg_ref, neg_ref);
-            float2 s2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-            for (int e = 0; e < 64; e += 2) {
-              const float2 t = __ffma2_rn(make_float2(x[e], x[e + 1]), sc2, nr2);
-              x[e] = ex2_approx(t.x);
-              x[e + 1] = ex2_approx(t.y);
-              s2[(e >> 1) & 1] = __fadd2_rn(s2[(e >> 1) & 1], make_float2(x[e], x[e + 1]));
-            }
-            ls[0] = s2[0].x, ls[1] = s2[0].y, ls[2] = s2[1].x, ls[3] = s2[1].y;
-          }
-          return (ls[0] + ls[1]) + (ls[2] + ls[3]);
+          for (int e = 0; e < 64; ++e) m4[e & 3] = fmaxf(m4[e & 3], x[e]);
+          return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * scale_log2;
         };
         if (kt == 0) {
           const float mx = row_max();
           m_ref = mx == -INFINITY ? 0.f : mx;
         }
-        float lsum = to_probabilities();
-        // No maximum is tracked on the way: a logit far above the reference shows in the sum (each of the 64 terms
-        // is at most the largest one), and anything below 2^16 is harmless for bf16 P and the fp32 accumulators.
-        // Above it - rare - the reference is raised to the tile's true maximum, the output and the sum so far are
-        // rescaled, and the tile is redone from the logits still in tensor memory.
-        if (kt > 0 && __any_sync(0xffffffffu, !(lsum <= OVERFLOW_GUARD))) {
-          ld32(ts, x);
-          ld32(ts + 32, x + 32);
-          wait_ld();
-          const float mx = row_max();
-          const float raise = fmaxf(mx - m_ref, 0.f);  // lanes that triggered nothing keep their reference (raise 0)
+        float lsum;
+#pragma unroll 1
+        for (bool redone = false;; redone = true) {
+          // x <- exp2(x * scale - m_ref) (one FMA and one ex2.approx per element; ex2 maps -inf to +0) and their sum, in packed
+          // fp32 pairs (fma.rn.f32x2 / add.rn.f32x2): half the issue slots for the FMA and the sum
+          const float2 sc2 = make_float2(scale_log2, scale_log2), nr2 = make_float2(-m_ref, -m_ref);
+          float2 s2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+          for (int e = 0; e < 64; e += 2) {
+            const float2 t = __ffma2_rn(make_float2(x[e], x[e + 1]), sc2, nr2);
+            x[e] = ex2_approx(t.x);
+            x[e + 1] = ex2_approx(t.y);
+            s2[(e >> 1) & 1] = __fadd2_rn(s2[(e >> 1) & 1], make_float2(x[e], x[e + 1]));
+          }
+          lsum = (s2[0].x + s2[0].y) + (s2[1].x + s2[1].y);
+          // No maximum is tracked on the way: a logit far above the reference shows in the sum (each of the 64 terms
+          // is at most the largest one), and anything below 2^16 is harmless for bf16 P and the fp32 accumulators.
+          // Above it - rare - the reference is raised to the tile's true maximum, the output and the sum so far are
+          // rescaled, and the tile is redone from the logits still in tensor memory.
+          if (kt == 0 || redone || !__any_sync(0xffffffffu, !(lsum <= OVERFLOW_GUARD))) break;
+          load_logits();
+          const float raise = fmaxf(row_max() - m_ref, 0.f);  // lanes that triggered nothing keep their reference (raise 0)
           const float f = exp2f(-raise);
           m_ref += raise;
           l_run *= f;
@@ -446,8 +466,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             wait_st();
           }
-          lsum = to_probabilities();
         }
+        if (!ok) break;
         l_run += lsum;
         if (want_o) {
           // P as bf16 pairs over the first 32 of this thread's 64 S columns (all of them are in registers by now):
@@ -462,17 +482,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           wait_st();
           if (w.kt0 + kt == w.nkt_all - 1 && half == 0) {
             // slots beyond the row tile's last visible key may hold anything: they get probability zero, and zero
-            // times a non-finite value would still poison the product, so clear those V rows of the last tile
-            // (thread `row` of the first half clears key `row`)
+            // times a non-finite value would still poison the product, so clear those V rows of the last tile (the 128
+            // threads of the first half, eight to a row: a row per thread puts all of a warp's stores on four banks)
             const int first_bad = w.maxpos - (w.kt0 + kt) * ATC_BN + 1;
             const int vs = it % L::KV_STAGES;
             const bool landed = mbar_wait(v_full(vs), (it / L::KV_STAGES) & 1, abort_flag, status);  // the V tile must have landed before rows of it are cleared
-            if (landed && row >= first_bad) {
+            if (landed) {
               unsigned char* sv = base_ptr + L::KV_OFF + vs * L::KV_STAGE + (D / 64) * L::SUB;
+#pragma unroll 1
+              for (int v = max(first_bad, 0) * 8 + row; v < ATC_BN * 8; v += 128)
 #pragma unroll
-              for (int j = 0; j < D / 64; ++j)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(sv + j * L::SUB + row * 128 + c * 16) = make_uint4(0, 0, 0, 0);
+                for (int j = 0; j < D / 64; ++j) *reinterpret_cast<uint4*>(sv + j * L::SUB + v * 16) = make_uint4(0, 0, 0, 0);
             }
             fence_async_smem();
           }
@@ -547,6 +567,8 @@ attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int
   const int rows_total = M * G;
   const int fr = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int g = blockIdx.y, lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_launch_dependents();
   if (fr >= rows_total) return;
   const int r0 = (fr / ATC_BM) * ATC_BM;
   const int last_tok = min(M - 1, (r0 + ATC_BM - 1) / G);
@@ -694,8 +716,8 @@ int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M,
   A3_LAUNCHED();
   if (n_split > 1) {
     dim3 cgrid(cdiv((long long)M * G, 4), Hkv);
-    if (D == 128) attention_combine_kernel<128><<<cgrid, 128, 0, st>>>(pos, M, kv_len, Hq, Hkv, tiles_per_split, rows_pad, part_o, part_ml, o, lse);
-    else attention_combine_kernel<64><<<cgrid, 128, 0, st>>>(pos, M, kv_len, Hq, Hkv, tiles_per_split, rows_pad, part_o, part_ml, o, lse);
+    A3_CUDA(launch_pdl(D == 128 ? attention_combine_kernel<128> : attention_combine_kernel<64>, cgrid, dim3(128), 0, st, pos, M, kv_len, Hq, Hkv,
+                       tiles_per_split, rows_pad, part_o, part_ml, o, lse));
     A3_LAUNCHED();
   }
   return A3_OK;

@@ -410,12 +410,12 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           const int first_bad = max(w.maxpos[0], w.maxpos[1]) - key0 + 1;
           const uint32_t vit = it + t;
           const bool landed = mbar_wait(v_full(vit & 1), (vit >> 1) & 1, abort_flag, status);
-          if (landed && row >= first_bad) {
+          if (landed) {  // eight threads to a row (a row per thread puts all of a warp's stores on four banks)
             unsigned char* sv = base_ptr + L::V_OFF + (vit & 1) * L::TILE;
+#pragma unroll 1
+            for (int v = max(first_bad, 0) * 8 + row; v < ATC_BN * 8; v += 128)
 #pragma unroll
-            for (int j = 0; j < D / 64; ++j)
-#pragma unroll
-              for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(sv + j * L::SUB + row * 128 + c * 16) = make_uint4(0, 0, 0, 0);
+              for (int j = 0; j < D / 64; ++j) *reinterpret_cast<uint4*>(sv + j * L::SUB + v * 16) = make_uint4(0, 0, 0, 0);
           }
           fence_async_smem();
         }
