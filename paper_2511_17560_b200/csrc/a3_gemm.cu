@@ -455,9 +455,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();  // the peer's barriers exist before anything is signalled on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
   // as in the persistent kernel: the weights may be read before the preceding kernel has finished (see GemmArgs)
-  if (warp >= 2 || !p.early) pdl_wait();
+  if (warp != 0 || !p.early) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own rows of A, own half of B
@@ -481,7 +483,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       };
       const int early = p.early ? min(STAGES, KT) : 0;
       for (int kb = 0; kb < early; ++kb) load_weights(kb, kb);
-      if (p.early) pdl_wait();
+      if (p.early) {
+        pdl_wait();
+        pdl_launch_dependents();
+      }
       int issued = early;
       for (int kb = 0; kb < KT; ++kb) {
         const int s = kb % STAGES;

@@ -15,8 +15,9 @@
 //     token tile), accumulators are double-buffered in tensor memory (2 x N <= 512 columns), so the epilogue of a
 //     unit runs under the main loop of the next one; a ring stage holds two k-blocks (one barrier hand-shake and one
 //     commit per eight instructions: the single issuing thread, not the pipe, was the limit with one).
-// SwiGLU epilogue: the two halves meet through shared memory (see below); a warp writes 32 consecutive features of
-// one token (64 bytes) per instruction.  Measured at Llama-8B width: tensor pipe 97 % active at 5 152 rows.
+// Epilogues: accumulator lanes are features, so values go through shared memory once, where gate meets up and a rotation
+// pair its other half, and leave token by token in 16-byte stores.  Measured at Llama-8B width: tensor pipe 97 % active at
+// 5 152 rows.
 // No load uses cluster multicast.  Every wait is bounded (see a3_tc.cuh): a waiter that gives up raises the CTA's
 // abort flag and the device status bit, all roles leave their loops, tensor memory is released and the CTA returns.
 #include <cuda.h>
@@ -34,14 +35,11 @@ constexpr int SP_SUB = 2;  // k-blocks of 64 per ring stage: one barrier hand-sh
 constexpr int SP_FEAT = 64;                              // features per CTA (64 gate lanes + 64 up lanes)
 constexpr int SP_A_BYTES = 2 * SP_FEAT * TC_BK * 2;      // 16 KiB: gate rows, then up rows
 // Exchange buffers of the epilogues, which take `chunk` tokens at a time (32 where that costs no ring stage, else 16 or 8: see
-// set_stages).  SwiGLU: per warp set two buffers of float [chunk][64 features]; QKV and residual: per warp set four
-// quarters of [chunk][32 features] fp32, 16 bytes apart in the banks.
-__host__ __device__ constexpr int sp_set_floats(int epi, int chunk) {
-  return epi == EPI_SWIGLU ? 2 * chunk * SP_FEAT : 4 * (chunk * 32 + 4);
-}
-// both sets, 256-byte aligned, and for QKV the checked positions of a chunk's tokens per set behind them
-__host__ __device__ constexpr int sp_xch_floats_bytes(int epi, int chunk) { return (2 * sp_set_floats(epi, chunk) * 4 + 255) & ~255; }
-__host__ __device__ constexpr int sp_xch_bytes(int epi, int chunk) { return sp_xch_floats_bytes(epi, chunk) + (epi == EPI_QKV ? 256 : 0); }
+// set_stages): per warp set four quarters of [chunk][32 lanes] fp32, 16 bytes apart in the banks.
+__host__ __device__ constexpr int sp_set_floats(int chunk) { return 4 * (chunk * 32 + 4); }
+// both sets, 256-byte aligned, and for QKV the checked positions of each set's tokens behind them
+__host__ __device__ constexpr int sp_xch_floats_bytes(int chunk) { return (2 * sp_set_floats(chunk) * 4 + 255) & ~255; }
+__host__ __device__ constexpr int sp_xch_bytes(int epi, int chunk) { return sp_xch_floats_bytes(chunk) + (epi == EPI_QKV ? 1024 : 0); }
 constexpr int SP_SMEM_LIMIT = 227 * 1024;
 
 struct SpParams {
@@ -72,9 +70,6 @@ struct SpParams {
 __device__ __forceinline__ void named_bar_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-__device__ __forceinline__ void named_bar_arrive(int id, int threads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 // arrives on the barrier at the same shared-memory offset in CTA `cta` of the cluster
 __device__ __forceinline__ void mbar_arrive_in_cta(uint32_t bar, uint32_t cta) {
   uint32_t remote;
@@ -91,14 +86,34 @@ __device__ __forceinline__ void sp_ld_chunk(uint32_t taddr, int w, float* v) {
     for (int i = 0; i < CH / 8; ++i)
       if (w >= 8 * i + 8) tc_ld8(taddr + 8 * i, v + 8 * i);
   }
-  tc_wait_ld();
+  tc_wait_ld_of<CH>(v);
 }
 // f(std::integral_constant<int, chunk>) for the chunk of this launch
 template <bool MAY_8, typename F>
 __device__ __forceinline__ bool sp_with_chunk(int chunk, F f) {
   if (chunk == 32) return f(std::integral_constant<int, 32>());
-  if (!MAY_8 || chunk == 16) return f(std::integral_constant<int, 16>());
-  return f(std::integral_constant<int, 8>());
+  if constexpr (MAY_8) {
+    if (chunk == 8) return f(std::integral_constant<int, 8>());
+  }
+  return f(std::integral_constant<int, 16>());
+}
+
+// Stores of the first `valid` of CH tokens, eight at a time without a branch in between: a branch around every store makes
+// a block of its own of every token's arithmetic, and its latency (exchange, exponential, reciprocal: 160 clocks) was paid
+// token by token - 5 000 clocks for the 32 of a chunk.
+template <int CH, typename F>
+__device__ __forceinline__ void sp_store_tokens(int valid, F store) {
+#pragma unroll
+  for (int i = 0; i < CH; i += 8) {
+    if (valid >= i + 8) {
+#pragma unroll
+      for (int e = i; e < i + 8; ++e) store(e);
+    } else {
+#pragma unroll
+      for (int e = i; e < i + 8; ++e)
+        if (e < valid) store(e);
+    }
+  }
 }
 
 // Unit u -> (feature block, token tile).  Units are numbered in groups of `group` feature blocks, token tiles next,
@@ -178,8 +193,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tmem_full(b), 1);
-      // SwiGLU: the gate warps and the up warps of both warp sets of each CTA; residual and QKV: every epilogue warp
-      mbar_init(tmem_empty(b), EPI == EPI_SWIGLU && !SPLIT ? 8 : 16);
+      mbar_init(tmem_empty(b), 16);  // every epilogue warp of both CTAs
     }
     abort_flag[0] = 0;
     abort_flag[1] = 0;
@@ -195,11 +209,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   cluster_sync_all();  // the peer's barriers exist before anything is signalled on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
-  // Only the threads that touch what earlier kernels wrote wait for them: the producer before the first token tile, the
-  // epilogue warps.  The weights are nobody's output, so the producer has already filled the ring's weight half by then
-  // (16 KiB x 2 per stage and CTA, most of what a launch of few rows spends its first microseconds on).
-  if (warp >= 2 || !p.early) pdl_wait();
+  // The weights are nobody's output: the producer fills the ring's weight half before it waits for the preceding kernel
+  // (16 KiB x 2 per stage and CTA, most of what a launch of few rows spends its first microseconds on); everybody else
+  // waits here.
+  if (warp != 0 || !p.early) {
+    pdl_wait();
+    pdl_launch_dependents();  // from here on: a launch never runs ahead of more than the one before it
+  }
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own gate/up rows, own half of the token tile
@@ -260,6 +276,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           for (int i = 0; i < early; ++i) load_weights(i, kb0 + i * SP_SUB);
           issued = early;
           pdl_wait();
+          pdl_launch_dependents();
         }
         for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
           if (kbg >= early) {
@@ -382,100 +399,93 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         __syncwarp();
         sp_ld_chunk<32>(trow + c * 32, w, v);
         const int valid = f < p.F ? min(w, p.M - (t0 + c * 32)) : 0;
-#pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (e < valid) prow[(size_t)(c * 32 + e) * p.F] = v[e];
+        float* pc = prow + (size_t)(c * 32) * p.F;
+        sp_store_tokens<32>(valid, [&](int e) { pc[(size_t)e * p.F] = v[e]; });
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
     }
   } else if (EPI == EPI_SWIGLU) {
-    // ---------------- epilogue: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31.
-    // Lanes 0..63 hold the gate rows of this CTA's 64 features, lanes 64..127 their up rows.  Warp set 0 (warps
-    // 2..5) takes the first half of the token columns, set 1 (warps 6..9) the second.  Inside a set the two halves of
-    // silu(g) * u meet through shared memory, 32 tokens at a time, in two buffers: on even chunks the up warps write
-    // buffer 0 and the gate warps combine and store, on odd chunks the gate warps write buffer 1 and the up warps
-    // combine and store.  Named barriers of a set: "buffer written" (writers arrive, readers wait) and "buffer read"
-    // (readers arrive, writers wait before writing it again) per buffer; each is used by the same 64 + 64 threads in
-    // strict alternation, so no phase can be overtaken.
+    // ---------------- epilogue, silu(gate) * up: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31: lanes
+    // 0..63 hold the gate rows of this CTA's 64 features, lanes 64..127 their up rows.  Warp set 0 (warps 2..5) takes the
+    // first half of the token columns, set 1 (warps 6..9) the second, a chunk at a time in two phases as in the QKV
+    // epilogue: feature-major out of tensor memory into shared memory, then token-major, a thread taking 8 features of a
+    // token: their gates, their ups and one 16-byte store.
     const int quarter = warp & 3;
     const int set = (warp - 2) >> 2;
-    const bool up_warp = quarter >= 2;
-    const int feat = (quarter & 1) * 32 + lane;  // feature within this CTA's 64
     const int ep_tid = (warp - 2) * 32 + lane;
-    const int set_n = p.tok_n >> 1;              // token columns of a set (multiple of 8)
-    const int my_units = pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0;
-    const int bar_written = 2 + set * 4, bar_read = 4 + set * 4, bar_group = 10 + set * 2 + (up_warp ? 0 : 1);
+    const int st = quarter * 32 + lane;  // thread within the set
+    const int set_n = p.tok_n >> 1;      // token columns of a set (multiple of 8)
+    const int bar_set = 2 + set;
     sp_with_chunk<true>(p.chunk, [&](auto chunk) {
-      constexpr int CH = decltype(chunk)::value;
-      const int n_chunks = (set_n + CH - 1) / CH, total_chunks = my_units * n_chunks;
-      float* xset = xch + set * sp_set_floats(EPI, CH);
-      int it = 0, cc = 0;
+      constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4, PASSES = (CH + 15) / 16;
+      const int n_chunks = (set_n + CH - 1) / CH;
+      float* xset = xch + set * sp_set_floats(CH);
+      float* xmine = xset + quarter * QUARTER + lane;
+      // phase 2 assignment: token e2 (+ 16 per pass; half of the threads idle in chunks of 8), features 8 (st & 7) .. + 7
+      const int e2 = st >> 3, fg = st & 7;
+      const float* xg = xset + (fg >> 2) * QUARTER + (fg & 3) * 8;
+      const float* xu = xg + 2 * QUARTER;
+      int it = 0;
       for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
         const int b = it & 1;
+        int fb, tt;
+        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        const int t0 = tt * p.tok_n + set * set_n;
+        const int valid = min(set_n, p.M - t0);  // tokens of this set that exist (may be <= 0)
+        bf16* out = p.C + (size_t)max(t0, 0) * p.ldc + fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + fg * 8;
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
         tc_fence_after();
         const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
-        int fb, tt;
-        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
-        const int f = fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + feat;
-        const int t0 = tt * p.tok_n + set * set_n;
-        bf16* out = p.C + f;
 #pragma unroll 1
-        for (int c = 0; c < n_chunks; ++c, ++cc) {
-          const int buf = cc & 1;
-          const int w = min(CH, set_n - c * CH);
-          float* xb = xset + buf * (CH * SP_FEAT);
+        for (int c = 0; c < n_chunks; ++c) {
           float v[CH];
           __syncwarp();
-          sp_ld_chunk<CH>(trow + c * CH, w, v);
-          const bool writer = up_warp == (buf == 0);
-          if (writer) {
-            if (cc >= 2) named_bar_sync(bar_read + buf, 128);  // the readers are done with what this buffer held
-            if (w == CH) {
+          sp_ld_chunk<CH>(trow + c * CH, min(CH, set_n - c * CH), v);
 #pragma unroll
-              for (int e = 0; e < CH; ++e) xb[e * SP_FEAT + feat] = v[e];
-            } else {
+          for (int e = 0; e < CH; ++e) xmine[e * 32] = v[e];
+          named_bar_sync(bar_set, 128);
+          uint4 r[PASSES];
 #pragma unroll
-              for (int e = 0; e < CH; ++e)
-                if (e < w) xb[e * SP_FEAT + feat] = v[e];
-            }
-            named_bar_arrive(bar_written + buf, 128);
-          } else {
-            named_bar_sync(bar_written + buf, 128);
-            bf16* orow = out + (size_t)(t0 + c * CH) * p.ldc;
-            const int valid = min(w, p.M - (t0 + c * CH));  // tokens of this chunk that exist
+          for (int pass = 0; pass < PASSES; ++pass) {
+            const int e = min(e2 + 16 * pass, CH - 1);
+            float g[8], up[8];
+            *reinterpret_cast<float4*>(g) = *reinterpret_cast<const float4*>(xg + e * 32);
+            *reinterpret_cast<float4*>(g + 4) = *reinterpret_cast<const float4*>(xg + e * 32 + 4);
+            *reinterpret_cast<float4*>(up) = *reinterpret_cast<const float4*>(xu + e * 32);
+            *reinterpret_cast<float4*>(up + 4) = *reinterpret_cast<const float4*>(xu + e * 32 + 4);
 #pragma unroll
-            for (int e = 0; e < CH; ++e) {
-              const float o = xb[e * SP_FEAT + feat];
-              const float g = up_warp ? o : v[e], uv = up_warp ? v[e] : o;
-              const float r = silu_mul(g, uv);
-              if (e < valid) orow[(size_t)e * p.ldc] = __float2bfloat16_rn(r);
-            }
-            if (cc + 2 < total_chunks) named_bar_arrive(bar_read + buf, 128);  // nobody waits for the last two
+            for (int k = 0; k < 8; ++k) g[k] = silu_mul(g[k], up[k]);
+            r[pass] = pack8(g);
           }
+#pragma unroll
+          for (int pass = 0; pass < PASSES; ++pass) {
+            const int e = e2 + 16 * pass;
+            if (e < CH && c * CH + e < valid) *reinterpret_cast<uint4*>(out + (size_t)(c * CH + e) * p.ldc) = r[pass];
+          }
+          named_bar_sync(bar_set, 128);  // everybody has read this chunk's values
         }
-        // this half of the set has read its part of the accumulator (wait::ld in sp_ld_chunk): one arrival per half,
-        // set and CTA on the leader's barrier hands it back to the MMA issuer
+        // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
-        named_bar_sync(bar_group, 64);
-        if (lane == 0 && (quarter == 0 || quarter == 2)) mbar_arrive_in_cta(tmem_empty(b), 0);
+        __syncwarp();
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
       }
       return true;
     });
   } else if (EPI == EPI_QKV) {
     // ---------------- epilogue, q / k / v heads: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31,
     // lane = feature of this CTA's head; warp set 0 (warps 2..5) takes the first half of the token columns, set 1 the
-    // second.  32 tokens at a time, in two phases around a named barrier of the set's 128 threads:
-    //   1. feature-major: every warp reads its 32 features x 32 tokens from tensor memory, adds the bias and parks the
-    //      values in shared memory; the first warp also fetches and checks the tokens' positions;
+    // second.  While the unit's main loop runs, the set fetches and checks the positions of its tokens and the table rows
+    // of its first chunk.  Then a chunk of tokens at a time, in two phases around a named barrier of the set's 128 threads:
+    //   1. feature-major: every warp reads its 32 features x chunk from tensor memory, adds the bias and parks the
+    //      values in shared memory;
     //   2. token-major: a thread takes 8 consecutive features of the head's first half and the 8 that lie 64 further of
-    //      ONE token (both halves of its rotation pairs, whichever the pairing), rotates them with 16-byte loads of the
-    //      token's table row and writes two 16-byte vectors: a warp stores 512 contiguous-by-row bytes per instruction
-    //      where a lane-per-feature epilogue stores 64.
+    //      ONE token (both halves of its rotation pairs, whichever the pairing), rotates them with the token's table row,
+    //      fetched a chunk ahead in 16-byte loads, and writes two 16-byte vectors: a warp stores 512 contiguous-by-row
+    //      bytes per instruction where a lane-per-feature epilogue stores 64.
     const int quarter = warp & 3;
     const int set = (warp - 2) >> 2;
     const int ep_tid = (warp - 2) * 32 + lane;
@@ -483,11 +493,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int set_n = p.tok_n >> 1;
     const int bar_set = 2 + set;
     sp_with_chunk<false>(p.chunk, [&](auto chunk) {
-      constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4;
+      constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4, PASSES = CH / 16;
       const int n_chunks = (set_n + CH - 1) / CH;
-      float* xset = xch + set * sp_set_floats(EPI, CH);
-      int* posbuf = reinterpret_cast<int*>(base_ptr + xch_off + sp_xch_floats_bytes(EPI, CH)) + set * 32;
-      // phase 2 assignment: token e2 (+16 in the second pass), features f0 .. f0 + 7 and 64 + f0 .. 64 + f0 + 7
+      float* xset = xch + set * sp_set_floats(CH);
+      int* posbuf = reinterpret_cast<int*>(base_ptr + xch_off + sp_xch_floats_bytes(CH)) + set * 128;
+      // phase 2 assignment: token e2 (+ 16 per pass), features f0 .. f0 + 7 and 64 + f0 .. 64 + f0 + 7
       const int e2 = st >> 3, f0 = (st & 7) * 8;
       const float* xlo = xset + (f0 >> 5) * QUARTER + (f0 & 31);
       const float* xhi = xset + (2 + (f0 >> 5)) * QUARTER + (f0 & 31);
@@ -506,6 +516,33 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         const int t0 = tt * p.tok_n + set * set_n;
         const float bias = p.bias[sg] ? __bfloat162float(p.bias[sg][head_in_seg * 128 + quarter * 32 + lane]) : 0.f;
         const bool rotate = kind != 2;
+        {  // positions of the set's tokens, checked: -1 where nothing is to be written
+          int ps = -1;
+          if (st < set_n && t0 + st < p.M) {
+            ps = p.pos[t0 + st];
+            if (ps < 0 || ps >= p.kv_len || ps >= p.max_pos) {
+              if (live) atomicOr(p.status, A3_DEV_BAD_POSITION);
+              ps = -1;
+            }
+          }
+          posbuf[st] = live ? ps : -1;
+        }
+        named_bar_sync(bar_set, 128);
+        // (cos, sin) of this thread's rotation pairs of a chunk: four vectors per pass.  Half-split pairs (i, i + 64): frequencies
+        // f0 .. f0 + 7; adjacent pairs (2i, 2i + 1): f0/2 .. f0/2 + 3 for the first eight features, 32 higher for the others
+        float4 tab[4 * PASSES];
+        auto fetch = [&](int c) {
+          if (!rotate) return;
+#pragma unroll
+          for (int pass = 0; pass < PASSES; ++pass) {
+            const int e = c * CH + e2 + 16 * pass;
+            const float2* row = p.tab + (size_t)max(posbuf[min(e, 127)], 0) * 64;
+            const float4* lo = reinterpret_cast<const float4*>(row + (p.layout == 0 ? f0 : f0 >> 1));
+            const float4* hi = reinterpret_cast<const float4*>(row + (p.layout == 0 ? f0 + 4 : 32 + (f0 >> 1)));
+            tab[4 * pass] = __ldg(lo), tab[4 * pass + 1] = __ldg(lo + 1), tab[4 * pass + 2] = __ldg(hi), tab[4 * pass + 3] = __ldg(hi + 1);
+          }
+        };
+        fetch(0);
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
@@ -513,30 +550,16 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
         for (int c = 0; c < n_chunks; ++c) {
-          const int w = min(CH, set_n - c * CH);
-          const int valid = min(w, p.M - (t0 + c * CH));  // tokens of this chunk that exist (may be <= 0)
           float v[CH];
           __syncwarp();
-          sp_ld_chunk<CH>(trow + c * CH, w, v);
-          if (quarter == 0) {  // positions of the chunk's tokens, checked: -1 where nothing is to be written
-            int ps = -1;
-            if (lane < valid) {
-              ps = p.pos[t0 + c * CH + lane];
-              if (ps < 0 || ps >= p.kv_len || ps >= p.max_pos) {
-                if (live) atomicOr(p.status, A3_DEV_BAD_POSITION);
-                ps = -1;
-              }
-            }
-            posbuf[lane] = ps;
-          }
+          sp_ld_chunk<CH>(trow + c * CH, min(CH, set_n - c * CH), v);
 #pragma unroll
           for (int e = 0; e < CH; ++e) xmine[e * 32] = v[e] + bias;
           named_bar_sync(bar_set, 128);
+          uint4 out_lo[PASSES], out_hi[PASSES];
 #pragma unroll
-          for (int pass = 0; pass < CH / 16; ++pass) {
+          for (int pass = 0; pass < PASSES; ++pass) {
             const int e = e2 + 16 * pass;
-            const int ps = posbuf[e];
-            if (ps < 0 || !live) continue;
             float a[8], bq[8], ra[8], rb[8];
             *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(xlo + e * 32);
             *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(xlo + e * 32 + 4);
@@ -546,23 +569,20 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
 #pragma unroll
               for (int k = 0; k < 8; ++k) ra[k] = a[k], rb[k] = bq[k];
             } else if (p.layout == 0) {
-              // pairs (i, i + 64): the thread's first 8 features rotate with the 8 that lie 64 further, frequencies f0 .. f0 + 7
-              const float4* tr = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + f0);
+              // the thread's first 8 features rotate with the 8 that lie 64 further
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
-                const float4 t = __ldg(tr + k);  // (cos, sin) of two frequencies
+                const float4 t = tab[4 * pass + k];  // (cos, sin) of two frequencies
                 ra[2 * k] = a[2 * k] * t.x - bq[2 * k] * t.y;
                 rb[2 * k] = a[2 * k] * t.y + bq[2 * k] * t.x;
                 ra[2 * k + 1] = a[2 * k + 1] * t.z - bq[2 * k + 1] * t.w;
                 rb[2 * k + 1] = a[2 * k + 1] * t.w + bq[2 * k + 1] * t.z;
               }
             } else {
-              // pairs (2i, 2i + 1): both groups of 8 hold four pairs of their own, frequencies f0/2 .. and 32 + f0/2 ..
-              const float4* tl = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + (f0 >> 1));
-              const float4* th = reinterpret_cast<const float4*>(p.tab + (size_t)ps * 64 + 32 + (f0 >> 1));
+              // both groups of 8 hold four pairs of their own
 #pragma unroll
               for (int k = 0; k < 2; ++k) {
-                const float4 t = __ldg(tl + k), u4 = __ldg(th + k);
+                const float4 t = tab[4 * pass + k], u4 = tab[4 * pass + 2 + k];
                 ra[4 * k] = a[4 * k] * t.x - a[4 * k + 1] * t.y;
                 ra[4 * k + 1] = a[4 * k] * t.y + a[4 * k + 1] * t.x;
                 ra[4 * k + 2] = a[4 * k + 2] * t.z - a[4 * k + 3] * t.w;
@@ -573,10 +593,19 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
                 rb[4 * k + 3] = bq[4 * k + 2] * u4.w + bq[4 * k + 3] * u4.z;
               }
             }
-            bf16* dst = kind == 0 ? p.q_out + (size_t)(t0 + c * CH + e) * (p.Hq * 128) + head_in_seg * 128
+            out_lo[pass] = pack8(ra);
+            out_hi[pass] = pack8(rb);
+          }
+          if (c + 1 < n_chunks) fetch(c + 1);
+#pragma unroll
+          for (int pass = 0; pass < PASSES; ++pass) {
+            const int e = c * CH + e2 + 16 * pass;
+            const int ps = e < set_n ? posbuf[e] : -1;
+            if (ps < 0) continue;
+            bf16* dst = kind == 0 ? p.q_out + (size_t)(t0 + e) * (p.Hq * 128) + head_in_seg * 128
                       : (kind == 1 ? p.k_cache : p.v_cache) + (size_t)ps * (p.Hkv * 128) + head_in_seg * 128;
-            *reinterpret_cast<uint4*>(dst + f0) = pack8(ra);
-            *reinterpret_cast<uint4*>(dst + 64 + f0) = pack8(rb);
+            *reinterpret_cast<uint4*>(dst + f0) = out_lo[pass];
+            *reinterpret_cast<uint4*>(dst + 64 + f0) = out_hi[pass];
           }
           named_bar_sync(bar_set, 128);  // everybody has read this chunk's values and positions
         }
@@ -605,7 +634,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     sp_with_chunk<true>(p.chunk, [&](auto chunk) {
       constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4;
       const int n_chunks = (set_n + CH - 1) / CH;
-      float* xset = xch + set * sp_set_floats(EPI, CH);
+      float* xset = xch + set * sp_set_floats(CH);
       float* xmine = xset + quarter * QUARTER + lane;
       const float* xrow = xset + (fg >> 2) * QUARTER + (fg & 3) * 8;
       int it = 0;
@@ -621,7 +650,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         uint4 old[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-          old[i] = i * 8 + e2 < valid ? *reinterpret_cast<const uint4*>(crow + (size_t)(i * 8 + e2) * p.ldc) : make_uint4(0, 0, 0, 0);
+          old[i] = i * 8 + e2 < valid ? __ldcg(reinterpret_cast<const uint4*>(crow + (size_t)(i * 8 + e2) * p.ldc)) : make_uint4(0, 0, 0, 0);
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads

@@ -136,6 +136,13 @@ __device__ __forceinline__ void tc_ld8(uint32_t taddr, float* v) {
                : "r"(taddr)
                : "memory");
 }
+// waits for the loads above; the registers go through the instruction, so that no use of them can be scheduled ahead of it
+template <int N>
+__device__ __forceinline__ void tc_wait_ld_of(float* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
+}
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major [rows][64] bf16 tile written by TMA with the 128-byte swizzle:
