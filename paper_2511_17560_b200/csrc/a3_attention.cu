@@ -348,10 +348,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const bool row_ok = fr < rows_total;
       const int tok = row_ok ? fr / G : 0;
       const int hq = pl.g * G + (row_ok ? fr % G : 0);
-      uint4 qv[D / 16];  // this thread's half of the Q row, on its way while the positions are read
+      // the item's Q rows, on their way while the positions are read: consecutive threads take consecutive 16-byte chunks
+      uint4 qv[D / 16];
+      const int st = threadIdx.x - 64;  // of the 256 threads
+      QRow qrow(pl.r0 + st / (D / 8), 256 / (D / 8), G);
 #pragma unroll
-      for (int c = 0; c < D / 16; ++c)
-        qv[c] = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + ((size_t)tok * Hq + hq) * D) + half * (D / 16) + c) : make_uint4(0, 0, 0, 0);
+      for (int j = 0; j < D / 16; ++j, qrow.next())
+        qv[j] = qrow.tok < M ? __ldcg(reinterpret_cast<const uint4*>(q + ((size_t)qrow.tok * Hq + pl.g * G + qrow.head) * D) + st % (D / 8))
+                             : make_uint4(0, 0, 0, 0);
       const AtcItem w = atc_item(pl, pos, M, G, kv_len, tiles_per_split, n_split == 1);
       if (!w.valid) continue;
       const int lim = row_ok ? min(pos[tok], kv_len - 1) : -1;
@@ -369,13 +373,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         continue;
       }
 
-      // Q row -> shared memory, swizzled K-major sub-tiles (each thread copies half of the row's 16-byte chunks).
+      // Q rows -> shared memory, swizzled K-major sub-tiles.
       // The previous item's S MMAs have all completed (their last s_full was waited for), so the Q buffer is free.
       {
 #pragma unroll
-        for (int cc = 0; cc < D / 16; ++cc) {
-          const int c = half * (D / 16) + cc;
-          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (c / 8) * L::SUB + swz(row, c % 8)) = qv[cc];
+        for (int j = 0; j < D / 16; ++j) {
+          const int qr = (st + 256 * j) / (D / 8), qc = st % (D / 8);
+          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (qc / 8) * L::SUB + swz(qr, qc % 8)) = qv[j];
         }
         fence_async_smem();
         mbar_arrive(q_ready);
@@ -578,7 +582,7 @@ attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int
   if (n_active <= 1) return;  // written directly by the attention kernel
   float m = -INFINITY;
   for (int z = 0; z < n_active; ++z) {
-    const float2 ml = part_ml[((size_t)z * Hkv + g) * rows_pad + fr];
+    const float2 ml = __ldcg(part_ml + ((size_t)z * Hkv + g) * rows_pad + fr);
     if (ml.y > 0.f) m = fmaxf(m, ml.x);
   }
   constexpr int PER = D / 32;
@@ -588,14 +592,14 @@ attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int
   float l = 0.f;
   for (int z = 0; z < n_active; ++z) {
     const size_t prow = ((size_t)z * Hkv + g) * rows_pad + fr;
-    const float2 ml = part_ml[prow];
+    const float2 ml = __ldcg(part_ml + prow);
     if (!(ml.y > 0.f)) continue;
     const float w = exp2f(ml.x - m);
     l += ml.y * w;
     if (o) {
       const float* src = part_o + prow * D + lane * PER;
 #pragma unroll
-      for (int e = 0; e < PER; ++e) acc[e] += src[e] * w;
+      for (int e = 0; e < PER; ++e) acc[e] += __ldcg(src + e) * w;
     }
   }
   const int tok = fr / G, hq = g * G + fr % G;

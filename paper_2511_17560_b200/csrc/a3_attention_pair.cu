@@ -299,14 +299,17 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const int lim = row_ok ? min(pos[tok], kv_len - 1) : -1;
       const int nkt = w.nkt[x];
 
-      // Q row -> shared memory, swizzled K-major sub-tiles.  The previous item's S_X MMAs have all completed (their
+      // Q rows -> shared memory, swizzled K-major sub-tiles.  The previous item's S_X MMAs have all completed (their
       // last s_full was waited for), so the buffer is free.  Every thread arrives, also when its row tile is empty.
       {
-        const uint4* src = reinterpret_cast<const uint4*>(q + ((size_t)tok * Hq + hq) * D);
+        // consecutive threads of the row tile take consecutive 16-byte chunks
+        QRow qrow(w.r0[x] + row / (D / 8), 128 / (D / 8), G);
 #pragma unroll
-        for (int c = 0; c < D / 8; ++c) {
-          const uint4 v = (row_ok && nkt > 0) ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
-          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + x * L::TILE + (c / 8) * L::SUB + swz(row, c % 8)) = v;
+        for (int j = 0; j < D / 8; ++j, qrow.next()) {
+          const int qr = (row + 128 * j) / (D / 8), qc = row % (D / 8);
+          const uint4 v = (qrow.tok < M && nkt > 0) ? __ldcg(reinterpret_cast<const uint4*>(q + ((size_t)qrow.tok * Hq + w.g * G + qrow.head) * D) + qc)
+                                                    : make_uint4(0, 0, 0, 0);
+          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + x * L::TILE + (qc / 8) * L::SUB + swz(qr, qc % 8)) = v;
         }
         fence_async_smem();
         mbar_arrive(q_ready);
@@ -405,8 +408,8 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         }
         // Slots beyond the last visible key of the pair may hold anything (probability zero times a non-finite
         // value would still poison the product): clear those V rows of the last key tile before the first P V that
-        // reads it - row tile A does it when it walks to the last tile (its P V is issued first), else B.
-        if (t == w.T - 1 && x == (w.nkt[0] == w.T ? 0 : 1)) {
+        // reads it - each row tile that walks there before its own, since neither waits for the other.
+        if (t == w.T - 1) {
           const int first_bad = max(w.maxpos[0], w.maxpos[1]) - key0 + 1;
           const uint32_t vit = it + t;
           const bool landed = mbar_wait(v_full(vit & 1), (vit >> 1) & 1, abort_flag, status);

@@ -140,6 +140,20 @@ __host__ __device__ constexpr uint32_t idesc(int n, int b_mn) {
 }
 // byte offset of element chunk (16 bytes) j of row r inside a [rows][64] bf16 sub-tile with the 128-byte swizzle
 __device__ __forceinline__ uint32_t swz(int r, int j) { return (uint32_t)(r * 128 + ((j ^ (r & 7)) << 4)); }
+
+// The packed row that a thread copies into the Q tile, stepped by a fixed number of rows without a division per step.
+struct QRow {
+  int tok, head, dt, dh, G;
+  __device__ __forceinline__ QRow(int row, int step, int g) : tok(row / g), head(row % g), dt(step / g), dh(step % g), G(g) {}
+  __device__ __forceinline__ void next() {
+    tok += dt;
+    head += dh;
+    if (head >= G) {
+      head -= G;
+      ++tok;
+    }
+  }
+};
 }  // namespace atc
 
 // 2^v for a pair on the FMA pipe: v = n + f with n integer and |f| <= 1/2 (magic-number rounding), 2^f by a cubic

@@ -359,7 +359,7 @@ rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gain, floa
 #pragma unroll
   for (int i = 0; i < RN_VPT; ++i) {
     const int idx = threadIdx.x + i * RN_THREADS;
-    v[i] = idx < row_vecs ? __ldg(xr + idx) : make_uint4(0, 0, 0, 0);
+    v[i] = idx < row_vecs ? __ldcg(xr + idx) : make_uint4(0, 0, 0, 0);
   }
 #pragma unroll
   for (int i = 0; i < RN_VPT; ++i) {
@@ -370,7 +370,7 @@ rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gain, floa
   }
   for (int idx = threadIdx.x + RN_VPT * RN_THREADS; idx < row_vecs; idx += RN_THREADS) {
     float f[8];
-    unpack8(__ldg(xr + idx), f);
+    unpack8(__ldcg(xr + idx), f);
 #pragma unroll
     for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
   }
@@ -398,7 +398,7 @@ rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gain, floa
   }
   for (int idx = threadIdx.x + RN_VPT * RN_THREADS; idx < row_vecs; idx += RN_THREADS) {
     float f[8], g[8], r[8];
-    unpack8(__ldg(xr + idx), f);
+    unpack8(__ldcg(xr + idx), f);
     unpack8(__ldg(gain + idx), g);
 #pragma unroll
     for (int e = 0; e < 8; ++e) r[e] = f[e] * inv * g[e];
@@ -467,7 +467,7 @@ add_slices_rmsnorm_kernel(uint4* __restrict__ x, const float4* __restrict__ part
   for (int i = 0; i < RS_VPT; ++i) {
     const int idx = threadIdx.x + i * RS_THREADS;
     v[i] = make_uint4(0, 0, 0, 0);
-    if (idx < row_vecs) xr[idx] = v[i] = add_slices8<SLICES>(xr[idx], pr + 2 * idx, stride, slices);
+    if (idx < row_vecs) xr[idx] = v[i] = add_slices8<SLICES>(__ldcg(xr + idx), pr + 2 * idx, stride, slices);
   }
 #pragma unroll
   for (int i = 0; i < RS_VPT; ++i) {
@@ -477,7 +477,7 @@ add_slices_rmsnorm_kernel(uint4* __restrict__ x, const float4* __restrict__ part
     for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
   }
   for (int idx = threadIdx.x + RS_VPT * RS_THREADS; idx < row_vecs; idx += RS_THREADS) {  // wider rows: kept in x, read again below
-    const uint4 t = add_slices8<SLICES>(xr[idx], pr + 2 * idx, stride, slices);
+    const uint4 t = add_slices8<SLICES>(__ldcg(xr + idx), pr + 2 * idx, stride, slices);
     xr[idx] = t;
     float f[8];
     unpack8(t, f);
