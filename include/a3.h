@@ -339,7 +339,7 @@ int a3_fuse_request_host(const a3_handle* h, const a3_request* req, const a3_hos
  *   k_layer, v_layer: dev [kv_len][Hkv][D], kv_len = n_ctx + nq;
  *   k_out, v_out: dev [C'][Hkv][D], C' = n_system + k + nq: entry c of head g is source slot kept_out[g][c];
  *   kept_out: dev [Hkv][C'] int32 (ascending per head) or NULL.
- * ws: a3_evict_workspace_bytes(h, kv_len), borrowed.  Four launches, no allocation, no synchronisation. */
+ * ws: a3_evict_workspace_bytes(h, kv_len), borrowed.  At most four launches, no allocation, no synchronisation. */
 int a3_evict_count(int capacity, int n_system, int n_ctx, int n_question);
 size_t a3_evict_workspace_bytes(const a3_handle* h, int kv_len);
 int a3_evict_layer(const a3_handle* h, const void* q_window, const int32_t* q_pos, int nq, const float* lse,

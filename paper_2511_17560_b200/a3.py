@@ -362,9 +362,9 @@ class A3:
         kv_len = k_layer.shape[0]
         Cp = n_system + evict_count(capacity, n_system, n_ctx, nq) + nq
         Hkv, D = self.shape.n_kv_heads, self.shape.head_dim
-        k_out = torch.zeros((Cp, Hkv, D), dtype=torch.bfloat16, device=k_layer.device)
-        v_out = torch.zeros_like(k_out)
-        kept = torch.full((Hkv, Cp), -1, dtype=torch.int32, device=k_layer.device)
+        k_out = torch.empty((Cp, Hkv, D), dtype=torch.bfloat16, device=k_layer.device)  # the gather writes every entry
+        v_out = torch.empty_like(k_out)
+        kept = torch.empty((Hkv, Cp), dtype=torch.int32, device=k_layer.device)
         ws = self.workspace(int(_load().a3_evict_workspace_bytes(self._h, kv_len)))
         _check(_load().a3_evict_layer(self._h, _ptr(q_window), _ptr(q_pos), nq, _ptr(lse), _ptr(k_layer), _ptr(v_layer), kv_len,
                                       n_system, n_ctx, capacity, pool, _ptr(k_out), _ptr(v_out), _ptr(kept), _ptr(ws), ws.numel(),

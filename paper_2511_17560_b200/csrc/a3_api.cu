@@ -582,32 +582,36 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
                           r->kept_out ? r->kept_out + (size_t)l * m.n_kv_heads * c_evicted : nullptr, w.evict, w.evict_bytes, stream);
   };
 
+  // R: the selection (or the caller's rows, which are checked) and the question rows
+  auto selected_rows = [&]() -> int {
+    if (!r->forced_re) return topk_rows(h, r->scores_out, r->n_system, r->n_ctx, p, r->n_ctx, nq, r->rows_out, st);
+    if (p > 0) A3_CUDA(cudaMemcpyAsync(r->rows_out, r->forced_re, (size_t)p * 4, cudaMemcpyDeviceToDevice, st));
+    A3_TRY(iota_rows(h, r->rows_out + p, r->n_ctx, nq, st));
+    return check_rows(h, r->rows_out, M, n, st);
+  };
+
   if (r->score_source == A3_SCORES_CACHED_KEYS) {
     // Scores against the recovered cached keys: every layer is position-recovered; only the question rows pass
     // through the leading blocks; rows [Re, Q] are recomputed through every layer from the embeddings.
     A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, 0, m.n_layers, stream));
-    A3_TRY(iota_rows(h, w.all_pos, 0, n, st));
-    const int32_t* q_pos = w.all_pos + r->n_ctx;
-    A3_CUDA(cudaMemsetAsync(r->scores_out, 0, (size_t)n * 4, st));
+    const int32_t* q_pos = w.all_pos;  // [nq]
     if (nq > 0) {
       bf16* xq = w.x_all;  // [nq][d] scratch for the question rows
-      A3_CUDA(cudaMemcpyAsync(xq, (const bf16*)r->x0 + (size_t)r->n_ctx * m.d_model, (size_t)nq * m.d_model * 2, cudaMemcpyDeviceToDevice, st));
+      A3_TRY(enter_rows(h, (const bf16*)r->x0 + (size_t)r->n_ctx * m.d_model, nq, nullptr, nq, (const bf16*)h->layers[0].attn_norm, m.rms_eps,
+                        m.d_model, xq, lw.a, w.all_pos, r->n_ctx, st));
       for (int l = 0; l < ls; ++l)
-        A3_TRY(recompute_layer_impl(h, l, xq, q_pos, nq, kl(l), vl(l), n, nullptr, lw, st, l > 0, (const bf16*)h->layers[l + 1].attn_norm));
-      if (ls == 0) A3_TRY(rmsnorm_rows(h, xq, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, nq, m.d_model, lw.a, st));
+        A3_TRY(recompute_layer_impl(h, l, xq, q_pos, nq, kl(l), vl(l), n, nullptr, lw, st, true, (const bf16*)h->layers[l + 1].attn_norm));
       A3_TRY(qkv_project(h, ls, lw.a, q_pos, nq, 0, lw.q, kl(ls), vl(ls), n, st));
       A3_TRY(scores_with_stats(h, lw.q, q_pos, nq, kl(ls), n, r->n_system, r->n_ctx, w.lse_q, lw.attn_part, lw.attn_part_bytes,
                                r->scores_out, st));
+    } else {
+      A3_CUDA(cudaMemsetAsync(r->scores_out, 0, (size_t)n * 4, st));
     }
-    if (p > 0) {
-      if (r->forced_re) A3_CUDA(cudaMemcpyAsync(r->rows_out, r->forced_re, (size_t)p * 4, cudaMemcpyDeviceToDevice, st));
-      else A3_TRY(a3_topk_select(h, r->scores_out, r->n_system, r->n_ctx, p, r->rows_out, stream));
-    }
-    A3_TRY(iota_rows(h, r->rows_out + p, r->n_ctx, nq, st));
+    A3_TRY(selected_rows());
     if (M == 0) return A3_OK;
-    A3_TRY(check_rows(h, r->rows_out, M, n, st));
-    A3_TRY(a3_gather_rows(h, r->x0, n, r->rows_out, M, m.d_model, r->x_out, stream));
-    for (int l = 0; l < m.n_layers; ++l) A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, l > 0, true));
+    A3_TRY(enter_rows(h, (const bf16*)r->x0, n, r->rows_out, M, (const bf16*)h->layers[0].attn_norm, m.rms_eps, m.d_model, (bf16*)r->x_out, lw.a,
+                      nullptr, 0, st));
+    for (int l = 0; l < m.n_layers; ++l) A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, true, true));
     return A3_OK;
   }
 
@@ -619,17 +623,18 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
                             m.n_layers, stream));
   // leading full blocks: the whole input through layers 0..select_layer-1
   const int panels = x0_panels(n);
-  A3_TRY(iota_rows(h, w.all_pos, 0, n, st));
+  const bool norm_panels = ls > 0 || panels == 1;
   for (int i = 0; i < panels; ++i) {
     const int r0 = x0_panel_begin(n, i, panels), r1 = x0_panel_begin(n, i + 1, panels);
+    bf16* x = w.x_all + (size_t)r0 * m.d_model;
     if (x0_ready) A3_CUDA(cudaStreamWaitEvent(st, x0_ready[i], 0));
-    A3_CUDA(cudaMemcpyAsync(w.x_all + (size_t)r0 * m.d_model, (const bf16*)r->x0 + (size_t)r0 * m.d_model, (size_t)(r1 - r0) * m.d_model * 2,
-                            cudaMemcpyDeviceToDevice, st));
+    A3_TRY(enter_rows(h, (const bf16*)r->x0 + (size_t)r0 * m.d_model, r1 - r0, nullptr, r1 - r0,
+                      norm_panels ? (const bf16*)h->layers[0].attn_norm : nullptr, m.rms_eps, m.d_model, x, lw.a, w.all_pos + r0, r0, st));
     if (ls > 0) {
       // block 0 on this panel of rows: they attend to the rows before them, whose K/V the earlier panels have written
       if (i == 0) A3_TRY(feed_to(ls + 1 + FEED_AHEAD));  // a full block is long: several layers' copies fit under it
-      if (i + 1 < panels) A3_TRY(recompute_layer_impl(h, 0, w.x_all + (size_t)r0 * m.d_model, w.all_pos + r0, r1 - r0, kl(0), vl(0), n, nullptr, lw, st));
-      else A3_TRY(layer_step(0, w.x_all + (size_t)r0 * m.d_model, w.all_pos + r0, r1 - r0, false, panels == 1));
+      if (i + 1 < panels) A3_TRY(recompute_layer_impl(h, 0, x, w.all_pos + r0, r1 - r0, kl(0), vl(0), n, nullptr, lw, st, true));
+      else A3_TRY(layer_step(0, x, w.all_pos + r0, r1 - r0, true, panels == 1));
     }
   }
   for (int l = 1; l < ls; ++l) {
@@ -638,21 +643,18 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
   }
   A3_TRY(feed_to(ls + 1 + FEED_AHEAD));
   // selection layer: true K, V for all rows, queries of the question rows, scores, Re (Eq. 3)
-  if (ls == 0 || (ls == 1 && panels > 1))  // otherwise the last full block left the norm of all rows
+  if (ls <= 1 && panels > 1)  // otherwise the norm of all rows is there already
     A3_TRY(rmsnorm_rows(h, w.x_all, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, n, m.d_model, lw.a, st));
   A3_TRY(qkv_project(h, ls, lw.a, w.all_pos, n, r->n_ctx, lw.q, kl(ls), vl(ls), n, st));
-  A3_CUDA(cudaMemsetAsync(r->scores_out, 0, (size_t)n * 4, st));
+  // (the score pass writes every slot)
+  if (r->selector == A3_SELECT_VALUE_DEVIATION || nq == 0) A3_CUDA(cudaMemsetAsync(r->scores_out, 0, (size_t)n * 4, st));
   if (r->selector == A3_SELECT_VALUE_DEVIATION) {
     A3_TRY(value_deviation(h, r->chunks, r->n_chunks, r->max_chunk_len, ls, vl(ls), r->n_system, r->n_ctx, r->scores_out, st));
   } else if (nq > 0) {
     A3_TRY(scores_with_stats(h, lw.q, w.all_pos + r->n_ctx, nq, kl(ls), n, r->n_system, r->n_ctx, w.lse_q, lw.attn_part,
                              lw.attn_part_bytes, r->scores_out, st));
   }
-  if (p > 0) {
-    if (r->forced_re) A3_CUDA(cudaMemcpyAsync(r->rows_out, r->forced_re, (size_t)p * 4, cudaMemcpyDeviceToDevice, st));
-    else A3_TRY(a3_topk_select(h, r->scores_out, r->n_system, r->n_ctx, p, r->rows_out, stream));
-  }
-  A3_TRY(iota_rows(h, r->rows_out + p, r->n_ctx, nq, st));
+  A3_TRY(selected_rows());
   if (M == 0) {
     A3_TRY(feed_to(m.n_layers));
     if (layer_ready)
@@ -662,8 +664,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
       }
     return A3_OK;
   }
-  A3_TRY(check_rows(h, r->rows_out, M, n, st));
-  A3_TRY(a3_gather_rows(h, w.x_all, n, r->rows_out, M, m.d_model, r->x_out, stream));
+  A3_TRY(enter_rows(h, w.x_all, n, r->rows_out, M, (const bf16*)h->layers[ls].attn_norm, m.rms_eps, m.d_model, (bf16*)r->x_out, lw.a, nullptr, 0, st));
   // layers select_layer..L-1 on rows [Re, Q] only (Eq. 4, Eq. 5)
   for (int l = ls; l < m.n_layers; ++l) {
     A3_TRY(feed_to(l + FEED_AHEAD));
@@ -671,7 +672,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
       A3_CUDA(cudaStreamWaitEvent(st, layer_ready[l], 0));
       A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, l, l + 1, stream));
     }
-    A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, l > ls, true));
+    A3_TRY(layer_step(l, (bf16*)r->x_out, r->rows_out, M, true, true));
   }
   return A3_OK;
 }

@@ -2,9 +2,9 @@
 // per layer and per KV head the C - |S| - |Q| document tokens with the most question-window attention are kept
 // (SnapKV's strategy) and the layer's cache is compacted.
 //
-// One layer = four launches: per-head votes (the score kernel of Eq. 3 without the sum over KV heads, fed with
-// the question rows' queries and log-sum-exps of that layer), optional max pooling, one top-k CTA per KV head,
-// and a gather that writes the compact cache [C'][Hkv][D] (bound by HBM: each kept row is read and written once).
+// One layer = three launches: per-head votes (the score kernel of Eq. 3 without the sum over KV heads, fed with
+// the question rows' queries and log-sum-exps of that layer), one top-k CTA per KV head, which pools the votes as it reads
+// them (a kernel of its own does where they do not fit its shared memory), and a gather that writes the compact cache [C'][Hkv][D] (bound by HBM: each kept row is read and written once).
 #include "a3_internal.cuh"
 
 namespace a3 {
@@ -36,13 +36,18 @@ __global__ void __launch_bounds__(128)
 evict_gather_kernel(const uint4* __restrict__ kc, const uint4* __restrict__ vc, int kv_len, const int32_t* __restrict__ sel, int k,
                     int n_system, int n_ctx, int Hkv, int head_vecs, uint4* __restrict__ k_out, uint4* __restrict__ v_out,
                     int32_t* __restrict__ kept, int C, uint32_t* status) {
+  pdl_wait();
   const int c = blockIdx.x;
   const int row_vecs = Hkv * head_vecs;
   for (int v = threadIdx.x; v < row_vecs; v += blockDim.x) {
     const int g = v / head_vecs;
     const int src = evict_source(c, g, sel, k, n_system, n_ctx);
     if (src < 0 || src >= kv_len) {
-      if (v % head_vecs == 0) atomicOr(status, A3_DEV_BAD_POSITION);
+      if (v % head_vecs == 0) {
+        atomicOr(status, A3_DEV_BAD_POSITION);
+        if (kept) kept[(size_t)g * C + c] = -1;
+      }
+      k_out[(size_t)c * row_vecs + v] = v_out[(size_t)c * row_vecs + v] = make_uint4(0, 0, 0, 0);
       continue;
     }
     k_out[(size_t)c * row_vecs + v] = __ldcs(kc + (size_t)src * row_vecs + v);
@@ -90,13 +95,14 @@ extern "C" int a3_evict_layer(const a3_handle* h, const void* q_window, const in
     if (nq > 0) A3_TRY(scores_pass(h, (const bf16*)q_window, q_pos, nq, (const bf16*)k_layer, kv_len, n_system, n_ctx, lse, nullptr, st, votes));
     else A3_CUDA(cudaMemsetAsync(votes, 0, (size_t)m.n_kv_heads * kv_len * 4, st));
     const float* src = votes;
-    if (pool > 1) {
+    const bool pool_in_topk = topk_can_pool(n_ctx - n_system);
+    if (pool > 1 && !pool_in_topk) {
       ProfScope prof(h, A3_K_ROWS, st);
       pool_scores_kernel<<<dim3(cdiv(kv_len, 256), m.n_kv_heads), 256, 0, st>>>(votes, pooled, kv_len, n_system, n_ctx, pool / 2);
       A3_LAUNCHED();
       src = pooled;
     }
-    A3_TRY(topk_batched(h, src, (size_t)kv_len, m.n_kv_heads, n_system, n_ctx, k, sel, (size_t)k, st));
+    A3_TRY(topk_batched(h, src, (size_t)kv_len, m.n_kv_heads, n_system, n_ctx, k, pool_in_topk ? pool : 1, sel, (size_t)k, st));
   } else if (k > 0) {
     // everything fits: the selection is every document slot (no votes needed)
     for (int g = 0; g < m.n_kv_heads; ++g) A3_TRY(iota_rows(h, sel + (size_t)g * k, n_system, k, st));
@@ -104,8 +110,8 @@ extern "C" int a3_evict_layer(const a3_handle* h, const void* q_window, const in
   if (C == 0) return A3_OK;
   {
     ProfScope prof(h, A3_K_ROWS, st);
-    evict_gather_kernel<<<C, 128, 0, st>>>((const uint4*)k_layer, (const uint4*)v_layer, kv_len, sel, k, n_system, n_ctx, m.n_kv_heads,
-                                           m.head_dim / 8, (uint4*)k_out, (uint4*)v_out, kept_out, C, h->dev_status);
+    A3_CUDA(launch_pdl(evict_gather_kernel, dim3(C), dim3(128), 0, st, (const uint4*)k_layer, (const uint4*)v_layer, kv_len, sel, k, n_system, n_ctx,
+                       m.n_kv_heads, m.head_dim / 8, (uint4*)k_out, (uint4*)v_out, kept_out, C, h->dev_status));
     A3_LAUNCHED();
   }
   return A3_OK;

@@ -132,6 +132,11 @@ int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps,
 int add_slices_rmsnorm(const a3_handle* h, bf16* x, const float* part, int slices, const bf16* gain, float eps, int M, int d, bf16* out,
                        cudaStream_t st);
 
+// Rows entering a layer: x_dst[r] = src[rows ? rows[r] : r]; out[r] = rmsnorm of it * gain (gain null: no norm); pos_out[r] =
+// pos_base + r (null: no positions).
+int enter_rows(const a3_handle* h, const bf16* src, int n_src, const int32_t* rows, int M, const bf16* gain, float eps, int d, bf16* x_dst,
+               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st);
+
 enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_SWIGLU = 1, EPI_QKV = 2 };
 
 struct GemmSegment {
@@ -194,9 +199,14 @@ int scores_with_stats(const a3_handle* h, const bf16* q, const int32_t* q_pos, i
 
 int scores_pass(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len,
                 int cand_begin, int cand_end, const float* lse, float* scores, cudaStream_t st, float* per_head = nullptr);
+// a3_topk_select of the k best candidates, followed by the slots tail_begin .. tail_begin + tail - 1 (the question's)
+int topk_rows(const a3_handle* h, const float* scores, int cand_begin, int cand_end, int k, int tail_begin, int tail, int32_t* idx_out,
+              cudaStream_t st);
 // `batches` independent selections, one CTA each: scores + b*score_stride -> idx_out + b*idx_stride
+// (pool > 1, odd: of the running maximum over `pool` neighbouring candidates instead of the scores themselves)
 int topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,
-                 int k, int32_t* idx_out, size_t idx_stride, cudaStream_t st);
+                 int k, int pool, int32_t* idx_out, size_t idx_stride, cudaStream_t st);
+bool topk_can_pool(int n_cand);  // ... as long as the candidates fit its shared memory
 
 // scores[slot] = |v_true[slot] - cached value of that slot|^2 for candidate slots covered by a chunk (others untouched)
 int value_deviation(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len, int layer, const bf16* v_true,

@@ -231,8 +231,8 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int key0 = blockIdx.x * 128;
-  // gridDim.y == 1: all KV heads, summed (Eq. 3); gridDim.y == Hkv: one KV head per CTA (per-head votes only)
-  const int g_begin = gridDim.y == 1 ? 0 : blockIdx.y, g_end = gridDim.y == 1 ? p.Hkv : blockIdx.y + 1;
+  // gridDim.y == 1: all KV heads, summed (Eq. 3); more: a share of the KV heads per CTA (per-head votes only)
+  const int g_begin = p.Hkv * blockIdx.y / gridDim.y, g_end = p.Hkv * (blockIdx.y + 1) / gridDim.y;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -476,7 +476,14 @@ static int launch_scores_tc(const a3_handle* h, const bf16* q, const int32_t* q_
   const int smem = L::smem_bytes(G * nq_tile);
   static SmemAttrOnce attr;
   A3_TRY(smem_attr_once(attr, h->device, scores_tc_kernel<D>, L::smem_bytes(256)));
-  dim3 grid(cdiv(kv_len, 128), (per_head && !scores) ? Hkv : 1);
+  dim3 grid(cdiv(kv_len, 128), 1);
+  if (per_head && !scores) {
+    // Heads need no sum: as many shares of them as leave one CTA per SM (a CTA holds 165 KiB of shared memory, and its tables
+    // cost as much as two heads: 41 key tiles x 8 heads as 328 CTAs in three waves take 14.5 us, as 123 CTAs 10.7)
+    const int sms = h->sm_count > 0 ? h->sm_count : 148;
+    const int shares = sms / (int)grid.x;
+    grid.y = shares < 1 ? 1 : shares > Hkv ? Hkv : shares;
+  }
   A3_CUDA(launch_pdl(scores_tc_kernel<D>, grid, dim3(STC_THREADS), (size_t)smem, st, tK, tQ, p));
   A3_LAUNCHED();
   return A3_OK;

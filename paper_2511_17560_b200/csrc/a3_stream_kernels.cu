@@ -414,6 +414,90 @@ int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps,
   return A3_OK;
 }
 
+// Row r of a request on its way into a layer: x_dst[r] = src[rows ? rows[r] : r], out[r] = RMSNorm of it (gain given), and
+// pos_out[r] = pos_base + r.  What a copy, an index kernel, a gather and a norm would each launch for; a thread keeps its
+// vectors in registers between the two stores.  Rows out of range are flagged and skipped.
+__global__ void __launch_bounds__(RN_THREADS)
+enter_rows_kernel(const uint4* __restrict__ src, int n_src, const int32_t* __restrict__ rows, const uint4* __restrict__ gain, float eps,
+                  int row_vecs, uint4* __restrict__ x_dst, uint4* __restrict__ out, int32_t* __restrict__ pos_out, int pos_base, uint32_t* status) {
+  pdl_wait();
+  pdl_launch_dependents();
+  uint4 gv[RN_VPT];
+#pragma unroll
+  for (int i = 0; i < RN_VPT; ++i) {
+    const int idx = threadIdx.x + i * RN_THREADS;
+    gv[i] = gain && idx < row_vecs ? __ldg(gain + idx) : make_uint4(0, 0, 0, 0);
+  }
+  const int r = blockIdx.x;
+  const int s = rows ? __ldcg(rows + r) : r;
+  if (pos_out && threadIdx.x == 0) pos_out[r] = pos_base + r;
+  if (s < 0 || s >= n_src) {
+    if (threadIdx.x == 0) atomicOr(status, A3_DEV_BAD_POSITION);
+    return;
+  }
+  const uint4* xr = src + (size_t)s * row_vecs;
+  uint4* xo = x_dst + (size_t)r * row_vecs;
+  uint4 v[RN_VPT];
+  float ss = 0.f;
+#pragma unroll
+  for (int i = 0; i < RN_VPT; ++i) {
+    const int idx = threadIdx.x + i * RN_THREADS;
+    v[i] = idx < row_vecs ? __ldcg(xr + idx) : make_uint4(0, 0, 0, 0);
+  }
+  auto squares = [&](const uint4& t) {
+    float f[8];
+    unpack8(t, f);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
+  };
+#pragma unroll
+  for (int i = 0; i < RN_VPT; ++i) {
+    const int idx = threadIdx.x + i * RN_THREADS;
+    if (idx < row_vecs) xo[idx] = v[i];
+    squares(v[i]);
+  }
+  for (int idx = threadIdx.x + RN_VPT * RN_THREADS; idx < row_vecs; idx += RN_THREADS) {
+    const uint4 t = __ldcg(xr + idx);
+    xo[idx] = t;
+    squares(t);
+  }
+  if (!gain) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  __shared__ float part[RN_THREADS / 32];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < RN_THREADS / 32; ++w) tot += part[w];
+  const float inv = rsqrtf(tot / (float)(row_vecs * 8) + eps);
+  uint4* orow = out + (size_t)r * row_vecs;
+  auto scaled = [&](const uint4& xv, const uint4& gain_v, int idx) {
+    float f[8], g[8];
+    unpack8(xv, f);
+    unpack8(gain_v, g);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) f[e] = f[e] * inv * g[e];
+    orow[idx] = pack8(f);
+  };
+#pragma unroll
+  for (int i = 0; i < RN_VPT; ++i) {
+    const int idx = threadIdx.x + i * RN_THREADS;
+    if (idx < row_vecs) scaled(v[i], gv[i], idx);
+  }
+  for (int idx = threadIdx.x + RN_VPT * RN_THREADS; idx < row_vecs; idx += RN_THREADS) scaled(__ldcg(xr + idx), __ldg(gain + idx), idx);
+}
+
+int enter_rows(const a3_handle* h, const bf16* src, int n_src, const int32_t* rows, int M, const bf16* gain, float eps, int d, bf16* x_dst,
+               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st) {
+  if (M <= 0) return A3_OK;
+  ProfScope prof(h, A3_K_ROWS, st);
+  A3_CUDA(launch_pdl(enter_rows_kernel, dim3(M), dim3(RN_THREADS), 0, st, (const uint4*)src, n_src, rows, (const uint4*)gain, eps, d / 8,
+                     (uint4*)x_dst, (uint4*)out, pos_out, pos_base, h->dev_status));
+  A3_LAUNCHED();
+  return A3_OK;
+}
+
 // x += the k-slices of a residual GEMM (fp32, summed in slice order, rounded once), then RMSNorm of the new row: what the
 // split GEMM saves in its k-loop is not spent again on a pass of its own.  One CTA per row, a thread keeps its vectors in
 // registers; the slices' loads (two 16-byte vectors per slice and bf16 vector) are all in flight together.  Bound by the

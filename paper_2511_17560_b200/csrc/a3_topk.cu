@@ -23,7 +23,7 @@ __device__ __forceinline__ uint32_t score_key(float s) {
 }
 
 template <bool IN_SMEM>
-__device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t* __restrict__ keys, int cand_begin, int n, int k,
+__device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t* __restrict__ keys, int cand_begin, int n, int k, int half_pool,
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
   __shared__ unsigned int hist[256];
   __shared__ unsigned int whist[TK_HISTS][256];
@@ -37,7 +37,10 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
   bool nonfinite = false;
 #pragma unroll 4
   for (int i = tid; i < n; i += TK_THREADS) {
-    const float v = s[i];
+    float v = __ldcg(s + i);
+    if (IN_SMEM && half_pool > 0) {  // running maximum, cut at the candidate range
+      for (int j = max(0, i - half_pool); j <= min(n - 1, i + half_pool); ++j) v = fmaxf(v, s[j]);
+    }
     if (!(fabsf(v) <= 3.0e38f)) nonfinite = true;
     if (IN_SMEM) keys[i] = score_key(v);
   }
@@ -144,26 +147,27 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
 
 __global__ void __launch_bounds__(TK_THREADS)
 topk_select_kernel(const float* __restrict__ scores, int cand_begin, int n, int k, int32_t* __restrict__ idx_out, uint32_t* status,
-                   size_t score_stride, size_t idx_stride, int in_smem) {
+                   size_t score_stride, size_t idx_stride, int in_smem, int half_pool, int tail_begin, int tail) {
   extern __shared__ uint32_t tk_keys[];
   pdl_wait();
   pdl_launch_dependents();
   // one CTA per independent selection (the per-head selections of the eviction step; a single one for Eq. 3)
   const float* s = scores + blockIdx.x * score_stride + cand_begin;
   int32_t* out = idx_out + blockIdx.x * idx_stride;
-  if (in_smem) topk_body<true>(s, tk_keys, cand_begin, n, k, out, status);
-  else topk_body<false>(s, tk_keys, cand_begin, n, k, out, status);
+  for (int i = threadIdx.x; i < tail; i += TK_THREADS) out[k + i] = tail_begin + i;
+  if (in_smem) topk_body<true>(s, tk_keys, cand_begin, n, k, half_pool, out, status);
+  else topk_body<false>(s, tk_keys, cand_begin, n, k, 0, out, status);
 }
 
 static int launch_topk(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int n, int k,
-                       int32_t* idx_out, size_t idx_stride, cudaStream_t st) {
+                       int half_pool, int tail_begin, int tail, int32_t* idx_out, size_t idx_stride, cudaStream_t st) {
   const int in_smem = n <= TK_SMEM_KEYS ? 1 : 0;
   const size_t smem = in_smem ? (size_t)n * 4 : 0;
   static SmemAttrOnce attr;
   A3_TRY(smem_attr_once(attr, h->device, topk_select_kernel, TK_SMEM_KEYS * 4));
   ProfScope prof(h, A3_K_TOPK, st);
   A3_CUDA(launch_pdl(topk_select_kernel, dim3(batches), dim3(TK_THREADS), smem, st, scores, cand_begin, n, k, idx_out, h->dev_status,
-                     score_stride, idx_stride, in_smem));
+                     score_stride, idx_stride, in_smem, half_pool, tail_begin, tail));
   A3_LAUNCHED();
   return A3_OK;
 }
@@ -179,13 +183,21 @@ extern "C" int a3_topk_select(const a3_handle* h, const float* scores, int cand_
   if (k > n) k = n;
   if (k == 0) return A3_OK;
   if (!scores || !idx_out) return A3_EINVAL;
-  return launch_topk(h, scores, 0, 1, cand_begin, n, k, idx_out, 0, (cudaStream_t)stream);
+  return launch_topk(h, scores, 0, 1, cand_begin, n, k, 0, 0, 0, idx_out, 0, (cudaStream_t)stream);
 }
 
+int a3::topk_rows(const a3_handle* h, const float* scores, int cand_begin, int cand_end, int k, int tail_begin, int tail, int32_t* idx_out,
+                  cudaStream_t st) {
+  if (k <= 0) return iota_rows(h, idx_out, tail_begin, tail, st);
+  return launch_topk(h, scores, 0, 1, cand_begin, cand_end - cand_begin, k, 0, tail_begin, tail, idx_out, 0, st);
+}
+
+bool a3::topk_can_pool(int n_cand) { return n_cand <= TK_SMEM_KEYS; }
+
 int a3::topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,
-                     int k, int32_t* idx_out, size_t idx_stride, cudaStream_t st) {
+                     int k, int pool, int32_t* idx_out, size_t idx_stride, cudaStream_t st) {
   const int n = cand_end - cand_begin;
   if (k > n) k = n;
   if (k <= 0 || batches <= 0) return A3_OK;
-  return launch_topk(h, scores, score_stride, batches, cand_begin, n, k, idx_out, idx_stride, st);
+  return launch_topk(h, scores, score_stride, batches, cand_begin, n, k, pool > 1 ? pool / 2 : 0, 0, 0, idx_out, idx_stride, st);
 }
