@@ -30,17 +30,21 @@
 namespace a3 {
 
 constexpr int ATC_THREADS = 320;  // TMA warp, MMA warp, 8 softmax warps (two threads per row)
-template <int D>
+template <int D, int CS = 1>
 struct AtcLayout {
   static constexpr int SUB = 128 * 64 * 2;           // one [128][64] bf16 sub-tile: 16 KiB
   static constexpr int Q_BYTES = (D / 64) * SUB;
   static constexpr int KV_STAGE = 2 * (D / 64) * SUB;  // K then V
-  static constexpr int KV_STAGES = 3;
+  static constexpr int KV_STAGES = CS == 1 ? 3 : 2;
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = Q_BYTES;
   static constexpr int BAR_OFF = KV_OFF + KV_STAGES * KV_STAGE;
   static constexpr int XCH_OFF = BAR_OFF + 256;          // float2 exchange[2 halves][128 rows]
-  static constexpr int SMEM_BYTES = XCH_OFF + 2048;      // the dynamic shared window must be 1024-byte aligned (checked)
+  // clusters: the row statistics of every CTA and the output blocks of 32 columns that the others send to this one
+  static constexpr int STATS_OFF = XCH_OFF + 2048;                      // float2 [CS][128]
+  static constexpr int OWN_BLOCKS = (D / 32) / CS;                      // output blocks that a CTA merges and stores
+  static constexpr int RECV_OFF = STATS_OFF + (CS > 1 ? CS * 1024 : 0);  // float4 [CS - 1][OWN_BLOCKS][8][128 rows]
+  static constexpr int SMEM_BYTES = RECV_OFF + (CS - 1) * OWN_BLOCKS * 16384;  // the dynamic shared window must be 1024-byte aligned (checked)
 };
 
 // One unit of work: a 128-row tile of one KV head and one segment of its key tiles.  Where it lies follows from its number
@@ -90,18 +94,32 @@ __device__ __forceinline__ AtcItem atc_item(const AtcPlace& pl, const int32_t* _
   it.partial = n_active > 1;
   return it;
 }
+// The segment of CTA `rank` of a cluster: at least one key tile, all of it masked where the row tile does not reach it.
+__device__ __forceinline__ AtcItem atc_cluster_item(const AtcPlace& pl, int rank, const int32_t* __restrict__ pos, int M, int G, int kv_len,
+                                                    int tiles_per_split) {
+  AtcItem it = atc_item(pl, pos, M, G, kv_len, 1 << 30, true);
+  it.kt0 = rank * tiles_per_split;
+  it.nkt = max(1, min(tiles_per_split, it.nkt_all - it.kt0));
+  return it;
+}
 
 // Persistent kernel: one CTA per SM walks its share of the items.  Item i of round r goes to CTA (i mod C) on even
 // rounds and to CTA C-1-(i mod C) on odd ones, so every CTA gets a mix of long and short items without any atomic.
 // Barrier phases and buffer indices follow counters that run across items (`it`: key tiles, `qn`: items with work),
 // so the TMA producer keeps prefetching the next item's K/V while the current one drains.
-template <int D>
+//
+// CS > 1: launches with few items.  A cluster of CS CTAs takes one item, each CTA a segment of its key tiles (there is one
+// round).  At the end every CTA sends its unnormalised output, 32 columns at a time, to the CTA that owns these columns
+// (distributed shared memory), and its row statistics to all; behind one cluster barrier the owners merge the segments in
+// their order and store.  With partial results through global memory and a kernel of its own for the merge (the other
+// split, kept for the statistics pass and for comparisons) the split costs 7 us, as much as eight key tiles.
+template <int D, int CS = 1>
 __global__ void __launch_bounds__(ATC_THREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const bf16* __restrict__ q, const int32_t* __restrict__ pos, int M, int kv_len, bf16* __restrict__ o,
                     float* __restrict__ lse, int Hq, int Hkv, float scale_log2, uint32_t* status,
                     int n_split, int tiles_per_split, float* __restrict__ part_o, float2* __restrict__ part_ml) {
-  using L = AtcLayout<D>;
+  using L = AtcLayout<D, CS>;
   using namespace atc;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
@@ -136,8 +154,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int rows_total = M * G;
   const int row_tiles = (rows_total + ATC_BM - 1) / ATC_BM;
   const int rows_pad = row_tiles * ATC_BM;
-  const int n_items = row_tiles * n_split * Hkv;
-  const int C = gridDim.x, cta = blockIdx.x;
+  const int n_items = row_tiles * n_split * Hkv;  // CS > 1: n_split is 1
+  const int C = gridDim.x / CS, cta = blockIdx.x / CS;
+  const int rank = CS > 1 ? (int)cluster_rank() : 0;
   const bool want_o = o != nullptr;
   // item of round r for this CTA, or -1
   auto item_index = [&](int r) {
@@ -149,7 +168,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   // and its first K tile are requested without waiting for the positions: of the 13 400 clocks that a launch with one key
   // tile took from there, 5 600 went by before its first product (3 900 now).
   const AtcPlace first = atc_place(item_index(0) < 0 ? 0 : item_index(0), Hkv, row_tiles, n_split);
-  const bool k_ahead = n_split == 1 && item_index(0) >= 0;  // an unsplit item starts at key tile 0
+  const bool k_ahead = n_split == 1 && item_index(0) >= 0;  // the first key tile is then known: 0, or the segment's
+  auto item_of = [&](int r, int i) {
+    const AtcPlace pl = r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split);
+    return CS > 1 ? atc_cluster_item(pl, rank, pos, M, G, kv_len, tiles_per_split)
+                  : atc_item(pl, pos, M, G, kv_len, tiles_per_split, n_split == 1);
+  };
+  if (CS > 1) cluster_arrive();  // waited for before the first access to another CTA's shared memory
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < L::KV_STAGES; ++i) {
@@ -181,6 +206,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   pdl_wait();  // the set-up above overlapped the previous kernel's tail; positions, Q and the cache are read below
   pdl_launch_dependents();
   const uint32_t tmem_s0 = tmem_base, tmem_o = tmem_base + 256;
+  // CS > 1: what the softmax threads keep for the merge behind the cluster barrier
+  constexpr int BLOCKS = D / 64;  // blocks of 32 output columns per thread
+  float keep[CS > 1 ? BLOCKS * 32 : 1];
+  bool merge = false, cluster_met = false;
 
   if (warp == 0) {
     // ---------------- TMA producer (the whole warp walks, one elected lane issues)
@@ -199,11 +228,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
       __syncwarp();
     };
-    if (k_ahead) load_k(first.g, 0);
+    if (k_ahead) load_k(first.g, rank * tiles_per_split * ATC_BN);
     for (int r = 0; r < rounds && ok; ++r) {
       const int i = item_index(r);
       if (i < 0) continue;
-      const AtcItem w = atc_item(r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split), pos, M, G, kv_len, tiles_per_split, n_split == 1);
+      const AtcItem w = item_of(r, i);
       const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0), row0 = __shfl_sync(0xffffffffu, w.kt0 * ATC_BN, 0);
       for (int kt = 0; kt < nkt; ++kt) {
         const uint32_t sv = base + L::KV_OFF + s * L::KV_STAGE + (D / 64) * L::SUB;
@@ -263,7 +292,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     for (int r = 0; r < rounds && ok; ++r) {
       const int i = item_index(r);
       if (i < 0) continue;
-      const AtcItem w = atc_item(r == 0 ? first : atc_place(i, Hkv, row_tiles, n_split), pos, M, G, kv_len, tiles_per_split, n_split == 1);
+      const AtcItem w = item_of(r, i);
       const int nkt = __shfl_sync(0xffffffffu, w.valid ? w.nkt : 0, 0);
       if (nkt == 0) continue;
       ok = mbar_wait_warp(q_ready, qn & 1, abort_flag, status);
@@ -356,7 +385,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int j = 0; j < D / 16; ++j, qrow.next())
         qv[j] = qrow.tok < M ? __ldcg(reinterpret_cast<const uint4*>(q + ((size_t)qrow.tok * Hq + pl.g * G + qrow.head) * D) + st % (D / 8))
                              : make_uint4(0, 0, 0, 0);
-      const AtcItem w = atc_item(pl, pos, M, G, kv_len, tiles_per_split, n_split == 1);
+      const AtcItem w = item_of(r, i);
       if (!w.valid) continue;
       const int lim = row_ok ? min(pos[tok], kv_len - 1) : -1;
       const size_t prow = ((size_t)w.z * Hkv + w.g) * (size_t)rows_pad + fr;  // partial-result row
@@ -484,7 +513,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           }
           st32(ts, reinterpret_cast<const float*>(pk));
           wait_st();
-          if (w.kt0 + kt == w.nkt_all - 1 && half == 0) {
+          if (w.kt0 + kt >= w.nkt_all - 1 && half == 0) {
             // slots beyond the row tile's last visible key may hold anything: they get probability zero, and zero
             // times a non-finite value would still poison the product, so clear those V rows of the last tile (the 128
             // threads of the first half, eight to a row: a row per thread puts all of a warp's stores on four banks)
@@ -526,6 +555,36 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         if (!ok) break;
         fence_after();
         bf16* dst = o + ((size_t)tok * Hq + hq) * D + half * (D / 2);
+        if constexpr (CS > 1) {
+          const float fa = half == 0 ? f_mine : f_other, fb = half == 0 ? f_other : f_mine;
+          cluster_wait();  // every CTA of the cluster runs
+          cluster_met = true;
+#pragma unroll
+          for (int c = 0; c < BLOCKS; ++c) {
+            float t[32], u[32];
+            ld32(tmem_o + lane_addr + half * (D / 2) + c * 32, t);
+            ld32(tmem_o + D + lane_addr + half * (D / 2) + c * 32, u);
+            wait_ld();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) t[e] = fmaf(t[e], fa, u[e] * fb);
+            const int block = half * BLOCKS + c, owner = block / L::OWN_BLOCKS;
+            if (owner == rank) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) keep[c * 32 + e] = t[e];
+            } else {
+              const int from = rank < owner ? rank : rank - 1;
+              const uint32_t dst_s = map_to_cta(base + L::RECV_OFF + ((from * L::OWN_BLOCKS + block % L::OWN_BLOCKS) * 8 * 128 + row) * 16, owner);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) st_cluster4(dst_s + j * 128 * 16, t[4 * j], t[4 * j + 1], t[4 * j + 2], t[4 * j + 3]);
+            }
+          }
+          if (half == 0) {
+#pragma unroll
+            for (int z = 0; z < CS; ++z) st_cluster2(map_to_cta(base + L::STATS_OFF + (rank * 128 + row) * 8, z), m_ref, l_run);
+          }
+          merge = true;
+          break;  // one item
+        }
         const float fa = (half == 0 ? f_mine : f_other) * (w.partial ? 1.f : inv), fb = (half == 0 ? f_other : f_mine) * (w.partial ? 1.f : inv);
 #pragma unroll 1
         for (int c = 0; c < D / 64; ++c) {  // this thread's half of the output columns, from both accumulators
@@ -552,6 +611,62 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       if (half == 0) {
         if (row_ok && w.partial) part_ml[prow] = make_float2(m_ref, l_run);
         if (row_ok && !w.partial && lse) lse[(size_t)tok * Hq + hq] = l_run > 0.f ? (m_ref + log2f(l_run)) * ATC_LN2 : -INFINITY;
+      }
+    }
+  }
+  if constexpr (CS > 1) {
+    if (!cluster_met) cluster_wait();
+    cluster_arrive();
+    cluster_wait();  // everything sent has arrived; from here on a CTA reads its own shared memory only
+    if (merge) {
+      const int half = (warp - 2) >> 2, row = (warp & 3) * 32 + lane;
+      const int fr = first.r0 + row;
+      const float2* stats = reinterpret_cast<const float2*>(base_ptr + L::STATS_OFF) + row;
+      float m = -INFINITY, l = 0.f, wz[CS];
+#pragma unroll
+      for (int z = 0; z < CS; ++z)
+        if (stats[z * 128].y > 0.f) m = fmaxf(m, stats[z * 128].x);
+#pragma unroll
+      for (int z = 0; z < CS; ++z) {
+        const float2 ml = stats[z * 128];
+        wz[z] = ml.y > 0.f ? exp2f(ml.x - m) : 0.f;
+        l += ml.y * wz[z];
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      if (fr < rows_total) {
+        const int tok = fr / G, hq = first.g * G + fr % G;
+#pragma unroll
+        for (int c = 0; c < BLOCKS; ++c) {
+          const int block = half * BLOCKS + c;
+          if (block / L::OWN_BLOCKS != rank) continue;
+          float acc[32];
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+#pragma unroll
+          for (int z = 0; z < CS; ++z) {
+            if (!(wz[z] > 0.f)) continue;  // a segment without a visible key: nothing of it counts
+            const float w = wz[z] * inv;
+            if (z == rank) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) acc[e] = fmaf(keep[c * 32 + e], w, acc[e]);
+            } else {
+              const int from = z < rank ? z : z - 1;
+              const float4* src = reinterpret_cast<const float4*>(base_ptr + L::RECV_OFF) + (from * L::OWN_BLOCKS + block % L::OWN_BLOCKS) * 8 * 128 + row;
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float4 v = src[j * 128];
+                acc[4 * j] = fmaf(v.x, w, acc[4 * j]);
+                acc[4 * j + 1] = fmaf(v.y, w, acc[4 * j + 1]);
+                acc[4 * j + 2] = fmaf(v.z, w, acc[4 * j + 2]);
+                acc[4 * j + 3] = fmaf(v.w, w, acc[4 * j + 3]);
+              }
+            }
+          }
+          uint4* dst = reinterpret_cast<uint4*>(o + ((size_t)tok * Hq + hq) * D + block * 32);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) dst[j] = pack8(acc + 8 * j);
+        }
+        if (lse && rank == 0 && half == 0) lse[(size_t)tok * Hq + hq] = l > 0.f ? (m + log2f(l)) * ATC_LN2 : -INFINITY;
       }
     }
   }
@@ -663,6 +778,28 @@ size_t attention_part_bytes(const a3_handle* h) {
   return 4 * rows * ((size_t)h->m.head_dim + 2) * sizeof(float);
 }
 
+// CTAs per item of a launch with few items (1: no clusters).  A key tile takes 0.85 us, the merge about 1.5: two CTAs pay from
+// six key tiles on (Llama width, 144 rows over 826 slots: layer 66.4 -> 65.8 us; 60 rows over 800: 59.2 -> 60.1), four from
+// eight (60 rows over 2 000 slots 69.5 -> 60.0, 280 rows over 1 900 with two 78.2 -> 73.4).  33 clusters of four CTAs with
+// this much shared memory are resident at a time (a cluster stays inside one group of SMs), hence the tenth.
+static int cluster_size(int items, int tiles, int sms, int D) {
+  if (D == 128 && items * 4 <= sms - sms / 10 && tiles >= 8) return 4;
+  if (items * 2 <= sms && tiles >= 6) return 2;
+  return 1;
+}
+template <int D, int CS>
+static int launch_cluster(const a3_handle* h, const CUtensorMap& tK, const CUtensorMap& tV, const bf16* q, const int32_t* pos, int M, int kv_len,
+                          bf16* o, float* lse, int items, float scale_log2, cudaStream_t st) {
+  using L = AtcLayout<D, CS>;
+  static SmemAttrOnce attr;
+  A3_TRY(smem_attr_once(attr, h->device, attention_tc_kernel<D, CS>, L::SMEM_BYTES));
+  A3_CUDA(launch_pdl_cluster(CS, attention_tc_kernel<D, CS>, dim3(items * CS), dim3(ATC_THREADS), (size_t)L::SMEM_BYTES, st, tK, tV, q, pos, M, kv_len, o,
+                             lse, h->m.n_q_heads, h->m.n_kv_heads, scale_log2, h->dev_status, 1, cdiv(cdiv(kv_len, ATC_BN), CS), (float*)nullptr,
+                             (float2*)nullptr));
+  A3_LAUNCHED();
+  return A3_OK;
+}
+
 int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M, const bf16* k, const bf16* v,
                       int kv_len, bf16* o, float* lse, void* part, size_t part_bytes, cudaStream_t st) {
   if (M <= 0) return A3_OK;
@@ -681,6 +818,16 @@ int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M,
     if (use_pair && o && D == 128) {
       const int s = attention_rows_pair(h, tK, tV, q, pos, M, kv_len, o, lse, st);
       if (s != A3_EUNSUPPORTED) return s;
+    }
+  }
+  const int sms_all = h->sm_count > 0 ? h->sm_count : 148;
+  if (o && h->opt[A3_OPT_ATTN_SPLIT] == 0 && h->opt[A3_OPT_ATTN_MAX_CTAS] == 0) {
+    const int cs = cluster_size((int)grid.x * Hkv, cdiv(kv_len, ATC_BN), sms_all, D);
+    if (cs > 1) {
+      ProfScope prof(h, A3_K_ATTENTION, st);
+      if (D == 128 && cs == 4) return launch_cluster<128, 4>(h, tK, tV, q, pos, M, kv_len, o, lse, (int)grid.x * Hkv, scale_log2, st);
+      if (D == 128) return launch_cluster<128, 2>(h, tK, tV, q, pos, M, kv_len, o, lse, (int)grid.x * Hkv, scale_log2, st);
+      return launch_cluster<64, 2>(h, tK, tV, q, pos, M, kv_len, o, lse, (int)grid.x * Hkv, scale_log2, st);
     }
   }
   // split over the keys when the grid would leave SMs idle behind a few long row tiles
