@@ -162,9 +162,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
               const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmW, const SpParams p) {
   constexpr int ROWS = EPI == EPI_SWIGLU ? SP_FEAT : 2 * SP_FEAT;  // output features per CTA
-  extern __shared__ unsigned char smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // same offset in both CTAs of the pair
-  unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const uint32_t base = smem_u32(smem_raw);  // same offset in both CTAs of the pair
+  unsigned char* base_ptr = smem_raw;
+  if (base & 1023u) {  // the swizzled tiles need a 1024-byte aligned window; uniform for the launch, nothing is set up yet
+    if (threadIdx.x == 0) atomicOr(p.status, A3_DEV_WAIT_EXHAUSTED);
+    return;
+  }
   const int S = p.stages;
   const int xch_off = S * p.stage_bytes, bar_off = xch_off + (SPLIT ? 0 : sp_xch_bytes(EPI, p.chunk));
   // barriers (8 bytes each): full[8] (used in the leader), empty[8], tmem_full[2], tmem_empty[2] (used in the leader)
@@ -778,23 +782,25 @@ int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) 
 }
 
 // Ring depth and epilogue chunk of a launch: the widest chunk among those that leave the ring deepest (a stage more is 8 %
-// at 513 rows, where 32-token chunks leave three stages of 176 tokens and 8-token chunks four).  Returns the dynamic
-// shared memory.
+// at 513 rows, where 32-token chunks leave three stages of 176 tokens and 8-token chunks four), but no deeper than a pair
+// has stages to run through.  Returns the dynamic shared memory.
 static int set_stages(SpParams& p, int epi, bool split) {
   p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
   p.stages = 0;
+  const long long steps = (long long)cdiv(p.n_units, p.n_pairs) * (p.K / TC_BK / SP_SUB);
+  const int useful = steps < SP_MAX_STAGES ? (int)steps : SP_MAX_STAGES;
   int xch = 0;
   for (int chunk = 32; chunk >= (epi == EPI_QKV ? 16 : 8); chunk /= 2) {
     const int x = split ? 0 : sp_xch_bytes(epi, chunk);
-    int stages = (SP_SMEM_LIMIT - x - 256 - 1024) / p.stage_bytes;
-    if (stages > SP_MAX_STAGES) stages = SP_MAX_STAGES;
+    int stages = (SP_SMEM_LIMIT - x - 256) / p.stage_bytes;
+    if (stages > useful) stages = useful;
     if (stages > p.stages) {
       p.stages = stages;
       p.chunk = chunk;
       xch = x;
     }
   }
-  return p.stages * p.stage_bytes + xch + 256 + 1024;
+  return p.stages * p.stage_bytes + xch + 256;
 }
 
 int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st) {
