@@ -22,10 +22,146 @@ __device__ __forceinline__ uint32_t score_key(float s) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);  // larger float <=> larger key
 }
 
+// Sums the private histograms and finds the bin of the element of rank `remaining` (1-based, from the top); the caller's
+// prefix and remaining move on to that bin.  All threads.
+__device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned int* warp_tot, unsigned int* s_prefix,
+                                         unsigned int* s_remaining, int shift, uint32_t& prefix, unsigned int& remaining) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned int v = 0;
+  if (tid < 256) {
+#pragma unroll
+    for (int w = 0; w < TK_HISTS; ++w) v += whist[w][tid];
+    // suffix sums over the bins: S[d] = count of elements with digit >= d; the k-th element's digit is the largest d
+    // with S[d] >= remaining
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int t = __shfl_down_sync(0xffffffffu, v, o);
+      if (lane + o < 32) v += t;
+    }
+    if (lane == 0) warp_tot[warp] = v;
+  }
+  __syncthreads();
+  if (tid < 256) {
+    unsigned int above = 0;  // elements in the bins of higher warps
+    for (int w = warp + 1; w < 8; ++w) above += warp_tot[w];
+    const unsigned int next = __shfl_down_sync(0xffffffffu, v, 1);
+    const unsigned int S_d = v + above, S_next = lane == 31 ? above : next + above;  // S[d], S[d + 1]
+    if (S_d >= remaining && S_next < remaining) {
+      *s_prefix = prefix | ((uint32_t)tid << shift);
+      *s_remaining = remaining - S_next;
+    }
+  }
+  __syncthreads();
+  prefix = *s_prefix;
+  remaining = *s_remaining;
+}
+
+// Up to KPT x 1 024 candidates, which is every request of a few thousand tokens: a thread keeps its keys (slots tid, tid +
+// 1 024, ...) in registers through all passes.  With half_pool the keys are of the running maximum over the neighbouring
+// candidates, taken from a copy of the scores in shared memory.  Bound by the chain of block barriers, three per pass:
+// 5 120 candidates take 5.4 us where the passes over shared memory below took 10.
+template <int KPT>
+__device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __restrict__ raw, int cand_begin, int n, int k, int half_pool,
+                                          int32_t* __restrict__ idx_out, uint32_t* status) {
+  __shared__ unsigned int whist[2][TK_HISTS][256];  // passes alternate: one is cleared while the other counts
+  __shared__ unsigned int warp_tot[8];
+  __shared__ unsigned int s_prefix, s_remaining;
+  __shared__ unsigned int cnt[2][KPT * TK_WARPS];  // greater-than and equal candidates of (round, warp), in slot order
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float v[KPT];
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) v[j] = tid + j * TK_THREADS < n ? __ldcg(s + tid + j * TK_THREADS) : 0.f;
+  for (int i = tid; i < TK_HISTS * 256; i += TK_THREADS) (&whist[0][0][0])[i] = 0;
+  if (half_pool > 0) {
+#pragma unroll
+    for (int j = 0; j < KPT; ++j)
+      if (tid + j * TK_THREADS < n) raw[tid + j * TK_THREADS] = v[j];
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const int i = tid + j * TK_THREADS;
+      if (i < n)
+        for (int t = max(0, i - half_pool); t <= min(n - 1, i + half_pool); ++t) v[j] = fmaxf(v[j], raw[t]);
+    }
+  }
+  uint32_t key[KPT];
+  bool nonfinite = false;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool live = tid + j * TK_THREADS < n;
+    nonfinite = nonfinite || (live && !(fabsf(v[j]) <= 3.0e38f));
+    key[j] = score_key(v[j]);
+  }
+  if (nonfinite) atomicOr(status, A3_DEV_NONFINITE_SCORE);
+  uint32_t prefix = 0, mask = 0;
+  unsigned int remaining = (unsigned int)k;
+  __syncthreads();
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 24 - 8 * pass;
+    unsigned int* mine = whist[pass & 1][warp % TK_HISTS];
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const bool in = tid + j * TK_THREADS < n && (key[j] & mask) == prefix;
+      if (!__any_sync(0xffffffffu, in)) continue;  // the rule behind the first passes
+      const uint32_t digit = in ? (key[j] >> shift) & 255u : 0xFFFFFFFFu;
+      const uint32_t first = __shfl_sync(0xffffffffu, digit, 0);
+      if (__all_sync(0xffffffffu, digit == first)) {
+        if (lane == 0) atomicAdd(&mine[digit], 32u);
+      } else if (in) {
+        atomicAdd(&mine[digit], 1u);
+      }
+    }
+    for (int i = tid; i < TK_HISTS * 256; i += TK_THREADS) (&whist[(pass & 1) ^ 1][0][0])[i] = 0;
+    __syncthreads();
+    topk_bin(whist[pass & 1], warp_tot, &s_prefix, &s_remaining, shift, prefix, remaining);
+    mask |= 255u << shift;
+  }
+  // ordered emission
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool live = tid + j * TK_THREADS < n;
+    const unsigned int bgt = __ballot_sync(0xffffffffu, live && key[j] > prefix), beq = __ballot_sync(0xffffffffu, live && key[j] == prefix);
+    if (lane == 0) {
+      cnt[0][j * TK_WARPS + warp] = __popc(bgt);
+      cnt[1][j * TK_WARPS + warp] = __popc(beq);
+    }
+  }
+  __syncthreads();
+  if (warp < 2) {  // exclusive prefix sums, warp 0 the greater ones, warp 1 the equal ones
+    unsigned int run = 0;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const unsigned int c = cnt[warp][j * TK_WARPS + lane];
+      unsigned int x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+      }
+      cnt[warp][j * TK_WARPS + lane] = run + x - c;
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+  }
+  __syncthreads();
+  const unsigned int lt_mask = (1u << lane) - 1u;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const int i = tid + j * TK_THREADS;
+    const bool gt = i < n && key[j] > prefix, eq = i < n && key[j] == prefix;
+    const unsigned int bgt = __ballot_sync(0xffffffffu, gt), beq = __ballot_sync(0xffffffffu, eq);
+    const unsigned int my_gt = cnt[0][j * TK_WARPS + warp] + __popc(bgt & lt_mask);
+    const unsigned int my_eq = cnt[1][j * TK_WARPS + warp] + __popc(beq & lt_mask);
+    if (gt || (eq && my_eq < remaining)) {
+      const unsigned int o = my_gt + (my_eq < remaining ? my_eq : remaining);
+      if (o < (unsigned int)k) idx_out[o] = cand_begin + i;
+    }
+  }
+}
+
 template <bool IN_SMEM>
 __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t* __restrict__ keys, int cand_begin, int n, int k, int half_pool,
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
-  __shared__ unsigned int hist[256];
   __shared__ unsigned int whist[TK_HISTS][256];
   __shared__ unsigned int warp_tot[8];
   __shared__ unsigned int s_prefix, s_remaining;
@@ -68,40 +204,7 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
       }
     }
     __syncthreads();
-    if (tid < 256) {
-      unsigned int v = 0;
-#pragma unroll
-      for (int w = 0; w < TK_HISTS; ++w) v += whist[w][tid];
-      hist[tid] = v;
-    }
-    __syncthreads();
-    // suffix sums over the bins: S[d] = count of elements with digit >= d; the k-th element's digit is the largest d
-    // with S[d] >= remaining
-    if (tid < 256) {
-      unsigned int v = hist[tid];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int t = __shfl_down_sync(0xffffffffu, v, o);
-        if (lane + o < 32) v += t;
-      }
-      if (lane == 0) warp_tot[warp] = v;
-      __syncwarp();
-      hist[tid] = v;  // suffix sum within this warp's 32 bins
-    }
-    __syncthreads();
-    if (tid < 256) {
-      unsigned int above = 0;  // elements in the bins of higher warps
-      for (int w = warp + 1; w < 8; ++w) above += warp_tot[w];
-      const unsigned int S_d = hist[tid] + above;
-      const unsigned int S_next = lane == 31 ? above : hist[tid + 1] + above;  // S[d + 1]
-      if (S_d >= remaining && S_next < remaining) {
-        s_prefix = prefix | ((uint32_t)tid << shift);
-        s_remaining = remaining - S_next;
-      }
-    }
-    __syncthreads();
-    prefix = s_prefix;
-    remaining = s_remaining;
+    topk_bin(whist, warp_tot, &s_prefix, &s_remaining, shift, prefix, remaining);
     mask |= 255u << shift;
   }
   // `remaining` = how many elements equal to the threshold key are taken (lowest slots first)
@@ -145,6 +248,8 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
   }
 }
 
+// REGS > 0: at most REGS x 1 024 candidates, in registers; 0: any number, in shared memory or re-read from global memory
+template <int REGS>
 __global__ void __launch_bounds__(TK_THREADS)
 topk_select_kernel(const float* __restrict__ scores, int cand_begin, int n, int k, int32_t* __restrict__ idx_out, uint32_t* status,
                    size_t score_stride, size_t idx_stride, int in_smem, int half_pool, int tail_begin, int tail) {
@@ -155,6 +260,10 @@ topk_select_kernel(const float* __restrict__ scores, int cand_begin, int n, int 
   const float* s = scores + blockIdx.x * score_stride + cand_begin;
   int32_t* out = idx_out + blockIdx.x * idx_stride;
   for (int i = threadIdx.x; i < tail; i += TK_THREADS) out[k + i] = tail_begin + i;
+  if constexpr (REGS > 0) {
+    topk_regs<REGS>(s, reinterpret_cast<float*>(tk_keys), cand_begin, n, k, half_pool, out, status);
+    return;
+  }
   if (in_smem) topk_body<true>(s, tk_keys, cand_begin, n, k, half_pool, out, status);
   else topk_body<false>(s, tk_keys, cand_begin, n, k, 0, out, status);
 }
@@ -162,12 +271,30 @@ topk_select_kernel(const float* __restrict__ scores, int cand_begin, int n, int 
 static int launch_topk(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int n, int k,
                        int half_pool, int tail_begin, int tail, int32_t* idx_out, size_t idx_stride, cudaStream_t st) {
   const int in_smem = n <= TK_SMEM_KEYS ? 1 : 0;
-  const size_t smem = in_smem ? (size_t)n * 4 : 0;
-  static SmemAttrOnce attr;
-  A3_TRY(smem_attr_once(attr, h->device, topk_select_kernel, TK_SMEM_KEYS * 4));
   ProfScope prof(h, A3_K_TOPK, st);
-  A3_CUDA(launch_pdl(topk_select_kernel, dim3(batches), dim3(TK_THREADS), smem, st, scores, cand_begin, n, k, idx_out, h->dev_status,
-                     score_stride, idx_stride, in_smem, half_pool, tail_begin, tail));
+  auto go = [&](auto kernel, size_t smem) {
+    return launch_pdl(kernel, dim3(batches), dim3(TK_THREADS), smem, st, scores, cand_begin, n, k, idx_out, h->dev_status, score_stride, idx_stride,
+                      in_smem, half_pool, tail_begin, tail);
+  };
+  const size_t raw = half_pool > 0 ? (size_t)n * 4 : 0;
+  // half a microsecond per key and thread: as few keys per thread as the candidates need
+  if (n <= TK_THREADS) {
+    A3_CUDA(go(topk_select_kernel<1>, raw));
+  } else if (n <= 3 * TK_THREADS) {
+    A3_CUDA(go(topk_select_kernel<3>, raw));
+  } else if (n <= 5 * TK_THREADS) {
+    static SmemAttrOnce attr5;
+    A3_TRY(smem_attr_once(attr5, h->device, topk_select_kernel<5>, 5 * TK_THREADS * 4));
+    A3_CUDA(go(topk_select_kernel<5>, raw));
+  } else if (n <= 8 * TK_THREADS) {
+    static SmemAttrOnce attr8;
+    A3_TRY(smem_attr_once(attr8, h->device, topk_select_kernel<8>, 8 * TK_THREADS * 4));
+    A3_CUDA(go(topk_select_kernel<8>, raw));
+  } else {
+    static SmemAttrOnce attr;
+    A3_TRY(smem_attr_once(attr, h->device, topk_select_kernel<0>, TK_SMEM_KEYS * 4));
+    A3_CUDA(go(topk_select_kernel<0>, in_smem ? (size_t)n * 4 : 0));
+  }
   A3_LAUNCHED();
   return A3_OK;
 }

@@ -99,3 +99,47 @@ def test_attention_keys_shared_by_a_cluster(a3mod, shape, kv_len, M):
     assert eng.device_status() & a3mod.DEV_BAD_POSITION
     assert torch.isfinite(dX.float()).all()
     eng.close()
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 3071, 3072, 3073, 5119, 5121, 8192, 8193])
+def test_topk_at_the_register_sizes(a3mod, n):
+    """Candidate counts around those at which a thread holds one key more, with ties across the threshold and k = 1, n - 1."""
+    eng, _, dev = make_engine(a3mod, W.TINY)
+    s = (np.random.default_rng(n).integers(0, 37, size=n) / 32.0).astype(np.float32)
+    for k in (1, n // 7, n - 1):
+        got = eng.topk_select(torch.from_numpy(s).to(dev), 0, n, k).cpu().numpy()
+        assert got.tolist() == O.topk_select(s.astype(np.float64), 0, n, k).tolist()
+    assert eng.device_status() == 0
+    eng.close()
+
+
+@pytest.mark.parametrize("n_ctx,pool", [(900, 3), (3073, 7), (5120, 5), (8200, 7)])
+def test_pooled_selection_of_the_eviction(a3mod, n_ctx, pool):
+    """Pooling inside the selection: votes in registers, and (8 200 candidates) in shared memory."""
+    m = W.TINY_GQA
+    eng, _, dev = make_engine(a3mod, m, seed=n_ctx)
+    model, nq, n_system, capacity = oracle_model(m), 9, 5, 300
+    rng = np.random.default_rng(n_ctx)
+    K, V = (W.bf16_round(rng.standard_normal((n_ctx + nq, m.n_kv_heads, m.head_dim), dtype=np.float32)) for _ in range(2))
+    q = W.bf16_round(rng.standard_normal((nq, m.n_q_heads, m.head_dim), dtype=np.float32))
+    pos = np.arange(n_ctx, n_ctx + nq)
+    dq, dK, dpos = to_dev(q, dev), to_dev(K, dev), torch.from_numpy(pos.astype(np.int32)).to(dev)
+    s = np.einsum("jhd,ihd->jhi", q.astype(np.float64), np.repeat(K, m.n_q_heads // m.n_kv_heads, axis=1).astype(np.float64)) / np.sqrt(m.head_dim)
+    s[np.broadcast_to(np.arange(n_ctx + nq)[None, None, :] > pos[:, None, None], s.shape)] = -np.inf
+    lse = np.log(np.exp(s).sum(axis=2)).astype(np.float32)
+    k_out, v_out, kept = eng.evict_layer(dq, dpos, torch.from_numpy(lse).to(dev), dK, to_dev(V, dev), n_system, n_ctx, capacity, pool)
+    assert eng.device_status() == 0
+    votes = O.pool_scores(O.eviction_scores(q, pos, K, model, n_system, n_ctx), n_system, n_ctx, pool)
+    k = capacity - n_system - nq
+    for g in range(m.n_kv_heads):
+        idx = kept[g].cpu().numpy()
+        assert idx[:n_system].tolist() == list(range(n_system)) and idx[-nq:].tolist() == list(range(n_ctx, n_ctx + nq))
+        sel = idx[n_system:n_system + k]
+        assert (np.diff(sel) > 0).all()
+        v = votes[g][n_system:n_ctx]
+        thr = np.sort(v)[-k]
+        inside = np.isin(np.arange(n_system, n_ctx), sel)
+        # votes are sums of fp32 exponentials: 1e-3 relative, as for the scores
+        assert (v[inside] >= thr * (1 - 2e-3)).all() and (v[~inside] <= thr * (1 + 2e-3)).all()
+        assert torch.equal(k_out[:, g], dK[kept[g].long(), g])
+    eng.close()
