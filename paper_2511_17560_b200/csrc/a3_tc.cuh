@@ -201,6 +201,17 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
                ::"r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar)
                : "memory");
 }
+// the same for data that nobody reads again (policy: l2_evict_first): its lines are the first to leave L2
+__device__ __forceinline__ void tma_load_3d_pair_once(uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar, uint64_t policy) {
+  asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+               ::"r"(dst), "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar), "l"(policy)
+               : "memory");
+}
+__device__ __forceinline__ uint64_t l2_evict_first() {
+  uint64_t policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  return policy;
+}
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(cta_mask) : "memory");
 }
