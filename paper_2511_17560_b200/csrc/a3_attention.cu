@@ -352,6 +352,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const uint32_t tmem_oh = tmem_o + half * D;  // this thread's accumulator
+    // 16-byte chunk c of this half of row `rw` of the Q buffer (swizzled K-major sub-tiles)
+    constexpr int ROW_CHUNKS = D / 16;
+    auto row_chunk = [&](int rw, int c) {
+      const int col = half * ROW_CHUNKS + c;
+      return reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (col / 8) * L::SUB + swz(rw, col % 8));
+    };
     constexpr float OVERFLOW_GUARD = 65536.f;
     uint32_t it = 0, px = 0;  // running key tile; running count of pair exchanges (parity of the pair barrier)
     bool ok = true;
@@ -377,13 +383,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const bool row_ok = fr < rows_total;
       const int tok = row_ok ? fr / G : 0;
       const int hq = pl.g * G + (row_ok ? fr % G : 0);
-      // the item's Q rows, on their way while the positions are read: consecutive threads take consecutive 16-byte chunks
-      uint4 qv[D / 16];
-      const int st = threadIdx.x - 64;  // of the 256 threads
-      QRow qrow(pl.r0 + st / (D / 8), 256 / (D / 8), G);
+      // The item's Q rows, on their way while the positions are read: a warp takes its half of its 32 rows, consecutive lanes
+      // consecutive 16-byte chunks.  The output rows leave the same way (below), so a warp meets no other in this buffer.
+      uint4 qv[ROW_CHUNKS];
+      const int lane_row = quarter * 32 + lane / ROW_CHUNKS, lane_chunk = lane % ROW_CHUNKS;
+      QRow qrow(pl.r0 + lane_row, 32 / ROW_CHUNKS, G);
 #pragma unroll
-      for (int j = 0; j < D / 16; ++j, qrow.next())
-        qv[j] = qrow.tok < M ? __ldcg(reinterpret_cast<const uint4*>(q + ((size_t)qrow.tok * Hq + pl.g * G + qrow.head) * D) + st % (D / 8))
+      for (int j = 0; j < ROW_CHUNKS; ++j, qrow.next())
+        qv[j] = qrow.tok < M ? __ldcg(reinterpret_cast<const uint4*>(q + ((size_t)qrow.tok * Hq + pl.g * G + qrow.head) * D + half * (D / 2)) + lane_chunk)
                              : make_uint4(0, 0, 0, 0);
       const AtcItem w = item_of(r, i);
       if (!w.valid) continue;
@@ -405,11 +412,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       // Q rows -> shared memory, swizzled K-major sub-tiles.
       // The previous item's S MMAs have all completed (their last s_full was waited for), so the Q buffer is free.
       {
+        __syncwarp();  // the previous item's output rows have been read out of the buffer
 #pragma unroll
-        for (int j = 0; j < D / 16; ++j) {
-          const int qr = (st + 256 * j) / (D / 8), qc = st % (D / 8);
-          *reinterpret_cast<uint4*>(base_ptr + L::Q_OFF + (qc / 8) * L::SUB + swz(qr, qc % 8)) = qv[j];
-        }
+        for (int j = 0; j < ROW_CHUNKS; ++j) *row_chunk(lane_row + j * (32 / ROW_CHUNKS), lane_chunk) = qv[j];
         fence_async_smem();
         mbar_arrive(q_ready);
       }
@@ -554,7 +559,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         ok = __all_sync(0xffffffffu, mbar_wait(p_free(it_last & 1), (it_last >> 1) & 1, abort_flag, status));
         if (!ok) break;
         fence_after();
-        bf16* dst = o + ((size_t)tok * Hq + hq) * D + half * (D / 2);
         if constexpr (CS > 1) {
           const float fa = half == 0 ? f_mine : f_other, fb = half == 0 ? f_other : f_mine;
           cluster_wait();  // every CTA of the cluster runs
@@ -598,11 +602,23 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float4* pd = reinterpret_cast<float4*>(part_o + prow * D + half * (D / 2) + c * 32);
 #pragma unroll
             for (int j = 0; j < 8; ++j) pd[j] = make_float4(t[4 * j], t[4 * j + 1], t[4 * j + 2], t[4 * j + 3]);
-          } else if (row_ok) {
+          } else if (!w.partial) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) reinterpret_cast<uint4*>(dst + c * 32)[j] = pack8(t + 8 * j);
+            for (int j = 0; j < 4; ++j) *row_chunk(row, c * 4 + j) = pack8(t + 8 * j);
           }
           __syncwarp();
+        }
+        if (!w.partial) {
+          // through the Q buffer, which the item's last S MMA has read: a warp instruction touches four lines (D = 64: eight)
+          // where a row per lane touched 32.  A layer of 75 rows 89.6 -> 88.7 us, of 68 rows of a small model 42.0 -> 41.3: the
+          // 2 us from P V to the last store are a third of a one-tile launch.
+          QRow orow(pl.r0 + lane_row, 32 / ROW_CHUNKS, G);
+#pragma unroll
+          for (int j = 0; j < ROW_CHUNKS; ++j, orow.next()) {
+            const uint4 v = *row_chunk(lane_row + j * (32 / ROW_CHUNKS), lane_chunk);
+            if (orow.tok < M)
+              *(reinterpret_cast<uint4*>(o + ((size_t)orow.tok * Hq + pl.g * G + orow.head) * D + half * (D / 2)) + lane_chunk) = v;
+          }
         }
         // the next item's first P V overwrites O: it is issued only after this item's p_ready arrivals of all 256
         // threads for that tile, which each thread makes after the loads above
