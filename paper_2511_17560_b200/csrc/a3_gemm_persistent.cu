@@ -157,8 +157,10 @@ __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc
 // SPLIT: a launch with fewer units than CTA pairs cuts the k-loop of every unit into k_slices and the epilogue writes
 // the slice's fp32 sums to `part` instead; the kernel that follows (RMSNorm, which reads these rows anyway) adds the
 // slices in order.  See residual_slices below for when and why.
-template <int EPI, bool SPLIT = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SP_THREADS, 1)
+// KC = 2 (QKV of few rows): a cluster of two pairs per unit, each with half of the k-loop.  The epilogue needs whole sums: pair c
+// finishes the tokens of warp set c and receives the other pair's sums for them through distributed shared memory.
+template <int EPI, bool SPLIT = false, int KC = 1>
+__global__ void __cluster_dims__(2 * KC, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
               const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmW, const SpParams p) {
   constexpr int ROWS = EPI == EPI_SWIGLU ? SP_FEAT : 2 * SP_FEAT;  // output features per CTA
@@ -183,9 +185,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   float* xch = reinterpret_cast<float*>(base_ptr + xch_off);
 
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
+  const uint32_t crank = cluster_ctarank(), rank = crank & 1u;  // CTA of the cluster, CTA of the pair
+  const int kc = (int)(crank >> 1);                             // the pair's part of the k-loop (KC > 1)
+  const uint32_t pair_cta0 = crank & ~1u;
+  const uint16_t pair_mask = (uint16_t)(3u << pair_cta0);
   const bool leader = rank == 0;
-  const int pair = blockIdx.x >> 1;
+  const int pair = blockIdx.x / (2 * KC);
+  int merged = 0;  // KC > 1: how many of the two cluster barriers of the merge this warp has passed
   const int KT = p.K / TC_BK;  // a multiple of SP_SUB (checked by the launcher)
   const int half_n = p.tok_n >> 1;  // token rows this CTA loads per k-block (multiple of 8)
   const uint32_t b_bytes = (uint32_t)half_n * TC_BK * 2;
@@ -250,6 +256,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         sp_unit(SPLIT ? u / p.k_slices : u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
         if (SPLIT) {
           sp_slice(u % p.k_slices, p.k_slices, KT / SP_SUB, kb0, kb1);
+          kb0 *= SP_SUB;
+          kb1 = kb0 + kb1 * SP_SUB;
+        } else if (KC > 1) {
+          sp_slice(kc, KC, KT / SP_SUB, kb0, kb1);
           kb0 *= SP_SUB;
           kb1 = kb0 + kb1 * SP_SUB;
         }
@@ -332,6 +342,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, a_sub16 = SP_A_BYTES >> 4, b_sub16 = (uint32_t)half_n * (TC_BK * 2) >> 4;
       const uint32_t tmem_acc = __shfl_sync(0xffffffffu, tmem_base, 0);
       int per_unit = KT / SP_SUB, total = 0;
+      if (KC > 1) {
+        int first;
+        sp_slice(kc, KC, KT / SP_SUB, first, per_unit);
+      }
       if (SPLIT) {
         for (int u = pair, first; u < p.n_units; u += p.n_pairs) {
           int count;
@@ -367,8 +381,8 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
             const int j = i / (TC_BK / 16), k = i % (TC_BK / 16);
             tc_mma_pair_acc(d, da_s + (uint64_t)(j * a_sub16 + 2 * k), db_s + (uint64_t)(j * b_sub16 + 2 * k), idesc);
           }
-          tc_commit_pair(empty_bar(s), 3);  // frees this stage in both CTAs once the instructions above have read it
-          if (in_unit + 1 == per_unit) tc_commit_pair(tmem_full(it & 1), 3);  // publishes the accumulator in both CTAs
+          tc_commit_pair(empty_bar(s), pair_mask);  // frees this stage in both CTAs once the instructions above have read it
+          if (in_unit + 1 == per_unit) tc_commit_pair(tmem_full(it & 1), pair_mask);  // publishes the accumulator in both CTAs
         }
         __syncwarp();
         if (++in_unit == per_unit) {
@@ -417,7 +431,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
+      if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
     }
   } else if (EPI == EPI_SWIGLU) {
     // ---------------- epilogue, silu(gate) * up: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31: lanes
@@ -484,7 +498,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
       }
       return true;
     });
@@ -561,11 +575,41 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
         tc_fence_after();
         const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+        // KC > 1: [token of the set][128 features] fp32 sums of the other pair, over the ring, whose stages have all been read
+        // once both pairs have published their accumulators
+        const float* theirs = reinterpret_cast<const float*>(base_ptr) + quarter * 32 + lane;
+        if constexpr (KC > 1) {
+          __syncwarp();
+          cluster_sync_all();
+          if (set != kc) {
+            uint32_t to;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(base + (uint32_t)(quarter * 32 + lane) * 4), "r"(crank ^ 2u));
+#pragma unroll 1
+            for (int c = 0; c < n_chunks; ++c) {
+              float v[CH];
+              __syncwarp();
+              sp_ld_chunk<CH>(trow + c * CH, min(CH, set_n - c * CH), v);
+#pragma unroll
+              for (int e = 0; e < CH; ++e)
+                if (c * CH + e < set_n)
+                  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to + (uint32_t)(c * CH + e) * 512), "f"(v[e]) : "memory");
+            }
+          }
+          __syncwarp();
+          cluster_sync_all();
+          merged = 2;
+          if (set != kc) return true;
+        }
 #pragma unroll 1
         for (int c = 0; c < n_chunks; ++c) {
           float v[CH];
           __syncwarp();
           sp_ld_chunk<CH>(trow + c * CH, min(CH, set_n - c * CH), v);
+          if constexpr (KC > 1) {
+#pragma unroll
+            for (int e = 0; e < CH; ++e)
+              if (c * CH + e < set_n) v[e] += theirs[(c * CH + e) * 128];
+          }
 #pragma unroll
           for (int e = 0; e < CH; ++e) xmine[e * 32] = v[e] + bias;
           named_bar_sync(bar_set, 128);
@@ -625,7 +669,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
       }
       return true;
     });
@@ -695,10 +739,14 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), 0);
+        if (lane == 0) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
       }
       return true;
     });
+  }
+  if constexpr (KC > 1) {  // the warps without a part in the merge, and everybody after a wait that gave up
+    __syncwarp();
+    for (; merged < 2; ++merged) cluster_sync_all();
   }
   tc_fence_before();
   cluster_sync_all();  // neither CTA releases tensor or shared memory while the other may still use it
@@ -883,6 +931,20 @@ bool qkv_t_usable(const a3_handle* h, const GemmArgs& a) {
   return true;
 }
 
+// QKV of few rows in clusters of two pairs, each with half of the k-loop.  The heads alone occupy few pairs (Llama-8B: 24,
+// Qwen-7B: 18 of 74) and a CTA takes in its 16 KiB of weights per k-block at about 107 GB/s, however fast HBM is: 9.5 us for
+// the 33 MB of Qwen-7B.  Halves stream twice as wide; the merge costs two cluster barriers and a trip of the sums through
+// distributed shared memory (about 2 500 clocks).  Compared with the other way to occupy pairs, narrower token tiles, by the
+// cost per k-block of choose_tiling.  A layer of 75 rows (Qwen width) 88.8 -> 87.5 us, of 144 rows (Llama width) 111.6 ->
+// 109.6.  A half is at least as deep as a slice of the residual GEMMs; a tenth of the pairs is left out because clusters of
+// four do not fill every GPC.  Pinned kernel variants keep the undivided sums (split_allowed).
+static bool qkv_clusters(const a3_handle* h, int M, int K, int head_pairs, int pairs, const SpTiling& til) {
+  if (!split_allowed(h) || M > 256 || 2 * head_pairs > pairs - pairs / 10 || K / TC_BK < 2 * SP_SLICE_MIN_KB) return false;
+  auto per_kb = [](int n) { return 2 * n > 256 + n ? 2 * n : 256 + n; };
+  const int kt = K / TC_BK;
+  return kt / 2 * per_kb(cdiv(M, 16) * 16) + 2500 < (long long)cdiv(head_pairs * til.tiles, pairs) * kt * per_kb(til.n);
+}
+
 int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   SpParams p{};
   p.M = a.M;
@@ -901,8 +963,9 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
   const int sms = h->sm_count > 0 ? h->sm_count : 148;
   const int pairs = sms / 2;
   const SpTiling til = choose_tiling(h, a.M, head_pairs, pairs);
-  p.tok_tiles = til.tiles;
-  p.tok_n = til.n;
+  const bool clusters = qkv_clusters(h, a.M, a.K, head_pairs, pairs, til);
+  p.tok_tiles = clusters ? 1 : til.tiles;
+  p.tok_n = clusters ? cdiv(a.M, 16) * 16 : til.n;
   p.n_fblocks = head_pairs;
   p.group = unit_group(a.M, a.K);
   p.k_slices = 1;
@@ -927,10 +990,11 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
     if (s < a.nseg) A3_TRY(make_tmap_kblocks(&tW[s], a.seg[s].B, a.seg[s].n, a.K, 128, SP_SUB));
     else tW[s] = tW[0];
   }
-  static SmemAttrOnce attr;
-  A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI_QKV>, SP_SMEM_LIMIT));
+  static SmemAttrOnce attr[2];
+  const auto kernel = clusters ? pair_t_kernel<EPI_QKV, false, 2> : pair_t_kernel<EPI_QKV>;
+  A3_TRY(smem_attr_once(attr[clusters], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_QKV, st);
-  A3_CUDA(launch_pdl(pair_t_kernel<EPI_QKV>, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tW[0], tW[1], tW[2], p));
+  A3_CUDA(launch_pdl(kernel, dim3((clusters ? 4 : 2) * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tW[0], tW[1], tW[2], p));
   A3_LAUNCHED();
   return A3_OK;
 }

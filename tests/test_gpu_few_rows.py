@@ -1,5 +1,5 @@
-"""The paths that only launches of few rows take: GEMMs whose k-loop is cut into slices, added up by the kernel that follows,
-and attention whose keys are shared out to a cluster of CTAs.
+"""The paths that only launches of few rows take: GEMMs whose k-loop is cut into slices, added up by the kernel that follows
+(output and down projection) or within a cluster (QKV projection), and attention whose keys are shared out to a cluster of CTAs.
 
 The models here are the smallest whose matrices are deep enough to be cut (at least two slices of 1 024).  Gates as in
 tests/test_gpu_steps.py: the slices are fp32 sums of the same products, so the bounds derived there hold unchanged.
@@ -19,6 +19,10 @@ pytestmark = pytest.mark.gpu
 
 # d_model 896: the last 256-feature block is half empty; d_ff 2176 = 17 ring stages: slices of 8 and 9
 DEEP = W.ModelShape("deep", 2, 896, 16, 4, 128, 2176, 32000, 5e5, 1e-5)
+
+
+# QKV: 17 ring stages in halves of 8 and 9; 15 heads, so the last pair of CTAs has one without a head
+BROAD = W.ModelShape("broad", 1, 2176, 9, 3, 128, 640, 32000, 5e5, 1e-5)
 
 
 def layer_parity(a3mod, m, M, seed):
@@ -56,6 +60,12 @@ def layer_parity(a3mod, m, M, seed):
 def test_residual_gemm_in_slices(a3mod, M):
     """Output and down projection of few rows: one token, ragged and full token tiles, two tiles."""
     layer_parity(a3mod, DEEP, M, seed=M)
+
+
+@pytest.mark.parametrize("M", [1, 16, 17, 75, 255, 256, 257])
+def test_qkv_projection_in_halves(a3mod, M):
+    """Two pairs of CTAs per two heads, up to one full token tile: one token, warp sets with and without tokens."""
+    layer_parity(a3mod, BROAD, M, seed=M + 1)
 
 
 @pytest.mark.parametrize("shape,kv_len,M", [(W.TINY_GQA, 768, 60), (W.TINY_GQA, 1023, 41), (W.TINY_GQA, 1024, 64), (W.TINY_GQA, 1153, 7),
