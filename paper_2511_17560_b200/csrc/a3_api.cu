@@ -1,4 +1,5 @@
 // Handle lifetime, workspace carving and the orchestration of the fusion request (host code only).
+#include <algorithm>
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -452,9 +453,17 @@ struct HostFeed {
   const cudaEvent_t* layer_ready;  // [n_layers]
   const cudaEvent_t* x0_ready;     // [x0_panels(n)]: the embeddings of a panel of rows are on the device
   void* ctx;
-  int (*queue_layer)(void* ctx, int layer);  // queues the copies of one layer on the copy stream, records layer_ready[layer]
-  int next;                                  // first layer whose copies are not queued yet
+  int (*queue_layers)(void* ctx, int l0, int l1);  // queues the copies of layers l0 .. l1 - 1 on the copy stream, records their layer_ready
+  int next;                                        // first layer whose copies are not queued yet
+  int group;                                       // layers per copy, at most; the first groups are smaller: 1, 2, 4, ...
 };
+// Layers per copy for chunks of `slice` bytes a layer: copies of 4 MB.  640 copies of 1 MB reach 45.7 GB/s, of 4 MB 52.5, of
+// 64 MB 55.2 (a second copy stream changes nothing), but a layer is ready only when its whole group is,
+// hence the small first groups.  Ten chunks of 512 tokens from host memory, Llama-8B width: 15.94 -> 14.93 ms a request.
+static int feed_group(size_t slice) {
+  const size_t g = slice ? (4u << 20) / slice : 1;
+  return g < 1 ? 1 : g > 8 ? 8 : (int)g;
+}
 static int fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size_t ws_bytes, a3_stream stream, HostFeed* feed);
 }
 
@@ -530,8 +539,10 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
   // copies of the layers up to `upto` are on their way (host-buffer entry only)
   auto feed_to = [&](int upto) -> int {
     while (feed && feed->next <= upto && feed->next < h->m.n_layers) {
-      A3_TRY(feed->queue_layer(feed->ctx, feed->next));
-      ++feed->next;
+      const int sent = feed->next - (r->select_layer + 1) + 1;
+      const int l1 = std::min(feed->next + std::min(feed->group, sent), h->m.n_layers);
+      A3_TRY(feed->queue_layers(feed->ctx, feed->next, l1));
+      feed->next = l1;
     }
     return A3_OK;
   };
@@ -838,17 +849,17 @@ extern "C" int a3_fuse_request_host(const a3_handle* h, const a3_request* req, c
     cudaEvent_t* layer_ready;
   } fc{href, io, req->n_chunks, row, cs, hp->layer_ready};
   HostFeed feed{hp->layer_ready, hp->x0_ready, &fc,
-                [](void* ctx, int l) -> int {
+                [](void* ctx, int l0, int l1) -> int {
                   FeedCtx* f = (FeedCtx*)ctx;
-                  for (int c = 0; c < f->n_chunks; ++c) {
-                    const size_t slice = (size_t)f->href[c].len * f->row;
-                    A3_CUDA(cudaMemcpyAsync((char*)f->href[c].k_src + l * slice, (const char*)f->io->chunk_k[c] + l * slice, slice, cudaMemcpyHostToDevice, f->cs));
-                    A3_CUDA(cudaMemcpyAsync((char*)f->href[c].v_src + l * slice, (const char*)f->io->chunk_v[c] + l * slice, slice, cudaMemcpyHostToDevice, f->cs));
+                  for (int c = 0; c < f->n_chunks; ++c) {  // a chunk's layers lie one after the other on both sides
+                    const size_t slice = (size_t)f->href[c].len * f->row, from = l0 * slice, bytes = (l1 - l0) * slice;
+                    A3_CUDA(cudaMemcpyAsync((char*)f->href[c].k_src + from, (const char*)f->io->chunk_k[c] + from, bytes, cudaMemcpyHostToDevice, f->cs));
+                    A3_CUDA(cudaMemcpyAsync((char*)f->href[c].v_src + from, (const char*)f->io->chunk_v[c] + from, bytes, cudaMemcpyHostToDevice, f->cs));
                   }
-                  A3_CUDA(cudaEventRecord(f->layer_ready[l], f->cs));
+                  for (int l = l0; l < l1; ++l) A3_CUDA(cudaEventRecord(f->layer_ready[l], f->cs));
                   return A3_OK;
                 },
-                req->select_layer + 1};
+                req->select_layer + 1, feed_group(row * (size_t)req->n_ctx / (size_t)(req->n_chunks > 0 ? req->n_chunks : 1))};
   if (status == A3_OK) status = fuse_impl(h, &r, ws, ws_bytes, stream, &feed);
   const int M = r.n_recompute + r.n_question;
   if (status == A3_OK && M > 0) {
