@@ -151,7 +151,7 @@ typedef struct {
  * (every variant must meet the same tolerances; some pairs are bit-identical) and for measurements.  They are plain
  * fields of the handle: set them while no call on the handle is in flight. */
 typedef enum {
-  A3_OPT_ATTN_SPLIT = 0,        /* attention, one row tile per CTA: key segments per row tile; 0 = choose (default) */
+  A3_OPT_ATTN_SPLIT = 0,        /* attention, one row tile per CTA: key segments per row tile; 0 = choose, also clusters of CTAs that share them (default) */
   A3_OPT_ATTN_PAIR,             /* two-row-tile attention kernel: -1 choose (default), 0 never, 1 whenever supported */
   A3_OPT_ATTN_MAX_CTAS,         /* cap on the persistent attention grid; 0 = one CTA per SM (default) */
   A3_OPT_SWIGLU_NARROW,         /* one-CTA gate/up GEMM: 0 uniform tiles, 1 narrower last wave (default), 16..120 forced width */
@@ -164,7 +164,7 @@ typedef enum {
   A3_OPT_GEMM_STAGES_SWIGLU,
   A3_OPT_GEMM_STAGES_QKV,
   A3_OPT_SCORES_KERNEL,         /* relevance scores: 0 choose (default), 1 the tcgen05 kernel, 2 the warp-level MMA kernel */
-  A3_OPT_QKV_T,                 /* persistent CTA-pair QKV projection (one head per CTA): 0 never, 1 whenever the shape allows (default) */
+  A3_OPT_QKV_T,                 /* persistent CTA-pair QKV projection (one head per CTA): 0 never, 1 whenever the shape allows, few rows in clusters of two pairs (default) */
   A3_OPT_GEMM_TILING,           /* persistent CTA-pair GEMMs, token tiles: 0 widths that balance the pairs' loads (default), 1 even split */
   A3_OPT_COUNT
 } a3_option;

@@ -314,6 +314,13 @@ static int qkv_project(const a3_handle* h, int layer, const bf16* a, const int32
   g.nseg = 2;
   g.seg[0] = {(const bf16*)w.wk, (const bf16*)w.bk, kvd, 1};
   g.seg[1] = {(const bf16*)w.wv, (const bf16*)w.bv, kvd, 2};
+  if (q_first < M && h->opt[A3_OPT_GEMM_BN_QKV] == 0) {  // one launch for both where the kernel can
+    GemmArgs both = g;
+    both.q_first = q_first;
+    both.nseg = 3;
+    both.seg[2] = {(const bf16*)w.wq, (const bf16*)w.bq, qd, 0};
+    if (qkv_t_usable(h, both)) return gemm_qkv_t(h, both, st);
+  }
   A3_TRY(gemm_bf16(h, EPI_QKV, g, st));
   if (q_first < M) {
     g.A = a + (size_t)q_first * m.d_model;

@@ -172,6 +172,7 @@ struct GemmArgs {
   bf16* v_cache;
   const int32_t* pos;  // [M] cache slot = RoPE position of each row
   int kv_len;
+  int q_first;         // > 0: queries only of the rows from here on (q_out starts with them); segments k, v, q; gemm_qkv_t only
 };
 
 // SwiGLU GEMM with the weights as the M-side operand of a CTA pair, persistent (a3_swiglu_pair.cu).

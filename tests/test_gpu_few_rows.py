@@ -153,3 +153,30 @@ def test_pooled_selection_of_the_eviction(a3mod, n_ctx, pool):
         assert (v[inside] >= thr * (1 - 2e-3)).all() and (v[~inside] <= thr * (1 + 2e-3)).all()
         assert torch.equal(k_out[:, g], dK[kept[g].long(), g])
     eng.close()
+
+
+@pytest.mark.parametrize("shape,n_ctx,nq", [(W.TINY_GQA, 300, 1), (W.TINY_GQA, 511, 40), (W.TINY_GQA, 100, 300), (W.TINY_G7, 7, 5),
+                                            (W.TINY_G7, 250, 33)])
+def test_late_queries_ride_along(a3mod, shape, n_ctx, nq):
+    """Selection layer: the question rows' queries in the launch of everybody's keys and values (one or more token tiles of
+    them, an odd number of heads) against launches of their own on the tile kernel: the same bits."""
+    m, dev, n = shape, torch.device("cuda:0"), n_ctx + nq
+    eng = a3mod.A3(m, W.make_weights_device(m, dev, 0), n + 8)
+    g = torch.Generator(device=dev)
+    g.manual_seed(n)
+    ck, cv = (torch.randn(m.n_layers, n_ctx, m.n_kv_heads, m.head_dim, device=dev, generator=g).bfloat16() for _ in range(2))
+    x0 = torch.randn(n, m.d_model, device=dev, generator=g).bfloat16()
+    tab = a3mod.chunk_table([ck], [cv], [0])
+    res = []
+    for qkv_t in (1, 0):
+        eng.set_option(a3mod.OPT_QKV_T, qkv_t)
+        K, V = (torch.zeros(m.n_layers, n, m.n_kv_heads, m.head_dim, device=dev, dtype=torch.bfloat16) for _ in range(2))
+        rq, out = eng.make_request(tab, 1, n_ctx, n_ctx, nq, x0, K, V, ratio=0.0, select_layer=0)
+        eng.fuse_request(rq)
+        assert eng.device_status() == 0
+        res.append((K[0, :n_ctx], V[0, :n_ctx], out["scores"][:n_ctx]))
+    eng.set_option(a3mod.OPT_QKV_T, 1)
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+    assert float(res[0][2].abs().max()) > 0
+    eng.close()
