@@ -175,7 +175,8 @@ __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc
 // slices in order.  See residual_slices below for when and why.
 // KC = 2 (QKV of few rows): a cluster of two pairs per unit, each with half of the k-loop.  The epilogue needs whole sums: pair c
 // finishes the tokens of warp set c and receives the other pair's sums for them through distributed shared memory.
-template <int EPI, bool SPLIT = false, int KC = 1>
+// ONCE: one token tile, every weight is read once in the whole launch (see the producer).
+template <int EPI, bool SPLIT, int KC, bool ONCE>
 __global__ void __cluster_dims__(2 * KC, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
               const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmW, const SpParams p) {
@@ -253,13 +254,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         if (EPI != EPI_RESIDUAL) tmap_prefetch(&tmU);
         if (EPI == EPI_QKV) tmap_prefetch(&tmW);
       }
-      // With one token tile every weight is read once in the whole launch, and a layer of weights is several times L2: first
-      // out, so that they do not displace what the kernels hand on (rows, partial sums, the cache) and their code.  A layer of
-      // 144 rows at Llama-8B width 115.6 -> 111.7 us, of 75 rows at Qwen-7B width 91.3 -> 89.6.  With two token tiles
-      // (280 rows) a policy on every load cost 2 %: 138.1 -> 140.5.
-      const uint64_t once = l2_evict_first();
+      // ONCE: a layer of weights is several times L2 and nobody reads them again: first out, so that they do not displace what
+      // the kernels hand on (rows, partial sums, the cache) and their code.  A layer of 144 rows at Llama-8B width 115.6 ->
+      // 111.7 us, of 75 rows at Qwen-7B width 91.3 -> 89.6.  With two token tiles a policy on every load costs (280 rows 138.1
+      // -> 140.5), and so does choosing per load (270 rows, Qwen width 122.7 -> 123.6): hence an instance of its own.
+      const uint64_t once = ONCE ? l2_evict_first() : 0;
       auto load = [&](uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
-        if (p.tok_tiles == 1) tma_load_3d_pair_once(dst, map, y, z, bar, once);
+        if (ONCE) tma_load_3d_pair_once(dst, map, y, z, bar, once);
         else tma_load_3d_pair(dst, map, y, z, bar);
       };
       int kbg = 0, issued = 0;
@@ -896,10 +897,12 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   CUtensorMap tX, tG;
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB));
-  static SmemAttrOnce attr;
-  A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI_RESIDUAL, true>, SP_SMEM_LIMIT));
+  static SmemAttrOnce attr[2];
+  const bool once = p.tok_tiles == 1;
+  const auto kernel = once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true> : pair_t_kernel<EPI_RESIDUAL, true, 1, false>;
+  A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
-  A3_CUDA(launch_pdl(pair_t_kernel<EPI_RESIDUAL, true>, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tG, tG, p));
+  A3_CUDA(launch_pdl(kernel, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tG, tG, p));
   A3_LAUNCHED();
   return A3_OK;
 }
@@ -930,10 +933,12 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, ROWS, EPI == EPI_SWIGLU ? 1 : SP_SUB));
   if (EPI == EPI_SWIGLU) A3_TRY(make_tmap_kblocks(&tU, a.B2, p.F, a.K, ROWS, 1));
   else tU = tG;
-  static SmemAttrOnce attr;
-  A3_TRY(smem_attr_once(attr, h->device, pair_t_kernel<EPI>, SP_SMEM_LIMIT));
+  static SmemAttrOnce attr[2];
+  const bool once = p.tok_tiles == 1;
+  const auto kernel = once ? pair_t_kernel<EPI, false, 1, true> : pair_t_kernel<EPI, false, 1, false>;
+  A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, EPI == EPI_SWIGLU ? A3_K_GEMM_SWIGLU : A3_K_GEMM_RESIDUAL, st);
-  A3_CUDA(launch_pdl(pair_t_kernel<EPI>, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tU, tU, p));
+  A3_CUDA(launch_pdl(kernel, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tU, tU, p));
   A3_LAUNCHED();
   return A3_OK;
 }
@@ -1024,9 +1029,12 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
     if (s < a.nseg) A3_TRY(make_tmap_kblocks(&tW[s], a.seg[s].B, a.seg[s].n, a.K, 128, SP_SUB));
     else tW[s] = tW[0];
   }
-  static SmemAttrOnce attr[2];
-  const auto kernel = clusters ? pair_t_kernel<EPI_QKV, false, 2> : pair_t_kernel<EPI_QKV>;
-  A3_TRY(smem_attr_once(attr[clusters], h->device, kernel, SP_SMEM_LIMIT));
+  static SmemAttrOnce attr[3];
+  const int variant = clusters ? 2 : p.tok_tiles == 1;
+  const auto kernel = variant == 2   ? pair_t_kernel<EPI_QKV, false, 2, true>
+                      : variant == 1 ? pair_t_kernel<EPI_QKV, false, 1, true>
+                                     : pair_t_kernel<EPI_QKV, false, 1, false>;
+  A3_TRY(smem_attr_once(attr[variant], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_QKV, st);
   A3_CUDA(launch_pdl(kernel, dim3((clusters ? 4 : 2) * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tW[0], tW[1], tW[2], p));
   A3_LAUNCHED();
