@@ -4,9 +4,9 @@
 // KV head are packed into the row dimension (flat row r -> token r / G, head r % G); one CTA owns 128 flat rows of
 // one KV head and walks the keys in tiles of 128 up to the largest position among its rows.
 //
-//   warp 0 (one lane)   TMA producer: K and V tiles of the cache ([slots][Hkv*D] seen as a 2-D tensor, 128-byte
+//   warp 0              TMA producer: K and V tiles of the cache ([slots][Hkv*D] seen as a 2-D tensor, 128-byte
 //                       swizzle), a ring of three stages each.
-//   warp 1 (one lane)   tcgen05.mma issuer: S = Q K^T (128 x 128 x D) into one of two TMEM buffers, and, once the
+//   warp 1              tcgen05.mma issuer: S = Q K^T (128 x 128 x D) into one of two TMEM buffers, and, once the
 //                       probabilities of a tile are back in tensor memory, O~ += P V (128 x D x 128; P is the A
 //                       operand read from TMEM, V an MN-major operand in shared memory) accumulated in TMEM.
 //                       S of tile t+1 is issued before P V of tile t, so the tensor core works while the
@@ -20,6 +20,8 @@
 //                       rescaled in TMEM and the tile redone.  At the end of an item the two partial softmaxes of
 //                       a row are merged, normalised and stored.
 // TMEM (512 columns): S buffers at 0 and 128, the two output accumulators at 256 and 256 + D.
+// Warps 0 and 1 walk their loops whole, one elected lane issuing.  With few row tiles (CS = 2 or 4, see cluster_size) a cluster
+// of CTAs shares the keys of an item and merges through distributed shared memory.
 // Statistics are fp32 in the exp2 domain.  Every mbarrier wait is bounded (see a3_gemm.cu); there is no block-
 // wide or named barrier inside the loops, so a role that gives up cannot strand another.
 #include <cuda.h>

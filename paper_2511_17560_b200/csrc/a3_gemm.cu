@@ -607,9 +607,9 @@ static int launch_pair(const a3_handle* h, const GemmArgs& a, const TcParams& p,
 // Tile width / pipeline depth per epilogue [EPI_RESIDUAL, EPI_SWIGLU, EPI_QKV] -> {BN, STAGES}; BN = 0 lets the
 // launcher choose (a3_set_option pins a choice on a handle for cross-checks).  Measured on B200 at Llama-8B width:
 // two co-resident CTAs per SM (256/2, 128/3) overlap one tile's epilogue with the other's main loop and win when
-// the grid has several waves.  The CTA-pair kernel wins for the residual GEMMs (N = d_model: few tiles, one CTA per
-// SM); for SwiGLU and QKV its extra all-padding row tile at 804 rows (7 -> 8) costs more than the halved B traffic
-// saves: under the power cap the tensor work, not the L2 port, sets the pace.
+// the grid has several waves.  The CTA-pair kernel was the better one for the residual GEMMs (N = d_model: few tiles, one
+// CTA per SM); for SwiGLU and QKV its extra all-padding row tile at 804 rows (7 -> 8) cost more than the halved B traffic
+// saved.  All three yield to the persistent kernels (a3_gemm_persistent.cu) where those take the shape.
 // A3_OPT_SWIGLU_NARROW: 0: no narrower last wave in the SwiGLU grid; 1: choose; 16..120: that width on half the tiles.
 
 template <int EPI>
@@ -643,7 +643,7 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
     const int m_tiles = cdiv(a.M, TC_BM), sms = h->sm_count > 0 ? h->sm_count : 148;
     if (epi == EPI_RESIDUAL) {
       // the CTA-pair kernel (bn 512 selects it): measured 5-7 % faster than one CTA per 128 x 224/256 tile at
-      // Llama-8B width for 804 and 5 152 rows
+      // Llama-8B width for 804 and 5 152 rows.  Depths that are no multiple of 128 come here.
       (void)m_tiles;
       (void)sms;
       bn = 512;

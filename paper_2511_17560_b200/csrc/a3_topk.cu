@@ -1,6 +1,6 @@
 // Selection Re = top_p(s) (Eq. 3): block-radix select on the order-preserving integer image of the fp32 scores.
-// One CTA per score array.  The scores are read from global memory once, as integer keys into shared memory (up to
-// TK_SMEM_KEYS of them; longer arrays are re-read from global memory in every pass).  Four 8-bit histogram passes
+// One CTA per score array.  The scores are read from global memory once, as integer keys into registers (up to 8 192, see
+// topk_regs) or shared memory (up to TK_SMEM_KEYS of them; longer arrays are re-read from global memory in every pass).  Four 8-bit histogram passes
 // find the key of the k-th largest score: the warps count into TK_HISTS private histograms (a warp whose lanes all
 // hold the same digit - the rule in the first pass, since the scores of one request share their leading bits - adds
 // 32 with one instruction instead of serialising 32 atomics on one bin), the histograms are summed, and the bin of
