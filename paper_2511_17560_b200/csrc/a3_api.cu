@@ -453,12 +453,19 @@ namespace a3 {
 // on the first panel while the others are still on their way.
 constexpr int X0_PANELS = 4;
 constexpr int X0_PANEL_MIN_ROWS = 16384;  // shorter inputs: one panel
-static inline int x0_panels(int n) { return n >= X0_PANEL_MIN_ROWS ? X0_PANELS : 1; }
 static inline int x0_panel_begin(int n, int i, int panels) { return i >= panels ? n : (int)((long long)n * i / panels) & ~127; }
+static inline int x0_panels(const a3_request* r) {
+  const int n = r->n_ctx + r->n_question;
+  if (n < X0_PANEL_MIN_ROWS) return 1;
+  // eviction of block 0 takes the question rows' queries and log-sum-exps from the workspace, which holds those of the last
+  // panel only: a question that reaches further back keeps the block whole
+  if (r->evict_capacity > 0 && r->n_ctx < x0_panel_begin(n, X0_PANELS - 1, X0_PANELS)) return 1;
+  return X0_PANELS;
+}
 
 struct HostFeed {
   const cudaEvent_t* layer_ready;  // [n_layers]
-  const cudaEvent_t* x0_ready;     // [x0_panels(n)]: the embeddings of a panel of rows are on the device
+  const cudaEvent_t* x0_ready;     // [x0_panels]: the embeddings of a panel of rows are on the device
   void* ctx;
   int (*queue_layers)(void* ctx, int l0, int l1);  // queues the copies of layers l0 .. l1 - 1 on the copy stream, records their layer_ready
   int next;                                        // first layer whose copies are not queued yet
@@ -640,7 +647,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, ls + 1,
                             m.n_layers, stream));
   // leading full blocks: the whole input through layers 0..select_layer-1
-  const int panels = x0_panels(n);
+  const int panels = x0_panels(r);
   const bool norm_panels = ls > 0 || panels == 1;
   for (int i = 0; i < panels; ++i) {
     const int r0 = x0_panel_begin(n, i, panels), r1 = x0_panel_begin(n, i + 1, panels);
@@ -836,7 +843,7 @@ extern "C" int a3_fuse_request_host(const a3_handle* h, const a3_request* req, c
   // the descriptor array is pageable host memory: this copy returns only once it has been staged
   if (status == A3_OK && req->n_chunks > 0)
     note(cudaMemcpyAsync(dref, href, sizeof(a3_chunk_ref) * req->n_chunks, cudaMemcpyHostToDevice, cs));
-  const int panels = x0_panels(n);
+  const int panels = x0_panels(req);
   for (int i = 0; i < panels && status == A3_OK; ++i) {
     const int r0 = x0_panel_begin(n, i, panels), r1 = x0_panel_begin(n, i + 1, panels);
     if (note(cudaMemcpyAsync(x0 + (size_t)r0 * m.d_model * 2, (const char*)io->x0 + (size_t)r0 * m.d_model * 2, (size_t)(r1 - r0) * m.d_model * 2,
