@@ -363,9 +363,9 @@ class A3:
         kv_len = k_layer.shape[0]
         Cp = n_system + evict_count(capacity, n_system, n_ctx, nq) + nq
         Hkv, D = self.shape.n_kv_heads, self.shape.head_dim
-        k_out = k_layer.new_empty((Cp, Hkv, D))  # the gather writes every entry
-        v_out = k_layer.new_empty((Cp, Hkv, D))
-        kept = q_pos.new_empty((Hkv, Cp))
+        k_out = k_layer.new_empty((Cp, Hkv, D), dtype=torch.bfloat16)  # the gather writes every entry
+        v_out = torch.empty_like(k_out)
+        kept = k_layer.new_empty((Hkv, Cp), dtype=torch.int32)  # not q_pos's type and device: without question rows nobody reads q_pos
         ws = self.workspace(int(_load().a3_evict_workspace_bytes(self._h, kv_len)))
         _check(_load().a3_evict_layer(self._h, _ptr(q_window), _ptr(q_pos), nq, _ptr(lse), _ptr(k_layer), _ptr(v_layer), kv_len,
                                       n_system, n_ctx, capacity, pool, _ptr(k_out), _ptr(v_out), _ptr(kept), _ptr(ws), ws.numel(),
