@@ -4,7 +4,7 @@
 //
 // One layer = three launches: per-head votes (the score kernel of Eq. 3 without the sum over KV heads, fed with
 // the question rows' queries and log-sum-exps of that layer), one top-k CTA per KV head, which pools the votes as it reads
-// them (a kernel of its own does where they do not fit its shared memory), and a gather that writes the compact cache [C'][Hkv][D] (bound by HBM: each kept row is read and written once).
+// them (a kernel of its own before it does for many candidates or wide windows, see topk_can_pool), and a gather that writes the compact cache [C'][Hkv][D] (bound by HBM: each kept row is read and written once).
 #include "a3_internal.cuh"
 
 namespace a3 {
@@ -95,7 +95,7 @@ extern "C" int a3_evict_layer(const a3_handle* h, const void* q_window, const in
     if (nq > 0) A3_TRY(scores_pass(h, (const bf16*)q_window, q_pos, nq, (const bf16*)k_layer, kv_len, n_system, n_ctx, lse, nullptr, st, votes));
     else A3_CUDA(cudaMemsetAsync(votes, 0, (size_t)m.n_kv_heads * kv_len * 4, st));
     const float* src = votes;
-    const bool pool_in_topk = topk_can_pool(n_ctx - n_system);
+    const bool pool_in_topk = topk_can_pool(n_ctx - n_system, pool);
     if (pool > 1 && !pool_in_topk) {
       ProfScope prof(h, A3_K_ROWS, st);
       pool_scores_kernel<<<dim3(cdiv(kv_len, 256), m.n_kv_heads), 256, 0, st>>>(votes, pooled, kv_len, n_system, n_ctx, pool / 2);

@@ -215,7 +215,7 @@ int topk_rows(const a3_handle* h, const float* scores, int cand_begin, int cand_
 // (pool > 1, odd: of the running maximum over `pool` neighbouring candidates instead of the scores themselves)
 int topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,
                  int k, int pool, int32_t* idx_out, size_t idx_stride, cudaStream_t st);
-bool topk_can_pool(int n_cand);  // ... as long as the candidates fit its shared memory
+bool topk_can_pool(int n_cand, int pool);  // ... where that is the faster way (pool_scores_kernel does it otherwise)
 
 // scores[slot] = |v_true[slot] - cached value of that slot|^2 for candidate slots covered by a chunk (others untouched)
 int value_deviation(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len, int layer, const bf16* v_true,

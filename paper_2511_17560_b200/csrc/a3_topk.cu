@@ -160,7 +160,7 @@ __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __
 }
 
 template <bool IN_SMEM>
-__device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t* __restrict__ keys, int cand_begin, int n, int k, int half_pool,
+__device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t* __restrict__ keys, int cand_begin, int n, int k,
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
   __shared__ unsigned int whist[TK_HISTS][256];
   __shared__ unsigned int warp_tot[8];
@@ -173,10 +173,7 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
   bool nonfinite = false;
 #pragma unroll 4
   for (int i = tid; i < n; i += TK_THREADS) {
-    float v = __ldcg(s + i);
-    if (IN_SMEM && half_pool > 0) {  // running maximum, cut at the candidate range
-      for (int j = max(0, i - half_pool); j <= min(n - 1, i + half_pool); ++j) v = fmaxf(v, s[j]);
-    }
+    const float v = __ldcg(s + i);
     if (!(fabsf(v) <= 3.0e38f)) nonfinite = true;
     if (IN_SMEM) keys[i] = score_key(v);
   }
@@ -264,8 +261,8 @@ topk_select_kernel(const float* __restrict__ scores, int cand_begin, int n, int 
     topk_regs<REGS>(s, reinterpret_cast<float*>(tk_keys), cand_begin, n, k, half_pool, out, status);
     return;
   }
-  if (in_smem) topk_body<true>(s, tk_keys, cand_begin, n, k, half_pool, out, status);
-  else topk_body<false>(s, tk_keys, cand_begin, n, k, 0, out, status);
+  if (in_smem) topk_body<true>(s, tk_keys, cand_begin, n, k, out, status);
+  else topk_body<false>(s, tk_keys, cand_begin, n, k, out, status);
 }
 
 static int launch_topk(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int n, int k,
@@ -319,7 +316,13 @@ int a3::topk_rows(const a3_handle* h, const float* scores, int cand_begin, int c
   return launch_topk(h, scores, 0, 1, cand_begin, cand_end - cand_begin, k, 0, tail_begin, tail, idx_out, 0, st);
 }
 
-bool a3::topk_can_pool(int n_cand) { return n_cand <= TK_SMEM_KEYS; }
+// Pooling inside the selection saves a launch (2.5 us) and costs every thread its keys x the width in shared-memory reads, in
+// the one CTA of a head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, inside against
+// apart (us): 2 000 candidates 17.1 / 19.7 at width 7, 18.7 / 20.2 at 63, 20.7 / 21.6 at 127, 24.8 / 22.6 at 255; 5 120
+// candidates 21.8 / 24.3 at 7, 24.3 / 24.3 at 45, 25.9 / 24.3 at 63; 8 192 candidates 25.9 / 27.4 at 7, 26.9 / 27.4 at 21, 27.9 /
+// 27.4 at 31.  The line is where the two meet, within half a microsecond.  Candidates that do not fit the registers would read their window from global
+// memory, which loses at every width (12 000 candidates 39.2 / 38.7 at 3, 32 768 79.1 / 70.9 at 7, 215 / 82 at 255).
+bool a3::topk_can_pool(int n_cand, int pool) { return n_cand <= 8 * TK_THREADS && (long long)n_cand * pool <= 250 * TK_THREADS; }
 
 int a3::topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,
                      int k, int pool, int32_t* idx_out, size_t idx_stride, cudaStream_t st) {

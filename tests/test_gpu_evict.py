@@ -64,3 +64,34 @@ def test_votes_of_a_question_longer_than_the_last_panel(a3mod, nq):
         check_kept(kept[0, h].cpu().numpy(), votes[h], 0, n_ctx, nq)
         assert torch.equal(k_evicted[0, :, h], K[0][kept[0, h].long(), h])
     eng.close()
+
+
+def evict_setup(a3mod, m, n_ctx, nq, seed):
+    eng, _, dev = make_engine(a3mod, m, seed=seed)
+    rng = np.random.default_rng(seed)
+    K, V = (W.bf16_round(rng.standard_normal((n_ctx + nq, m.n_kv_heads, m.head_dim), dtype=np.float32)) for _ in range(2))
+    q = W.bf16_round(rng.standard_normal((nq, m.n_q_heads, m.head_dim), dtype=np.float32))
+    pos = np.arange(n_ctx, n_ctx + nq)
+    s = np.einsum("jhd,ihd->jhi", q.astype(np.float64), np.repeat(K, m.n_q_heads // m.n_kv_heads, axis=1).astype(np.float64)) / np.sqrt(m.head_dim)
+    s[np.broadcast_to(np.arange(n_ctx + nq)[None, None, :] > pos[:, None, None], s.shape)] = -np.inf
+    lse = torch.from_numpy(np.log(np.exp(s).sum(axis=2)).astype(np.float32)).to(dev)
+    return eng, q, pos, K, (to_dev(q, dev), torch.from_numpy(pos.astype(np.int32)).to(dev), lse, to_dev(K, dev), to_dev(V, dev))
+
+
+@pytest.mark.parametrize("n_cand,pool,launches", [(95, 1001, 3), (700, 2001, 4), (900, 255, 3), (1024, 249, 3), (1024, 251, 4), (5120, 49, 3),
+                                                  (5120, 51, 4), (8192, 31, 3), (8192, 33, 4), (8193, 3, 4), (20000, 7, 4)])
+def test_wide_pooling(a3mod, n_cand, pool, launches):
+    """Windows as wide as the candidates and wider, both sides of the line between pooling inside the selection and apart."""
+    m, nq, n_system = W.TINY_GQA, 9, 5
+    n_ctx = n_system + n_cand
+    eng, q, pos, K, args = evict_setup(a3mod, m, n_ctx, nq, n_cand + pool)
+    k = n_cand // 3
+    a3mod.launch_count(reset=True)
+    k_out, v_out, kept = eng.evict_layer(*args, n_system, n_ctx, n_system + nq + k, pool)
+    assert a3mod.launch_count() == launches
+    assert eng.device_status() == 0
+    votes = O.pool_scores(O.eviction_scores(q.astype(np.float64), pos, K.astype(np.float64), oracle_model(m), n_system, n_ctx), n_system, n_ctx, pool)
+    for h in range(m.n_kv_heads):
+        check_kept(kept[h].cpu().numpy(), votes[h], n_system, n_ctx, nq)
+        assert torch.equal(k_out[:, h], args[3][kept[h].long(), h]) and torch.equal(v_out[:, h], args[4][kept[h].long(), h])
+    eng.close()
