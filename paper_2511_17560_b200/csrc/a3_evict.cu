@@ -24,10 +24,11 @@ pool_scores_kernel(const float* __restrict__ in, float* __restrict__ out, int kv
   out[(size_t)blockIdx.y * kv_len + i] = v;
 }
 
-// kept slot c of head g: S, then the selected documents (ascending), then Q
+// kept slot c of head g: S, then the selected documents (ascending), then Q.  The selection is read past L1: it is the result of
+// the kernel that the gather's CTAs may have become resident next to.
 __device__ __forceinline__ int evict_source(int c, int g, const int32_t* __restrict__ sel, int k, int n_system, int n_ctx) {
   if (c < n_system) return c;
-  if (c < n_system + k) return sel[(size_t)g * k + (c - n_system)];
+  if (c < n_system + k) return __ldcg(sel + (size_t)g * k + (c - n_system));
   return n_ctx + (c - n_system - k);
 }
 

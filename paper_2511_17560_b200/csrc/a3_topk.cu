@@ -167,7 +167,8 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
   __shared__ unsigned int s_prefix, s_remaining;
   __shared__ unsigned int warp_gt[TK_WARPS], warp_eq[TK_WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  auto key_at = [&](int i) -> uint32_t { return IN_SMEM ? keys[i] : score_key(s[i]); };
+  // past L1: this CTA may have become resident while the kernel that writes the scores was still running
+  auto key_at = [&](int i) -> uint32_t { return IN_SMEM ? keys[i] : score_key(__ldcg(s + i)); };
 
   // ---- load: scores -> keys (shared memory), non-finite scores flagged
   bool nonfinite = false;
@@ -320,8 +321,9 @@ int a3::topk_rows(const a3_handle* h, const float* scores, int cand_begin, int c
 // the one CTA of a head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, inside against
 // apart (us): 2 000 candidates 17.1 / 19.7 at width 7, 18.7 / 20.2 at 63, 20.7 / 21.6 at 127, 24.8 / 22.6 at 255; 5 120
 // candidates 21.8 / 24.3 at 7, 24.3 / 24.3 at 45, 25.9 / 24.3 at 63; 8 192 candidates 25.9 / 27.4 at 7, 26.9 / 27.4 at 21, 27.9 /
-// 27.4 at 31.  The line is where the two meet, within half a microsecond.  Candidates that do not fit the registers would read their window from global
-// memory, which loses at every width (12 000 candidates 39.2 / 38.7 at 3, 32 768 79.1 / 70.9 at 7, 215 / 82 at 255).
+// 27.4 at 31.  The line is where the two meet, within half a microsecond.  Candidates that do not fit the registers would read
+// their window from global memory, which loses at every width (12 000 candidates 39.2 / 38.7 at 3, 32 768 79.1 / 70.9 at 7,
+// 215 / 82 at 255).
 bool a3::topk_can_pool(int n_cand, int pool) { return n_cand <= 8 * TK_THREADS && (long long)n_cand * pool <= 250 * TK_THREADS; }
 
 int a3::topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,
