@@ -156,8 +156,6 @@ __device__ __forceinline__ void tc_epilogue_row(const TcParams& p, uint32_t trow
     }
 }
 
-// Old values of this thread's row of C for the residual epilogue: issued before the accumulator is waited for, so
-// the global-memory latency (a row per lane: uncoalesced, L2-resident) hides behind the main loop.
 // Position of this thread's row (checked; -1 if unusable) and, for q and k tiles, the row's D/2 (cos, sin) pairs into
 // `pre`: issued before the accumulator is waited for, like the residual rows below.
 __device__ __forceinline__ int tc_prefetch_rope(const TcParams& p, int gr, bool row_ok, int seg, uint4 (&pre)[32]) {
@@ -177,6 +175,9 @@ __device__ __forceinline__ int tc_prefetch_rope(const TcParams& p, int gr, bool 
   return ps;
 }
 
+// Old values of this thread's row of C for the residual epilogue: issued before the accumulator is waited for, so
+// the global-memory latency (a row per lane: uncoalesced, L2-resident) hides behind the main loop.  Not through the read-only
+// path: this kernel writes the same rows.
 template <int BN>
 __device__ __forceinline__ void tc_prefetch_residual(const TcParams& p, int gr, bool row_ok, int nt, uint4 (&pre)[BN / 8]) {
   const int n0 = nt * BN;
@@ -185,7 +186,7 @@ __device__ __forceinline__ void tc_prefetch_residual(const TcParams& p, int gr, 
     const bool col_ok = row_ok && n0 + c * 32 < p.N;
     const uint4* src = reinterpret_cast<const uint4*>(p.C + (size_t)(col_ok ? gr : 0) * p.ldc + (col_ok ? n0 + c * 32 : 0));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) pre[c * 4 + i] = col_ok ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
+    for (int i = 0; i < 4; ++i) pre[c * 4 + i] = col_ok ? __ldcg(src + i) : make_uint4(0, 0, 0, 0);
   }
 }
 
