@@ -4,7 +4,8 @@
 //
 // One layer = three launches: per-head votes (the score kernel of Eq. 3 without the sum over KV heads, fed with
 // the question rows' queries and log-sum-exps of that layer), one top-k CTA per KV head, which pools the votes as it reads
-// them (a kernel of its own before it does for many candidates or wide windows, see topk_can_pool), and a gather that writes the compact cache [C'][Hkv][D] (bound by HBM: each kept row is read and written once).
+// them (a kernel of its own before it does for many candidates or wide windows, see topk_can_pool), and a gather that writes the compact cache
+// [C'][Hkv][D] (bound by HBM: each kept row is read and written once); the gather alone where everything fits.
 #include "a3_internal.cuh"
 
 namespace a3 {
@@ -24,10 +25,11 @@ pool_scores_kernel(const float* __restrict__ in, float* __restrict__ out, int kv
   out[(size_t)blockIdx.y * kv_len + i] = v;
 }
 
-// kept slot c of head g: S, then the selected documents (ascending), then Q.  The selection is read past L1: it is the result of
+// kept slot c of head g: S, then the selected documents (ascending), then Q; slot c itself where everything is kept (no
+// selection given).  The selection is read past L1: it is the result of
 // the kernel that the gather's CTAs may have become resident next to.
 __device__ __forceinline__ int evict_source(int c, int g, const int32_t* __restrict__ sel, int k, int n_system, int n_ctx) {
-  if (c < n_system) return c;
+  if (!sel || c < n_system) return c;
   if (c < n_system + k) return __ldcg(sel + (size_t)g * k + (c - n_system));
   return n_ctx + (c - n_system - k);
 }
@@ -105,8 +107,7 @@ extern "C" int a3_evict_layer(const a3_handle* h, const void* q_window, const in
     }
     A3_TRY(topk_batched(h, src, (size_t)kv_len, m.n_kv_heads, n_system, n_ctx, k, pool_in_topk ? pool : 1, sel, (size_t)k, st));
   } else if (k > 0) {
-    // everything fits: the selection is every document slot (no votes needed)
-    for (int g = 0; g < m.n_kv_heads; ++g) A3_TRY(iota_rows(h, sel + (size_t)g * k, n_system, k, st));
+    sel = nullptr;  // everything fits: no votes, no selection
   }
   if (C == 0) return A3_OK;
   {

@@ -95,3 +95,18 @@ def test_wide_pooling(a3mod, n_cand, pool, launches):
         check_kept(kept[h].cpu().numpy(), votes[h], n_system, n_ctx, nq)
         assert torch.equal(k_out[:, h], args[3][kept[h].long(), h]) and torch.equal(v_out[:, h], args[4][kept[h].long(), h])
     eng.close()
+
+
+@pytest.mark.parametrize("n_system,n_cand,nq,more", [(0, 300, 9, 0), (5, 95, 9, 40), (7, 1, 0, 0), (0, 33, 0, 5)])
+def test_everything_fits(a3mod, n_system, n_cand, nq, more):
+    """Capacity for the whole cache, or for more: a copy, in one launch (the header promises at most four)."""
+    m = W.TINY_GQA
+    n_ctx = n_system + n_cand
+    eng, _, _, _, (q, pos, lse, K, V) = evict_setup(a3mod, m, n_ctx, nq, n_cand)
+    a3mod.launch_count(reset=True)
+    k_out, v_out, kept = eng.evict_layer(q, pos, lse, K, V, n_system, n_ctx, n_ctx + nq + more, 7)
+    assert a3mod.launch_count() == 1
+    assert eng.device_status() == 0
+    assert torch.equal(k_out, K) and torch.equal(v_out, V)
+    assert torch.equal(kept, torch.arange(n_ctx + nq, dtype=torch.int32, device=kept.device).expand(m.n_kv_heads, -1))
+    eng.close()
