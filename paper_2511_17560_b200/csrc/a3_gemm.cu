@@ -456,11 +456,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();  // the peer's barriers exist before anything is signalled on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // as in the persistent kernel: the weights may be read before the preceding kernel has finished (see GemmArgs)
-  if (warp != 0 || !p.early) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own rows of A, own half of B
@@ -476,27 +473,19 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       tmap_prefetch(&tmA);
       tmap_prefetch(mapB);
-      auto load_weights = [&](int s, int kb) {
+      int issued = 0;
+      for (int kb = 0; kb < KT; ++kb) {
+        const int s = kb % STAGES;
+        const uint32_t ph = (kb / STAGES) & 1;
+        if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status)) break;
+        const uint32_t sa = base + s * L::STAGE_BYTES, sb = sa + L::A_BYTES;
+        const uint32_t full_leader = full_bar(s) & PAIR_LEADER_MASK;
         // The leader announces the bytes of both CTAs.  A copy of the peer may complete before that: the phase
         // cannot end early, because the leader's own arrival is still pending until its expect_tx.
         if (leader) mbar_expect_tx(full_bar(s), 2 * L::STAGE_BYTES);
-        tma_load_2d_pair(base + s * L::STAGE_BYTES + L::A_BYTES, mapB, kb * TC_BK, brow0, full_bar(s) & PAIR_LEADER_MASK);
-      };
-      const int early = p.early ? min(STAGES, KT) : 0;
-      for (int kb = 0; kb < early; ++kb) load_weights(kb, kb);
-      if (p.early) {
-        pdl_wait();
-        pdl_launch_dependents();
-      }
-      int issued = early;
-      for (int kb = 0; kb < KT; ++kb) {
-        const int s = kb % STAGES;
-        if (kb >= early) {
-          if (!mbar_wait(empty_bar(s), ((kb / STAGES) & 1) ^ 1, abort_flag, p.status)) break;
-          load_weights(s, kb);
-        }
-        tma_load_2d_pair(base + s * L::STAGE_BYTES, &tmA, kb * TC_BK, m0, full_bar(s) & PAIR_LEADER_MASK);
-        issued = max(issued, kb + 1);
+        tma_load_2d_pair(sa, &tmA, kb * TC_BK, m0, full_leader);
+        tma_load_2d_pair(sb, mapB, kb * TC_BK, brow0, full_leader);
+        issued = kb + 1;
       }
       if (*abort_flag) {
         // let the copies already issued land before the CTA can exit (bounded)
@@ -610,7 +599,9 @@ static int launch_pair(const a3_handle* h, const GemmArgs& a, const TcParams& p,
 // two co-resident CTAs per SM (256/2, 128/3) overlap one tile's epilogue with the other's main loop and win when
 // the grid has several waves.  The CTA-pair kernel was the better one for the residual GEMMs (N = d_model: few tiles, one
 // CTA per SM); for SwiGLU and QKV its extra all-padding row tile at 804 rows (7 -> 8) cost more than the halved B traffic
-// saved.  All three yield to the persistent kernels (a3_gemm_persistent.cu) where those take the shape.
+// saved.  By default only the QKV projection at head dimension 64 comes here: every other GEMM of a model that a3_create
+// accepts (widths and depths multiples of 128) goes to the persistent kernels (a3_gemm_persistent.cu), and these tiles, the
+// CTA-pair kernel among them, are what the options pin for comparisons.
 // A3_OPT_SWIGLU_NARROW: 0: no narrower last wave in the SwiGLU grid; 1: choose; 16..120: that width on half the tiles.
 
 template <int EPI>
@@ -644,7 +635,7 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
     const int m_tiles = cdiv(a.M, TC_BM), sms = h->sm_count > 0 ? h->sm_count : 148;
     if (epi == EPI_RESIDUAL) {
       // the CTA-pair kernel (bn 512 selects it): measured 5-7 % faster than one CTA per 128 x 224/256 tile at
-      // Llama-8B width for 804 and 5 152 rows.  Depths that are no multiple of 128 come here.
+      // Llama-8B width for 804 and 5 152 rows
       (void)m_tiles;
       (void)sms;
       bn = 512;
@@ -749,7 +740,6 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
   p.max_pos = h->m.max_positions;
   p.tab = h->rope_tab;
   p.status = h->dev_status;
-  p.early = a.early_weights;
   if (pair) bn = 512;
   if (epi == EPI_RESIDUAL) return dispatch_tc<EPI_RESIDUAL>(h, a, p, tiles, bn, stages, st);
   if (epi == EPI_SWIGLU) return dispatch_tc<EPI_SWIGLU>(h, a, p, tiles, bn, stages, st);

@@ -26,7 +26,6 @@ struct TcParams {
   int Hq, Hkv, D, layout, max_pos;
   const float2* tab;
   uint32_t* status;
-  int early;  // CTA-pair kernel: GemmArgs::early_weights
   // SwiGLU with a narrower last wave: column tiles 0..y_wide-1 hold BN/2 features, the rest g_narrow (0: all wide)
   int y_wide, g_narrow;
 };
