@@ -176,6 +176,10 @@ extern "C" int a3_create(a3_handle** out, const a3_model_desc* m, const a3_layer
   memcpy(h->layers, layers, sizeof(a3_layer_weights) * m->n_layers);
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device);
+  int l2 = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
+  const long long qd = (long long)m->n_q_heads * m->head_dim, kvd = (long long)m->n_kv_heads * m->head_dim;
+  h->stack_over_l2 = 2ll * m->n_layers * m->d_model * (2 * qd + 2 * kvd + 3ll * m->d_ff) > l2;
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->rope_tab, (size_t)m->max_positions * (m->head_dim / 2) * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, 256);
   if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, 256);
@@ -446,7 +450,7 @@ extern "C" int a3_query_scores(const a3_handle* h, const void* q_rows, const int
 namespace a3 {
 // The host-buffer entry feeds the request: layer_ready[l] is the event after which layer l's chunk caches are in device
 // memory; position recovery of layer l is queued behind it, just before the layer needs the cache.  The copies
-// themselves are queued a few layers ahead of the compute launches that need them (queue_layer), not all up front:
+// themselves are queued a few layers ahead of the compute launches that need them (queue_layers), not all up front:
 // thousands of small copies take the host tens of milliseconds to queue, which would otherwise delay the first launch.
 // The first full block walks a long input in row panels (same panels whatever the entry point, so that every entry
 // point arrives at the same bits): the host-buffer entry copies the embeddings panel by panel and the block starts

@@ -175,7 +175,7 @@ __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc
 // slices in order.  See residual_slices below for when and why.
 // KC = 2 (QKV of few rows): a cluster of two pairs per unit, each with half of the k-loop.  The epilogue needs whole sums: pair c
 // finishes the tokens of warp set c and receives the other pair's sums for them through distributed shared memory.
-// ONCE: one token tile, every weight is read once in the whole launch (see the producer).
+// ONCE: every weight is read once and leaves L2 first (see weights_once and the producer).
 template <int EPI, bool SPLIT, int KC, bool ONCE>
 __global__ void __cluster_dims__(2 * KC, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
@@ -254,10 +254,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         if (EPI != EPI_RESIDUAL) tmap_prefetch(&tmU);
         if (EPI == EPI_QKV) tmap_prefetch(&tmW);
       }
-      // ONCE: a layer of weights is several times L2 and nobody reads them again: first out, so that they do not displace what
-      // the kernels hand on (rows, partial sums, the cache) and their code.  A layer of 144 rows at Llama-8B width 115.6 ->
-      // 111.7 us, of 75 rows at Qwen-7B width 91.3 -> 89.6.  With two token tiles a policy on every load costs (280 rows 138.1
-      // -> 140.5), and so does choosing per load (270 rows, Qwen width 122.7 -> 123.6): hence an instance of its own.
+      // ONCE (see weights_once): first out, so that they do not displace what the kernels hand on (rows, partial sums, the
+      // cache) and their code.  A layer of 144 rows at Llama-8B width 115.6 -> 111.7 us, of 75 rows at Qwen-7B width 91.3 -> 89.6.
+      // With two token tiles a policy on every load costs (280 rows 138.1 -> 140.5), and so does choosing per load (270 rows,
+      // Qwen width 122.7 -> 123.6): hence an instance of its own.
       const uint64_t once = ONCE ? l2_evict_first() : 0;
       auto load = [&](uint32_t dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
         if (ONCE) tma_load_3d_pair_once(dst, map, y, z, bar, once);
@@ -350,7 +350,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: the leader alone, for both CTAs.
-    // The whole warp walks the loop, one elected lane issues (see uniform_warp in a3_tc.cuh).  Back to back at 804 rows x
+    // The whole warp walks the loop, one elected lane issues (see uniform_warp).  Back to back at 804 rows x
     // 28 672 columns 167 -> 156 us, at 133 rows 54.3 -> 51.1, a single unit alone (no contention) 19.7 -> 16.0.
     if (leader) {
       const uint32_t idesc = idesc_bf16_pair(p.tok_n);
@@ -855,6 +855,13 @@ int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) 
   return choose_slices(M, N, K, blocks, pairs, part_bytes);
 }
 
+// Weights that nobody finds in L2 again: one token tile, so that the launch reads each of them once, and a stack of layers
+// beyond L2, so that the next request does not either.  A model that L2 holds wants its weights left there: one layer of 90 MB
+// back to back, 13 rows 42.7 us with the normal policy against 46.8, 75 rows 48.9 / 53.0, 200 rows 71.4 / 71.4; 18 MB in three
+// layers no difference; two layers of 180 MB 45.3 / 44.2, 52.0 / 50.7 and 69.4 / 67.5.  The QKV projection in clusters marks its
+// weights always: with the normal policy for a model that L2 holds the 90 MB layer took 43.3 and 50.4 us.
+static bool weights_once(const a3_handle* h, int tok_tiles) { return tok_tiles == 1 && h->stack_over_l2; }
+
 // Ring depth and epilogue chunk of a launch: the widest chunk among those that leave the ring deepest (a stage more is 8 %
 // at 513 rows, where 32-token chunks leave three stages of 176 tokens and 8-token chunks four), but no deeper than a pair
 // has stages to run through.  Returns the dynamic shared memory.
@@ -898,7 +905,7 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB));
   static SmemAttrOnce attr[2];
-  const bool once = p.tok_tiles == 1;
+  const bool once = weights_once(h, p.tok_tiles);
   const auto kernel = once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true> : pair_t_kernel<EPI_RESIDUAL, true, 1, false>;
   A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
@@ -934,7 +941,7 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   if (EPI == EPI_SWIGLU) A3_TRY(make_tmap_kblocks(&tU, a.B2, p.F, a.K, ROWS, 1));
   else tU = tG;
   static SmemAttrOnce attr[2];
-  const bool once = p.tok_tiles == 1;
+  const bool once = weights_once(h, p.tok_tiles);
   const auto kernel = once ? pair_t_kernel<EPI, false, 1, true> : pair_t_kernel<EPI, false, 1, false>;
   A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, EPI == EPI_SWIGLU ? A3_K_GEMM_SWIGLU : A3_K_GEMM_RESIDUAL, st);
@@ -1030,7 +1037,7 @@ int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st) {
     else tW[s] = tW[0];
   }
   static SmemAttrOnce attr[3];
-  const int variant = clusters ? 2 : p.tok_tiles == 1;
+  const int variant = clusters ? 2 : weights_once(h, p.tok_tiles);
   const auto kernel = variant == 2   ? pair_t_kernel<EPI_QKV, false, 2, true>
                       : variant == 1 ? pair_t_kernel<EPI_QKV, false, 1, true>
                                      : pair_t_kernel<EPI_QKV, false, 1, false>;

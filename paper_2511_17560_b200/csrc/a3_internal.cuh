@@ -20,6 +20,7 @@ struct a3_handle {
   uint32_t* dev_status;      // dev, 1 word (+ padding)
   int device;
   int sm_count;
+  bool stack_over_l2;        // the weights of all layers do not fit in L2: one pass over the layers never finds them there
   void* tmaps;               // host-side tensor-map cache (a3_gemm.cu)
   a3::Profiler* prof;        // null unless a3_profile_enable is on
   void* host_pipe;           // copy stream + events of a3_fuse_request_host, created on first use
@@ -175,7 +176,7 @@ struct GemmArgs {
   int q_first;         // > 0: queries only of the rows from here on (q_out starts with them); segments k, v, q; gemm_qkv_t only
 };
 
-// SwiGLU GEMM with the weights as the M-side operand of a CTA pair, persistent (a3_swiglu_pair.cu).
+// SwiGLU GEMM with the weights as the M-side operand of a CTA pair, persistent (a3_gemm_persistent.cu).
 bool swiglu_pair_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_swiglu_pair(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
 // C += A B^T with the same kernel structure (weights on the M side, persistent CTA pairs).

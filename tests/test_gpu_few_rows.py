@@ -25,6 +25,11 @@ DEEP = W.ModelShape("deep", 2, 896, 16, 4, 128, 2176, 32000, 5e5, 1e-5)
 BROAD = W.ModelShape("broad", 1, 2176, 9, 3, 128, 640, 32000, 5e5, 1e-5)
 
 
+# two layers are 243 MB, more than L2: every weight of a launch of one token tile leaves L2 first; down projection in 8 slices,
+# which the adding kernel takes in its loop
+BEYOND_L2 = W.ModelShape("beyond_l2", 2, 2048, 16, 4, 128, 8192, 32000, 5e5, 1e-5)
+
+
 def layer_parity(a3mod, m, M, seed):
     eng, layers, dev = make_engine(a3mod, m, seed=seed, w_std=0.05 * (512 / m.d_model) ** 0.5)
     model, weights = oracle_model(m), oracle_weights(layers)
@@ -66,6 +71,12 @@ def test_residual_gemm_in_slices(a3mod, M):
 def test_qkv_projection_in_halves(a3mod, M):
     """Two pairs of CTAs per two heads, up to one full token tile: one token, warp sets with and without tokens."""
     layer_parity(a3mod, BROAD, M, seed=M + 1)
+
+
+@pytest.mark.parametrize("M", [1, 75, 256, 257])
+def test_layer_of_a_stack_beyond_l2(a3mod, M):
+    """One token tile (the instances that mark the weights) and two (those that do not)."""
+    layer_parity(a3mod, BEYOND_L2, M, seed=M + 2)
 
 
 @pytest.mark.parametrize("shape,kv_len,M", [(W.TINY_GQA, 768, 60), (W.TINY_GQA, 1023, 41), (W.TINY_GQA, 1024, 64), (W.TINY_GQA, 1153, 7),
