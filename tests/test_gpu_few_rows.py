@@ -79,6 +79,43 @@ def test_layer_of_a_stack_beyond_l2(a3mod, M):
     layer_parity(a3mod, BEYOND_L2, M, seed=M + 2)
 
 
+# rows of more than 4 096 values: what the threads of the adding kernel do not keep in registers is read again; both of a layer's
+# residual products in two slices
+LONG_ROWS = W.ModelShape("long_rows", 1, 4224, 16, 4, 128, 2176, 32000, 5e5, 1e-5)
+
+
+@pytest.mark.parametrize("M", [1, 17])
+def test_slices_added_to_long_rows(a3mod, M):
+    layer_parity(a3mod, LONG_ROWS, M, seed=M + 3)
+
+
+@pytest.mark.parametrize("d_model", [4224, 8448])
+def test_long_rows_enter_a_request(a3mod, d_model):
+    """Copied, gathered and normed by one kernel: the request that recomputes everything is the layer-by-layer prefill, bit for
+    bit, and its first keys are the oracle's."""
+    m = W.ModelShape("long_rows", 2, d_model, 2, 1, 128, 256, 1000, 1e4, 1e-5)
+    eng, layers, dev = make_engine(a3mod, m, seed=d_model, w_std=0.05 * (512 / d_model) ** 0.5)
+    n_ctx, nq = 61, 9
+    n = n_ctx + nq
+    g = torch.Generator(device=dev)
+    g.manual_seed(d_model)
+    ck, cv = (torch.randn(m.n_layers, n_ctx, m.n_kv_heads, m.head_dim, device=dev, generator=g).bfloat16() for _ in range(2))
+    x0 = torch.randn(n, d_model, device=dev, generator=g).bfloat16()
+    K, V = (torch.zeros(m.n_layers, n, m.n_kv_heads, m.head_dim, device=dev, dtype=torch.bfloat16) for _ in range(2))
+    rq, out = eng.make_request(a3mod.chunk_table([ck], [cv], [0]), 1, n_ctx, n_ctx, nq, x0, K, V, ratio=1.0)
+    eng.fuse_request(rq)
+    x, Kp, Vp = x0.clone(), torch.zeros_like(K), torch.zeros_like(V)
+    pos = torch.arange(n, dtype=torch.int32, device=dev)
+    for layer in range(m.n_layers):
+        eng.recompute_layer(layer, x, pos, Kp[layer], Vp[layer])
+    assert eng.device_status() == 0
+    assert torch.equal(K, Kp) and torch.equal(V, Vp) and torch.equal(out["x"], x)
+    Ko, Vo, _ = O.full_prefill(f64(x0), oracle_weights(layers), oracle_model(m), rnd=O.round_bf16)
+    check_kv(f64(K[0]), Ko[0], "first layer's K")
+    check_kv(f64(V[0]), Vo[0], "first layer's V")
+    eng.close()
+
+
 @pytest.mark.parametrize("shape,kv_len,M", [(W.TINY_GQA, 768, 60), (W.TINY_GQA, 1023, 41), (W.TINY_GQA, 1024, 64), (W.TINY_GQA, 1153, 7),
                                             (W.TINY_GQA, 3000, 300), (W.TINY_G7, 1200, 55), (W.TINY, 700, 33), (W.TINY, 770, 128)])
 def test_attention_keys_shared_by_a_cluster(a3mod, shape, kv_len, M):

@@ -14,8 +14,17 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("n_layers,select_layer,lens", [(2, 1, (40, 30)), (3, 0, (1, 64)), (4, 1, (33, 70, 5)), (9, 1, (48, 16)),
                                                         (14, 2, (20, 31, 12)), (12, 1, ())])
 def test_groups_of_layers_match_the_device_entry(a3mod, n_layers, select_layer, lens):
-    m = replace(W.TINY_GQA, n_layers=n_layers)
-    dev, n_ctx, nq = torch.device("cuda:0"), sum(lens), 9
+    compare_entries(a3mod, replace(W.TINY_GQA, n_layers=n_layers), select_layer, lens)
+
+
+# 2 KB of keys a token: slices of 4.1 MB, 2.1, 1.4, 1.0 and 0.7 are copied one, one, three, four and five layers at a time
+@pytest.mark.parametrize("n_layers,lens", [(5, (2007,)), (6, (1025, 1030)), (9, (650, 700)), (13, (512, 512)), (12, (400, 300))])
+def test_large_slices_are_copied_in_smaller_groups(a3mod, n_layers, lens):
+    compare_entries(a3mod, W.ModelShape("broad_cache", n_layers, 128, 8, 8, 128, 128, 1000, 1e4, 1e-5), 1, lens)
+
+
+def compare_entries(a3mod, m, select_layer, lens):
+    dev, n_layers, n_ctx, nq = torch.device("cuda:0"), m.n_layers, sum(lens), 9
     n = n_ctx + nq
     eng = a3mod.A3(m, W.make_weights_device(m, dev, 0), n + 8)
     g = torch.Generator(device=dev)
