@@ -695,11 +695,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
 // One warp per (flat row, KV head) of a row tile that was split over the keys: merges the segments' partial results
 // in segment order (fixed, so the result is reproducible): O = sum_z O_z 2^(m_z - m) / sum_z l_z 2^(m_z - m).
+// The partial results come from the preceding kernel, which this one may have become resident next to: their pointers are not
+// __restrict__, so that the loads are ordinary ones and not of the read-only path.  They are kept in L1 all the same: a segment's
+// statistics are read twice, and by four rows from one line (129 segments through L2 each time: 8 us more).
 template <int D>
 __global__ void __launch_bounds__(128)
 attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int Hq, int Hkv, int tiles_per_split, int rows_pad,
-                         const float* __restrict__ part_o, const float2* __restrict__ part_ml, bf16* __restrict__ o,
-                         float* __restrict__ lse) {
+                         const float* part_o, const float2* part_ml, bf16* __restrict__ o, float* __restrict__ lse) {
   const int G = Hq / Hkv;
   const int rows_total = M * G;
   const int fr = blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -715,7 +717,7 @@ attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int
   if (n_active <= 1) return;  // written directly by the attention kernel
   float m = -INFINITY;
   for (int z = 0; z < n_active; ++z) {
-    const float2 ml = __ldcg(part_ml + ((size_t)z * Hkv + g) * rows_pad + fr);
+    const float2 ml = part_ml[((size_t)z * Hkv + g) * rows_pad + fr];
     if (ml.y > 0.f) m = fmaxf(m, ml.x);
   }
   constexpr int PER = D / 32;
@@ -725,14 +727,14 @@ attention_combine_kernel(const int32_t* __restrict__ pos, int M, int kv_len, int
   float l = 0.f;
   for (int z = 0; z < n_active; ++z) {
     const size_t prow = ((size_t)z * Hkv + g) * rows_pad + fr;
-    const float2 ml = __ldcg(part_ml + prow);
+    const float2 ml = part_ml[prow];
     if (!(ml.y > 0.f)) continue;
     const float w = exp2f(ml.x - m);
     l += ml.y * w;
     if (o) {
       const float* src = part_o + prow * D + lane * PER;
 #pragma unroll
-      for (int e = 0; e < PER; ++e) acc[e] += __ldcg(src + e) * w;
+      for (int e = 0; e < PER; ++e) acc[e] += src[e] * w;
     }
   }
   const int tok = fr / G, hq = g * G + fr % G;

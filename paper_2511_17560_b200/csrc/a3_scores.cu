@@ -260,7 +260,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   // tables: log-sum-exps in the exp2 domain in packed order per KV head, and each packed row's position
   for (int i = threadIdx.x; i < p.Hkv * rows_g; i += STC_THREADS) {
     const int g = i / rows_g, r = i - g * rows_g;
-    l2tab[i] = __ldcg(p.lse + (size_t)(r / G) * p.Hq + g * G + r % G) * ATC_LOG2E;
+    l2tab[i] = p.lse[(size_t)(r / G) * p.Hq + g * G + r % G] * ATC_LOG2E;
   }
   for (int r = threadIdx.x; r < rows_g; r += STC_THREADS) postab[r] = min(p.q_pos[r / G], p.kv_len - 1);
   __syncthreads();
