@@ -232,7 +232,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int key0 = blockIdx.x * 128;
   // gridDim.y == 1: all KV heads, summed (Eq. 3); more: a share of the KV heads per CTA (per-head votes only)
-  const int g_begin = p.Hkv * blockIdx.y / gridDim.y, g_end = p.Hkv * (blockIdx.y + 1) / gridDim.y;
+  const int g_begin = gridDim.y == 1 ? 0 : p.Hkv * blockIdx.y / gridDim.y, g_end = gridDim.y == 1 ? p.Hkv : p.Hkv * (blockIdx.y + 1) / gridDim.y;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
