@@ -33,8 +33,9 @@ if ROOT not in sys.path:
 # DRAM bytes (read + write) per launch of the dominant kernel classes from the ncu captures summarised under profiles/
 # (gemm_kernels_llama8b_2layer.txt: SwiGLU GEMM of a sparse layer, M = 804, and of the full block, M = 5152).  Used for `roofline.traffic` of the workloads they were captured on.
 NCU_TRAFFIC = {("llama8b_10x512", "gemm_swiglu"): {"sparse": 244.2e6 + 19.3e6, "full": 415.4e6 + 141.8e6},
-               # attention_and_selection_kernels_llama8b_64x512_2layer.txt: sparse rows (4 952) and the full causal block (32 800)
-               ("llama8b_64x512", "attention"): {"sparse": 419.97e6 + 35.71e6, "full": 2208.55e6 + 265.24e6}}
+               # attention_and_selection_kernels_llama8b_64x512_2layer.txt: sparse rows (4 952) and the full causal block (32 800 rows in
+               # four panels, a launch each)
+               ("llama8b_64x512", "attention"): {"sparse": 391.48e6 + 35.12e6, "full": 2230.77e6 + 235.11e6, "full_launches": 4}}
 
 METRIC = "context_tokens_fused_per_s"
 UNIT = "tokens/s"
@@ -45,7 +46,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 
 
 def load_peaks():
-    """Measured peaks of this machine (generated file) and the SM clock the sustained matmul figure was taken at."""
+    """Measured peaks of the device (file beside this one) and the SM clock the sustained matmul figure was taken at."""
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
         try:
@@ -489,7 +490,8 @@ class RequestWorkload:
         if t:
             nf = self.r.select_layer
             # launch-weighted mean over the class's launches: the leading full blocks, then one sparse-row launch per later layer
-            traffic = (t["full"] * nf + t["sparse"] * (self.m.n_layers - nf)) / self.m.n_layers
+            sparse = self.m.n_layers - nf
+            traffic = (t["full"] * nf + t["sparse"] * sparse) / (t.get("full_launches", 1) * nf + sparse)
         return {"kernel": top, "bound": tk.get("bound"), "achieved": tk.get("achieved"),
                 "peak": peaks["bf16_tflops_sustained"] if tk.get("bound") == "tensor" else peaks["hbm_gbs"],
                 "unit": tk.get("unit"), "frac": tk.get("frac"), "frac_burst": tk.get("frac_burst"),

@@ -173,7 +173,7 @@ def test_topk_at_the_register_sizes(a3mod, n):
 
 @pytest.mark.parametrize("n_ctx,pool", [(900, 3), (3073, 7), (5120, 5), (8200, 7)])
 def test_pooled_selection_of_the_eviction(a3mod, n_ctx, pool):
-    """Pooling inside the selection: votes in registers, and (8 200 candidates) in shared memory."""
+    """Pooling inside the selection, and (8 200 candidates) by the kernel of its own."""
     m = W.TINY_GQA
     eng, _, dev = make_engine(a3mod, m, seed=n_ctx)
     model, nq, n_system, capacity = oracle_model(m), 9, 5, 300
