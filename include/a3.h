@@ -316,7 +316,7 @@ int a3_fuse_batch(const a3_handle* h, const a3_request* reqs, int n_requests, vo
 
 /* a3_fuse_request with the chunk caches and embeddings in HOST memory (pinned memory lets the copies
  * overlap the compute): copies them to `staging` (dev, a3_host_staging_bytes) on a copy stream the
- * handle creates on first use, layer by layer, while `stream` computes; builds the chunk descriptors,
+ * handle creates on first use, a few layers at a time, while `stream` computes; builds the chunk descriptors,
  * fuses, copies rows_out and x_out back to the host and waits for both streams - also when it returns an
  * error after the first copy was queued, so the host buffers and the staging area are free on return whatever
  * the status.  Chunk caches of layers up to select_layer are not copied: those layers are recomputed for every

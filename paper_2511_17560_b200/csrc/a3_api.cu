@@ -787,8 +787,8 @@ static void host_pipe_destroy(a3_handle* h) {
 }
 }  // namespace a3
 
-// Copies run on the handle's own copy stream, layer by layer, while the compute stream works: the embeddings go
-// first (the full block needs only them), then each layer's chunk caches; position recovery of a layer is queued
+// Copies run on the handle's own copy stream while the compute stream works: the embeddings go first (the full block
+// needs only them), then the chunk caches, a few layers at a time (feed_group); position recovery of a layer is queued
 // behind that layer's copy.  Layers up to the selection layer are never copied: their caches are recomputed.
 extern "C" int a3_fuse_request_host(const a3_handle* h, const a3_request* req, const a3_host_io* io, void* staging,
                                     size_t staging_bytes, void* ws, size_t ws_bytes, a3_stream stream) {

@@ -58,8 +58,8 @@ __device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned in
 
 // Up to KPT x 1 024 candidates, which is every request of a few thousand tokens: a thread keeps its keys (slots tid, tid +
 // 1 024, ...) in registers through all passes.  With half_pool the keys are of the running maximum over the neighbouring
-// candidates, taken from a copy of the scores in shared memory.  Bound by the chain of block barriers, three per pass:
-// 5 120 candidates take 7.1 us where the passes over shared memory below took 10.6, 356 take 4.3 instead of 6.3.
+// candidates, taken from a copy of the scores in shared memory.  Bound by the chain of block barriers, three per pass: back
+// to back 5 120 candidates take 7.6 us where the passes over shared memory below took 10.6, 900 take 5.0 instead of 7.0.
 template <int KPT>
 __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __restrict__ raw, int cand_begin, int n, int k, int half_pool,
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
@@ -275,9 +275,8 @@ static int launch_topk(const a3_handle* h, const float* scores, size_t score_str
                       in_smem, half_pool, tail_begin, tail);
   };
   const size_t raw = half_pool > 0 ? (size_t)n * 4 : 0;
-  // Half a microsecond per key and thread, hence instances of one, three, five and eight keys (900 candidates 4.9 us, 5 120 7.7,
-  // 8 192 9.9): the smallest that holds the candidates.  An instance for every count would save at most a microsecond more (5 121
-  // candidates take 9.2).
+  // 0.7 us per key and thread, hence instances of one, three, five and eight keys (back to back 900 candidates 5.0 us, 5 120 7.6,
+  // 8 192 9.9): the smallest that holds the candidates.  Those in between would save up to 1.5 us more (5 121 candidates take 9.1).
   if (n <= TK_THREADS) {
     A3_CUDA(go(topk_select_kernel<1>, raw));
   } else if (n <= 3 * TK_THREADS) {
