@@ -179,7 +179,7 @@ extern "C" int a3_create(a3_handle** out, const a3_model_desc* m, const a3_layer
   int l2 = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
   const long long qd = (long long)m->n_q_heads * m->head_dim, kvd = (long long)m->n_kv_heads * m->head_dim;
-  h->stack_over_l2 = 2ll * m->n_layers * m->d_model * (2 * qd + 2 * kvd + 3ll * m->d_ff) > l2;
+  h->stack_over_l2 = 2ll * m->n_layers * m->d_model * (2 * qd + 2 * kvd + 3ll * m->d_ff) > l2 / 4 * 3ll;
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->rope_tab, (size_t)m->max_positions * (m->head_dim / 2) * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, 256);
   if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, 256);

@@ -856,10 +856,12 @@ int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) 
 }
 
 // Weights that nobody finds in L2 again: one token tile, so that the launch reads each of them once, and a stack of layers
-// beyond L2, so that the next request does not either.  A model that L2 holds wants its weights left there: one layer of 90 MB
-// back to back, 13 rows 42.7 us with the normal policy against 46.8, 75 rows 48.9 / 53.0, 200 rows 71.4 / 71.4; 18 MB in three
-// layers no difference; two layers of 180 MB 45.3 / 44.2, 52.0 / 50.7 and 69.4 / 67.5.  The QKV projection in clusters marks its
-// weights always: with the normal policy for a model that L2 holds the 90 MB layer took 43.3 and 50.4 us.
+// beyond L2, so that the next request does not either.  A model that L2 holds wants its weights left there.  One layer back to
+// back, normal policy against marked weights (us, 13 / 75 / 200 rows): 78 MB 40.7 / 47.0 / 65.0 against 44.8 / 51.0 / 64.8; 90 MB
+// 42.7 / 49.7 / 69.4 and 46.9 / 53.5 / 71.4; 100 MB 44.8 / 52.0 / 73.2 and 48.9 / 55.5 / 71.4; 115 MB 50.9 / 58.9 / 76.0 and
+// 51.0 / 57.1 / 73.5; 131 MB 55.5 / 61.9 / 78.0 and 53.0 / 59.6 / 74.0; with heads of 64, 122 MB 66.1 / 72.0 / 85.5 and
+// 59.1 / 64.2 / 75.5; 18 MB in three layers no difference.  Hence the line at three quarters of L2.  The QKV projection in
+// clusters marks its weights always: with the normal policy the 90 MB layer took 43.3 and 50.4 us for 13 and 75 rows.
 static bool weights_once(const a3_handle* h, int tok_tiles) { return tok_tiles == 1 && h->stack_over_l2; }
 
 // Ring depth and epilogue chunk of a launch: the widest chunk among those that leave the ring deepest (a stage more is 8 %

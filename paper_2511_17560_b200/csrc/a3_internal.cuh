@@ -20,7 +20,7 @@ struct a3_handle {
   uint32_t* dev_status;      // dev, 1 word (+ padding)
   int device;
   int sm_count;
-  bool stack_over_l2;        // the weights of all layers do not fit in L2: one pass over the layers never finds them there
+  bool stack_over_l2;        // the weights of all layers do not fit in L2 beside what a request works on (see weights_once)
   void* tmaps;               // host-side tensor-map cache (a3_gemm.cu)
   a3::Profiler* prof;        // null unless a3_profile_enable is on
   void* host_pipe;           // copy stream + events of a3_fuse_request_host, created on first use
