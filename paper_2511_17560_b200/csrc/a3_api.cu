@@ -341,9 +341,10 @@ static int qkv_project(const a3_handle* h, int layer, const bf16* a, const int32
 // norm's kernel; otherwise the GEMM updates C itself and the norm follows.
 static int residual_then_norm(const a3_handle* h, const GemmArgs& g, const LayerWs& w, const bf16* next_gain, cudaStream_t st) {
   const a3_model_desc& m = h->m;
-  const int slices = residual_slices(h, g.M, g.seg[0].n, g.K, w.attn_part_bytes);
+  int tiles;
+  const int slices = residual_slices(h, g.M, g.seg[0].n, g.K, w.attn_part_bytes, &tiles);
   if (slices > 1) {  // the attention's partial results were consumed before the projection that follows it: their room is free
-    A3_TRY(gemm_residual_split(h, g, slices, (float*)w.attn_part, st));
+    A3_TRY(gemm_residual_split(h, g, slices, tiles, (float*)w.attn_part, st));
     return add_slices_rmsnorm(h, g.C, (const float*)w.attn_part, slices, next_gain, m.rms_eps, g.M, m.d_model, w.a, st);
   }
   A3_TRY(gemm_bf16(h, EPI_RESIDUAL, g, st));

@@ -41,17 +41,19 @@ __host__ __device__ constexpr int sp_set_floats(int chunk) { return 4 * (chunk *
 __host__ __device__ constexpr int sp_xch_floats_bytes(int chunk) { return (2 * sp_set_floats(chunk) * 4 + 255) & ~255; }
 __host__ __device__ constexpr int sp_xch_bytes(int epi, int chunk) { return sp_xch_floats_bytes(chunk) + (epi == EPI_QKV ? 1024 : 0); }
 constexpr int SP_SMEM_LIMIT = 227 * 1024;
+constexpr int SP_SLOTS = 3;  // accumulators in tensor memory, at most
 
 struct SpParams {
   int M, K, F;
-  int tok_tiles, tok_n;  // token tiles and tokens per tile (multiple of 16, at most 256)
+  int tok_tiles, tok_n;  // token tiles of a launch (TT > 1: groups of TT) and tokens per tile (multiple of 16, at most 256)
   int n_fblocks;         // feature blocks (one per CTA pair and unit): units = n_fblocks x tok_tiles
   int group;             // feature blocks per group of the unit order (1: feature blocks outermost)
   int early;             // the first ring stages' weights may be loaded before the preceding kernels are waited for
   int k_slices;          // SPLIT: slices of the k-loop per (feature block, token tile); 1 otherwise
   float* part;           // SPLIT: fp32 partial sums [k_slices][M][F]
   int n_units, n_pairs;
-  int stages, stage_bytes;  // ring depth; bytes per stage: SP_SUB k-blocks of weights, then SP_SUB of this CTA's half of the token tile
+  int stages, stage_bytes;  // ring depth; bytes per stage: SP_SUB / TT k-blocks of weights, then as many of this CTA's half of every token tile
+  int slot_cols;         // tensor-memory columns from one accumulator to the next
   int chunk;             // tokens per exchange of the epilogue: 32, 16 or (not QKV) 8
   bf16* C;
   int ldc;
@@ -176,11 +178,15 @@ __device__ __forceinline__ void tc_mma_pair_acc(uint32_t d_tmem, uint64_t a_desc
 // KC = 2 (QKV of few rows): a cluster of two pairs per unit, each with half of the k-loop.  The epilogue needs whole sums: pair c
 // finishes the tokens of warp set c and receives the other pair's sums for them through distributed shared memory.
 // ONCE: every weight is read once and leaves L2 first (see weights_once and the producer).
-template <int EPI, bool SPLIT, int KC, bool ONCE>
+// TT = 2 (just over 256 rows): a unit is two token tiles on one stream of weights, see two_tiles.  A ring stage is then one k-block:
+// eight instructions again.  Accumulators take turns in three slots of tensor memory instead of two.
+template <int EPI, bool SPLIT, int KC, bool ONCE, int TT = 1>
 __global__ void __cluster_dims__(2 * KC, 1, 1) __launch_bounds__(SP_THREADS, 1)
 pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
               const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmW, const SpParams p) {
   constexpr int ROWS = EPI == EPI_SWIGLU ? SP_FEAT : 2 * SP_FEAT;  // output features per CTA
+  constexpr int SUB = SP_SUB / TT;          // k-blocks per ring stage
+  constexpr int SLOTS = TT == 1 ? 2 : SP_SLOTS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);  // same offset in both CTAs of the pair
   unsigned char* base_ptr = smem_raw;
@@ -190,14 +196,14 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   }
   const int S = p.stages;
   const int xch_off = S * p.stage_bytes, bar_off = xch_off + (SPLIT ? 0 : sp_xch_bytes(EPI, p.chunk));
-  // barriers (8 bytes each): full[8] (used in the leader), empty[8], tmem_full[2], tmem_empty[2] (used in the leader)
+  // barriers (8 bytes each): full[8] (used in the leader), empty[8], tmem_full[3], tmem_empty[3] (used in the leader)
   const uint32_t bars = base + bar_off;
   auto full_bar = [&](int s) { return bars + 8u * s; };
   auto empty_bar = [&](int s) { return bars + 8u * (SP_MAX_STAGES + s); };
   auto tmem_full = [&](int b) { return bars + 8u * (2 * SP_MAX_STAGES + b); };
-  auto tmem_empty = [&](int b) { return bars + 8u * (2 * SP_MAX_STAGES + 2 + b); };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + bar_off + 8 * (2 * SP_MAX_STAGES + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + bar_off + 8 * (2 * SP_MAX_STAGES + 4) + 8);
+  auto tmem_empty = [&](int b) { return bars + 8u * (2 * SP_MAX_STAGES + SP_SLOTS + b); };
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + bar_off + 8 * (2 * SP_MAX_STAGES + 2 * SP_SLOTS));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + bar_off + 8 * (2 * SP_MAX_STAGES + 2 * SP_SLOTS) + 8);
   volatile int* ep_ok = abort_flag + 2;  // the epilogue's one waiter tells the other 127 threads how its wait ended
   float* xch = reinterpret_cast<float*>(base_ptr + xch_off);
 
@@ -209,7 +215,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   const bool leader = rank == 0;
   const int pair = blockIdx.x / (2 * KC);
   int merged = 0;  // KC > 1: how many of the two cluster barriers of the merge this warp has passed
-  const int KT = p.K / TC_BK;  // a multiple of SP_SUB (checked by the launcher)
+  const int KT = p.K / TC_BK, KS = KT / SUB;  // k-blocks (a multiple of SP_SUB, checked by the launcher) and ring stages of a k-loop
   const int half_n = p.tok_n >> 1;  // token rows this CTA loads per k-block (multiple of 8)
   const uint32_t b_bytes = (uint32_t)half_n * TC_BK * 2;
 
@@ -218,7 +224,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < SLOTS; ++b) {
       mbar_init(tmem_full(b), 1);
       mbar_init(tmem_empty(b), 16);  // every epilogue warp of both CTAs
     }
@@ -244,9 +250,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     pdl_launch_dependents();  // from here on: a launch never runs ahead of more than the one before it
   }
 
-  // The accumulator of unit u goes back to the MMA issuer, which takes it again two units later.  Behind a pair's last two units
-  // nobody waits, and an arrival still on its way must not find the leader gone (the last barrier orders no memory).
-  auto awaited = [&](int u) { return u + 2 * p.n_pairs < p.n_units; };
+  // Accumulators of this pair, numbered in order: number t lies in slot t % SLOTS.  It goes back to the MMA issuer, which takes the slot
+  // again SLOTS accumulators later.  Behind the last ones nobody waits, and an arrival still on its way must not find the leader
+  // gone (the last barrier orders no memory).
+  const int n_acc = pair < p.n_units ? TT * ((p.n_units - pair + p.n_pairs - 1) / p.n_pairs) : 0;
+  auto awaited = [&](int t) { return t + SLOTS < n_acc; };
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own gate/up rows, own half of the token tile
     // as a whole warp, one elected lane issuing; a stage's k-blocks of an operand are one copy of a 3-D map ([k-block][row][64])
@@ -275,13 +283,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         int fb, row0, kb0 = 0, kb1 = KT;
         sp_place<EPI>(p, SPLIT ? u / p.k_slices : u, fb, row0);
         if (SPLIT) {
-          sp_slice(u % p.k_slices, p.k_slices, KT / SP_SUB, kb0, kb1);
-          kb0 *= SP_SUB;
-          kb1 = kb0 + kb1 * SP_SUB;
+          sp_slice(u % p.k_slices, p.k_slices, KS, kb0, kb1);
+          kb0 *= SUB;
+          kb1 = kb0 + kb1 * SUB;
         } else if (KC > 1) {
-          sp_slice(kc, KC, KT / SP_SUB, kb0, kb1);
-          kb0 *= SP_SUB;
-          kb1 = kb0 + kb1 * SP_SUB;
+          sp_slice(kc, KC, KS, kb0, kb1);
+          kb0 *= SUB;
+          kb1 = kb0 + kb1 * SUB;
         }
         int f0 = fb * (2 * ROWS) + (int)rank * ROWS;
         const CUtensorMap* mapA = &tmG;
@@ -300,11 +308,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           // the leader announces the bytes of both CTAs; a copy of the peer that completes earlier cannot end the
           // phase, because the leader's own arrival is still pending until its expect_tx
           if (elect_one()) {
-            if (leader) mbar_expect_tx(full_bar(stage), 2 * SP_SUB * (SP_A_BYTES + b_bytes));
+            if (leader) mbar_expect_tx(full_bar(stage), 2 * SUB * (SP_A_BYTES + TT * b_bytes));
             if (EPI == EPI_SWIGLU) {
               // a k-block's operand is gate rows, then up rows
 #pragma unroll
-              for (int j = 0; j < SP_SUB; ++j) {
+              for (int j = 0; j < SUB; ++j) {
                 load(sa + j * SP_A_BYTES, &tmG, f0, kb + j, full_leader);
                 load(sa + j * SP_A_BYTES + SP_A_BYTES / 2, &tmU, f0, kb + j, full_leader);
               }
@@ -315,13 +323,13 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           __syncwarp();
         };
         if (early && kbg == 0) {
-          early = min(early, (kb1 - kb0) / SP_SUB);
-          for (int i = 0; i < early; ++i) load_weights(i, kb0 + i * SP_SUB);
+          early = min(early, (kb1 - kb0) / SUB);
+          for (int i = 0; i < early; ++i) load_weights(i, kb0 + i * SUB);
           issued = early;
           pdl_wait();
           pdl_launch_dependents();
         }
-        for (int kb = kb0; kb < kb1; kb += SP_SUB, ++kbg) {
+        for (int kb = kb0; kb < kb1; kb += SUB, ++kbg) {
           if (kbg >= early) {
             if (!mbar_wait_warp(empty_bar(s), ph ^ 1, abort_flag, p.status)) {
               ok = false;
@@ -329,8 +337,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
             }
             load_weights(s, kb);
           }
-          if (elect_one())
-            tma_load_3d_pair(base + s * p.stage_bytes + SP_SUB * SP_A_BYTES, &tmX, t0, kb, full_bar(s) & PAIR_LEADER_MASK);
+          if (elect_one()) {
+#pragma unroll
+            for (int j = 0; j < TT; ++j)
+              tma_load_3d_pair(base + s * p.stage_bytes + SUB * (SP_A_BYTES + j * b_bytes), &tmX, t0 + j * p.tok_n, kb, full_bar(s) & PAIR_LEADER_MASK);
+          }
           __syncwarp();
           issued = max(issued, kbg + 1);
           if (++s == S) {
@@ -357,37 +368,45 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     // 28 672 columns 167 -> 156 us, at 133 rows 54.3 -> 51.1, a single unit alone (no contention) 19.7 -> 16.0.
     if (leader) {
       const uint32_t idesc = idesc_bf16_pair(p.tok_n);
-      const uint64_t da0 = smem_desc_sw128(base), db0 = smem_desc_sw128(base + SP_SUB * SP_A_BYTES);
+      const uint64_t da0 = smem_desc_sw128(base), db0 = smem_desc_sw128(base + SUB * SP_A_BYTES);
       // descriptor address fields count 16-byte units: stage and k-step offsets are added to the first stage's
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, a_sub16 = SP_A_BYTES >> 4, b_sub16 = (uint32_t)half_n * (TC_BK * 2) >> 4;
       const uint32_t tmem_acc = __shfl_sync(0xffffffffu, tmem_base, 0);
-      int per_unit = KT / SP_SUB, total = 0;
+      int per_unit = KS, total = 0;
       if (KC > 1) {
         int first;
-        sp_slice(kc, KC, KT / SP_SUB, first, per_unit);
+        sp_slice(kc, KC, KS, first, per_unit);
       }
       if (SPLIT) {
         for (int u = pair, first; u < p.n_units; u += p.n_pairs) {
           int count;
-          sp_slice(u % p.k_slices, p.k_slices, KT / SP_SUB, first, count);
+          sp_slice(u % p.k_slices, p.k_slices, KS, first, count);
           total += count;
         }
       } else {
-        total = (pair < p.n_units ? (p.n_units - pair + p.n_pairs - 1) / p.n_pairs : 0) * per_unit;
+        total = n_acc / TT * per_unit;
       }
-      int s = 0, it = 0, in_unit = 0;
-      uint32_t ph = 0, stage_off = 0, d = tmem_acc;
+      int s = 0, u = pair, in_unit = 0, slot[TT];
+      uint32_t ph = 0, stage_off = 0, slot_ph = 1, d[TT];  // slot: of the next accumulator, phase in which it is found empty
+      int next_slot = 0;
       bool ok = total > 0;
       for (int g = 0; g < total && ok; ++g) {
         if (in_unit == 0) {
-          // the epilogues of both CTAs have drained this accumulator (first use: passes at once)
-          const int b = it & 1;
-          ok = mbar_wait_warp(tmem_empty(b), ((it >> 1) & 1) ^ 1, abort_flag, p.status);
+#pragma unroll
+          for (int j = 0; j < TT; ++j) {
+            // the epilogues of both CTAs have drained this accumulator (first use: passes at once)
+            slot[j] = next_slot;
+            ok = ok && mbar_wait_warp(tmem_empty(next_slot), slot_ph, abort_flag, p.status);
+            d[j] = tmem_acc + (uint32_t)(next_slot * p.slot_cols);
+            if (++next_slot == SLOTS) {
+              next_slot = 0;
+              slot_ph ^= 1;
+            }
+          }
           if (!ok) break;
-          d = tmem_acc + (uint32_t)b * 256u;
           if (SPLIT) {
             int first;
-            sp_slice((pair + it * p.n_pairs) % p.k_slices, p.k_slices, KT / SP_SUB, first, per_unit);
+            sp_slice(u % p.k_slices, p.k_slices, KS, first, per_unit);
           }
         }
         ok = mbar_wait_warp(full_bar(s), ph, abort_flag, p.status);
@@ -395,19 +414,26 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         tc_fence_after();
         const uint64_t da_s = da0 + stage_off, db_s = db0 + stage_off;
         if (elect_one()) {
-          tc_mma_pair_f16(d, da_s, db_s, idesc, in_unit != 0);
 #pragma unroll
-          for (int i = 1; i < SP_SUB * (TC_BK / 16); ++i) {
-            const int j = i / (TC_BK / 16), k = i % (TC_BK / 16);
-            tc_mma_pair_acc(d, da_s + (uint64_t)(j * a_sub16 + 2 * k), db_s + (uint64_t)(j * b_sub16 + 2 * k), idesc);
+          for (int j = 0; j < TT; ++j) {
+            const uint64_t db_j = db_s + (uint64_t)(j * SUB * b_sub16);
+            tc_mma_pair_f16(d[j], da_s, db_j, idesc, in_unit != 0);
+#pragma unroll
+            for (int i = 1; i < SUB * (TC_BK / 16); ++i) {
+              const int b = i / (TC_BK / 16), k = i % (TC_BK / 16);
+              tc_mma_pair_acc(d[j], da_s + (uint64_t)(b * a_sub16 + 2 * k), db_j + (uint64_t)(b * b_sub16 + 2 * k), idesc);
+            }
           }
           tc_commit_pair(empty_bar(s), pair_mask);  // frees this stage in both CTAs once the instructions above have read it
-          if (in_unit + 1 == per_unit) tc_commit_pair(tmem_full(it & 1), pair_mask);  // publishes the accumulator in both CTAs
+          if (in_unit + 1 == per_unit) {
+#pragma unroll
+            for (int j = 0; j < TT; ++j) tc_commit_pair(tmem_full(slot[j]), pair_mask);  // publishes the accumulators in both CTAs
+          }
         }
         __syncwarp();
         if (++in_unit == per_unit) {
           in_unit = 0;
-          ++it;
+          u += p.n_pairs;
         }
         stage_off += stage16;
         if (++s == S) {
@@ -426,19 +452,20 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int ep_tid = (warp - 2) * 32 + lane;
     const int set_n = p.tok_n >> 1;
     const int n_chunks = (set_n + 31) >> 5;
-    int it = 0;
-    for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
-      const int b = it & 1;
+    int b = 0;
+    uint32_t b_ph = 0;
+    for (int t = 0; t < n_acc; ++t) {
+      const int u = pair + t / TT * p.n_pairs;
       int fb, tt;
       sp_unit(u / p.k_slices, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
       const int f = fb * (2 * ROWS) + (int)rank * ROWS + quarter * 32 + lane;
-      const int t0 = tt * p.tok_n + set * set_n;
+      const int t0 = (tt * TT + t % TT) * p.tok_n + set * set_n;
       float* prow = p.part + ((size_t)(u % p.k_slices) * p.M + t0) * p.F + f;
-      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+      if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), b_ph, abort_flag, p.status) ? 1 : 0;
       named_bar_sync(1, 256);
       if (!ep_ok[0]) break;  // uniform for the 256 threads
       tc_fence_after();
-      const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
       for (int c = 0; c < n_chunks; ++c) {
         const int w = min(32, set_n - c * 32);
@@ -451,7 +478,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0 && awaited(u)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+      if (lane == 0 && awaited(t)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+      if (++b == SLOTS) {
+        b = 0;
+        b_ph ^= 1;
+      }
     }
   } else if (EPI == EPI_SWIGLU) {
     // ---------------- epilogue, silu(gate) * up: warps 2..9 of both CTAs; warp w may touch TMEM lanes 32*(w%4) .. +31: lanes
@@ -474,19 +505,19 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       const int e2 = st >> 3, fg = st & 7;
       const float* xg = xset + (fg >> 2) * QUARTER + (fg & 3) * 8;
       const float* xu = xg + 2 * QUARTER;
-      int it = 0;
-      for (int u = pair; u < p.n_units; u += p.n_pairs, ++it) {
-        const int b = it & 1;
+      int b = 0;
+      uint32_t b_ph = 0;
+      for (int t = 0; t < n_acc; ++t) {
         int fb, tt;
-        sp_unit(u, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
-        const int t0 = tt * p.tok_n + set * set_n;
+        sp_unit(pair + t / TT * p.n_pairs, p.n_fblocks, p.tok_tiles, p.group, fb, tt);
+        const int t0 = (tt * TT + t % TT) * p.tok_n + set * set_n;
         const int valid = min(set_n, p.M - t0);  // tokens of this set that exist (may be <= 0)
         bf16* out = p.C + (size_t)max(t0, 0) * p.ldc + fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + fg * 8;
-        if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
+        if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), b_ph, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
         for (int c = 0; c < n_chunks; ++c) {
           float v[CH];
@@ -518,7 +549,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0 && awaited(u)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+        if (lane == 0 && awaited(t)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+        if (++b == SLOTS) {
+          b = 0;
+          b_ph ^= 1;
+        }
       }
       return true;
     });
@@ -594,7 +629,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
         // KC > 1: [token of the set][128 features] fp32 sums of the other pair, over the ring, whose stages have all been read
         // once both pairs have published their accumulators
         const float* theirs = reinterpret_cast<const float*>(base_ptr) + quarter * 32 + lane;
@@ -689,7 +724,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0 && awaited(u)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+        if (lane == 0 && awaited(it)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
       }
       return true;
     });
@@ -732,7 +767,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         named_bar_sync(1, 256);
         if (!ep_ok[0]) return false;  // uniform for the 256 threads
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)b * 256u + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll
         for (int c = 0; c < 128 / CH; ++c) {
           if (c >= n_chunks) break;
@@ -759,7 +794,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         // this warp has read its part of the accumulator (wait::ld in sp_ld_chunk): it goes back to the MMA issuer
         tc_fence_before();
         __syncwarp();
-        if (lane == 0 && awaited(u)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
+        if (lane == 0 && awaited(it)) mbar_arrive_in_cta(tmem_empty(b), pair_cta0);
       }
       return true;
     });
@@ -804,6 +839,12 @@ bool residual_t_usable(const a3_handle* h, const GemmArgs& a) {
 // the weights and the output that stream through it, else 1.
 static int unit_group(int M, int K) { return (long long)M * K * 2 > (64ll << 20) ? 8 : 1; }
 
+// Two token tiles of n per unit on one stream of weights.  Just over 256 rows every weight goes to two units, and units that narrow
+// wait for their operands: 270 rows x 2 x (16 KiB of weights + 9 KiB of tokens) per k-block and CTA, 800 clocks for 576 of tensor time.
+// Together they take 16 + 18 KiB, 544 clocks, and each weight crosses to an SM once: SwiGLU of 270 rows (Qwen width) 67 -> 55 us.
+constexpr int SP_TWO_TILES_MAX = 160;  // tokens per tile: three accumulators in 512 columns
+static int two_tiles_per_kb(int n) { return 4 * n > 256 + 2 * n ? 4 * n : 256 + 2 * n; }
+
 struct SpTiling {
   int tiles, n;
 };
@@ -839,27 +880,44 @@ static bool split_allowed(const a3_handle* h) {
   return h->opt[A3_OPT_RESIDUAL_T] == 1 && h->opt[A3_OPT_QKV_T] == 1 && h->opt[A3_OPT_SWIGLU_PAIR] == 1 &&
          h->opt[A3_OPT_GEMM_TILING] == 0;
 }
-static int choose_slices(int M, int F, int K, int n_fblocks, int pairs, size_t part_bytes) {
+struct SpSlices {
+  int slices, tiles;  // tiles: token tiles per unit
+};
+static SpSlices choose_slices(int M, int F, int K, int n_fblocks, int pairs, size_t part_bytes) {
   const int tiles = cdiv(M, 256), n = cdiv(cdiv(M, tiles), 16) * 16, kt = K / TC_BK;
   const int per_kb = 2 * n > 256 + n ? 2 * n : 256 + n;
-  long long unsplit = (long long)kt * per_kb;
-  int best = 1;
+  long long least = (long long)kt * per_kb, least_two = least;
+  int two = 1;
+  SpSlices best{1, 1};
   for (int s = 2; s <= 16 && s * SP_SLICE_MIN_KB <= kt; ++s) {
     if ((size_t)s * M * F * 4 > part_bytes) break;
-    const long long cost = (long long)cdiv((long long)n_fblocks * tiles * s, pairs) * ((long long)cdiv(kt / SP_SUB, s) * SP_SUB * per_kb + 2000) +
-                           (long long)s * M * F * 8 / 3000 + 2000;
-    if (cost < unsplit) {
-      unsplit = cost;
-      best = s;
+    const long long sums = (long long)s * M * F * 8 / 3000 + 2000;
+    const long long cost = (long long)cdiv((long long)n_fblocks * tiles * s, pairs) * ((long long)cdiv(kt / SP_SUB, s) * SP_SUB * per_kb + 2000) + sums;
+    if (cost < least) {
+      least = cost;
+      best = SpSlices{s, 1};
+    }
+    if (tiles != 2 || n_fblocks * s > pairs) continue;  // two_tiles; one unit per pair: both accumulators of 256 columns are in use
+    const long long both = (long long)cdiv(kt, s) * two_tiles_per_kb(n) + 2000 + n * 20 + sums;
+    if (both < least_two) {
+      least_two = both;
+      two = s;
     }
   }
+  // A tenth is left out: slices twice as many cost more than their traffic.  Prefill (us), one tile per unit against two: Qwen-7B 272
+  // rows 4 739 / 4 588 (both five slices), 352 rows 5 342 / 5 232, 400 rows 5 938 / 5 921; Llama-8B (two slices against four) 272
+  // rows 5 200 / 5 231, 320 rows 5 486 / 5 547.
+  if (least_two * 10 < least * 9) best = SpSlices{two, 2};
   return best;
 }
-int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes) {
+int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes, int* tiles) {
+  *tiles = 1;
   if (!split_allowed(h) || h->opt[A3_OPT_GEMM_BN_RESIDUAL] != 0 || M <= 0 || K % (SP_SUB * TC_BK) || N % 32) return 1;
   const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2, blocks = cdiv(N, 4 * SP_FEAT);
   if (blocks * cdiv(M, 256) > pairs / 2) return 1;  // the pairs are busy with whole units
-  return choose_slices(M, N, K, blocks, pairs, part_bytes);
+  const SpSlices c = choose_slices(M, N, K, blocks, pairs, part_bytes);
+  *tiles = c.tiles;
+  return c.slices;
 }
 
 // Weights that nobody finds in L2 again: one token tile, so that the launch reads each of them once, and a stack of layers
@@ -874,13 +932,15 @@ static bool weights_once(const a3_handle* h, int tok_tiles) { return tok_tiles =
 // Ring depth and epilogue chunk of a launch: the widest chunk among those that leave the ring deepest (a stage more is 8 %
 // at 513 rows, where 32-token chunks leave three stages of 176 tokens and 8-token chunks four), but no deeper than a pair
 // has stages to run through.  Returns the dynamic shared memory.
-static int set_stages(SpParams& p, int epi, bool split) {
-  p.stage_bytes = SP_SUB * (SP_A_BYTES + (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
+static int set_stages(SpParams& p, int epi, bool split, int tt = 1) {
+  const int sub = SP_SUB / tt;
+  p.stage_bytes = sub * (SP_A_BYTES + tt * (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
+  p.slot_cols = tt == 1 || split ? 256 : SP_TWO_TILES_MAX;
   p.stages = 0;
-  const long long steps = (long long)cdiv(p.n_units, p.n_pairs) * (p.K / TC_BK / SP_SUB);
+  const long long steps = (long long)cdiv(p.n_units, p.n_pairs) * (p.K / TC_BK / sub);
   const int useful = steps < SP_MAX_STAGES ? (int)steps : SP_MAX_STAGES;
   int xch = 0;
-  for (int chunk = 32; chunk >= (epi == EPI_QKV ? 16 : 8); chunk /= 2) {
+  for (int chunk = 32; chunk >= (epi == EPI_QKV || tt == 2 ? 16 : 8); chunk /= 2) {
     const int x = split ? 0 : sp_xch_bytes(epi, chunk);
     int stages = (SP_SMEM_LIMIT - x - 256) / p.stage_bytes;
     if (stages > useful) stages = useful;
@@ -893,7 +953,7 @@ static int set_stages(SpParams& p, int epi, bool split) {
   return p.stages * p.stage_bytes + xch + 256;
 }
 
-int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st) {
+int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, int tiles, float* part, cudaStream_t st) {
   SpParams p{};
   p.M = a.M;
   p.K = a.K;
@@ -902,6 +962,7 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   p.n_fblocks = cdiv(p.F, 4 * SP_FEAT);
   p.tok_tiles = cdiv(a.M, 256);
   p.tok_n = cdiv(cdiv(a.M, p.tok_tiles), 16) * 16;
+  if (tiles == 2) p.tok_tiles = 1;
   p.k_slices = slices;
   p.early = a.early_weights;
   p.part = part;
@@ -909,18 +970,30 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float
   p.group = 1;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;
-  const int smem_bytes = set_stages(p, EPI_RESIDUAL, true);
+  const int smem_bytes = set_stages(p, EPI_RESIDUAL, true, tiles);
   CUtensorMap tX, tG;
-  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
-  A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB));
-  static SmemAttrOnce attr[2];
+  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB / tiles));
+  A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB / tiles));
+  static SmemAttrOnce attr[4];
   const bool once = weights_once(h, p.tok_tiles);
-  const auto kernel = once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true> : pair_t_kernel<EPI_RESIDUAL, true, 1, false>;
-  A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
+  const auto kernel = tiles == 2 ? (once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true, 2> : pair_t_kernel<EPI_RESIDUAL, true, 1, false, 2>)
+                                 : (once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true> : pair_t_kernel<EPI_RESIDUAL, true, 1, false>);
+  A3_TRY(smem_attr_once(attr[2 * (tiles - 1) + once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
   A3_CUDA(launch_pdl(kernel, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tG, tG, p));
   A3_LAUNCHED();
   return A3_OK;
+}
+
+// SwiGLU on two token tiles per unit: every unit costs half an epilogue more, which the third accumulator does not hide.  Prefill (us),
+// one tile per unit against two (Qwen-7B with the down projection's two tiles, see choose_slices): Qwen-7B 288 rows 4 705 / 4 378, 320
+// rows 4 934 / 4 709; Llama-8B, whose 112 feature blocks are two rounds for 1.5, 288 rows 5 152 / 5 063, 320 rows 5 390 / 5 368.  The
+// epilogue's chunks stay at 16 tokens or more: with 8, for the sake of one ring stage more, 320 rows gained nothing.
+static bool two_tiles(const a3_handle* h, int M, int K, int n_fblocks, int pairs, const SpTiling& til) {
+  const int n = cdiv(cdiv(M, 2), 16) * 16, kt = K / TC_BK;
+  if (M <= 256 || n > SP_TWO_TILES_MAX || h->opt[A3_OPT_GEMM_TILING] != 0) return false;
+  const int per_kb = 2 * til.n > 256 + til.n ? 2 * til.n : 256 + til.n;
+  return (long long)cdiv(n_fblocks, pairs) * (kt * two_tiles_per_kb(n) + 30 * n) < (long long)cdiv((long long)n_fblocks * til.tiles, pairs) * kt * per_kb;
 }
 
 template <int EPI>
@@ -933,8 +1006,9 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   const int sms = h->sm_count > 0 ? h->sm_count : 148;
   p.n_fblocks = cdiv(p.F, 2 * ROWS);
   const SpTiling til = choose_tiling(h, a.M, p.n_fblocks, sms / 2);
-  p.tok_tiles = til.tiles;
-  p.tok_n = til.n;
+  const int tt = EPI == EPI_SWIGLU && two_tiles(h, a.M, a.K, p.n_fblocks, sms / 2, til) ? 2 : 1;
+  p.tok_tiles = tt == 2 ? 1 : til.tiles;
+  p.tok_n = tt == 2 ? cdiv(cdiv(a.M, 2), 16) * 16 : til.n;
   p.n_units = p.n_fblocks * p.tok_tiles;
   p.group = unit_group(a.M, a.K);
   p.k_slices = 1;
@@ -943,16 +1017,19 @@ static int launch_pair_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st)
   p.C = a.C;
   p.ldc = a.ldc;
   p.status = h->dev_status;
-  const int smem_bytes = set_stages(p, EPI, false);
+  const int smem_bytes = set_stages(p, EPI, false, tt);
   CUtensorMap tX, tG, tU;
-  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB));
+  A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB / tt));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, ROWS, EPI == EPI_SWIGLU ? 1 : SP_SUB));
   if (EPI == EPI_SWIGLU) A3_TRY(make_tmap_kblocks(&tU, a.B2, p.F, a.K, ROWS, 1));
   else tU = tG;
-  static SmemAttrOnce attr[2];
+  static SmemAttrOnce attr[4];
   const bool once = weights_once(h, p.tok_tiles);
-  const auto kernel = once ? pair_t_kernel<EPI, false, 1, true> : pair_t_kernel<EPI, false, 1, false>;
-  A3_TRY(smem_attr_once(attr[once], h->device, kernel, SP_SMEM_LIMIT));
+  auto kernel = once ? pair_t_kernel<EPI, false, 1, true> : pair_t_kernel<EPI, false, 1, false>;
+  if constexpr (EPI == EPI_SWIGLU) {
+    if (tt == 2) kernel = once ? pair_t_kernel<EPI, false, 1, true, 2> : pair_t_kernel<EPI, false, 1, false, 2>;
+  }
+  A3_TRY(smem_attr_once(attr[2 * (tt - 1) + once], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, EPI == EPI_SWIGLU ? A3_K_GEMM_SWIGLU : A3_K_GEMM_RESIDUAL, st);
   A3_CUDA(launch_pdl(kernel, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tU, tU, p));
   A3_LAUNCHED();

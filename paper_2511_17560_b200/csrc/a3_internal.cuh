@@ -183,9 +183,10 @@ int gemm_swiglu_pair(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
 bool residual_t_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_residual_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
 // The same product of few rows, its k-loop cut into slices: fp32 partial sums [slices][M][N] for add_slices_rmsnorm.
-// residual_slices: how many slices suit the shape (1: use gemm_bf16), given room for part_bytes of partial sums.
-int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes);
-int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, float* part, cudaStream_t st);
+// residual_slices: how many slices suit the shape (1: use gemm_bf16), given room for part_bytes of partial sums, and how many token
+// tiles share a stream of weights.
+int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes, int* tiles);
+int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, int tiles, float* part, cudaStream_t st);
 // QKV projection (bias, RoPE, scatter in the epilogue) with one head per CTA of a pair
 bool qkv_t_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_qkv_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st);

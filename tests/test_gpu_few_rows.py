@@ -79,6 +79,27 @@ def test_layer_of_a_stack_beyond_l2(a3mod, M):
     layer_parity(a3mod, BEYOND_L2, M, seed=M + 2)
 
 
+# one layer that L2 holds; 38 feature blocks of SwiGLU, 8 of the down projection (38 ring stages, slices of 4 or 5)
+TWO_TILES = W.ModelShape("two_tiles", 1, 2048, 16, 4, 128, 4864, 32000, 5e5, 1e-5)
+
+
+@pytest.mark.parametrize("m", [BEYOND_L2, TWO_TILES], ids=lambda m: m.name)
+@pytest.mark.parametrize("M", [257, 289, 320, 321, 471])
+def test_two_token_tiles_on_one_stream_of_weights(a3mod, m, M):
+    """Just over 256 rows, up to 320 for SwiGLU and to 512 for the slices: the oracle's layer, and the gate/up product, whose sums
+    stay whole, bit for bit that of one tile per unit."""
+    layer_parity(a3mod, m, M, seed=M + 4)
+    eng, _, dev = make_engine(a3mod, m, seed=M, w_std=0.05)
+    g = torch.Generator(device=dev)
+    g.manual_seed(M)
+    x = torch.randn(M, m.d_model, device=dev, generator=g).bfloat16()
+    both = eng.swiglu_rows(0, x)
+    eng.set_option(a3mod.OPT_GEMM_TILING, 1)
+    assert torch.equal(both, eng.swiglu_rows(0, x))
+    assert eng.device_status() == 0
+    eng.close()
+
+
 # rows of more than 4 096 values: what the threads of the adding kernel do not keep in registers is read again; both of a layer's
 # residual products in two slices
 LONG_ROWS = W.ModelShape("long_rows", 1, 4224, 16, 4, 128, 2176, 32000, 5e5, 1e-5)
