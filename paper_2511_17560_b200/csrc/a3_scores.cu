@@ -16,7 +16,7 @@
 //   warp 0 (one lane)  TMA: the K tile of head g (two slots) and chunks of <= 256 packed question rows (two slots;
 //                      a 3-D box over q seen as [nq][Hq][D] lands as the packed K-major operand)
 //   warp 1 (one lane)  tcgen05.mma, accumulators double-buffered in tensor memory (2 x 256 columns)
-//   warps 2..5         one cache slot per thread: p = ex2(s * scale - lse), masked where slot > position, summed
+//   warps 2..9         two threads per cache slot: p = ex2(s * scale - lse), masked where slot > position, summed
 // scores_mma_kernel: the earlier warp-level mma.sync kernel, kept as the cross-check and for shapes the tcgen05
 // kernel does not take (more than 16 query heads per KV head, more than 4096 (row, head) pairs).
 #include <cuda.h>
@@ -180,7 +180,7 @@ scores_mma_kernel(const bf16* __restrict__ q, const int32_t* __restrict__ q_pos,
 }
 
 // ------------------------------------------------------------------ relevance scores on tcgen05
-constexpr int STC_THREADS = 192;
+constexpr int STC_ACC_THREADS = 256, STC_THREADS = 64 + STC_ACC_THREADS;
 constexpr int STC_MAX_PAIRS = 4096;  // (question row, query head) pairs whose log-sum-exps fit the shared-memory table
 
 struct StcParams {
@@ -195,13 +195,13 @@ struct StcParams {
   uint32_t* status;
 };
 
-// dynamic shared memory: [K slot 0][K slot 1][Q slot 0][Q slot 1][l2 table][position table][barriers]
+// dynamic shared memory: [K slot 0][K slot 1][Q slot 0][Q slot 1][l2 table][position table][barriers][sums of the second halves]
 template <int D>
 struct StcLayout {
   static constexpr int K_SLOT = (D / 64) * 128 * 128;  // [128 slots][64] bf16 sub-tiles
   __host__ __device__ static constexpr int q_slot(int n_cols) { return (D / 64) * n_cols * 128; }
   static constexpr int TAB_BYTES = STC_MAX_PAIRS * 4 + STC_MAX_PAIRS * 4;  // l2[Hkv][rows_g], position per packed row
-  static int smem_bytes(int n_cols) { return 2 * K_SLOT + 2 * q_slot(n_cols) + TAB_BYTES + 256 + 1024; }
+  static int smem_bytes(int n_cols) { return 2 * K_SLOT + 2 * q_slot(n_cols) + TAB_BYTES + 256 + 2 * 128 * 4 + 1024; }
 };
 
 template <int D>
@@ -217,7 +217,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   const int rows_g = p.nq * G;     // packed question rows of one KV head
   const int q_slot = L::q_slot(N);
   const uint32_t k_off = 0, q_off = 2 * L::K_SLOT, tab_off = q_off + 2 * q_slot, bar_off = tab_off + L::TAB_BYTES;
-  float* l2tab = reinterpret_cast<float*>(base_ptr + tab_off);                  // [Hkv][rows_g]: lse * log2(e)
+  float* l2tab = reinterpret_cast<float*>(base_ptr + tab_off);                  // [KV heads of this CTA][rows_g]: lse * log2(e)
   int* postab = reinterpret_cast<int*>(base_ptr + tab_off + STC_MAX_PAIRS * 4);  // [rows_g]: position of the packed row
   const uint32_t bars = base + bar_off;
   auto k_full = [&](int s) { return bars + 8u * s; };
@@ -226,8 +226,10 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   auto q_empty = [&](int s) { return bars + 8u * (6 + s); };
   auto t_full = [&](int b) { return bars + 8u * (8 + b); };
   auto t_empty = [&](int b) { return bars + 8u * (10 + b); };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + bar_off + 8 * 12);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + bar_off + 8 * 12 + 8);
+  auto x_full = [&](int quarter, int par) { return bars + 8u * (12 + 2 * quarter + par); };
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + bar_off + 8 * 20);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + bar_off + 8 * 20 + 8);
+  float* xch = reinterpret_cast<float*>(base_ptr + bar_off + 256);  // [2][128 slots]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int key0 = blockIdx.x * 128;
@@ -241,8 +243,9 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       mbar_init(q_full(i), 1);
       mbar_init(q_empty(i), 1);
       mbar_init(t_full(i), 1);
-      mbar_init(t_empty(i), 4);  // one arrival per accumulating warp
+      mbar_init(t_empty(i), 8);  // one arrival per accumulating warp
     }
+    for (int i = 0; i < 8; ++i) mbar_init(x_full(i >> 1, i & 1), 32);
     abort_flag[0] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -257,14 +260,6 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();  // everything above overlapped the previous kernel's tail; the log-sum-exps and K are read below
   pdl_launch_dependents();
-  // tables: log-sum-exps in the exp2 domain in packed order per KV head, and each packed row's position
-  for (int i = threadIdx.x; i < p.Hkv * rows_g; i += STC_THREADS) {
-    const int g = i / rows_g, r = i - g * rows_g;
-    l2tab[i] = p.lse[(size_t)(r / G) * p.Hq + g * G + r % G] * ATC_LOG2E;
-  }
-  for (int r = threadIdx.x; r < rows_g; r += STC_THREADS) postab[r] = min(p.q_pos[r / G], p.kv_len - 1);
-  __syncthreads();
-
   if (warp == 0) {
     // ---------------- TMA producer
     if (lane == 0) {
@@ -321,10 +316,21 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       }
     }
   } else {
-    // ---------------- accumulation: one cache slot per thread
-    const int quarter = warp & 3;
-    const int key = key0 + quarter * 32 + lane;
+    // ---------------- accumulation: two threads per cache slot, each with every second group of 32 packed rows; the first adds the
+    // second's sum (through shared memory) to its own.  The exponential unit takes 1 024 clocks for 128 rows of a tile; one warp per
+    // scheduler needed 1 860 for them.  With this and the tables built under the first copies, one layer's eviction of 5 120
+    // candidates, votes to gather, 18.8 -> 16.9 us together with the selection's changes.
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const int row = quarter * 32 + lane, key = key0 + row;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    // tables, while the first tiles are on their way: log-sum-exps in the exp2 domain in packed order per KV head, and each packed
+    // row's position
+    for (int i = threadIdx.x - 64; i < (g_end - g_begin) * rows_g; i += STC_ACC_THREADS) {
+      const int gi = i / rows_g, r = i - gi * rows_g;
+      l2tab[i] = p.lse[(size_t)(r / G) * p.Hq + (g_begin + gi) * G + r % G] * ATC_LOG2E;
+    }
+    for (int r = threadIdx.x - 64; r < rows_g; r += STC_ACC_THREADS) postab[r] = min(p.q_pos[r / G], p.kv_len - 1);
+    asm volatile("bar.sync 1, %0;" ::"n"(STC_ACC_THREADS) : "memory");  // nobody has waited for a tile yet
     // question rows sit behind the context, so only the key tiles that reach past the first question row need a mask
     const bool need_mask = key0 + 127 > postab[0];
     const bool vec_ok = (rows_g & 3) == 0;  // the table rows of every head start on a 16-byte boundary
@@ -334,7 +340,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     bool ok = true;
     for (int g = g_begin; g < g_end && ok; ++g) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const float* l2g = l2tab + g * rows_g;
+      const float* l2g = l2tab + (g - g_begin) * rows_g;
       for (int c = 0; c < p.n_chunks; ++c, ++st) {
         const int b = st & 1;
         ok = __all_sync(0xffffffffu, mbar_wait(t_full(b), (st >> 1) & 1, abort_flag, p.status));
@@ -344,7 +350,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         const int n_valid = min(N, rows_g - r0);  // packed rows beyond the question are zero-filled operands: skipped
         const int n32 = (n_valid + 31) >> 5;
 #pragma unroll 1
-        for (int cc = 0; cc < n32; ++cc) {
+        for (int cc = half; cc < n32; cc += 2) {
           float x[32];
           ld32(tmem_base + b * 256 + lane_addr + cc * 32, x);
           wait_ld();
@@ -384,16 +390,28 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             }
           }
         }
-        // this warp has read its part of the accumulator: hand it back to the MMA issuer
         fence_before();
+        float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        if (c == p.n_chunks - 1) {
+          // A slot of xch is written again two heads later, behind an accumulator that waits for all warps' arrivals below.
+          const int par = (g - g_begin) & 1;
+          if (half == 1) {
+            xch[par * 128 + row] = sum;
+            mbar_arrive(x_full(quarter, par));
+          } else {
+            ok = __all_sync(0xffffffffu, mbar_wait(x_full(quarter, par), ((g - g_begin) >> 1) & 1, abort_flag, p.status));
+            if (!ok) break;
+            sum += xch[par * 128 + row];
+            total += sum;
+            if (p.per_head && key < p.kv_len) p.per_head[(size_t)g * p.kv_len + key] = cand ? sum : 0.f;
+          }
+        }
+        // this warp has read its part of the accumulator: hand it back to the MMA issuer
         __syncwarp();
         if (lane == 0) mbar_arrive(t_empty(b));
       }
-      const float head_total = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      total += head_total;
-      if (p.per_head && key < p.kv_len) p.per_head[(size_t)g * p.kv_len + key] = cand ? head_total : 0.f;
     }
-    if (ok && p.scores && key < p.kv_len) p.scores[key] = cand ? total : 0.f;
+    if (ok && half == 0 && p.scores && key < p.kv_len) p.scores[key] = cand ? total : 0.f;
   }
   fence_before();
   __syncthreads();

@@ -1,11 +1,11 @@
 // Selection Re = top_p(s) (Eq. 3): block-radix select on the order-preserving integer image of the fp32 scores.
 // One CTA per score array.  The scores are read from global memory once, as integer keys into registers (up to 8 192, see
-// topk_regs) or shared memory (up to TK_SMEM_KEYS of them; longer arrays are re-read from global memory in every pass).  Four 8-bit histogram passes
+// topk_regs) or shared memory (up to TK_SMEM_KEYS of them; longer arrays are re-read from global memory in every pass).  Up to four 8-bit histogram passes
 // find the key of the k-th largest score: the warps count into TK_HISTS private histograms (a warp whose lanes all
 // hold the same digit - the rule in the first pass, since the scores of one request share their leading bits - adds
 // 32 with one instruction instead of serialising 32 atomics on one bin), the histograms are summed, and the bin of
 // the k-th element is found by a parallel suffix sum over the 256 bins.  The emission is
-// ordered: every warp owns a contiguous span of the slots, counts what it will emit, and after one exchange of the
+// ordered: every warp (in registers: every thread) owns a contiguous span of the slots, counts what it will emit, and after one exchange of the
 // 32 warp totals writes every slot above the threshold key plus, in slot order, as many slots equal to it as are
 // still needed.  The result is exact: ties go to the lower slot and the output is ascending.
 #include "a3_internal.cuh"
@@ -23,9 +23,9 @@ __device__ __forceinline__ uint32_t score_key(float s) {
 }
 
 // Sums the private histograms and finds the bin of the element of rank `remaining` (1-based, from the top); the caller's
-// prefix and remaining move on to that bin.  All threads.
-__device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned int* warp_tot, unsigned int* s_prefix,
-                                         unsigned int* s_remaining, int shift, uint32_t& prefix, unsigned int& remaining) {
+// prefix, remaining and count (of the keys in the bin) move on to that bin.  All threads.
+__device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned int* warp_tot, unsigned int* s_prefix, unsigned int* s_remaining,
+                                         unsigned int* s_count, int shift, uint32_t& prefix, unsigned int& remaining, unsigned int& count) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned int v = 0;
   if (tid < 256) {
@@ -43,66 +43,98 @@ __device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned in
   __syncthreads();
   if (tid < 256) {
     unsigned int above = 0;  // elements in the bins of higher warps
-    for (int w = warp + 1; w < 8; ++w) above += warp_tot[w];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) above += w > warp ? warp_tot[w] : 0;
     const unsigned int next = __shfl_down_sync(0xffffffffu, v, 1);
     const unsigned int S_d = v + above, S_next = lane == 31 ? above : next + above;  // S[d], S[d + 1]
     if (S_d >= remaining && S_next < remaining) {
       *s_prefix = prefix | ((uint32_t)tid << shift);
       *s_remaining = remaining - S_next;
+      *s_count = S_d - S_next;
     }
   }
   __syncthreads();
   prefix = *s_prefix;
   remaining = *s_remaining;
+  count = *s_count;
 }
 
-// Up to KPT x 1 024 candidates, which is every request of a few thousand tokens: a thread keeps its keys (slots tid, tid +
-// 1 024, ...) in registers through all passes.  With half_pool the keys are of the running maximum over the neighbouring
-// candidates, taken from a copy of the scores in shared memory.  Bound by the chain of block barriers, three per pass: back
-// to back 5 120 candidates take 7.6 us where the passes over shared memory below took 10.6, 900 take 5.0 instead of 7.0.
+// Up to KPT x 1 024 candidates, which is every request of a few thousand tokens: a thread keeps the keys of KPT consecutive slots in
+// registers, read once through shared memory.  With half_pool the keys are of the running maximum over the neighbouring candidates.
+// Bound by the chain of block barriers, three per pass, hence: as soon as the bin of the k-th largest key holds TK_LIST keys or
+// fewer, usually after two passes, these are listed and ranked by key and slot at once; consecutive slots make the emission one
+// scan over threads and let neighbouring windows share their middle.  With four passes always, a window per key and a count per warp
+// and round, the selection of 5 120 candidates at width 7 took 14 700 clocks: 1 050 for the loads, 2 600 the windows, 7 700 the
+// passes, 2 650 the emission.  Back to back, before and now (us): 300 candidates 4.2 / 2.7, 900 4.1 / 2.6, 2 000 5.6 / 3.7, 3 000 5.8 / 4.7,
+// 5 120 7.2 / 5.7, 8 192 9.2 / 8.3.
+constexpr int TK_LIST = 128;  // eight threads rank one key
+template <int KPT>
+__host__ __device__ constexpr int topk_at(int i) {  // place of slot i in shared memory: a thread's slots on banks of their own
+  return KPT % 2 == 0 ? i + i / KPT : i;
+}
 template <int KPT>
 __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __restrict__ raw, int cand_begin, int n, int k, int half_pool,
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
   __shared__ unsigned int whist[2][TK_HISTS][256];  // passes alternate: one is cleared while the other counts
-  __shared__ unsigned int warp_tot[8];
-  __shared__ unsigned int s_prefix, s_remaining;
-  __shared__ unsigned int cnt[2][KPT * TK_WARPS];  // greater-than and equal candidates of (round, warp), in slot order
+  __shared__ unsigned int warp_tot[TK_WARPS];
+  __shared__ unsigned int s_prefix, s_remaining, s_count, s_listed;
+  __shared__ uint32_t list_key[TK_LIST], s_key;
+  __shared__ int list_slot[TK_LIST], s_slot;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i0 = tid * KPT;
   float v[KPT];
 #pragma unroll
   for (int j = 0; j < KPT; ++j) v[j] = tid + j * TK_THREADS < n ? __ldcg(s + tid + j * TK_THREADS) : 0.f;
   for (int i = tid; i < TK_HISTS * 256; i += TK_THREADS) (&whist[0][0][0])[i] = 0;
-  if (half_pool > 0) {
+  if (tid == 0) s_listed = 0;
+  if (KPT > 1 || half_pool > 0) {
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
-      if (tid + j * TK_THREADS < n) raw[tid + j * TK_THREADS] = v[j];
+      if (tid + j * TK_THREADS < n) raw[topk_at<KPT>(tid + j * TK_THREADS)] = v[j];
     __syncthreads();
+    const float none = __int_as_float(0x7fffffff);  // fmaxf passes over NaN
+    auto get = [&](int i) { return i >= 0 && i < n ? raw[topk_at<KPT>(i)] : none; };
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const int i = tid + j * TK_THREADS;
-      if (i < n)
-        for (int t = max(0, i - half_pool); t <= min(n - 1, i + half_pool); ++t) v[j] = fmaxf(v[j], raw[t]);
+    for (int j = 0; j < KPT; ++j) v[j] = i0 + j < n ? raw[topk_at<KPT>(i0 + j)] : 0.f;
+    if (2 * half_pool + 1 >= KPT && half_pool > 0) {
+      // what all windows of the thread have in common, then what those before and those behind have besides
+      float mid = none, run = none;
+      for (int i = i0 + KPT - 1 - half_pool; i <= i0 + half_pool; ++i) mid = fmaxf(mid, get(i));
+#pragma unroll
+      for (int j = KPT - 2; j >= 0; --j) {
+        run = fmaxf(run, get(i0 + j - half_pool));
+        v[j] = fmaxf(v[j], run);
+      }
+      run = mid;
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) {
+        if (j > 0) run = fmaxf(run, get(i0 + j + half_pool));
+        v[j] = fmaxf(v[j], run);
+      }
+    } else if (half_pool > 0) {
+#pragma unroll
+      for (int j = 0; j < KPT; ++j)
+        for (int i = i0 + j - half_pool; i <= i0 + j + half_pool; ++i) v[j] = fmaxf(v[j], get(i));
     }
   }
   uint32_t key[KPT];
   bool nonfinite = false;
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    const bool live = tid + j * TK_THREADS < n;
-    nonfinite = nonfinite || (live && !(fabsf(v[j]) <= 3.0e38f));
+    nonfinite = nonfinite || (i0 + j < n && !(fabsf(v[j]) <= 3.0e38f));
     key[j] = score_key(v[j]);
   }
   if (nonfinite) atomicOr(status, A3_DEV_NONFINITE_SCORE);
   uint32_t prefix = 0, mask = 0;
-  unsigned int remaining = (unsigned int)k;
+  unsigned int remaining = (unsigned int)k, count = (unsigned int)n;  // keys with this prefix, and how many of them are taken
   __syncthreads();
 #pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
+  for (int pass = 0; pass < 4 && count > TK_LIST; ++pass) {
     const int shift = 24 - 8 * pass;
     unsigned int* mine = whist[pass & 1][warp % TK_HISTS];
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      const bool in = tid + j * TK_THREADS < n && (key[j] & mask) == prefix;
+      const bool in = i0 + j < n && (key[j] & mask) == prefix;
       if (!__any_sync(0xffffffffu, in)) continue;  // the rule behind the first passes
       const uint32_t digit = in ? (key[j] >> shift) & 255u : 0xFFFFFFFFu;
       const uint32_t first = __shfl_sync(0xffffffffu, digit, 0);
@@ -114,48 +146,63 @@ __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __
     }
     for (int i = tid; i < TK_HISTS * 256; i += TK_THREADS) (&whist[(pass & 1) ^ 1][0][0])[i] = 0;
     __syncthreads();
-    topk_bin(whist[pass & 1], warp_tot, &s_prefix, &s_remaining, shift, prefix, remaining);
+    topk_bin(whist[pass & 1], warp_tot, &s_prefix, &s_remaining, &s_count, shift, prefix, remaining, count);
     mask |= 255u << shift;
   }
-  // ordered emission
+  // taken: keys above `prefix`, and of those equal to it the `remaining` lowest slots - or, listed, exactly those up to a key and slot
+  const bool listed = count <= TK_LIST;
+  if (listed) {
 #pragma unroll
-  for (int j = 0; j < KPT; ++j) {
-    const bool live = tid + j * TK_THREADS < n;
-    const unsigned int bgt = __ballot_sync(0xffffffffu, live && key[j] > prefix), beq = __ballot_sync(0xffffffffu, live && key[j] == prefix);
-    if (lane == 0) {
-      cnt[0][j * TK_WARPS + warp] = __popc(bgt);
-      cnt[1][j * TK_WARPS + warp] = __popc(beq);
-    }
-  }
-  __syncthreads();
-  if (warp < 2) {  // exclusive prefix sums, warp 0 the greater ones, warp 1 the equal ones
-    unsigned int run = 0;
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const unsigned int c = cnt[warp][j * TK_WARPS + lane];
-      unsigned int x = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int t = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += t;
+    for (int j = 0; j < KPT; ++j)
+      if (i0 + j < n && (key[j] & mask) == prefix) {
+        const unsigned int at = atomicAdd(&s_listed, 1u);
+        list_key[at] = key[j];
+        list_slot[at] = i0 + j;
       }
-      cnt[warp][j * TK_WARPS + lane] = run + x - c;
-      run += __shfl_sync(0xffffffffu, x, 31);
+    __syncthreads();
+    const unsigned int c = tid >> 3;  // 1 024 threads: TK_LIST keys
+    unsigned int better = 0;
+    const uint32_t my_key = c < count ? list_key[c] : 0;
+    const int my_slot = c < count ? list_slot[c] : 0;
+    for (unsigned int t = tid & 7; t < count; t += 8) better += list_key[t] > my_key || (list_key[t] == my_key && list_slot[t] < my_slot);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) better += __shfl_xor_sync(0xffffffffu, better, o);
+    if (c < count && better == remaining - 1 && (tid & 7) == 0) {
+      s_key = my_key;
+      s_slot = my_slot;
     }
+    __syncthreads();
+    prefix = s_key;
   }
-  __syncthreads();
-  const unsigned int lt_mask = (1u << lane) - 1u;
+  const int last_slot = listed ? s_slot : 0;
+  // ordered emission: one scan of the counts, taken ones in the low half of the word and equal keys that wait for their turn in the high
+  unsigned int mine = 0;
+  bool gt[KPT], eq[KPT];
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    const int i = tid + j * TK_THREADS;
-    const bool gt = i < n && key[j] > prefix, eq = i < n && key[j] == prefix;
-    const unsigned int bgt = __ballot_sync(0xffffffffu, gt), beq = __ballot_sync(0xffffffffu, eq);
-    const unsigned int my_gt = cnt[0][j * TK_WARPS + warp] + __popc(bgt & lt_mask);
-    const unsigned int my_eq = cnt[1][j * TK_WARPS + warp] + __popc(beq & lt_mask);
-    if (gt || (eq && my_eq < remaining)) {
+    const bool live = i0 + j < n;
+    gt[j] = live && (key[j] > prefix || (listed && key[j] == prefix && i0 + j <= last_slot));
+    eq[j] = live && !listed && key[j] == prefix;
+    mine += (gt[j] ? 1u : 0u) + (eq[j] ? 0x10000u : 0u);
+  }
+  unsigned int upto = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int t = __shfl_up_sync(0xffffffffu, upto, o);
+    if (lane >= o) upto += t;
+  }
+  if (lane == 31) warp_tot[warp] = upto;
+  __syncthreads();
+  const unsigned int before = upto - mine + __reduce_add_sync(0xffffffffu, lane < warp ? warp_tot[lane] : 0u);
+  unsigned int my_gt = before & 0xFFFFu, my_eq = before >> 16;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    if (gt[j] || (eq[j] && my_eq < remaining)) {
       const unsigned int o = my_gt + (my_eq < remaining ? my_eq : remaining);
-      if (o < (unsigned int)k) idx_out[o] = cand_begin + i;
+      if (o < (unsigned int)k) idx_out[o] = cand_begin + i0 + j;
     }
+    my_gt += gt[j] ? 1 : 0;
+    my_eq += eq[j] ? 1 : 0;
   }
 }
 
@@ -164,7 +211,7 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
                                           int32_t* __restrict__ idx_out, uint32_t* status) {
   __shared__ unsigned int whist[TK_HISTS][256];
   __shared__ unsigned int warp_tot[8];
-  __shared__ unsigned int s_prefix, s_remaining;
+  __shared__ unsigned int s_prefix, s_remaining, s_count;
   __shared__ unsigned int warp_gt[TK_WARPS], warp_eq[TK_WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // past L1: this CTA may have become resident while the kernel that writes the scores was still running
@@ -182,6 +229,7 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
 
   // ---- radix select: after the loop `prefix` is the key of the k-th largest element
   uint32_t prefix = 0, mask = 0;
+  unsigned int count;
   unsigned int remaining = (unsigned int)k;  // rank (1-based, from the top) inside the current bucket
   const int n_round = (n + 31) & ~31;        // whole warps walk the array, so that the lanes can vote together
   for (int shift = 24; shift >= 0; shift -= 8) {
@@ -202,7 +250,7 @@ __device__ __forceinline__ void topk_body(const float* __restrict__ s, uint32_t*
       }
     }
     __syncthreads();
-    topk_bin(whist, warp_tot, &s_prefix, &s_remaining, shift, prefix, remaining);
+    topk_bin(whist, warp_tot, &s_prefix, &s_remaining, &s_count, shift, prefix, remaining, count);
     mask |= 255u << shift;
   }
   // `remaining` = how many elements equal to the threshold key are taken (lowest slots first)
@@ -274,21 +322,20 @@ static int launch_topk(const a3_handle* h, const float* scores, size_t score_str
     return launch_pdl(kernel, dim3(batches), dim3(TK_THREADS), smem, st, scores, cand_begin, n, k, idx_out, h->dev_status, score_stride, idx_stride,
                       in_smem, half_pool, tail_begin, tail);
   };
-  const size_t raw = half_pool > 0 ? (size_t)n * 4 : 0;
-  // 0.7 us per key and thread, hence instances of one, three, five and eight keys (back to back 900 candidates 5.0 us, 5 120 7.6,
-  // 8 192 9.9): the smallest that holds the candidates.  Those in between would save up to 1.5 us more (5 121 candidates take 9.1).
+  // Time grows with the keys per thread (back to back 900 candidates 2.6 us, 3 000 4.7, 5 120 5.7, 8 192 8.3), hence instances of one,
+  // three, five and eight: the smallest that holds the candidates.
   if (n <= TK_THREADS) {
-    A3_CUDA(go(topk_select_kernel<1>, raw));
+    A3_CUDA(go(topk_select_kernel<1>, half_pool > 0 ? (size_t)n * 4 : 0));
   } else if (n <= 3 * TK_THREADS) {
-    A3_CUDA(go(topk_select_kernel<3>, raw));
+    A3_CUDA(go(topk_select_kernel<3>, (size_t)n * 4));
   } else if (n <= 5 * TK_THREADS) {
     static SmemAttrOnce attr5;
     A3_TRY(smem_attr_once(attr5, h->device, topk_select_kernel<5>, 5 * TK_THREADS * 4));
-    A3_CUDA(go(topk_select_kernel<5>, raw));
+    A3_CUDA(go(topk_select_kernel<5>, (size_t)n * 4));
   } else if (n <= 8 * TK_THREADS) {
     static SmemAttrOnce attr8;
-    A3_TRY(smem_attr_once(attr8, h->device, topk_select_kernel<8>, 8 * TK_THREADS * 4));
-    A3_CUDA(go(topk_select_kernel<8>, raw));
+    A3_TRY(smem_attr_once(attr8, h->device, topk_select_kernel<8>, topk_at<8>(8 * TK_THREADS) * 4));
+    A3_CUDA(go(topk_select_kernel<8>, (size_t)topk_at<8>(n) * 4));
   } else {
     static SmemAttrOnce attr;
     A3_TRY(smem_attr_once(attr, h->device, topk_select_kernel<0>, TK_SMEM_KEYS * 4));
@@ -318,13 +365,11 @@ int a3::topk_rows(const a3_handle* h, const float* scores, int cand_begin, int c
   return launch_topk(h, scores, 0, 1, cand_begin, cand_end - cand_begin, k, 0, tail_begin, tail, idx_out, 0, st);
 }
 
-// Pooling inside the selection saves a launch (2.5 us) and costs every thread its keys x the width in shared-memory reads, in
-// the one CTA of a head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, inside against
-// apart (us): 2 000 candidates 17.1 / 19.7 at width 7, 18.7 / 20.2 at 63, 20.7 / 21.6 at 127, 24.8 / 22.6 at 255; 5 120
-// candidates 21.8 / 24.3 at 7, 24.3 / 24.3 at 45, 25.9 / 24.3 at 63; 8 192 candidates 25.9 / 27.4 at 7, 26.9 / 27.4 at 21, 27.9 /
-// 27.4 at 31.  The line is where the two meet, within half a microsecond.  Candidates that do not fit the registers would read
-// their window from global memory, which loses at every width (12 000 candidates 39.2 / 38.7 at 3, 32 768 79.1 / 70.9 at 7,
-// 215 / 82 at 255).
+// Pooling inside the selection saves a launch (2.5 us) and costs every thread its window in shared-memory reads, in the one CTA of a
+// head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, on either side of the line (us): 5 120
+// candidates 16.9 at width 7 and 18.0 at 45 inside, 19.3 at 63 and 20.1 at 129 apart; 2 000 candidates 12.1 at 7, 15.1 at 63 and 16.1
+// at 127 inside, 19.2 at 255 apart; 8 192 candidates 21.4 at 21 and 22.4 at 31 inside, 23.0 at 63 apart.  Candidates that do not fit
+// the registers would read their window from global memory, which loses at every width (32 768 79.1 / 70.9 at 7, 215 / 82 at 255).
 bool a3::topk_can_pool(int n_cand, int pool) { return n_cand <= 8 * TK_THREADS && (long long)n_cand * pool <= 250 * TK_THREADS; }
 
 int a3::topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,

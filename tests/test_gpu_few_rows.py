@@ -192,6 +192,23 @@ def test_topk_at_the_register_sizes(a3mod, n):
     eng.close()
 
 
+@pytest.mark.parametrize("n,near", [(1, 1), (128, 128), (129, 129), (3000, 128), (3000, 129), (8192, 127)])
+def test_topk_threshold_among_few_keys(a3mod, n, near):
+    """`near` keys that agree in their first 16 bits, some of them equal, around the threshold: what is ranked in a list and what is not."""
+    eng, _, dev = make_engine(a3mod, W.TINY)
+    rng = np.random.default_rng(n + near)
+    s = rng.uniform(2.0, 3.0, size=n).astype(np.float32) * rng.choice([1.0, 0.01], size=n).astype(np.float32)
+    at = rng.permutation(n)[:near]
+    s[at] = 1.0 + rng.integers(0, 2000, size=near).astype(np.float32) * 2.0 ** -23
+    above = int((s >= 2.0).sum())
+    for k in {max(above, 1), above + 1, above + near // 2, above + near}:
+        if 0 < k <= n:
+            got = eng.topk_select(torch.from_numpy(s).to(dev), 0, n, k).cpu().numpy()
+            assert got.tolist() == O.topk_select(s.astype(np.float64), 0, n, k).tolist(), k
+    assert eng.device_status() == 0
+    eng.close()
+
+
 @pytest.mark.parametrize("n_ctx,pool", [(900, 3), (3073, 7), (5120, 5), (8200, 7)])
 def test_pooled_selection_of_the_eviction(a3mod, n_ctx, pool):
     """Pooling inside the selection, and (8 200 candidates) by the kernel of its own."""
