@@ -21,6 +21,15 @@ struct FtBest {
 // total order: larger value first, then lower id; NaN never wins
 __device__ __forceinline__ bool ft_better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
 
+// The ticket must be zero when it is drawn from; the kernel leaves it at zero, but the workspace is the caller's and may have been used
+// for something else in between.  The projection starts beside this launch (programmatic dependent launch), which itself comes after
+// everything queued before, and waits for it only before it draws.  In place of a memset between the two, and with enter_rows beside position
+// recovery: request of 369 tokens on a small model 146.6 -> 144.7 us.
+__global__ void clear_ticket_kernel(unsigned int* ticket) {
+  pdl_launch_dependents();
+  *ticket = 0;
+}
+
 __global__ void __launch_bounds__(FT_THREADS, 2)
 first_token_kernel(const bf16* __restrict__ x, const bf16* __restrict__ gain, const uint4* __restrict__ w, int d, int vocab,
                    float eps, float* __restrict__ logits, int32_t* __restrict__ token, FtBest* __restrict__ cand,
@@ -111,6 +120,7 @@ first_token_kernel(const bf16* __restrict__ x, const bf16* __restrict__ gain, co
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    pdl_wait();  // the ticket is clear
     FtBest b = sbest[0];
     for (int i = 1; i < FT_WARPS; ++i)
       if (ft_better(sbest[i].v, sbest[i].i, b.v, b.i)) b = sbest[i];
@@ -165,9 +175,6 @@ extern "C" int a3_first_token(const a3_handle* h, const void* x_row, const void*
   cudaStream_t st = (cudaStream_t)stream;
   unsigned int* ticket = (unsigned int*)ws;
   FtBest* cand = (FtBest*)((char*)ws + 256);
-  // The ticket must be zero when the kernel starts; the kernel leaves it at zero, but the workspace is the
-  // caller's and may have been used for something else in between.
-  A3_CUDA(cudaMemsetAsync(ticket, 0, 4, st));
   const size_t smem = (size_t)d * 4;
   if (smem > 48 * 1024) A3_CUDA(cudaFuncSetAttribute(first_token_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
   int grid = h->sm_count * 2;
@@ -175,8 +182,10 @@ extern "C" int a3_first_token(const a3_handle* h, const void* x_row, const void*
   if (grid > need) grid = need;
   {
     ProfScope prof(h, A3_K_FIRST_TOKEN, st);
-    first_token_kernel<<<grid, FT_THREADS, smem, st>>>((const bf16*)x_row, (const bf16*)final_norm, (const uint4*)lm_head, d, vocab,
-                                                       h->m.rms_eps, logits_out, token_out, cand, ticket, h->dev_status);
+    clear_ticket_kernel<<<1, 1, 0, st>>>(ticket);
+    A3_LAUNCHED();
+    A3_CUDA(launch_pdl(first_token_kernel, dim3(grid), dim3(FT_THREADS), smem, st, (const bf16*)x_row, (const bf16*)final_norm, (const uint4*)lm_head,
+                       d, vocab, h->m.rms_eps, logits_out, token_out, cand, ticket, h->dev_status));
   }
   return launched();
 }

@@ -142,9 +142,9 @@ int add_slices_rmsnorm(const a3_handle* h, bf16* x, const float* part, int slice
                        cudaStream_t st);
 
 // Rows entering a layer: x_dst[r] = src[rows ? rows[r] : r]; out[r] = rmsnorm of it * gain (gain null: no norm); pos_out[r] =
-// pos_base + r (null: no positions).
+// pos_base + r (null: no positions).  beside: directly behind a launch of a3_rope_rerotate, which need not have finished.
 int enter_rows(const a3_handle* h, const bf16* src, int n_src, const int32_t* rows, int M, const bf16* gain, float eps, int d, bf16* x_dst,
-               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st);
+               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st, bool beside = false);
 
 enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_SWIGLU = 1, EPI_QKV = 2 };
 

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(RR_THREADS)
 rerotate_kernel(const a3_chunk_ref* __restrict__ chunks, char* __restrict__ kf, char* __restrict__ vf,
                 unsigned long long layer_stride, int kv_len, int max_chunk_len, int layer_begin, int row_elems, int tok_per_cta,
                 const float2* __restrict__ tab, int max_pos, uint32_t* status) {
+  pdl_launch_dependents();  // see enter_rows_kernel
   const a3_chunk_ref ch = chunks[blockIdx.y];
   const int t0 = blockIdx.x * tok_per_cta;
   if (ch.len < 0 && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, A3_DEV_BAD_POSITION);
@@ -417,11 +418,10 @@ int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps,
 // Row r of a request on its way into a layer: x_dst[r] = src[rows ? rows[r] : r], out[r] = RMSNorm of it (gain given), and
 // pos_out[r] = pos_base + r.  What a copy, an index kernel, a gather and a norm would each launch for; a thread keeps its
 // vectors in registers between the two stores.  Rows out of range are flagged and skipped.
-__global__ void __launch_bounds__(RN_THREADS)
-enter_rows_kernel(const uint4* __restrict__ src, int n_src, const int32_t* __restrict__ rows, const uint4* __restrict__ gain, float eps,
-                  int row_vecs, uint4* __restrict__ x_dst, uint4* __restrict__ out, int32_t* __restrict__ pos_out, int pos_base, uint32_t* status) {
-  pdl_wait();
-  pdl_launch_dependents();
+// beside: the launch before this one is position recovery, whose results nothing here touches and which itself comes after everything
+// queued earlier.  The two run side by side, and this one ends after the other: the launches that follow wait for both through it.
+__device__ __forceinline__ void enter_row(const uint4* src, int n_src, const int32_t* rows, const uint4* __restrict__ gain, float eps, int row_vecs,
+                                          uint4* x_dst, uint4* out, int32_t* pos_out, int pos_base, uint32_t* status) {
   uint4 gv[RN_VPT];
 #pragma unroll
   for (int i = 0; i < RN_VPT; ++i) {
@@ -488,12 +488,22 @@ enter_rows_kernel(const uint4* __restrict__ src, int n_src, const int32_t* __res
   for (int idx = threadIdx.x + RN_VPT * RN_THREADS; idx < row_vecs; idx += RN_THREADS) scaled(__ldcg(xr + idx), __ldg(gain + idx), idx);
 }
 
+__global__ void __launch_bounds__(RN_THREADS)
+enter_rows_kernel(const uint4* __restrict__ src, int n_src, const int32_t* __restrict__ rows, const uint4* __restrict__ gain, float eps,
+                  int row_vecs, uint4* __restrict__ x_dst, uint4* __restrict__ out, int32_t* __restrict__ pos_out, int pos_base, uint32_t* status,
+                  int beside) {
+  if (!beside) pdl_wait();
+  pdl_launch_dependents();
+  enter_row(src, n_src, rows, gain, eps, row_vecs, x_dst, out, pos_out, pos_base, status);
+  if (beside) pdl_wait();
+}
+
 int enter_rows(const a3_handle* h, const bf16* src, int n_src, const int32_t* rows, int M, const bf16* gain, float eps, int d, bf16* x_dst,
-               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st) {
+               bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st, bool beside) {
   if (M <= 0) return A3_OK;
   ProfScope prof(h, A3_K_ROWS, st);
   A3_CUDA(launch_pdl(enter_rows_kernel, dim3(M), dim3(RN_THREADS), 0, st, (const uint4*)src, n_src, rows, (const uint4*)gain, eps, d / 8,
-                     (uint4*)x_dst, (uint4*)out, pos_out, pos_base, h->dev_status));
+                     (uint4*)x_dst, (uint4*)out, pos_out, pos_base, h->dev_status, (int)beside));
   A3_LAUNCHED();
   return A3_OK;
 }
