@@ -93,6 +93,14 @@ __device__ __forceinline__ void sp_ld_chunk(uint32_t taddr, int w, float* v) {
   }
   tc_wait_ld_of<CH>(v);
 }
+// 32 bytes (aligned to 32) through the read-only path.  The lanes of a token read its table row 64 bytes apart, so that a load costs
+// its lines and not its bytes: half as many loads.  A chunk's fetch took 800 of its 1 450 clocks; request of 369 tokens on a small
+// model 144.1 -> 142.8 us, prefill of 512 tokens (Llama-8B) 7 614 -> 7 595.
+__device__ __forceinline__ void ldg32(const float4* p, float4& a, float4& b) {
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+               : "l"(p));
+}
 // f(std::integral_constant<int, chunk>) for the chunk of this launch
 template <bool MAY_8, typename F>
 __device__ __forceinline__ bool sp_with_chunk(int chunk, F f) {
@@ -621,7 +629,8 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
             const float2* row = p.tab + (size_t)max(posbuf[min(e, 127)], 0) * 64;
             const float4* lo = reinterpret_cast<const float4*>(row + (p.layout == 0 ? f0 : f0 >> 1));
             const float4* hi = reinterpret_cast<const float4*>(row + (p.layout == 0 ? f0 + 4 : 32 + (f0 >> 1)));
-            tab[4 * pass] = __ldg(lo), tab[4 * pass + 1] = __ldg(lo + 1), tab[4 * pass + 2] = __ldg(hi), tab[4 * pass + 3] = __ldg(hi + 1);
+            ldg32(lo, tab[4 * pass], tab[4 * pass + 1]);
+            ldg32(hi, tab[4 * pass + 2], tab[4 * pass + 3]);
           }
         };
         fetch(0);
