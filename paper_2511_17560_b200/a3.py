@@ -359,17 +359,18 @@ class A3:
 
     def evict_layer(self, q_window, q_pos, lse, k_layer, v_layer, n_system, n_ctx, capacity, pool=1):
         """`ex` for one layer; returns (k_out, v_out, kept) with C' = n_system + k + nq entries per head."""
-        nq = q_pos.shape[0]
-        kv_len = k_layer.shape[0]
-        Cp = n_system + evict_count(capacity, n_system, n_ctx, nq) + nq
-        Hkv, D = self.shape.n_kv_heads, self.shape.head_dim
-        k_out = k_layer.new_empty((Cp, Hkv, D), dtype=torch.bfloat16)  # the gather writes every entry
+        # the call is shorter on the device than on the host: no conversions and checks of what is made right here
+        lib, m = _load(), self.shape
+        nq, kv_len = q_pos.shape[0], k_layer.shape[0]
+        Cp = n_system + lib.a3_evict_count(capacity, n_system, n_ctx, nq) + nq
+        k_out = k_layer.new_empty((Cp, m.n_kv_heads, m.head_dim), dtype=torch.bfloat16)  # the gather writes every entry
         v_out = torch.empty_like(k_out)
-        kept = k_layer.new_empty((Hkv, Cp), dtype=torch.int32)  # not q_pos's type and device: without question rows nobody reads q_pos
-        ws = self.workspace(int(_load().a3_evict_workspace_bytes(self._h, kv_len)))
-        _check(_load().a3_evict_layer(self._h, _ptr(q_window), _ptr(q_pos), nq, _ptr(lse), _ptr(k_layer), _ptr(v_layer), kv_len,
-                                      n_system, n_ctx, capacity, pool, _ptr(k_out), _ptr(v_out), _ptr(kept), _ptr(ws), ws.numel(),
-                                      _stream()), "a3_evict_layer")
+        kept = k_layer.new_empty((m.n_kv_heads, Cp), dtype=torch.int32)  # not q_pos's type and device: without question rows nobody reads q_pos
+        ws = self.workspace(lib.a3_evict_workspace_bytes(self._h, kv_len))
+        status = lib.a3_evict_layer(self._h, _ptr(q_window), _ptr(q_pos), nq, _ptr(lse), _ptr(k_layer), _ptr(v_layer), kv_len, n_system, n_ctx,
+                                    capacity, pool, k_out.data_ptr(), v_out.data_ptr(), kept.data_ptr(), ws.data_ptr(), ws.numel(), _stream())
+        if status != A3_OK:
+            raise A3Error(status, "a3_evict_layer")
         return k_out, v_out, kept
 
     def first_token(self, x_row, final_norm, lm_head, want_logits=True):
