@@ -821,7 +821,8 @@ static int launch_cluster(const a3_handle* h, const CUtensorMap& tK, const CUten
 }
 
 int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M, const bf16* k, const bf16* v,
-                      int kv_len, bf16* o, float* lse, void* part, size_t part_bytes, cudaStream_t st) {
+                      int kv_len, bf16* o, float* lse, void* part, size_t part_bytes, cudaStream_t st, StatsSplit* unmerged) {
+  if (unmerged) *unmerged = StatsSplit{};
   if (M <= 0) return A3_OK;
   const int Hq = h->m.n_q_heads, Hkv = h->m.n_kv_heads, D = h->m.head_dim;
   const int G = Hq / Hkv;
@@ -885,7 +886,9 @@ int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M,
     A3_CUDA(launch_pdl(attention_tc_kernel<64>, dim3(n_ctas), dim3(ATC_THREADS), (size_t)AtcLayout<64>::SMEM_BYTES, st, tK, tV, q, pos, M, kv_len, o,
                        lse, Hq, Hkv, scale_log2, h->dev_status, n_split, tiles_per_split, part_o, part_ml));
   A3_LAUNCHED();
-  if (n_split > 1) {
+  if (n_split > 1 && unmerged) {
+    *unmerged = StatsSplit{part_ml, tiles_per_split, rows_pad};
+  } else if (n_split > 1) {
     dim3 cgrid(cdiv((long long)M * G, 4), Hkv);
     A3_CUDA(launch_pdl(D == 128 ? attention_combine_kernel<128> : attention_combine_kernel<64>, cgrid, dim3(128), 0, st, pos, M, kv_len, Hq, Hkv,
                        tiles_per_split, rows_pad, part_o, part_ml, o, lse));

@@ -197,8 +197,13 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
 // Causal attention of M rows (at cache slots pos[m]) over a [kv_len][Hkv][D] cache.
 // q: [M][Hq][D]; o: [M][Hq][D] (may be null: statistics only); lse: [M][Hq] or null.
 // part / part_bytes: optional scratch for partial results when the keys are split across CTAs (attention_part_bytes).
+// unmerged (statistics only): where the keys were split, the segments' statistics are left as they are and described there.
+struct StatsSplit {
+  const float2* part_ml;  // [segment][Hkv][rows_pad] (reference, sum), null: not split, lse is complete
+  int tiles_per_split, rows_pad;
+};
 int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M, const bf16* k, const bf16* v,
-                   int kv_len, bf16* o, float* lse, void* part, size_t part_bytes, cudaStream_t st);
+                   int kv_len, bf16* o, float* lse, void* part, size_t part_bytes, cudaStream_t st, StatsSplit* unmerged = nullptr);
 size_t attention_part_bytes(const a3_handle* h);
 // Statistics-only calls (o == null) split the keys of the few question row tiles over the SMs; the partial row
 // statistics of nq rows need at most this much of `part` (a fixed cap, so that every caller - whatever scratch it
@@ -208,8 +213,11 @@ size_t stats_part_bytes(const a3_handle* h, int nq);
 int scores_with_stats(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len, int cand_begin,
                       int cand_end, float* lse, void* part, size_t part_bytes, float* scores, cudaStream_t st);
 
+// split: the row statistics as the statistics pass left them (rows whose keys were not split are in lse), where the shape allows it.
+bool scores_merge_statistics(const a3_handle* h, int nq);
 int scores_pass(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len,
-                int cand_begin, int cand_end, const float* lse, float* scores, cudaStream_t st, float* per_head = nullptr);
+                int cand_begin, int cand_end, const float* lse, float* scores, cudaStream_t st, float* per_head = nullptr,
+                const StatsSplit* split = nullptr);
 // a3_topk_select of the k best candidates, followed by the slots tail_begin .. tail_begin + tail - 1 (the question's)
 int topk_rows(const a3_handle* h, const float* scores, int cand_begin, int cand_end, int k, int tail_begin, int tail, int32_t* idx_out,
               cudaStream_t st);
