@@ -156,7 +156,7 @@ typedef enum {
   A3_OPT_ATTN_MAX_CTAS,         /* cap on the persistent attention grid; 0 = one CTA per SM (default) */
   A3_OPT_SWIGLU_NARROW,         /* one-CTA gate/up GEMM: 0 uniform tiles, 1 narrower last wave (default), 16..120 forced width */
   A3_OPT_SWIGLU_PAIR,           /* persistent CTA-pair gate/up GEMM: 0 never, 1 whenever the shape allows (default) */
-  A3_OPT_RESIDUAL_T,            /* persistent CTA-pair C += A B^T: 0 never, 1 whenever the shape allows, few rows in k-slices (default), 2 never in k-slices */
+  A3_OPT_RESIDUAL_T,            /* persistent CTA-pair C += A B^T: 0 never, 1 whenever the shape allows, few rows in k-slices (default), 2 never in k-slices, 3 as 1 with one token tile per slice (the same sums) */
   A3_OPT_GEMM_BN_RESIDUAL,      /* tile width of the tile GEMMs per epilogue; 0 = choose; 512 = the 256 x 256 CTA-pair tile */
   A3_OPT_GEMM_BN_SWIGLU,
   A3_OPT_GEMM_BN_QKV,
@@ -364,6 +364,15 @@ const char* a3_status_string(int status);
 int a3_last_cuda_error(void);
 /* Number of kernel launches this library has queued since the counter was last reset (host counter). */
 uint64_t a3_launch_count(int reset);
+
+/* How the GEMMs of a layer of `rows` rows are cut by default for a model on a device of sm_count SMs: the rules by which the launches
+ * choose, for tests and measurements.  Host only, needs no device. */
+typedef struct {
+  int32_t swiglu_tiles;           /* gate/up: token tiles per unit of work that share one stream of weights, 1 or 2 */
+  int32_t out_slices, out_tiles;  /* output projection: slices of its k-loop (1: undivided), token tiles per unit */
+  int32_t down_slices, down_tiles; /* down projection */
+} a3_layer_plan;
+int a3_plan_layer(const a3_model_desc* model, int sm_count, int rows, a3_layer_plan* out);
 
 /* Per-kernel-class device timing with CUDA events recorded on the launching stream around every launch.
  * a3_profile_enable(h, max_records > 0) allocates the event pool (not a hot call) and starts recording;

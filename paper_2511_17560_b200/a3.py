@@ -74,12 +74,16 @@ EXPORTS = ("a3_create", "a3_destroy", "a3_set_option", "a3_scores_workspace_byte
            "a3_evict_count", "a3_evict_workspace_bytes", "a3_evict_layer", "a3_chunk_edge_rows", "a3_random_rows", "a3_fuse_request", "a3_fuse_batch", "a3_fuse_request_host",
            "a3_graph_capture", "a3_graph_launch", "a3_graph_kernel_count", "a3_graph_destroy",
            "a3_device_status", "a3_status_string", "a3_last_cuda_error", "a3_launch_count", "a3_profile_enable",
-           "a3_profile_read", "a3_kernel_class_name")
+           "a3_profile_read", "a3_kernel_class_name", "a3_plan_layer")
 K_CLASSES = 10
 
 
 class ProfileEntry(C.Structure):
     _fields_ = [("launches", C.c_uint64), ("ms", C.c_double)]
+
+
+class LayerPlan(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("swiglu_tiles", "out_slices", "out_tiles", "down_slices", "down_tiles")]
 
 
 def _load():
@@ -137,6 +141,7 @@ def _load():
     lib.a3_profile_read.argtypes = [vp, C.POINTER(ProfileEntry), vp]
     lib.a3_kernel_class_name.argtypes = [i32]
     lib.a3_kernel_class_name.restype = C.c_char_p
+    lib.a3_plan_layer.argtypes = [C.POINTER(ModelDesc), i32, i32, C.POINTER(LayerPlan)]
     _lib = lib
     return lib
 
@@ -229,6 +234,15 @@ def chunk_table(chunk_k: Sequence[torch.Tensor], chunk_v: Sequence[torch.Tensor]
     raw = np.frombuffer(bytes(arr), dtype=np.uint8).copy()
     dev = device if device is not None else (chunk_k[0].device if len(chunk_k) else "cuda")
     return torch.from_numpy(raw).to(dev)
+
+
+def plan_layer(shape, rows: int, sm_count: int = 148) -> Dict[str, int]:
+    """How the GEMMs of a layer of `rows` rows are cut by default (a3_plan_layer); needs no device."""
+    desc = ModelDesc(shape.n_layers, shape.d_model, shape.n_q_heads, shape.n_kv_heads, shape.head_dim, shape.d_ff,
+                     float(shape.rope_theta), float(shape.rms_eps), int(shape.rope_layout), 1)
+    plan = LayerPlan()
+    _check(_load().a3_plan_layer(C.byref(desc), int(sm_count), int(rows), C.byref(plan)), "a3_plan_layer")
+    return {n: int(getattr(plan, n)) for n, _ in LayerPlan._fields_}
 
 
 class A3:

@@ -142,6 +142,29 @@ extern "C" int a3_recompute_count(double ratio, int n, int n_candidates) {
   return (int)p;
 }
 
+static void default_options(int* opt) {
+  opt[A3_OPT_ATTN_PAIR] = -1;
+  opt[A3_OPT_SWIGLU_NARROW] = 1;
+  opt[A3_OPT_SWIGLU_PAIR] = 1;
+  opt[A3_OPT_RESIDUAL_T] = 1;
+  opt[A3_OPT_QKV_T] = 1;
+  opt[A3_OPT_GEMM_BN_SWIGLU] = 256;  // the one-CTA gate/up kernel runs two CTAs per SM: 256 columns, 2 stages
+  opt[A3_OPT_GEMM_STAGES_SWIGLU] = 2;
+}
+
+extern "C" int a3_plan_layer(const a3_model_desc* m, int sm_count, int rows, a3_layer_plan* out) {
+  if (!m || !out || sm_count < 2 || rows < 0 || m->d_model <= 0 || m->n_q_heads <= 0 || m->head_dim <= 0 || m->d_ff <= 0) return A3_EINVAL;
+  a3_handle h{};
+  h.m = *m;
+  h.sm_count = sm_count;
+  default_options(h.opt);
+  const size_t part_bytes = attention_part_bytes(&h);  // as carve_layer_ws hands it to the residual products
+  out->swiglu_tiles = swiglu_tiles(&h, rows, m->d_model, m->d_ff);
+  out->out_slices = residual_slices(&h, rows, m->d_model, m->n_q_heads * m->head_dim, part_bytes, &out->out_tiles);
+  out->down_slices = residual_slices(&h, rows, m->d_model, m->d_ff, part_bytes, &out->down_tiles);
+  return A3_OK;
+}
+
 extern "C" int a3_create(a3_handle** out, const a3_model_desc* m, const a3_layer_weights* layers) {
   if (!out || !m || !layers) return A3_EINVAL;
   *out = nullptr;
@@ -165,13 +188,7 @@ extern "C" int a3_create(a3_handle** out, const a3_model_desc* m, const a3_layer
   a3_handle* h = (a3_handle*)calloc(1, sizeof(a3_handle));
   if (!h) return A3_EINVAL;
   h->m = *m;
-  h->opt[A3_OPT_ATTN_PAIR] = -1;
-  h->opt[A3_OPT_SWIGLU_NARROW] = 1;
-  h->opt[A3_OPT_SWIGLU_PAIR] = 1;
-  h->opt[A3_OPT_RESIDUAL_T] = 1;
-  h->opt[A3_OPT_QKV_T] = 1;
-  h->opt[A3_OPT_GEMM_BN_SWIGLU] = 256;  // the one-CTA gate/up kernel runs two CTAs per SM: 256 columns, 2 stages
-  h->opt[A3_OPT_GEMM_STAGES_SWIGLU] = 2;
+  default_options(h->opt);
   h->layers = (a3_layer_weights*)malloc(sizeof(a3_layer_weights) * m->n_layers);
   memcpy(h->layers, layers, sizeof(a3_layer_weights) * m->n_layers);
   cudaError_t e = cudaGetDevice(&h->device);

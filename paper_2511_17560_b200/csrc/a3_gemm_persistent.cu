@@ -158,10 +158,14 @@ __device__ __forceinline__ void sp_place(const SpParams& p, int u, int& fb, int&
   row0 = tt * p.tok_n;
 }
 
-// SPLIT: ring stages [first, first + count) of slice ks of a k-loop of `steps` stages
-__device__ __forceinline__ void sp_slice(int ks, int k_slices, int steps, int& first, int& count) {
-  first = (int)((long long)steps * ks / k_slices);
-  count = (int)((long long)steps * (ks + 1) / k_slices) - first;
+// Ring stages [first, first + count) of slice ks of a k-loop of kt k-blocks.  The cuts lie between groups of SP_SUB k-blocks whatever a
+// stage holds (SP_SUB / TT of them), so that the partial sums of a slice do not depend on how many token tiles share its weights.
+template <int TT>
+__device__ __forceinline__ void sp_slice(int ks, int k_slices, int kt, int& first, int& count) {
+  const long long groups = kt / SP_SUB;
+  const int g0 = (int)(groups * ks / k_slices);
+  first = g0 * TT;
+  count = ((int)(groups * (ks + 1) / k_slices) - g0) * TT;
 }
 
 // D += A B over the CTA pair (accumulating form: no predicate to set up)
@@ -291,11 +295,11 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         int fb, row0, kb0 = 0, kb1 = KT;
         sp_place<EPI>(p, SPLIT ? u / p.k_slices : u, fb, row0);
         if (SPLIT) {
-          sp_slice(u % p.k_slices, p.k_slices, KS, kb0, kb1);
+          sp_slice<TT>(u % p.k_slices, p.k_slices, KT, kb0, kb1);
           kb0 *= SUB;
           kb1 = kb0 + kb1 * SUB;
         } else if (KC > 1) {
-          sp_slice(kc, KC, KS, kb0, kb1);
+          sp_slice<TT>(kc, KC, KT, kb0, kb1);
           kb0 *= SUB;
           kb1 = kb0 + kb1 * SUB;
         }
@@ -383,12 +387,12 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       int per_unit = KS, total = 0;
       if (KC > 1) {
         int first;
-        sp_slice(kc, KC, KS, first, per_unit);
+        sp_slice<TT>(kc, KC, KT, first, per_unit);
       }
       if (SPLIT) {
         for (int u = pair, first; u < p.n_units; u += p.n_pairs) {
           int count;
-          sp_slice(u % p.k_slices, p.k_slices, KS, first, count);
+          sp_slice<TT>(u % p.k_slices, p.k_slices, KT, first, count);
           total += count;
         }
       } else {
@@ -414,7 +418,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           if (!ok) break;
           if (SPLIT) {
             int first;
-            sp_slice(u % p.k_slices, p.k_slices, KS, first, per_unit);
+            sp_slice<TT>(u % p.k_slices, p.k_slices, KT, first, per_unit);
           }
         }
         ok = mbar_wait_warp(full_bar(s), ph, abort_flag, p.status);
@@ -886,7 +890,7 @@ static SpTiling choose_tiling(const a3_handle* h, int M, int n_fblocks, int pair
 // Pinned kernel variants (a3_set_option) are compared bit for bit and therefore keep the undivided sums.
 constexpr int SP_SLICE_MIN_KB = 16;
 static bool split_allowed(const a3_handle* h) {
-  return h->opt[A3_OPT_RESIDUAL_T] == 1 && h->opt[A3_OPT_QKV_T] == 1 && h->opt[A3_OPT_SWIGLU_PAIR] == 1 &&
+  return (h->opt[A3_OPT_RESIDUAL_T] == 1 || h->opt[A3_OPT_RESIDUAL_T] == 3) && h->opt[A3_OPT_QKV_T] == 1 && h->opt[A3_OPT_SWIGLU_PAIR] == 1 &&
          h->opt[A3_OPT_GEMM_TILING] == 0;
 }
 struct SpSlices {
@@ -895,28 +899,26 @@ struct SpSlices {
 static SpSlices choose_slices(int M, int F, int K, int n_fblocks, int pairs, size_t part_bytes) {
   const int tiles = cdiv(M, 256), n = cdiv(cdiv(M, tiles), 16) * 16, kt = K / TC_BK;
   const int per_kb = 2 * n > 256 + n ? 2 * n : 256 + n;
-  long long least = (long long)kt * per_kb, least_two = least;
-  int two = 1;
+  auto depth = [&](int s) { return (long long)cdiv(kt / SP_SUB, s) * SP_SUB; };  // k-blocks of the deepest slice
+  auto sums = [&](int s) { return (long long)s * M * F * 8 / 3000 + 2000; };
+  long long least = (long long)kt * per_kb;
   SpSlices best{1, 1};
   for (int s = 2; s <= 16 && s * SP_SLICE_MIN_KB <= kt; ++s) {
     if ((size_t)s * M * F * 4 > part_bytes) break;
-    const long long sums = (long long)s * M * F * 8 / 3000 + 2000;
-    const long long cost = (long long)cdiv((long long)n_fblocks * tiles * s, pairs) * ((long long)cdiv(kt / SP_SUB, s) * SP_SUB * per_kb + 2000) + sums;
+    const long long cost = (long long)cdiv((long long)n_fblocks * tiles * s, pairs) * (depth(s) * per_kb + 2000) + sums(s);
     if (cost < least) {
       least = cost;
       best = SpSlices{s, 1};
     }
-    if (tiles != 2 || n_fblocks * s > pairs) continue;  // two_tiles; one unit per pair: both accumulators of 256 columns are in use
-    const long long both = (long long)cdiv(kt, s) * two_tiles_per_kb(n) + 2000 + n * 20 + sums;
-    if (both < least_two) {
-      least_two = both;
-      two = s;
-    }
   }
-  // A tenth is left out: slices twice as many cost more than their traffic.  Prefill (us), one tile per unit against two: Qwen-7B 272
-  // rows 4 739 / 4 588 (both five slices), 352 rows 5 342 / 5 232, 400 rows 5 938 / 5 921; Llama-8B (two slices against four) 272
-  // rows 5 200 / 5 231, 320 rows 5 486 / 5 547.
-  if (least_two * 10 < least * 9) best = SpSlices{two, 2};
+  // The same slices with both tiles on one stream of weights (two_tiles), one unit per pair: both accumulators of 256 columns are in
+  // use.  Not with more slices for the sake of it, which would change the sums and lost where it was tried: a layer of 257 rows in two
+  // slices against five of two tiles 103.7 / 105.1 us at 3 200 x 10 112, 106.9 / 107.6 at 3 328 x 10 624; prefill (us) of Llama-8B in
+  // two slices against four, 272 rows 5 200 / 5 231, 320 rows 5 486 / 5 547.  Qwen-7B, five slices either way: a layer 156.4 / 150.9
+  // at 257 rows, 163.9 / 158.8 at 272, 175.6 / 172.1 at 320, 192.9 / 191.7 at 352, hence the tenth that is left out.
+  if (tiles == 2 && best.slices > 1 && n_fblocks * best.slices <= pairs &&
+      (depth(best.slices) * two_tiles_per_kb(n) + 2000 + n * 20 + sums(best.slices)) * 10 < least * 9)
+    best.tiles = 2;
   return best;
 }
 int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes, int* tiles) {
@@ -925,7 +927,7 @@ int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes, 
   const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2, blocks = cdiv(N, 4 * SP_FEAT);
   if (blocks * cdiv(M, 256) > pairs / 2) return 1;  // the pairs are busy with whole units
   const SpSlices c = choose_slices(M, N, K, blocks, pairs, part_bytes);
-  *tiles = c.tiles;
+  *tiles = h->opt[A3_OPT_RESIDUAL_T] == 3 ? 1 : c.tiles;
   return c.slices;
 }
 
@@ -1003,6 +1005,12 @@ static bool two_tiles(const a3_handle* h, int M, int K, int n_fblocks, int pairs
   if (M <= 256 || n > SP_TWO_TILES_MAX || h->opt[A3_OPT_GEMM_TILING] != 0) return false;
   const int per_kb = 2 * til.n > 256 + til.n ? 2 * til.n : 256 + til.n;
   return (long long)cdiv(n_fblocks, pairs) * (kt * two_tiles_per_kb(n) + 30 * n) < (long long)cdiv((long long)n_fblocks * til.tiles, pairs) * kt * per_kb;
+}
+
+// Token tiles per unit of the gate/up GEMM by default (a3_plan_layer)
+int swiglu_tiles(const a3_handle* h, int M, int K, int F) {
+  const int pairs = (h->sm_count > 0 ? h->sm_count : 148) / 2, n_fblocks = cdiv(F, 2 * SP_FEAT);
+  return M > 0 && two_tiles(h, M, K, n_fblocks, pairs, choose_tiling(h, M, n_fblocks, pairs)) ? 2 : 1;
 }
 
 template <int EPI>

@@ -179,12 +179,13 @@ struct GemmArgs {
 // SwiGLU GEMM with the weights as the M-side operand of a CTA pair, persistent (a3_gemm_persistent.cu).
 bool swiglu_pair_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_swiglu_pair(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
+int swiglu_tiles(const a3_handle* h, int M, int K, int F);
 // C += A B^T with the same kernel structure (weights on the M side, persistent CTA pairs).
 bool residual_t_usable(const a3_handle* h, const GemmArgs& a);
 int gemm_residual_t(const a3_handle* h, const GemmArgs& a, cudaStream_t st);
 // The same product of few rows, its k-loop cut into slices: fp32 partial sums [slices][M][N] for add_slices_rmsnorm.
 // residual_slices: how many slices suit the shape (1: use gemm_bf16), given room for part_bytes of partial sums, and how many token
-// tiles share a stream of weights.
+// tiles share a stream of weights (1 or 2; the slices, and with them the sums, are the same either way).
 int residual_slices(const a3_handle* h, int M, int N, int K, size_t part_bytes, int* tiles);
 int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, int tiles, float* part, cudaStream_t st);
 // QKV projection (bias, RoPE, scatter in the epilogue) with one head per CTA of a pair

@@ -100,6 +100,39 @@ def test_two_token_tiles_on_one_stream_of_weights(a3mod, m, M):
     eng.close()
 
 
+# the widths at which a slice of the down projection takes two token tiles: five slices of Qwen-7B's to 352 rows, of 3 200 x 13 440 at 257
+QWEN_LAYER = replace(W.QWEN7B, n_layers=1)
+TWO_TILE_SLICES = W.ModelShape("two_tile_slices", 1, 3200, 16, 4, 128, 13440, 32000, 5e5, 1e-5)
+
+
+@pytest.mark.parametrize("m,M", [(QWEN_LAYER, M) for M in (257, 270, 289, 320, 321, 352)] + [(TWO_TILE_SLICES, 257)])
+def test_slices_of_two_token_tiles(a3mod, m, M):
+    """The same slices with one token tile each: bit for bit, since neither their number nor the cuts of the k-loop depend on it.
+    Undivided sums: within what one rounding of the hidden row leaves (hidden_rows_scale's gates)."""
+    assert a3mod.plan_layer(m, M)["down_tiles"] == 2
+    dev = torch.device("cuda:0")
+    eng = a3mod.A3(m, W.make_weights_device(m, dev, M), M)
+    g = torch.Generator(device=dev)
+    g.manual_seed(M)
+    x0 = torch.randn(M, m.d_model, device=dev, generator=g).bfloat16()
+    pos = torch.arange(M, dtype=torch.int32, device=dev)
+    outs = {}
+    for residual in (1, 3, 2):
+        eng.set_option(a3mod.OPT_RESIDUAL_T, residual)
+        x, K, V = x0.clone(), *(torch.zeros(M, m.n_kv_heads, m.head_dim, device=dev, dtype=torch.bfloat16) for _ in range(2))
+        eng.recompute_layer(0, x, pos, K, V)
+        assert eng.device_status() == 0
+        outs[residual] = x
+    assert torch.equal(outs[1], outs[3])
+    exact = f64(outs[2])
+    check_kv(f64(outs[1]), exact, "hidden rows", scale=hidden_rows_scale(exact))
+    eng.close()
+
+
+def test_two_token_tiles_of_a_slice_against_the_oracle(a3mod):
+    layer_parity(a3mod, TWO_TILE_SLICES, 257, seed=11)
+
+
 # rows of more than 4 096 values: what the threads of the adding kernel do not keep in registers is read again; both of a layer's
 # residual products in two slices
 LONG_ROWS = W.ModelShape("long_rows", 1, 4224, 16, 4, 128, 2176, 32000, 5e5, 1e-5)
