@@ -987,17 +987,21 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, int t
   p.part = part;
   p.n_units = p.n_fblocks * p.tok_tiles * slices;
   p.group = 1;
+  // two tiles: accumulators of 256 columns, of which tensor memory holds two, so one unit per pair (choose_slices sees to both)
+  if (tiles == 2 && (p.n_units > pairs || a.M <= 256 || a.M > 512)) return A3_EINVAL;
   p.n_pairs = p.n_units < pairs ? p.n_units : pairs;
   p.status = h->dev_status;
   const int smem_bytes = set_stages(p, EPI_RESIDUAL, true, tiles);
   CUtensorMap tX, tG;
   A3_TRY(make_tmap_kblocks(&tX, a.A, a.M, a.K, p.tok_n / 2, SP_SUB / tiles));
   A3_TRY(make_tmap_kblocks(&tG, a.seg[0].B, p.F, a.K, 2 * SP_FEAT, SP_SUB / tiles));
-  static SmemAttrOnce attr[4];
-  const bool once = weights_once(h, p.tok_tiles);
-  const auto kernel = tiles == 2 ? (once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true, 2> : pair_t_kernel<EPI_RESIDUAL, true, 1, false, 2>)
-                                 : (once ? pair_t_kernel<EPI_RESIDUAL, true, 1, true> : pair_t_kernel<EPI_RESIDUAL, true, 1, false>);
-  A3_TRY(smem_attr_once(attr[2 * (tiles - 1) + once], h->device, kernel, SP_SMEM_LIMIT));
+  // (Two tiles mark their weights always: the smallest layer that takes them is more than twice L2.)
+  static SmemAttrOnce attr[3];
+  const int variant = tiles == 2 ? 2 : weights_once(h, p.tok_tiles);
+  const auto kernel = variant == 2   ? pair_t_kernel<EPI_RESIDUAL, true, 1, true, 2>
+                      : variant == 1 ? pair_t_kernel<EPI_RESIDUAL, true, 1, true>
+                                     : pair_t_kernel<EPI_RESIDUAL, true, 1, false>;
+  A3_TRY(smem_attr_once(attr[variant], h->device, kernel, SP_SMEM_LIMIT));
   ProfScope prof(h, A3_K_GEMM_RESIDUAL, st);
   A3_CUDA(launch_pdl(kernel, dim3(2 * p.n_pairs), dim3(SP_THREADS), (size_t)smem_bytes, st, tX, tG, tG, tG, p));
   A3_LAUNCHED();

@@ -40,6 +40,8 @@ def test_slices_do_not_depend_on_the_tiles_that_share_weights(rows):
                 assert tiles in (1, 2)
                 if tiles == 2:
                     assert 256 < rows <= 512 and slices > 1 and -(-d_model // 256) * slices <= PAIRS
+                    # their weights are marked to leave L2 first: the layer is beyond its three quarters (weights_once) by far
+                    assert 2 * d_model * 3 * d_ff > 2 * 126 * 2 ** 20
 
 
 @pytest.mark.parametrize("rows,down", [(75, (5, 1)), (256, (5, 1)), (257, (5, 2)), (270, (5, 2)), (352, (5, 2)), (368, (2, 1)), (512, (2, 1))])
