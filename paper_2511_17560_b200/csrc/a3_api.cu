@@ -440,7 +440,7 @@ namespace a3 {
 int scores_with_stats(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len, int cand_begin,
                       int cand_end, float* lse, void* part, size_t part_bytes, float* scores, cudaStream_t st) {
   StatsSplit split{};
-  if (nq > 0) A3_TRY(attention_rows(h, q, q_pos, nq, k, k, kv_len, nullptr, lse, part, part_bytes, st, scores_merge_statistics(h, nq) ? &split : nullptr));
+  if (nq > 0) A3_TRY(attention_rows(h, q, q_pos, nq, k, k, kv_len, nullptr, lse, part, part_bytes, st, &split));
   return scores_pass(h, q, q_pos, nq, k, kv_len, cand_begin, cand_end, lse, scores, st, nullptr, &split);
 }
 }  // namespace a3

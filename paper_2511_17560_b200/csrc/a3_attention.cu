@@ -886,7 +886,7 @@ int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M,
     A3_CUDA(launch_pdl(attention_tc_kernel<64>, dim3(n_ctas), dim3(ATC_THREADS), (size_t)AtcLayout<64>::SMEM_BYTES, st, tK, tV, q, pos, M, kv_len, o,
                        lse, Hq, Hkv, scale_log2, h->dev_status, n_split, tiles_per_split, part_o, part_ml));
   A3_LAUNCHED();
-  if (n_split > 1 && unmerged) {
+  if (n_split > 1 && unmerged && scores_merge_statistics(h, M, kv_len, n_split)) {
     *unmerged = StatsSplit{part_ml, tiles_per_split, rows_pad};
   } else if (n_split > 1) {
     dim3 cgrid(cdiv((long long)M * G, 4), Hkv);

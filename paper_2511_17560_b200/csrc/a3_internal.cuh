@@ -198,9 +198,10 @@ int gemm_bf16(const a3_handle* h, GemmEpilogue epi, const GemmArgs& a, cudaStrea
 // Causal attention of M rows (at cache slots pos[m]) over a [kv_len][Hkv][D] cache.
 // q: [M][Hq][D]; o: [M][Hq][D] (may be null: statistics only); lse: [M][Hq] or null.
 // part / part_bytes: optional scratch for partial results when the keys are split across CTAs (attention_part_bytes).
-// unmerged (statistics only): where the keys were split, the segments' statistics are left as they are and described there.
+// unmerged (statistics only): where the keys were split and the score kernel is to merge the segments (scores_merge_statistics), their
+// statistics are left as they are and described there.
 struct StatsSplit {
-  const float2* part_ml;  // [segment][Hkv][rows_pad] (reference, sum), null: not split, lse is complete
+  const float2* part_ml;  // [segment][Hkv][rows_pad] (reference, sum), null: lse is complete
   int tiles_per_split, rows_pad;
 };
 int attention_rows(const a3_handle* h, const bf16* q, const int32_t* pos, int M, const bf16* k, const bf16* v,
@@ -215,7 +216,7 @@ int scores_with_stats(const a3_handle* h, const bf16* q, const int32_t* q_pos, i
                       int cand_end, float* lse, void* part, size_t part_bytes, float* scores, cudaStream_t st);
 
 // split: the row statistics as the statistics pass left them (rows whose keys were not split are in lse), where the shape allows it.
-bool scores_merge_statistics(const a3_handle* h, int nq);
+bool scores_merge_statistics(const a3_handle* h, int nq, int kv_len, int segments);
 int scores_pass(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len,
                 int cand_begin, int cand_end, const float* lse, float* scores, cudaStream_t st, float* per_head = nullptr,
                 const StatsSplit* split = nullptr);

@@ -329,7 +329,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     for (int i = threadIdx.x - 64; i < (g_end - g_begin) * rows_g; i += STC_ACC_THREADS) {
       const int g = g_begin + i / rows_g, r = i % rows_g;
       // Segments that the statistics pass left for this row: merged here, as attention_combine_kernel would in a launch of its own
-      // (every CTA does it for itself, while its first tiles are on their way).  Request of 369 tokens on a small model 142.9 -> 141.4 us.
+      // (every CTA does it for itself, while its first tiles are on their way; see scores_merge_statistics).
       int n_active = 0;
       if (p.split.part_ml) {
         const int maxpos = min(p.q_pos[min(p.nq - 1, (r / ATC_BM * ATC_BM + ATC_BM - 1) / G)], p.kv_len - 1);
@@ -537,9 +537,20 @@ static int launch_scores_tc(const a3_handle* h, const bf16* q, const int32_t* q_
   return A3_OK;
 }
 
-bool scores_merge_statistics(const a3_handle* h, int nq) {
+// Whether the score kernel merges the statistics pass's segments or a launch between the two does.  Merged inside, a launch (2.5 us) is
+// saved, but every CTA walks the segments of all (row, head) pairs: in one round of its accumulating threads under the first copies,
+// whatever their number; each further round, by more pairs than threads or by more key tiles than SMs, delays the CTA by what it reads.
+// Statistics, merge and scores, inside against apart (us).  One round: 256 pairs over 813 slots 14.9 / 17.3, 5 128 18.7 / 21.2, 18 708
+// 25.2 / 28.1 (Llama-8B heads), 252 over 17 880 24.3 / 27.9 (Qwen-7B), 256 over 18 764 in 74 segments 25.5 / 33.0 (two KV heads).  Two
+// rounds of pairs: 384 x 3 segments 12.8 / 14.3, 504 x 7 18.9 / 18.7, 448 x 7 17.1 / 17.4, 384 x 14 23.0 / 22.5, 504 x 18 22.9 / 20.8, 512
+// x 20 21.1 / 19.8.  Two rounds of tiles: 256 x 18 42.7 / 44.5, 252 x 34 38.6 / 35.4, 256 x 53 32.2 / 27.3.  More: 1 024 pairs over 5 152
+// slots 30.6 / 25.9, 1 792 over 17 935 48.8 / 43.5, 1 024 over 32 800 in two rounds of tiles 70.1 / 49.8.
+bool scores_merge_statistics(const a3_handle* h, int nq, int kv_len, int segments) {
   int nq_tile, n_chunks;
-  return h->opt[A3_OPT_SCORES_KERNEL] != 2 && stc_shape(h, nq, &nq_tile, &n_chunks);
+  if (h->opt[A3_OPT_SCORES_KERNEL] == 2 || !stc_shape(h, nq, &nq_tile, &n_chunks)) return false;
+  const int passes = cdiv((long long)nq * h->m.n_q_heads, STC_ACC_THREADS), waves = cdiv(cdiv(kv_len, 128), h->sm_count > 0 ? h->sm_count : 148);
+  if (passes * waves == 1) return true;
+  return passes * waves == 2 && segments <= (waves == 2 ? 20 : 8);
 }
 
 int scores_pass(const a3_handle* h, const bf16* q, const int32_t* q_pos, int nq, const bf16* k, int kv_len,

@@ -299,3 +299,34 @@ def test_late_queries_ride_along(a3mod, shape, n_ctx, nq):
         assert torch.equal(a, b)
     assert float(res[0][2].abs().max()) > 0
     eng.close()
+
+
+HEADS_32_8 = W.ModelShape("heads_32_8", 1, 128, 32, 8, 128, 128, 1000, 5e5, 1e-5)
+HEADS_28_4 = W.ModelShape("heads_28_4", 1, 128, 28, 4, 128, 128, 1000, 1e6, 1e-6)
+HEADS_4_2 = W.ModelShape("heads_4_2", 1, 128, 4, 2, 128, 128, 1000, 5e5, 1e-5)
+
+
+@pytest.mark.parametrize("m,n_ctx,nq,launches", [(HEADS_32_8, 805, 8, 3), (HEADS_32_8, 805, 9, 3), (HEADS_32_8, 805, 17, 4), (HEADS_32_8, 1200, 9, 4),
+                                                 (HEADS_32_8, 5120, 32, 4), (HEADS_32_8, 18930, 8, 3), (HEADS_32_8, 18960, 8, 3), (HEADS_32_8, 32768, 32, 4),
+                                                 (HEADS_28_4, 17871, 9, 3), (HEADS_28_4, 17871, 64, 4), (HEADS_28_4, 19000, 9, 4),
+                                                 (HEADS_4_2, 356, 13, 3), (HEADS_4_2, 18800, 64, 3), (HEADS_4_2, 19000, 64, 4)])
+def test_statistics_merged_where_that_is_shorter(a3mod, m, n_ctx, nq, launches):
+    """Position check, statistics and scores, and a merge between the last two unless the score kernel merges the segments in one
+    round (or a second one over few segments): the same scores as the warp-level kernel's, which always has them merged before."""
+    eng, n = a3mod.A3(m, W.make_weights_device(m, torch.device("cuda:0"), 0), n_ctx + nq), n_ctx + nq
+    g = torch.Generator(device=eng.device)
+    g.manual_seed(n)
+    q = torch.randn(nq, m.n_q_heads, m.head_dim, device=eng.device, generator=g).bfloat16()
+    k = torch.randn(n, m.n_kv_heads, m.head_dim, device=eng.device, generator=g).bfloat16()
+    pos = torch.arange(n_ctx, n, dtype=torch.int32, device=eng.device)
+    a3mod.launch_count(reset=True)
+    scores = eng.query_scores(q, pos, k, 3, n_ctx)
+    assert a3mod.launch_count() == launches
+    eng.set_option(a3mod.OPT_SCORES_KERNEL, 2)
+    other = eng.query_scores(q, pos, k, 3, n_ctx)
+    assert eng.device_status() == 0
+    # A logit (up to 2^6 before its scale of 2^-3.5) is summed in fp32 in eight steps, each off by at most 2^-23 of it: 5.4e-6 in the
+    # exponent; ex2.approx 2^-22, the log-sum-exp no more.  Both kernels: below 2e-5, and the sums add terms of one sign.
+    assert torch.allclose(scores, other, rtol=2e-5, atol=0)
+    assert float(scores[3:n_ctx].min()) > 0 and float(scores[:3].abs().max()) == 0 == float(scores[n_ctx:].abs().max())
+    eng.close()
