@@ -99,7 +99,9 @@ __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __
     if (2 * half_pool + 1 >= KPT && half_pool > 0) {
       // what all windows of the thread have in common, then what those before and those behind have besides
       float mid = none, run = none;
-      for (int i = i0 + KPT - 1 - half_pool; i <= i0 + half_pool; ++i) mid = fmaxf(mid, get(i));
+      const int m0 = max(0, i0 + KPT - 1 - half_pool), m1 = i0 < n ? min(n - 1, i0 + half_pool) : -1;
+#pragma unroll 4
+      for (int i = m0; i <= m1; ++i) mid = fmaxf(mid, raw[topk_at<KPT>(i)]);
 #pragma unroll
       for (int j = KPT - 2; j >= 0; --j) {
         run = fmaxf(run, get(i0 + j - half_pool));

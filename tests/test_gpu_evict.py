@@ -97,6 +97,36 @@ def test_wide_pooling(a3mod, n_cand, pool, launches):
     eng.close()
 
 
+@pytest.mark.parametrize("n_cand,pool", [(8, 31999), (40, 6399), (128, 1999), (300, 853)])
+def test_windows_reach_no_further_than_the_candidates(a3mod, n_cand, pool):
+    """A window wider than the candidates costs what one that just covers them costs (a walk along its whole width takes 3 to 100
+    times as long), and keeps the same."""
+    m, nq = W.TINY_GQA, 9
+    eng, _, _, _, args = evict_setup(a3mod, m, n_cand, nq, n_cand)
+    kept, us = [], []
+    for width in (2 * n_cand - 1, pool):
+        call = lambda: eng.evict_layer(*args, 0, n_cand, nq + n_cand // 2, width)
+        kept.append(call())
+        graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=stream):
+            for _ in range(20):
+                call()
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            graph.replay()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        us.append(min(times))
+    assert eng.device_status() == 0
+    for a, b in zip(*kept):
+        assert torch.equal(a, b)
+    assert us[1] < 1.5 * us[0], us
+    eng.close()
+
+
 @pytest.mark.parametrize("n_system,n_cand,nq,more", [(0, 300, 9, 0), (5, 95, 9, 40), (7, 1, 0, 0), (0, 33, 0, 5)])
 def test_everything_fits(a3mod, n_system, n_cand, nq, more):
     """Capacity for the whole cache, or for more: a copy, in one launch (the header promises at most four)."""
