@@ -114,9 +114,22 @@ __device__ __forceinline__ void topk_regs(const float* __restrict__ s, float* __
         v[j] = fmaxf(v[j], run);
       }
     } else if (half_pool > 0) {
+      // windows narrower than the thread's slots: those and the few on either side, in registers
+      constexpr int HM = KPT > 2 ? (KPT - 2) / 2 : 0;  // 2 half_pool + 1 < KPT
+      float e[KPT + 2 * HM];
 #pragma unroll
-      for (int j = 0; j < KPT; ++j)
-        for (int i = i0 + j - half_pool; i <= i0 + j + half_pool; ++i) v[j] = fmaxf(v[j], get(i));
+      for (int j = 0; j < KPT; ++j) e[HM + j] = i0 + j < n ? v[j] : none;
+#pragma unroll
+      for (int d = 1; d <= HM; ++d) {
+        e[HM - d] = get(i0 - d);
+        e[HM + KPT - 1 + d] = get(i0 + KPT - 1 + d);
+      }
+#pragma unroll
+      for (int d = 1; d <= HM; ++d)
+        if (d <= half_pool) {
+#pragma unroll
+          for (int j = 0; j < KPT; ++j) v[j] = fmaxf(v[j], fmaxf(e[HM + j - d], e[HM + j + d]));
+        }
     }
   }
   uint32_t key[KPT];

@@ -97,6 +97,48 @@ def test_wide_pooling(a3mod, n_cand, pool, launches):
     eng.close()
 
 
+@pytest.mark.parametrize("n_cand,pool", [(3073, 3), (4000, 3), (4000, 5), (4000, 7), (5120, 3), (5121, 3), (5121, 5), (5121, 7), (6000, 7), (8191, 5),
+                                         (8192, 3), (8192, 7), (8192, 9)])
+def test_narrow_windows(a3mod, n_cand, pool):
+    """Windows narrower than the five or eight slots of a thread, at both ends of these sizes and beside the first wider one."""
+    m, nq, n_system = W.TINY_GQA, 9, 5
+    n_ctx, k = n_system + n_cand, n_cand // 5
+    eng, q, pos, K, args = evict_setup(a3mod, m, n_ctx, nq, n_cand + pool)
+    k_out, _, kept = eng.evict_layer(*args, n_system, n_ctx, n_system + nq + k, pool)
+    assert eng.device_status() == 0
+    votes = O.pool_scores(O.eviction_scores(q.astype(np.float64), pos, K.astype(np.float64), oracle_model(m), n_system, n_ctx), n_system, n_ctx, pool)
+    for h in range(m.n_kv_heads):
+        check_kept(kept[h].cpu().numpy(), votes[h], n_system, n_ctx, nq)
+        assert torch.equal(k_out[:, h], args[3][kept[h].long(), h])
+    eng.close()
+
+
+@pytest.mark.parametrize("n_cand,pool", [(900, 1), (900, 3), (2000, 5), (4000, 3), (5121, 7), (8192, 7), (8192, 9), (9000, 3)])
+def test_votes_that_are_no_numbers(a3mod, n_cand, pool):
+    """Infinite votes win their windows, NaN votes are passed over where a window has others and win where it has not, and either is
+    flagged.  Alone, at the ends of the candidates and in a run as wide as a window."""
+    m, nq, n_system = W.TINY_GQA, 9, 5
+    n_ctx, k, group = n_system + n_cand, n_cand // 5, m.n_q_heads // m.n_kv_heads
+    eng, q, pos, K, (dq, dpos, lse, dK, dV) = evict_setup(a3mod, m, n_ctx, nq, n_cand * 3 + pool)
+    votes = O.eviction_scores(q.astype(np.float64), pos, K.astype(np.float64), oracle_model(m), n_system, n_ctx)
+    nan = [n_system, n_system + 333] + list(range(n_system + 600, n_system + 600 + pool))
+    inf = [n_system + 100, n_system + 334, n_ctx - 1]
+    dK[nan] = float("nan")
+    for g in range(m.n_kv_heads):
+        dK[inf, g] = 300 * dq[0, g * group]  # a logit in the thousands
+    votes[:, nan], votes[:, inf] = np.nan, np.inf
+    k_out, _, kept = eng.evict_layer(dq, dpos, lse, dK, dV, n_system, n_ctx, n_system + nq + k, pool)
+    assert eng.device_status() == 2  # A3_DEV_NONFINITE_SCORE
+    for h in range(m.n_kv_heads):
+        v = np.full(n_ctx, np.nan)
+        for i in range(n_system, n_ctx):
+            v[i] = np.fmax.reduce(votes[h, max(n_system, i - pool // 2):min(n_ctx, i + pool // 2 + 1)])
+        rank = np.where(np.isnan(v), 2e30, np.where(np.isinf(v), 1e30, v))  # NaN before infinity before the rest
+        check_kept(kept[h].cpu().numpy(), rank, n_system, n_ctx, nq)
+        assert torch.equal(k_out[:, h].view(torch.int16), dK[kept[h].long(), h].view(torch.int16))
+    eng.close()
+
+
 @pytest.mark.parametrize("n_cand,pool", [(8, 31999), (40, 6399), (128, 1999), (300, 853)])
 def test_windows_reach_no_further_than_the_candidates(a3mod, n_cand, pool):
     """A window wider than the candidates costs what one that just covers them costs (a walk along its whole width takes 3 to 100
