@@ -863,7 +863,8 @@ static int unit_group(int M, int K) { return (long long)M * K * 2 > (64ll << 20)
 // Two token tiles of n per unit on one stream of weights.  Just over 256 rows every weight goes to two units, and units that narrow
 // wait for their operands: 270 rows x 2 x (16 KiB of weights + 9 KiB of tokens) per k-block and CTA, 800 clocks for 576 of tensor time.
 // Together they take 16 + 18 KiB, 544 clocks, and each weight crosses to an SM once: SwiGLU of 270 rows (Qwen width) 67 -> 57 us, down projection 42 -> 31.5.
-constexpr int SP_TWO_TILES_MAX = 160;  // tokens per tile: three accumulators in 512 columns
+constexpr int SP_TWO_TILES_COLS = 160;  // columns from one accumulator to the next: three in 512
+constexpr int SP_TWO_TILES_MAX = 144;   // tokens per tile of SwiGLU, see two_tiles
 static int two_tiles_per_kb(int n) { return 4 * n > 256 + 2 * n ? 4 * n : 256 + 2 * n; }
 
 struct SpTiling {
@@ -954,7 +955,7 @@ static bool weights_once(const a3_handle* h, int tok_tiles) { return tok_tiles =
 static int set_stages(SpParams& p, int epi, bool split, int tt = 1) {
   const int sub = SP_SUB / tt;
   p.stage_bytes = sub * (SP_A_BYTES + tt * (p.tok_n / 2) * TC_BK * 2);  // tok_n / 2 is a multiple of 8: 1024-byte multiples
-  p.slot_cols = tt == 1 || split ? 256 : SP_TWO_TILES_MAX;
+  p.slot_cols = tt == 1 || split ? 256 : SP_TWO_TILES_COLS;
   p.stages = 0;
   const long long steps = (long long)cdiv(p.n_units, p.n_pairs) * (p.K / TC_BK / sub);
   const int useful = steps < SP_MAX_STAGES ? (int)steps : SP_MAX_STAGES;
@@ -1008,15 +1009,18 @@ int gemm_residual_split(const a3_handle* h, const GemmArgs& a, int slices, int t
   return A3_OK;
 }
 
-// SwiGLU on two token tiles per unit: every unit costs half an epilogue more, which the third accumulator does not hide.  Prefill (us),
-// one tile per unit against two (Qwen-7B with the down projection's two tiles, see choose_slices): Qwen-7B 288 rows 4 705 / 4 378, 320
-// rows 4 934 / 4 709; Llama-8B, whose 112 feature blocks are two rounds for 1.5, 288 rows 5 152 / 5 063, 320 rows 5 390 / 5 368.  The
-// epilogue's chunks stay at 16 tokens or more: with 8, for the sake of one ring stage more, 320 rows gained nothing.
+// SwiGLU on two token tiles per unit: every unit costs half an epilogue more, which the third accumulator does not hide, and a k-block
+// a fifth more than its operands take to arrive.  One layer of a stack beyond L2, one tile per unit against two (us): Llama-8B 257 rows
+// 142.1 / 137.6, 272 155.7 / 154.7, 288 157.3 / 156.1; Qwen-7B 257 rows 153.3 / 150.9, 272 159.8 / 158.8; 3 072 x 8 192 257 rows 85.3 /
+// 83.8, 288 88.1 / 87.0.  Where the model says one: 2 048 x 16 384 257 rows 92.9 / 94.5, 2 048 x 8 192 71.9 / 71.5 (SwiGLU alone, from
+// L2, 16.6 / 19.2), 1 536 x 8 960 62.0 / 61.3 (13.8 / 15.6).  Tiles of 160 lost at every width but the narrowest: 304 and 320 rows,
+// Llama-8B 163.7 / 167.2 and 162.3 / 166.4, Qwen-7B 163.6 / 165.3 and 169.1 / 172.1, 2 048 x 16 384 94.3 / 96.9 and 97.2 / 101.2.  The
+// epilogue's chunks stay at 16 tokens or more: with 8, for the sake of one ring stage more, nothing was gained.
 static bool two_tiles(const a3_handle* h, int M, int K, int n_fblocks, int pairs, const SpTiling& til) {
   const int n = cdiv(cdiv(M, 2), 16) * 16, kt = K / TC_BK;
   if (M <= 256 || n > SP_TWO_TILES_MAX || h->opt[A3_OPT_GEMM_TILING] != 0) return false;
   const int per_kb = 2 * til.n > 256 + til.n ? 2 * til.n : 256 + til.n;
-  return (long long)cdiv(n_fblocks, pairs) * (kt * two_tiles_per_kb(n) + 30 * n) < (long long)cdiv((long long)n_fblocks * til.tiles, pairs) * kt * per_kb;
+  return (long long)cdiv(n_fblocks, pairs) * (kt * two_tiles_per_kb(n) * 6 / 5 + 30 * n) < (long long)cdiv((long long)n_fblocks * til.tiles, pairs) * kt * per_kb;
 }
 
 // Token tiles per unit of the gate/up GEMM by default (a3_plan_layer)

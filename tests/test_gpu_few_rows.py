@@ -100,6 +100,38 @@ def test_two_token_tiles_on_one_stream_of_weights(a3mod, m, M):
     eng.close()
 
 
+# gate/up product: one, two and three units per pair of CTAs (64, 148 and 222 feature blocks, 74 pairs), the smallest depths at which a
+# unit takes two token tiles
+SWIGLU_UNITS = {units: W.ModelShape(f"units_{units}", 1, d_model, 1, 1, 128, d_ff, 1000, 1e4, 1e-5)
+                for units, d_model, d_ff in ((1, 2560, 8192), (2, 2560, 18944), (3, 2688, 28416))}
+
+
+@pytest.mark.parametrize("units", [1, 2, 3])
+@pytest.mark.parametrize("M", [257, 272, 288])
+def test_accumulators_of_two_token_tiles_take_turns(a3mod, units, M):
+    """Two, four and six accumulators in three slots of tensor memory: slots that are used once, that are taken again (behind a drained
+    accumulator, a unit astride the last and the first slot), all of them.  Bit for bit the product of one tile per unit."""
+    m, dev = SWIGLU_UNITS[units], torch.device("cuda:0")
+    assert a3mod.plan_layer(m, M)["swiglu_tiles"] == 2 and -(-m.d_ff // 128 // 74) == units
+    eng = a3mod.A3(m, W.make_weights_device(m, dev, units), M)
+    g = torch.Generator(device=dev)
+    g.manual_seed(M)
+    x = torch.randn(M, m.d_model, device=dev, generator=g).bfloat16()
+    both = eng.swiglu_rows(0, x)
+    again = eng.swiglu_rows(0, x)
+    eng.set_option(a3mod.OPT_GEMM_TILING, 1)
+    one = eng.swiglu_rows(0, x)
+    assert eng.device_status() == 0
+    assert torch.equal(both, one) and torch.equal(both, again)
+    w = eng._weights[0]
+    rows = torch.tensor([0, M // 2, 143, 144, M - 1], device=dev)
+    gate, up = (x[rows].double() @ w[name].double().T for name in ("w_gate", "w_up"))
+    want = torch.nn.functional.silu(gate) * up
+    # one bf16 rounding (2^-9 of the value) besides fp32 sums of d_model products, silu_mul's 2^-21 and its cancellation near zero
+    assert ((both[rows].double() - want).abs() <= 2 ** -8 * want.abs() + 1e-5 * want.abs().max()).all()
+    eng.close()
+
+
 # the widths at which a slice of the down projection takes two token tiles: five slices of Qwen-7B's to 352 rows, of 3 200 x 13 440 at 257
 QWEN_LAYER = replace(W.QWEN7B, n_layers=1)
 TWO_TILE_SLICES = W.ModelShape("two_tile_slices", 1, 3200, 16, 4, 128, 13440, 32000, 5e5, 1e-5)

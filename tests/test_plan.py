@@ -50,6 +50,14 @@ def test_down_projection_of_qwen(rows, down):
     assert (p["down_slices"], p["down_tiles"]) == down
 
 
+@pytest.mark.parametrize("d_model,d_ff,rows,tiles", [(4096, 14336, 256, 1), (4096, 14336, 257, 2), (4096, 14336, 288, 2), (4096, 14336, 289, 1),
+                                                     (4096, 14336, 320, 1), (3584, 18944, 270, 2), (3584, 18944, 304, 1), (3072, 8192, 272, 2),
+                                                     (2048, 16384, 257, 1), (2048, 16384, 320, 1), (2048, 8192, 272, 1), (1536, 8960, 272, 1)])
+def test_token_tiles_of_the_gate_and_up_product(d_model, d_ff, rows, tiles):
+    """Two on one stream of weights only where that was faster: from 257 to 288 rows, and not at the narrow widths."""
+    assert a3.plan_layer(replace(SHAPE, d_model=d_model, d_ff=d_ff, n_q_heads=d_model // 128), rows)["swiglu_tiles"] == tiles
+
+
 def test_bad_arguments():
     lib, desc, plan = a3._load(), a3.ModelDesc(1, 512, 4, 2, 128, 1408, 1e4, 1e-5, 0, 1), a3.LayerPlan()
     assert lib.a3_plan_layer(None, 148, 1, plan) == -1 and lib.a3_plan_layer(desc, 148, 1, None) == -1
