@@ -351,7 +351,7 @@ int a3_evict_layer(const a3_handle* h, const void* q_window, const int32_t* q_po
  * on ties).  x_row: dev [d_model] bf16, normally the last row of a3_fuse_request's x_out; final_norm: dev
  * [d_model] bf16; lm_head: dev [vocab][d_model] bf16, 16-byte aligned; logits_out: dev [vocab] fp32 or NULL;
  * token_out: dev int32.  ws: dev, 256-byte aligned, a3_first_token_workspace_bytes(h) bytes, borrowed for the
- * call.  One kernel launch (plus a 4-byte memset), no allocation, no synchronisation.  Non-finite logits set
+ * call.  Two kernel launches (one of them clears a counter), no allocation, no synchronisation.  Non-finite logits set
  * A3_DEV_NONFINITE_SCORE and never win. */
 size_t a3_first_token_workspace_bytes(const a3_handle* h);
 int a3_first_token(const a3_handle* h, const void* x_row, const void* final_norm, const void* lm_head, int vocab,

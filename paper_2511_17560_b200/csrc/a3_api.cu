@@ -638,18 +638,16 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     return check_rows(h, r->rows_out, M, n, st);
   };
 
-  // does position recovery from layer l on launch anything
-  auto recovers = [&](int l) { return l < m.n_layers && r->n_chunks > 0 && r->max_chunk_len > 0; };
-
   if (r->score_source == A3_SCORES_CACHED_KEYS) {
     // Scores against the recovered cached keys: every layer is position-recovered; only the question rows pass
     // through the leading blocks; rows [Re, Q] are recomputed through every layer from the embeddings.
-    A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, 0, m.n_layers, stream));
+    bool recovering;
+    A3_TRY(rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, 0, m.n_layers, st, &recovering));
     const int32_t* q_pos = w.all_pos;  // [nq]
     if (nq > 0) {
       bf16* xq = w.x_all;  // [nq][d] scratch for the question rows
       A3_TRY(enter_rows(h, (const bf16*)r->x0 + (size_t)r->n_ctx * m.d_model, nq, nullptr, nq, (const bf16*)h->layers[0].attn_norm, m.rms_eps,
-                        m.d_model, xq, lw.a, w.all_pos, r->n_ctx, st, recovers(0)));
+                        m.d_model, xq, lw.a, w.all_pos, r->n_ctx, st, recovering));
       for (int l = 0; l < ls; ++l)
         A3_TRY(recompute_layer_impl(h, l, xq, q_pos, nq, kl(l), vl(l), n, nullptr, lw, st, true, (const bf16*)h->layers[l + 1].attn_norm));
       A3_TRY(qkv_project(h, ls, lw.a, q_pos, nq, 0, lw.q, kl(ls), vl(ls), n, st));
@@ -669,9 +667,10 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
   // Position recovery (Eq. 2) in one launch.  Layers up to the selection layer are skipped: every row of their
   // caches is rewritten with true values below (full blocks; K/V of all rows at the selection layer), so the
   // recovered values would never be read.
+  bool recovering = false;
   if (!layer_ready && ls + 1 < m.n_layers)
-    A3_TRY(a3_rope_rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, ls + 1,
-                            m.n_layers, stream));
+    A3_TRY(rerotate(h, r->chunks, r->n_chunks, r->max_chunk_len, r->k_fused, r->v_fused, r->layer_stride, r->n_ctx, ls + 1, m.n_layers, st,
+                    &recovering));
   // leading full blocks: the whole input through layers 0..select_layer-1
   const int panels = x0_panels(r);
   const bool norm_panels = ls > 0 || panels == 1;
@@ -681,7 +680,7 @@ static int a3::fuse_impl(const a3_handle* h, const a3_request* r, void* ws, size
     if (x0_ready) A3_CUDA(cudaStreamWaitEvent(st, x0_ready[i], 0));
     A3_TRY(enter_rows(h, (const bf16*)r->x0 + (size_t)r0 * m.d_model, r1 - r0, nullptr, r1 - r0,
                       norm_panels ? (const bf16*)h->layers[0].attn_norm : nullptr, m.rms_eps, m.d_model, x, lw.a, w.all_pos + r0, r0, st,
-                      i == 0 && !layer_ready && recovers(ls + 1)));
+                      i == 0 && recovering));
     if (ls > 0) {
       // block 0 on this panel of rows: they attend to the rows before them, whose K/V the earlier panels have written
       if (i == 0) A3_TRY(feed_to(ls + 1 + FEED_AHEAD));  // a full block is long: several layers' copies fit under it

@@ -6,7 +6,8 @@
 // fp32 holding the bf16-rounded values a bf16 pipeline would store; a warp then walks four vocabulary rows at a
 // time with sixteen 16-byte streaming loads in flight per lane, reduces with shuffles, writes the fp32 logits and keeps
 // its best (value, lowest id).  The last CTA to finish (ticket counter) reduces the per-CTA candidates, so the
-// whole step is one launch and its result does not depend on the order in which CTAs finish.
+// step is this launch and a tiny one before it that clears the ticket, and its result does not depend on the order in which CTAs
+// finish.
 #include "a3_internal.cuh"
 
 namespace a3 {
@@ -182,7 +183,7 @@ extern "C" int a3_first_token(const a3_handle* h, const void* x_row, const void*
   if (grid > need) grid = need;
   {
     ProfScope prof(h, A3_K_FIRST_TOKEN, st);
-    clear_ticket_kernel<<<1, 1, 0, st>>>(ticket);
+    clear_ticket_kernel<<<1, 1, 0, st>>>(ticket);  // an ordinary launch: the projection, which writes beside it, relies on that
     A3_LAUNCHED();
     A3_CUDA(launch_pdl(first_token_kernel, dim3(grid), dim3(FT_THREADS), smem, st, (const bf16*)x_row, (const bf16*)final_norm, (const uint4*)lm_head,
                        d, vocab, h->m.rms_eps, logits_out, token_out, cand, ticket, h->dev_status));

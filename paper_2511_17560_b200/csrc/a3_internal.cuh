@@ -89,6 +89,11 @@ struct ProfScope {
 // the stream is still running; it must execute pdl_wait() before its first global-memory access (everything before
 // that - barrier and tensor-memory set-up, descriptor prefetch - overlaps the predecessor's tail) and it lets its own
 // successor do the same with pdl_launch_dependents().  Both instructions are no-ops under an ordinary launch.
+// Exceptions, which read and write before they wait (and wait before they end):
+//   * the pair GEMMs' first weights, which no launch writes;
+//   * first_token_kernel behind clear_ticket_kernel, and enter_rows_kernel with `beside` behind rerotate_kernel.  Those two
+//     predecessors start with an early trigger, touch nothing that the kernel beside them touches before its wait, and are ORDINARY
+//     launches: what was queued before them has ended.  They must not become programmatic ones, and nothing may be queued between.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -141,8 +146,12 @@ int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps,
 int add_slices_rmsnorm(const a3_handle* h, bf16* x, const float* part, int slices, const bf16* gain, float eps, int M, int d, bf16* out,
                        cudaStream_t st);
 
+// a3_rope_rerotate; `launched`: whether there was anything to launch.
+int rerotate(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len, void* k_fused, void* v_fused,
+             uint64_t layer_stride, int kv_len, int layer_begin, int layer_end, cudaStream_t st, bool* launched);
+
 // Rows entering a layer: x_dst[r] = src[rows ? rows[r] : r]; out[r] = rmsnorm of it * gain (gain null: no norm); pos_out[r] =
-// pos_base + r (null: no positions).  beside: directly behind a launch of a3_rope_rerotate, which need not have finished.
+// pos_base + r (null: no positions).  beside: directly behind a launch of rerotate, which need not have finished.
 int enter_rows(const a3_handle* h, const bf16* src, int n_src, const int32_t* rows, int M, const bf16* gain, float eps, int d, bf16* x_dst,
                bf16* out, int32_t* pos_out, int pos_base, cudaStream_t st, bool beside = false);
 

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(RR_THREADS)
 rerotate_kernel(const a3_chunk_ref* __restrict__ chunks, char* __restrict__ kf, char* __restrict__ vf,
                 unsigned long long layer_stride, int kv_len, int max_chunk_len, int layer_begin, int row_elems, int tok_per_cta,
                 const float2* __restrict__ tab, int max_pos, uint32_t* status) {
-  pdl_launch_dependents();  // see enter_rows_kernel
+  pdl_launch_dependents();  // see enter_rows_kernel, and rerotate for what this relies on
   const a3_chunk_ref ch = chunks[blockIdx.y];
   const int t0 = blockIdx.x * tok_per_cta;
   if (ch.len < 0 && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, A3_DEV_BAD_POSITION);
@@ -195,13 +195,9 @@ rerotate_kernel(const a3_chunk_ref* __restrict__ chunks, char* __restrict__ kf, 
   }
 }
 
-}  // namespace a3
-
-using namespace a3;
-
-extern "C" int a3_rope_rerotate(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len,
-                                void* k_fused, void* v_fused, uint64_t layer_stride, int kv_len, int layer_begin, int layer_end,
-                                a3_stream stream) {
+int rerotate(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len, void* k_fused, void* v_fused,
+             uint64_t layer_stride, int kv_len, int layer_begin, int layer_end, cudaStream_t st, bool* launched) {
+  *launched = false;
   if (!h || !chunks || !k_fused || !v_fused) return A3_EINVAL;
   if (n_chunks < 0 || max_chunk_len < 0 || kv_len < 0 || layer_begin < 0 || layer_end > h->m.n_layers || layer_begin > layer_end) return A3_EINVAL;
   if (((uintptr_t)k_fused & 15) || ((uintptr_t)v_fused & 15) || (layer_stride & 15)) return A3_EINVAL;
@@ -213,7 +209,8 @@ extern "C" int a3_rope_rerotate(const a3_handle* h, const a3_chunk_ref* chunks, 
   int tok = (int)((16 * 1024) / (row_elems * 2));
   if (tok < 1) tok = 1;
   dim3 grid(cdiv(max_chunk_len, tok), n_chunks, layer_end - layer_begin);
-  cudaStream_t st = (cudaStream_t)stream;
+  // Ordinary launches, not launch_pdl: they wait for everything queued before, and the kernel that runs beside them (enter_rows with
+  // `beside`), which writes buffers of the workspace that earlier launches read, relies on that.
 #define RR_LAUNCH(DD, LL)                                                                                             \
   rerotate_kernel<DD, LL><<<grid, RR_THREADS, 0, st>>>(chunks, (char*)k_fused, (char*)v_fused, layer_stride, kv_len,  \
                                                        max_chunk_len, layer_begin, row_elems, tok, h->rope_tab,      \
@@ -225,7 +222,19 @@ extern "C" int a3_rope_rerotate(const a3_handle* h, const a3_chunk_ref* chunks, 
   else RR_LAUNCH(64, 1);
 #undef RR_LAUNCH
   A3_LAUNCHED();
+  *launched = true;
   return A3_OK;
+}
+
+}  // namespace a3
+
+using namespace a3;
+
+extern "C" int a3_rope_rerotate(const a3_handle* h, const a3_chunk_ref* chunks, int n_chunks, int max_chunk_len,
+                                void* k_fused, void* v_fused, uint64_t layer_stride, int kv_len, int layer_begin, int layer_end,
+                                a3_stream stream) {
+  bool launched;
+  return rerotate(h, chunks, n_chunks, max_chunk_len, k_fused, v_fused, layer_stride, kv_len, layer_begin, layer_end, (cudaStream_t)stream, &launched);
 }
 
 // ------------------------------------------------------------------ value deviation (comparison selector)
@@ -418,8 +427,9 @@ int rmsnorm_rows(const a3_handle* h, const bf16* x, const bf16* gain, float eps,
 // Row r of a request on its way into a layer: x_dst[r] = src[rows ? rows[r] : r], out[r] = RMSNorm of it (gain given), and
 // pos_out[r] = pos_base + r.  What a copy, an index kernel, a gather and a norm would each launch for; a thread keeps its
 // vectors in registers between the two stores.  Rows out of range are flagged and skipped.
-// beside: the launch before this one is position recovery, whose results nothing here touches and which itself comes after everything
-// queued earlier.  The two run side by side, and this one ends after the other: the launches that follow wait for both through it.
+// beside: the launch directly before this one is position recovery, whose results nothing here touches and which itself comes after
+// everything queued earlier (rerotate).  The two run side by side, and this one ends after the other: the launches that follow wait for
+// both through it.
 __device__ __forceinline__ void enter_row(const uint4* src, int n_src, const int32_t* rows, const uint4* __restrict__ gain, float eps, int row_vecs,
                                           uint4* x_dst, uint4* out, int32_t* pos_out, int pos_base, uint32_t* status) {
   uint4 gv[RN_VPT];

@@ -20,3 +20,17 @@ def test_a_pair_that_gave_up_leaves_through_a_releasing_barrier():
     assert len(re.findall(r"gave_up = !sp_with_chunk<", kernel)) == 3 == len(re.findall(r"sp_with_chunk<", kernel))
     assert len(re.findall(r"if \(!ep_ok\[0\]\) return false;", kernel)) == 3
     assert re.search(r"if \(!ep_ok\[0\]\) \{\s*gave_up = true;\s*break;", kernel)
+
+
+def test_launches_that_others_run_beside_are_ordinary():
+    """rerotate_kernel and clear_ticket_kernel let their successors start early, which write before they wait: sound only because these
+    two waited for everything before them.  Only rerotate itself says whether there is such a launch to run beside."""
+    for name, kernel in (("a3_stream_kernels.cu", "rerotate_kernel"), ("a3_first_token.cu", "clear_ticket_kernel")):
+        text = source(name)
+        assert re.search(kernel + r"(<\w+, \w+>)?<<<", text)
+        assert not re.search(r"launch_pdl(_cluster)?\([^;]*" + kernel, text)
+    ticket = source("a3_first_token.cu").split("clear_ticket_kernel<<<")[1]
+    assert ticket.split("launch_pdl(")[0].count(";") == 2  # the launch and its check, nothing queued in between
+    for call in re.findall(r"enter_rows\([^;]*;", source("a3_api.cu")):
+        last = call.rsplit(",", 1)[1].strip(" \n);")
+        assert last in ("st", "recovering", "i == 0 && recovering"), last
