@@ -115,8 +115,8 @@ def test_narrow_windows(a3mod, n_cand, pool):
 
 @pytest.mark.parametrize("n_cand,pool", [(900, 1), (900, 3), (2000, 5), (4000, 3), (5121, 7), (8192, 7), (8192, 9), (9000, 3)])
 def test_votes_that_are_no_numbers(a3mod, n_cand, pool):
-    """Infinite votes win their windows, NaN votes are passed over where a window has others and win where it has not, and either is
-    flagged.  Alone, at the ends of the candidates and in a run as wide as a window."""
+    """Infinite votes win their windows, NaN votes are passed over where a window has others and come last where it has not, and either
+    is flagged.  Alone, at the ends of the candidates and in a run as wide as a window."""
     m, nq, n_system = W.TINY_GQA, 9, 5
     n_ctx, k, group = n_system + n_cand, n_cand // 5, m.n_q_heads // m.n_kv_heads
     eng, q, pos, K, (dq, dpos, lse, dK, dV) = evict_setup(a3mod, m, n_ctx, nq, n_cand * 3 + pool)
@@ -133,7 +133,7 @@ def test_votes_that_are_no_numbers(a3mod, n_cand, pool):
         v = np.full(n_ctx, np.nan)
         for i in range(n_system, n_ctx):
             v[i] = np.fmax.reduce(votes[h, max(n_system, i - pool // 2):min(n_ctx, i + pool // 2 + 1)])
-        rank = np.where(np.isnan(v), 2e30, np.where(np.isinf(v), 1e30, v))  # NaN before infinity before the rest
+        rank = np.where(np.isnan(v), -1.0, np.where(np.isinf(v), 1e30, v))  # infinity before the rest before NaN
         check_kept(kept[h].cpu().numpy(), rank, n_system, n_ctx, nq)
         assert torch.equal(k_out[:, h].view(torch.int16), dK[kept[h].long(), h].view(torch.int16))
     eng.close()
