@@ -267,8 +267,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   // gone (the last barrier orders no memory).
   const int n_acc = pair < p.n_units ? TT * ((p.n_units - pair + p.n_pairs - 1) / p.n_pairs) : 0;
   auto awaited = [&](int t) { return t + SLOTS < n_acc; };
-  // An epilogue that gave a wait up may have sent arrivals that the issuer, which then gave up as well, never took: see the last barrier.
-  bool gave_up = false;
+  // An epilogue that gives a wait up may have sent arrivals that the issuer, which has given up as well, never took.  (Every epilogue
+  // with such an arrival gives up: the accumulator that would have been computed in that slot, for which it waits, is never published.)
+  // Its fence and the last barrier order them before the leader goes.
+  auto give_up = [] { asm volatile("fence.acq_rel.cluster;" ::: "memory"); };
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs): own gate/up rows, own half of the token tile
     // as a whole warp, one elected lane issuing; a stage's k-blocks of an operand are one copy of a 3-D map ([k-block][row][64])
@@ -478,7 +480,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
       if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), b_ph, abort_flag, p.status) ? 1 : 0;
       named_bar_sync(1, 256);
       if (!ep_ok[0]) {  // uniform for the 256 threads
-        gave_up = true;
+        give_up();
         break;
       }
       tc_fence_after();
@@ -513,7 +515,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int st = quarter * 32 + lane;  // thread within the set
     const int set_n = p.tok_n >> 1;      // token columns of a set (multiple of 8)
     const int bar_set = 2 + set;
-    gave_up = !sp_with_chunk<true>(p.chunk, [&](auto chunk) {
+    sp_with_chunk<true>(p.chunk, [&](auto chunk) {
       constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4, PASSES = (CH + 15) / 16;
       const int n_chunks = (set_n + CH - 1) / CH;
       float* xset = xch + set * sp_set_floats(CH);
@@ -532,7 +534,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         bf16* out = p.C + (size_t)max(t0, 0) * p.ldc + fb * (2 * SP_FEAT) + (int)rank * SP_FEAT + fg * 8;
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), b_ph, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
-        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        if (!ep_ok[0]) {  // uniform for the 256 threads
+          give_up();
+          return false;
+        }
         tc_fence_after();
         const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
@@ -591,7 +596,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int st = quarter * 32 + lane;  // thread within the set
     const int set_n = p.tok_n >> 1;
     const int bar_set = 2 + set;
-    gave_up = !sp_with_chunk<false>(p.chunk, [&](auto chunk) {
+    sp_with_chunk<false>(p.chunk, [&](auto chunk) {
       constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4, PASSES = CH / 16;
       const int n_chunks = (set_n + CH - 1) / CH;
       float* xset = xch + set * sp_set_floats(CH);
@@ -645,7 +650,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         fetch(0);
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
-        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        if (!ep_ok[0]) {  // uniform for the 256 threads
+          give_up();
+          return false;
+        }
         tc_fence_after();
         const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
         // KC > 1: [token of the set][128 features] fp32 sums of the other pair, over the ring, whose stages have all been read
@@ -761,7 +769,7 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int bar_set = 2 + set;
     // phase 2 assignment: tokens e2, e2 + 8, .. of a chunk, features 8 (st & 15) .. + 7
     const int e2 = st >> 4, fg = st & 15;
-    gave_up = !sp_with_chunk<true>(p.chunk, [&](auto chunk) {
+    sp_with_chunk<true>(p.chunk, [&](auto chunk) {
       constexpr int CH = decltype(chunk)::value, QUARTER = CH * 32 + 4;
       const int n_chunks = (set_n + CH - 1) / CH;
       float* xset = xch + set * sp_set_floats(CH);
@@ -783,7 +791,10 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
           old[i] = i * 8 + e2 < valid ? __ldcg(reinterpret_cast<const uint4*>(crow + (size_t)(i * 8 + e2) * p.ldc)) : make_uint4(0, 0, 0, 0);
         if (ep_tid == 0) ep_ok[0] = mbar_wait(tmem_full(b), (it >> 1) & 1, abort_flag, p.status) ? 1 : 0;
         named_bar_sync(1, 256);
-        if (!ep_ok[0]) return false;  // uniform for the 256 threads
+        if (!ep_ok[0]) {  // uniform for the 256 threads
+          give_up();
+          return false;
+        }
         tc_fence_after();
         const uint32_t trow = tmem_base + (uint32_t)(b * p.slot_cols) + (uint32_t)(set * set_n) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll
@@ -825,11 +836,8 @@ pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
   // Neither CTA releases tensor or shared memory while the other may still use it.  Ordering execution is enough: the stores above
   // are for the kernels that follow, and a barrier that releases them first waited 700-900 clocks for their way to L2 in
   // every launch.  Request of 369 tokens on a small model 153.2 -> 146.1 us, prefill of 75 tokens (Qwen-7B) 2 924 -> 2 873, request
-  // of three passages (Llama-8B) 4 277 -> 4 219.  Not so for an epilogue that gave up: its arrivals for accumulators that the issuer did
-  // not take again are ordered before the leader goes.  (Every epilogue with such an arrival gives up: the accumulator that would
-  // have been computed in that slot, for which it waits, is never published.)
-  if (__any_sync(0xffffffffu, gave_up)) cluster_sync_all();
-  else cluster_sync_relaxed();
+  // of three passages (Llama-8B) 4 277 -> 4 219.  Arrivals at the leader that it does not wait for are ordered where they are given up.
+  cluster_sync_relaxed();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
 }
 

@@ -187,10 +187,10 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// the same without ordering memory: nobody waits for his global stores here
+// the same without ordering memory, except what a fence.acq_rel.cluster before it orders: nobody waits for his global stores here
 __device__ __forceinline__ void cluster_sync_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // this CTA's own copy into its own shared memory; the bytes are counted on the barrier at `bar` (a shared::cluster
 // address, here always the leader's)

@@ -10,16 +10,16 @@ def source(name):
     return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
 
 
-def test_a_pair_that_gave_up_leaves_through_a_releasing_barrier():
+def test_a_pair_that_gave_up_orders_its_arrivals():
     """The pair GEMMs' last cluster barrier orders no memory, which is sound only while every arrival sent to the leader is one it
-    waits for.  All four epilogues report a wait that gave up, and these warps take the barrier that does order."""
+    waits for.  All four epilogues fence where they give a wait up, and the barrier acquires."""
     kernel = source("a3_gemm_persistent.cu").split("pair_t_kernel(", 1)[1].split("bool swiglu_pair_usable", 1)[0]
-    last = [line.strip() for line in kernel.splitlines() if "cluster_sync_" in line][-2:]
-    assert last == ["if (__any_sync(0xffffffffu, gave_up)) cluster_sync_all();", "else cluster_sync_relaxed();"]
-    assert kernel.count("cluster_sync_relaxed") == 1
-    assert len(re.findall(r"gave_up = !sp_with_chunk<", kernel)) == 3 == len(re.findall(r"sp_with_chunk<", kernel))
-    assert len(re.findall(r"if \(!ep_ok\[0\]\) return false;", kernel)) == 3
-    assert re.search(r"if \(!ep_ok\[0\]\) \{\s*gave_up = true;\s*break;", kernel)
+    assert re.search(r"give_up = \[\] \{ asm volatile\(\"fence.acq_rel.cluster;\"", kernel)
+    left = re.findall(r"if \(!ep_ok\[0\]\) \{\s*(.*?)\s*\}", kernel, flags=re.S)
+    assert len(left) == 4 == len(re.findall(r"ep_ok\[0\] = mbar_wait", kernel))
+    assert all(re.match(r"give_up\(\);\s*(break|return false);", body) for body in left)
+    barrier = source("a3_tc.cuh").split("cluster_sync_relaxed()", 1)[1].split("}", 1)[0]
+    assert "arrive.relaxed" in barrier and "wait.acquire" in barrier
 
 
 def test_launches_that_others_run_beside_are_ordinary():
