@@ -95,7 +95,7 @@ __device__ __forceinline__ void sp_ld_chunk(uint32_t taddr, int w, float* v) {
 }
 // 32 bytes (aligned to 32) through the read-only path.  The lanes of a token read its table row 64 bytes apart, so that a load costs
 // its lines and not its bytes: half as many loads.  A chunk's fetch took 800 of its 1 450 clocks; request of 369 tokens on a small
-// model 144.1 -> 142.8 us, prefill of 512 tokens (Llama-8B) 7 614 -> 7 595.
+// model 144.1 -> 142.8 us (a prefill of 512 tokens at Llama-8B width does not show it: 0.25 % where two runs differ by 0.8).
 __device__ __forceinline__ void ldg32(const float4* p, float4& a, float4& b) {
   asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
@@ -870,7 +870,8 @@ static int unit_group(int M, int K) { return (long long)M * K * 2 > (64ll << 20)
 
 // Two token tiles of n per unit on one stream of weights.  Just over 256 rows every weight goes to two units, and units that narrow
 // wait for their operands: 270 rows x 2 x (16 KiB of weights + 9 KiB of tokens) per k-block and CTA, 800 clocks for 576 of tensor time.
-// Together they take 16 + 18 KiB, 544 clocks, and each weight crosses to an SM once: SwiGLU of 270 rows (Qwen width) 67 -> 57 us, down projection 42 -> 31.5.
+// Together they take 16 + 18 KiB, 576 clocks of tensor time, and each weight crosses to an SM once: inside a request of 270 rows (Qwen
+// width) SwiGLU 67 -> 57 us, down projection 42 -> 31.5; SwiGLU alone 65.4 -> 62.7.
 constexpr int SP_TWO_TILES_COLS = 160;  // columns from one accumulator to the next: three in 512
 constexpr int SP_TWO_TILES_MAX = 144;   // tokens per tile of SwiGLU, see two_tiles
 static int two_tiles_per_kb(int n) { return 4 * n > 256 + 2 * n ? 4 * n : 256 + 2 * n; }

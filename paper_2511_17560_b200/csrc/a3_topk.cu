@@ -66,7 +66,9 @@ __device__ __forceinline__ void topk_bin(unsigned int (*whist)[256], unsigned in
 // scan over threads and let neighbouring windows share their middle.  With four passes always, a window per key and a count per warp
 // and round, the selection of 5 120 candidates at width 7 took 14 700 clocks: 1 050 for the loads, 2 600 the windows, 7 700 the
 // passes, 2 650 the emission.  Back to back, before and now (us): 300 candidates 4.2 / 2.7, 900 4.1 / 2.6, 2 000 5.6 / 3.7, 3 000 5.8 / 4.7,
-// 5 120 7.2 / 5.7, 8 192 9.2 / 8.3.
+// 5 120 7.2 / 5.7, 8 192 9.2 / 8.3.  Windows, one layer's eviction of 8 192 slots, each slot's read by itself against neighbours in
+// registers: width 3 17.5 / 15.9, width 7 19.3 / 16.3 (two heads); of 300 slots at width 853, walked whole against to the last candidate, 34.7 /
+// 10.9.
 constexpr int TK_LIST = 128;  // eight threads rank one key
 template <int KPT>
 __host__ __device__ constexpr int topk_at(int i) {  // place of slot i in shared memory: a thread's slots on banks of their own
@@ -338,7 +340,8 @@ static int launch_topk(const a3_handle* h, const float* scores, size_t score_str
                       in_smem, half_pool, tail_begin, tail);
   };
   // Time grows with the keys per thread (back to back 900 candidates 2.6 us, 3 000 4.7, 5 120 5.7, 8 192 8.3), hence instances of one,
-  // three, five and eight: the smallest that holds the candidates.
+  // three, five and eight: the smallest that holds the candidates.  Those in between would save 0.4 us (2 000 candidates 4.4 / 4.0, 4 000
+  // 5.9 / 5.6), 1.0 (6 000 8.1 / 7.1) and 0.6 (7 000 8.2 / 7.7) and are left out.
   if (n <= TK_THREADS) {
     A3_CUDA(go(topk_select_kernel<1>, half_pool > 0 ? (size_t)n * 4 : 0));
   } else if (n <= 3 * TK_THREADS) {
@@ -380,11 +383,15 @@ int a3::topk_rows(const a3_handle* h, const float* scores, int cand_begin, int c
   return launch_topk(h, scores, 0, 1, cand_begin, cand_end - cand_begin, k, 0, tail_begin, tail, idx_out, 0, st);
 }
 
-// Pooling inside the selection saves a launch (2.5 us) and costs every thread its window in shared-memory reads, in the one CTA of a
-// head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, on either side of the line (us): 5 120
-// candidates 16.9 at width 7 and 18.0 at 45 inside, 19.3 at 63 and 20.1 at 129 apart; 2 000 candidates 12.1 at 7, 15.1 at 63 and 16.1
-// at 127 inside, 19.2 at 255 apart; 8 192 candidates 21.4 at 21 and 22.4 at 31 inside, 23.0 at 63 apart.  Candidates that do not fit
-// the registers would read their window from global memory, which loses at every width (32 768 79.1 / 70.9 at 7, 215 / 82 at 255).
+// Pooling inside the selection saves a launch (2.5 us) and costs every thread its windows in shared-memory reads, in the one CTA of a
+// head where the kernel of its own has the whole chip.  One layer's eviction, votes to gather, inside / apart (us; Llama-8B heads, two
+// heads).  On this side of the line: 300 candidates at width 255 11.7 / 13.8 and 10.7 / 12.7, 900 at 283 14.6 / 16.7 and 13.4 / 14.4, 1 024
+// at 249 14.3 / 15.2 and 13.3 / 13.9, 2 000 at 127 15.1 / 17.0 and 12.6 / 13.8, 5 120 at 7 16.2 / 17.5 and 12.7 / 14.0, at 49 17.2 / 18.1 and
+// 13.6 / 14.7, 8 192 at 7 20.6 / 21.9 and 15.9 / 17.5, at 31 22.0 / 22.9 and 16.7 / 17.6.  Beyond it inside has become the faster side too
+// since windows share their middle: 1 024 at 251 14.3 / 15.2 and 13.4 / 14.0, 2 000 at 191 14.1 / 16.4 and 13.1 / 14.2, 5 120 at 129 18.3 / 19.3
+// and 15.0 / 15.9, 8 192 at 63 23.1 / 23.7 and 18.5 / 19.2; the line stays where it was drawn against a window per key, and where
+// tests/test_gpu_evict.py counts launches on either side.  Candidates that do not fit the registers would read their window from global
+// memory, which loses at every width (32 768 79.1 / 70.9 at 7, 215 / 82 at 255).
 bool a3::topk_can_pool(int n_cand, int pool) { return n_cand <= 8 * TK_THREADS && (long long)n_cand * pool <= 250 * TK_THREADS; }
 
 int a3::topk_batched(const a3_handle* h, const float* scores, size_t score_stride, int batches, int cand_begin, int cand_end,

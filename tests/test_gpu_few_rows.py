@@ -79,15 +79,16 @@ def test_layer_of_a_stack_beyond_l2(a3mod, M):
     layer_parity(a3mod, BEYOND_L2, M, seed=M + 2)
 
 
-# one layer that L2 holds; 38 feature blocks of SwiGLU, 8 of the down projection (38 ring stages, slices of 4 or 5)
+# one layer that L2 holds; 38 feature blocks of SwiGLU, 8 of the down projection (38 ring stages in four slices)
 TWO_TILES = W.ModelShape("two_tiles", 1, 2048, 16, 4, 128, 4864, 32000, 5e5, 1e-5)
 
 
 @pytest.mark.parametrize("m", [BEYOND_L2, TWO_TILES], ids=lambda m: m.name)
 @pytest.mark.parametrize("M", [257, 289, 320, 321, 471])
 def test_two_token_tiles_on_one_stream_of_weights(a3mod, m, M):
-    """Just over 256 rows, up to 320 for SwiGLU and to 512 for the slices: the oracle's layer, and the gate/up product, whose sums
-    stay whole, bit for bit that of one tile per unit."""
+    """Row counts around those at which units take two token tiles, on widths that keep one tile per unit (the widths that take two:
+    test_accumulators_of_two_token_tiles_take_turns, test_slices_of_two_token_tiles): the oracle's layer, and the gate/up product bit
+    for bit whatever the tiling."""
     layer_parity(a3mod, m, M, seed=M + 4)
     eng, _, dev = make_engine(a3mod, m, seed=M, w_std=0.05)
     g = torch.Generator(device=dev)
